@@ -3,7 +3,7 @@
 // Rather than scattering element matrices with atomics, each (node, neighbour)
 // block is gathered from the (1, 2, 4 or 8) elements that contain both nodes:
 // every block is written once, in order, with no atomics, so assembly is
-// deterministic.  The element stiffness is integrated with 2x2x2 Gauss points.
+// deterministic.  The element integrals are in closed form (fem.cuh).
 #include "fem.cuh"
 #include "kernels.cuh"
 
@@ -27,9 +27,7 @@ __global__ void k_element_C(int nel, int n_mat, const double *__restrict__ C0,
     atomicCAS(&st->code, 0, GENEO_ERR_INVALID_ARG);
     m = 0;
   }
-  double C[36];
-  for (int i = 0; i < 36; ++i) C[i] = C0[36 * m + i];
-  rotate_voigt(C, th[e], ph ? ph[e] : 0.0, Cel + 36 * (size_t)e);
+  rotate_voigt(C0 + 36 * m, th[e], ph ? ph[e] : 0.0, Cel + 36 * (size_t)e);
 }
 
 __device__ __forceinline__ void node_ijk(int n, int nnx, int nny, int &i, int &j, int &k) {
@@ -39,94 +37,133 @@ __device__ __forceinline__ void node_ijk(int n, int nnx, int nny, int &i, int &j
   k = r / nny;
 }
 
-__device__ __forceinline__ bool slot_valid(int s, int i, int j, int k, int nnx, int nny, int nnz) {
-  int di = s % 3 - 1, dj = (s / 3) % 3 - 1, dk = s / 9 - 1;
-  return (unsigned)(i + di) < (unsigned)nnx && (unsigned)(j + dj) < (unsigned)nny &&
-         (unsigned)(k + dk) < (unsigned)nnz;
+// Blocks in the rows of the nodes before i on an axis of n nodes (n >= 2): a
+// node couples to three positions, an end node to two.  The row pointer of the
+// tensor-product pattern is a product of these, so it needs no scan (the
+// single-block scan that stood here took 0.53 ms of a 23.3 ms assembly with
+// 0.41 M nodes, 1.49 ms with 1.16 M).
+__device__ __forceinline__ int axis_rows_before(int i, int n) { return 3 * i - (i > 0) - (i == n); }
+__device__ __forceinline__ int axis_row(int i, int n) { return 3 - (i == 0) - (i == n - 1); }
+__device__ __forceinline__ int row_start(int i, int j, int k, int nnx, int nny, int nnz) {
+  const int tx = 3 * nnx - 2, ty = 3 * nny - 2, cy = axis_row(j, nny), cz = axis_row(k, nnz);
+  return tx * (ty * axis_rows_before(k, nnz) + cz * axis_rows_before(j, nny)) +
+         cz * cy * axis_rows_before(i, nnx);
 }
 
-__global__ void k_bsr_count(int nnx, int nny, int nnz, int32_t *__restrict__ cnt) {
-  int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= nnx * nny * nnz) return;
-  int i, j, k;
-  node_ijk(n, nnx, nny, i, j, k);
-  int cx = 1 + (i > 0) + (i < nnx - 1);
-  int cy = 1 + (j > 0) + (j < nny - 1);
-  int cz = 1 + (k > 0) + (k < nnz - 1);
-  cnt[n] = cx * cy * cz;
-}
+// Rows of the matrix, assembled with the Dirichlet set eliminated: one block
+// per kRowNodes consecutive nodes.  The sums over the elements are formed in
+// registers -- elasticity: lane = node, one warp per component pair (i, k);
+// Darcy: thread = node -- and staged in shared memory, from where the rows
+// (contiguous in `val`) are written coalesced, with the Dirichlet rows and
+// columns replaced by the identity and the lifting
+//   lift_i = -sum_{c in D} A_ic g_c on free rows, g_i on Dirichlet rows
+// formed on the way (kept so that a new load needs no eliminated columns).
+// FP64 issue bounds it: about 3,500 FP64 operations per node for elasticity,
+// 450 for Darcy.
+template <int NC>
+constexpr int kRowNodes = NC == 3 ? 32 : 128;
+template <int NC>
+constexpr int kRowThreads = NC == 3 ? 192 : 128;
+template <int NC>
+constexpr int kRowSmem = kRowNodes<NC> * 27 * (NC * NC * 8 + 4 + 1);
 
-// Exclusive scan of cnt[0..n) into out[0..n], one block (setup only).
-__global__ void k_scan_single(int n, const int32_t *__restrict__ cnt, int32_t *__restrict__ out) {
-  __shared__ int32_t sh[1024];
-  __shared__ int32_t carry;
-  if (threadIdx.x == 0) carry = 0;
-  __syncthreads();
-  for (int base = 0; base < n; base += 1024) {
-    int idx = base + threadIdx.x;
-    int v = idx < n ? cnt[idx] : 0;
-    sh[threadIdx.x] = v;
-    __syncthreads();
-    for (int o = 1; o < 1024; o <<= 1) {
-      int t = threadIdx.x >= o ? sh[threadIdx.x - o] : 0;
-      __syncthreads();
-      sh[threadIdx.x] += t;
-      __syncthreads();
-    }
-    if (idx < n) out[idx] = carry + sh[threadIdx.x] - v;
-    __syncthreads();
-    if (threadIdx.x == 1023) carry += sh[1023];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) out[n] = carry;
-}
-
-__global__ void k_bsr_fill(int nnx, int nny, int nnz, const int32_t *__restrict__ row_ptr,
-                           int32_t *__restrict__ col) {
-  int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= nnx * nny * nnz) return;
-  int i, j, k;
-  node_ijk(n, nnx, nny, i, j, k);
-  int pos = row_ptr[n];
-  for (int s = 0; s < 27; ++s) {
-    if (!slot_valid(s, i, j, k, nnx, nny, nnz)) continue;
-    int di = s % 3 - 1, dj = (s / 3) % 3 - 1, dk = s / 9 - 1;
-    col[pos++] = (i + di) + nnx * ((j + dj) + nny * (k + dk));
-  }
-}
-
-// One thread per (node, neighbour slot): sum the element blocks of the
-// elements shared by the two nodes.
-__global__ void k_assemble_values(int nx, int ny, int nz, const double *__restrict__ X,
-                                  const double *__restrict__ Y, const double *__restrict__ Z,
-                                  const double *__restrict__ Cel,
-                                  const int32_t *__restrict__ row_ptr,
-                                  double *__restrict__ val) {
-  int nnx = nx + 1, nny = ny + 1, nnz = nz + 1;
-  long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (long long)nnx * nny * nnz * 27) return;
-  int n = (int)(t / 27), s = (int)(t % 27);
-  int i, j, k;
-  node_ijk(n, nnx, nny, i, j, k);
-  if (!slot_valid(s, i, j, k, nnx, nny, nnz)) return;
-  int pos = row_ptr[n];
-  for (int q = 0; q < s; ++q) pos += slot_valid(q, i, j, k, nnx, nny, nnz);
-  int i2 = i + s % 3 - 1, j2 = j + (s / 3) % 3 - 1, k2 = k + s / 9 - 1;
-  double acc[9];
-  for (int q = 0; q < 9; ++q) acc[q] = 0.0;
-  for (int ez = max(max(k, k2) - 1, 0); ez <= min(min(k, k2), nz - 1); ++ez)
-    for (int ey = max(max(j, j2) - 1, 0); ey <= min(min(j, j2), ny - 1); ++ey)
-      for (int ex = max(max(i, i2) - 1, 0); ex <= min(min(i, i2), nx - 1); ++ex) {
-        int e = ex + nx * (ey + ny * ez);
-        int a = (i - ex) + 2 * (j - ey) + 4 * (k - ez);
-        int b = (i2 - ex) + 2 * (j2 - ey) + 4 * (k2 - ez);
-        double Kb[9];
-        element_block(Cel + 36 * (size_t)e, X[ex + 1] - X[ex], Y[ey + 1] - Y[ey],
-                      Z[ez + 1] - Z[ez], a, b, Kb);
-        for (int q = 0; q < 9; ++q) acc[q] += Kb[q];
+template <int NC>
+__global__ void __launch_bounds__(kRowThreads<NC>)
+    k_assemble_rows(int nx, int ny, int nz, const double *__restrict__ X,
+                    const double *__restrict__ Y, const double *__restrict__ Z,
+                    const double *__restrict__ coef, const uint8_t *__restrict__ mask,
+                    const double *__restrict__ g, double *__restrict__ lift,
+                    int32_t *__restrict__ row_ptr, int32_t *__restrict__ col,
+                    double *__restrict__ val) {
+  constexpr int N = kRowNodes<NC>, NC2 = NC * NC;
+  extern __shared__ __align__(16) double sv[];               // [N][27][NC2]
+  int *pos = reinterpret_cast<int *>(sv + N * 27 * NC2);     // [N][27] block index in val, or -1
+  uint8_t *mk = reinterpret_cast<uint8_t *>(pos + N * 27);   // [N][27] Dirichlet bits of the column node
+  const int nnx = nx + 1, nny = ny + 1, nnz = nz + 1, nnode = nnx * nny * nnz;
+  const int n0 = blockIdx.x * N, tid = threadIdx.x;
+  for (int e = tid; e < N * 27; e += kRowThreads<NC>) {
+    const int t = e / 27, s = e - 27 * t, n = n0 + t;
+    int p = -1;
+    uint8_t m = 0;
+    if (n < nnode) {
+      int i, j, k;
+      node_ijk(n, nnx, nny, i, j, k);
+      const int i2 = i + s % 3 - 1, j2 = j + (s / 3) % 3 - 1, k2 = k + s / 9 - 1;
+      const int first = row_start(i, j, k, nnx, nny, nnz);
+      if (s == 0) row_ptr[n] = first;
+      if (s == 0 && n == nnode - 1)
+        row_ptr[nnode] = first + axis_row(i, nnx) * axis_row(j, nny) * axis_row(k, nnz);
+      if ((unsigned)i2 < (unsigned)nnx && (unsigned)j2 < (unsigned)nny && (unsigned)k2 < (unsigned)nnz) {
+        const int dx = s % 3 - (i == 0), dy = (s / 3) % 3 - (j == 0), dz = s / 9 - (k == 0);
+        p = first + dx + axis_row(i, nnx) * (dy + axis_row(j, nny) * dz);
+        const int cn = i2 + nnx * (j2 + nny * k2);
+        col[p] = cn;
+        for (int c = 0; c < NC; ++c) m |= (uint8_t)((mask[NC * cn + c] != 0) << c);
       }
-  double *out = val + 9 * (size_t)pos;
-  for (int q = 0; q < 9; ++q) out[q] = acc[q];
+    }
+    pos[e] = p;
+    mk[e] = m;
+  }
+  const int t = NC == 3 ? (tid & 31) : tid, n = n0 + t;
+  if (n < nnode) {
+    int i, j, k;
+    node_ijk(n, nnx, nny, i, j, k);
+    const NodeAxis ax = node_axis(X, i, 0, nx), ay = node_axis(Y, j, 0, ny), az = node_axis(Z, k, 0, nz);
+    auto all = [](int, int, int) { return true; };
+    double acc[27];
+#pragma unroll
+    for (int s = 0; s < 27; ++s) acc[s] = 0.0;
+    double *out = sv + t * 27 * NC2;
+    if constexpr (NC == 3) {
+      int ci, ck, off[9];
+      component_pair(tid >> 5, ci, ck, off);
+      double acct[27];
+      if (ci != ck) {
+#pragma unroll
+        for (int s = 0; s < 27; ++s) acct[s] = 0.0;
+        elastic_rows<true>(coef, off, ax, ay, az, i, j, k, nx, ny, all, acc, acct);
+#pragma unroll
+        for (int s = 0; s < 27; ++s) {
+          out[9 * s + 3 * ci + ck] = acc[s];
+          out[9 * s + 3 * ck + ci] = acct[s];
+        }
+      } else {
+        elastic_rows<false>(coef, off, ax, ay, az, i, j, k, nx, ny, all, acc, acct);
+#pragma unroll
+        for (int s = 0; s < 27; ++s) out[9 * s + 4 * ci] = acc[s];
+      }
+    } else {
+      darcy_rows(coef, ax, ay, az, i, j, k, nx, ny, all, acc);
+#pragma unroll
+      for (int s = 0; s < 27; ++s) out[s] = acc[s];
+    }
+  }
+  __syncthreads();
+  if (lift)
+    for (int e = tid; e < N * NC; e += kRowThreads<NC>) {
+      const int t2 = e / NC, r = e - NC * t2, m = n0 + t2;
+      if (m >= nnode) break;
+      if (mk[27 * t2 + 13] >> r & 1) {
+        lift[NC * m + r] = g[NC * m + r];
+        continue;
+      }
+      double sum = 0.0;
+      for (int s = 0; s < 27; ++s) {
+        const int b = mk[27 * t2 + s];
+        if (!b) continue;
+        const int cn = m + s % 3 - 1 + nnx * ((s / 3) % 3 - 1 + nny * (s / 9 - 1));
+        for (int c = 0; c < NC; ++c)
+          if (b >> c & 1) sum += sv[(27 * t2 + s) * NC2 + NC * r + c] * g[NC * cn + c];
+      }
+      lift[NC * m + r] = -sum;
+    }
+  for (int e = tid; e < N * 27 * NC2; e += kRowThreads<NC>) {
+    const int b = e / NC2, q = e - NC2 * b, p = pos[b];
+    if (p < 0) continue;
+    const int t2 = b / 27, r = q / NC, c = q - NC * r;
+    const bool drop = (mk[27 * t2 + 13] >> r & 1) || (mk[b] >> c & 1);
+    val[(size_t)NC2 * p + q] = drop ? ((b - 27 * t2 == 13 && r == c) ? 1.0 : 0.0) : sv[e];
+  }
 }
 
 // Consistent nodal load of the traction (0, 0, -q) on the face z = z_max
@@ -163,88 +200,12 @@ __global__ void k_dirichlet_mark(int nd, const int32_t *__restrict__ dofs,
   g[d] = vals ? vals[t] : 0.0;
 }
 
-// Lifting of the Dirichlet data (Sec. 2, u = g on the clamped face):
-// lift_i = -sum_{c in D} A_ic g_c on free rows, lift_i = g_i on Dirichlet rows.
-// It is kept so that a new load reuses it without the eliminated columns.
-__global__ void k_dirichlet_lift(int nnode, int nc, const int32_t *__restrict__ row_ptr,
-                                 const int32_t *__restrict__ col, const double *__restrict__ val,
-                                 const uint8_t *__restrict__ mask, const double *__restrict__ g,
-                                 double *__restrict__ lift) {
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= nc * nnode) return;
-  int n = t / nc, r = t % nc;
-  if (mask[t]) {
-    lift[t] = g[t];
-    return;
-  }
-  double s = 0.0;
-  for (int p = row_ptr[n]; p < row_ptr[n + 1]; ++p) {
-    int cn = col[p];
-    for (int c = 0; c < nc; ++c)
-      if (mask[nc * cn + c]) s += val[(size_t)nc * nc * p + nc * r + c] * g[nc * cn + c];
-  }
-  lift[t] = -s;
-}
-
 // b_i = f_i + lift_i on free rows, b_i = g_i on Dirichlet rows.
 __global__ void k_apply_lift(int n3, const uint8_t *__restrict__ mask,
                              const double *__restrict__ lift, double *__restrict__ b) {
   int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n3) return;
   b[t] = mask[t] ? lift[t] : b[t] + lift[t];
-}
-
-// Zero Dirichlet rows and columns, unit diagonal (nc unknowns per node).
-__global__ void k_dirichlet_eliminate(int nnode, int nc, const int32_t *__restrict__ row_ptr,
-                                      const int32_t *__restrict__ col,
-                                      const uint8_t *__restrict__ mask,
-                                      double *__restrict__ val) {
-  int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= nnode) return;
-  bool anyrow = false;
-  for (int r = 0; r < nc; ++r) anyrow |= mask[nc * n + r] != 0;
-  for (int p = row_ptr[n]; p < row_ptr[n + 1]; ++p) {
-    int cn = col[p];
-    bool anycol = false;
-    for (int c = 0; c < nc; ++c) anycol |= mask[nc * cn + c] != 0;
-    if (!anyrow && !anycol) continue;
-    for (int r = 0; r < nc; ++r)
-      for (int c = 0; c < nc; ++c)
-        if (mask[nc * n + r] || mask[nc * cn + c])
-          val[(size_t)nc * nc * p + nc * r + c] = (cn == n && r == c) ? 1.0 : 0.0;
-  }
-}
-
-// ---- scalar Darcy problem (eqn:Darcy, eq-fe-darcy): one unknown per node ----
-
-// One thread per (node, neighbour slot), gathered from the shared elements.
-__global__ void k_assemble_values_darcy(int nx, int ny, int nz, const double *__restrict__ X,
-                                        const double *__restrict__ Y,
-                                        const double *__restrict__ Z,
-                                        const double *__restrict__ perm,
-                                        const int32_t *__restrict__ row_ptr,
-                                        double *__restrict__ val) {
-  int nnx = nx + 1, nny = ny + 1, nnz = nz + 1;
-  long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (long long)nnx * nny * nnz * 27) return;
-  int n = (int)(t / 27), s = (int)(t % 27);
-  int i, j, k;
-  node_ijk(n, nnx, nny, i, j, k);
-  if (!slot_valid(s, i, j, k, nnx, nny, nnz)) return;
-  int pos = row_ptr[n];
-  for (int q = 0; q < s; ++q) pos += slot_valid(q, i, j, k, nnx, nny, nnz);
-  int i2 = i + s % 3 - 1, j2 = j + (s / 3) % 3 - 1, k2 = k + s / 9 - 1;
-  double acc = 0.0;
-  for (int ez = max(max(k, k2) - 1, 0); ez <= min(min(k, k2), nz - 1); ++ez)
-    for (int ey = max(max(j, j2) - 1, 0); ey <= min(min(j, j2), ny - 1); ++ey)
-      for (int ex = max(max(i, i2) - 1, 0); ex <= min(min(i, i2), nx - 1); ++ex) {
-        int e = ex + nx * (ey + ny * ez);
-        int a = (i - ex) + 2 * (j - ey) + 4 * (k - ez);
-        int b = (i2 - ex) + 2 * (j2 - ey) + 4 * (k2 - ez);
-        acc += darcy_entry(perm + 3 * (size_t)e, X[ex + 1] - X[ex], Y[ey + 1] - Y[ey],
-                           Z[ez + 1] - Z[ez], a, b);
-      }
-  val[pos] = acc;
 }
 
 // b_n = int f N_n dx = sum over the elements of node n of f V_e / 8, plus nodal.
@@ -256,45 +217,42 @@ __global__ void k_load_darcy(int nx, int ny, int nz, const double *__restrict__ 
   if (n >= nnx * nny * (nz + 1)) return;
   int i, j, k;
   node_ijk(n, nnx, nny, i, j, k);
-  double v = 0.0;
-  if (f != 0.0)
-    for (int ez = max(k - 1, 0); ez <= min(k, nz - 1); ++ez)
-      for (int ey = max(j - 1, 0); ey <= min(j, ny - 1); ++ey)
-        for (int ex = max(i - 1, 0); ex <= min(i, nx - 1); ++ex)
-          v += f * (X[ex + 1] - X[ex]) * (Y[ey + 1] - Y[ey]) * (Z[ez + 1] - Z[ez]) * 0.125;
+  // the element volumes around a node sum to a product of the axis widths
+  const double wx = X[min(i + 1, nx)] - X[max(i - 1, 0)], wy = Y[min(j + 1, ny)] - Y[max(j - 1, 0)],
+               wz = Z[min(k + 1, nz)] - Z[max(k - 1, 0)];
+  const double v = f * wx * wy * wz * 0.125;
   b[n] = v + (nodal ? nodal[n] : 0.0);
 }
 
 // ---------------------------------------------------------------------------
+// Dirichlet mask and values, then the matrix rows with the set eliminated, the
+// pattern and the lifting; b = load (launched by the caller) plus the lifting.
+template <int NC>
+static int launch_rows(const AssemblyArgs &a, const double *coef, cudaStream_t s) {
+  const int T = 256, nnode = (a.nx + 1) * (a.ny + 1) * (a.nz + 1);
+  GENEO_CUDA_TRY(cudaMemsetAsync(a.mask, 0, NC * (size_t)nnode, s));
+  GENEO_CUDA_TRY(cudaMemsetAsync(a.g, 0, NC * (size_t)nnode * sizeof(double), s));
+  if (a.n_dir > 0) {
+    k_dirichlet_mark<<<(a.n_dir + T - 1) / T, T, 0, s>>>(a.n_dir, a.dir_dofs, a.dir_vals,
+                                                         NC * nnode, a.mask, a.g, a.status); GENEO_COUNT_LAUNCH();
+  }
+  if (int st = ensure_smem(k_assemble_rows<NC>, kRowSmem<NC>)) return st;
+  k_assemble_rows<NC><<<(nnode + kRowNodes<NC> - 1) / kRowNodes<NC>, kRowThreads<NC>, kRowSmem<NC>, s>>>(
+      a.nx, a.ny, a.nz, a.X, a.Y, a.Z, coef, a.mask, a.g, a.n_dir > 0 ? a.lift : nullptr,
+      a.row_ptr, a.col, a.val); GENEO_COUNT_LAUNCH();
+  return launch_load(a, s);
+}
+
 int launch_assembly(const AssemblyArgs &a, cudaStream_t s) {
-  const int T = 256;
-  int nnx = a.nx + 1, nny = a.ny + 1, nnz = a.nz + 1;
-  int nnode = nnx * nny * nnz;
-  int nel = a.nx * a.ny * a.nz;
+  const int nel = a.nx * a.ny * a.nz, T = 128;
   k_material_base<<<(a.n_mat + 63) / 64, 64, 0, s>>>(a.n_mat, a.mats, a.C0); GENEO_COUNT_LAUNCH();
   k_element_C<<<(nel + T - 1) / T, T, 0, s>>>(nel, a.n_mat, a.C0, a.emat, a.theta, a.phi,
                                               a.Cel, a.status); GENEO_COUNT_LAUNCH();
-  k_bsr_count<<<(nnode + T - 1) / T, T, 0, s>>>(nnx, nny, nnz, a.cnt); GENEO_COUNT_LAUNCH();
-  k_scan_single<<<1, 1024, 0, s>>>(nnode, a.cnt, a.row_ptr); GENEO_COUNT_LAUNCH();
-  k_bsr_fill<<<(nnode + T - 1) / T, T, 0, s>>>(nnx, nny, nnz, a.row_ptr, a.col); GENEO_COUNT_LAUNCH();
-  long long nt = (long long)nnode * 27;
-  k_assemble_values<<<(unsigned)((nt + 127) / 128), 128, 0, s>>>(
-      a.nx, a.ny, a.nz, a.X, a.Y, a.Z, a.Cel, a.row_ptr, a.val); GENEO_COUNT_LAUNCH();
-  k_load<<<(nnode + T - 1) / T, T, 0, s>>>(a.nx, a.ny, a.nz, a.X, a.Y, a.top_pressure,
-                                           a.nodal, a.b); GENEO_COUNT_LAUNCH();
-  GENEO_CUDA_TRY(cudaMemsetAsync(a.mask, 0, 3 * (size_t)nnode, s));
-  GENEO_CUDA_TRY(cudaMemsetAsync(a.g, 0, 3 * (size_t)nnode * sizeof(double), s));
-  if (a.n_dir > 0) {
-    k_dirichlet_mark<<<(a.n_dir + T - 1) / T, T, 0, s>>>(a.n_dir, a.dir_dofs, a.dir_vals,
-                                                         3 * nnode, a.mask, a.g, a.status); GENEO_COUNT_LAUNCH();
-    k_dirichlet_lift<<<(3 * nnode + T - 1) / T, T, 0, s>>>(nnode, 3, a.row_ptr, a.col, a.val,
-                                                           a.mask, a.g, a.lift); GENEO_COUNT_LAUNCH();
-    k_apply_lift<<<(3 * nnode + T - 1) / T, T, 0, s>>>(3 * nnode, a.mask, a.lift, a.b); GENEO_COUNT_LAUNCH();
-    k_dirichlet_eliminate<<<(nnode + T - 1) / T, T, 0, s>>>(nnode, 3, a.row_ptr, a.col, a.mask,
-                                                            a.val); GENEO_COUNT_LAUNCH();
-  }
-  GENEO_CUDA_TRY(cudaGetLastError());
-  return GENEO_OK;
+  return launch_rows<3>(a, a.Cel, s);
+}
+
+int launch_assembly_darcy(const AssemblyArgs &a, cudaStream_t s) {
+  return launch_rows<1>(a, a.perm, s);
 }
 
 // Stress recovery at the element centres: sigma_e = C_e B(0) u_e (Voigt order
@@ -352,33 +310,6 @@ int launch_load(const AssemblyArgs &a, cudaStream_t s) {
   }
   if (a.n_dir > 0) {
     k_apply_lift<<<(nc * nnode + T - 1) / T, T, 0, s>>>(nc * nnode, a.mask, a.lift, a.b); GENEO_COUNT_LAUNCH();
-  }
-  GENEO_CUDA_TRY(cudaGetLastError());
-  return GENEO_OK;
-}
-
-int launch_assembly_darcy(const AssemblyArgs &a, cudaStream_t s) {
-  const int T = 256;
-  int nnx = a.nx + 1, nny = a.ny + 1, nnz = a.nz + 1;
-  int nnode = nnx * nny * nnz;
-  k_bsr_count<<<(nnode + T - 1) / T, T, 0, s>>>(nnx, nny, nnz, a.cnt); GENEO_COUNT_LAUNCH();
-  k_scan_single<<<1, 1024, 0, s>>>(nnode, a.cnt, a.row_ptr); GENEO_COUNT_LAUNCH();
-  k_bsr_fill<<<(nnode + T - 1) / T, T, 0, s>>>(nnx, nny, nnz, a.row_ptr, a.col); GENEO_COUNT_LAUNCH();
-  long long nt = (long long)nnode * 27;
-  k_assemble_values_darcy<<<(unsigned)((nt + 127) / 128), 128, 0, s>>>(
-      a.nx, a.ny, a.nz, a.X, a.Y, a.Z, a.perm, a.row_ptr, a.val); GENEO_COUNT_LAUNCH();
-  k_load_darcy<<<(nnode + T - 1) / T, T, 0, s>>>(a.nx, a.ny, a.nz, a.X, a.Y, a.Z, a.top_pressure,
-                                                 a.nodal, a.b); GENEO_COUNT_LAUNCH();
-  GENEO_CUDA_TRY(cudaMemsetAsync(a.mask, 0, (size_t)nnode, s));
-  GENEO_CUDA_TRY(cudaMemsetAsync(a.g, 0, (size_t)nnode * sizeof(double), s));
-  if (a.n_dir > 0) {
-    k_dirichlet_mark<<<(a.n_dir + T - 1) / T, T, 0, s>>>(a.n_dir, a.dir_dofs, a.dir_vals, nnode,
-                                                         a.mask, a.g, a.status); GENEO_COUNT_LAUNCH();
-    k_dirichlet_lift<<<(nnode + T - 1) / T, T, 0, s>>>(nnode, 1, a.row_ptr, a.col, a.val, a.mask,
-                                                       a.g, a.lift); GENEO_COUNT_LAUNCH();
-    k_apply_lift<<<(nnode + T - 1) / T, T, 0, s>>>(nnode, a.mask, a.lift, a.b); GENEO_COUNT_LAUNCH();
-    k_dirichlet_eliminate<<<(nnode + T - 1) / T, T, 0, s>>>(nnode, 1, a.row_ptr, a.col, a.mask,
-                                                            a.val); GENEO_COUNT_LAUNCH();
   }
   GENEO_CUDA_TRY(cudaGetLastError());
   return GENEO_OK;

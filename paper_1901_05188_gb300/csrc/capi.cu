@@ -126,7 +126,6 @@ void plan_assemble(Arena &A, geneo_ctx *c, int nx, int ny, int nz, int n_mat, in
   c->Z = A.take<double>(nz + 1);
   c->C0 = elastic ? A.take<double>(36 * (size_t)std::max(n_mat, 1)) : nullptr;
   c->Cel = elastic ? A.take<double>(36 * (size_t)nel) : nullptr;
-  c->cnt = A.take<int32_t>(nnode);
   c->row_ptr = A.take<int32_t>(nnode + 1);
   c->col = A.take<int32_t>(nnzb);
   c->val = A.take<double>((size_t)nc * nc * nnzb);
@@ -407,7 +406,6 @@ static void fill_common_args(geneo_ctx *c, AssemblyArgs &a, int n_dir, const gen
   a.dir_vals = (n_dir > 0 && dir->value) ? c->dir_vals : nullptr;
   a.nodal = nodal_load ? c->nodal : nullptr;
   a.top_pressure = scalar;
-  a.cnt = c->cnt;
   a.row_ptr = c->row_ptr;
   a.col = c->col;
   a.val = c->val;

@@ -34,7 +34,7 @@ struct geneo_ctx {
   size_t ws0_bound_bytes = 0;
   double *X = nullptr, *Y = nullptr, *Z = nullptr;
   double *Cel = nullptr, *C0 = nullptr;
-  int32_t *row_ptr = nullptr, *col = nullptr, *cnt = nullptr;
+  int32_t *row_ptr = nullptr, *col = nullptr;
   double *val = nullptr, *b = nullptr, *g = nullptr;
   double *lift = nullptr;                  // Dirichlet lifting (kept for new loads)
   double *sig = nullptr;                   // element stresses (6 per element), output staging

@@ -85,67 +85,132 @@ __global__ void k_pou_interior(const SubDesc *subs, const int *cand, int co0, in
   wloc[S.v_int + t] = x;
 }
 
-__global__ void __launch_bounds__(128)
+// S_j = A_Omega_j - sigma B_j in band tiles (lower part) and B_j as 27-slot
+// rows, from the rows of the node's elements inside Omega_j (fem.cuh): one
+// block per kNeuNodes consecutive local nodes, summed in registers (elasticity:
+// lane = node, one warp per component pair) and staged in shared memory, from
+// where B's rows are written coalesced and S's entries column by column.  The
+// overlap elements' rows are summed only in blocks that have some.  FP64 issue
+// bounds it, as for the global matrix.
+template <int NC>
+constexpr int kNeuNodes = NC == 3 ? 32 : 128;
+template <int NC>
+constexpr int kNeuThreads = NC == 3 ? 192 : 128;
+template <int NC>
+constexpr int kNeuSmem = kNeuNodes<NC> * 27 * (NC * NC * 8 + 4 + 1);
+
+template <int NC>
+__global__ void __launch_bounds__(kNeuThreads<NC>)
     k_neumann_assemble(const SubDesc *subs, const BandLayout *lay, int nx, int ny, int nz,
                        const double *__restrict__ X, const double *__restrict__ Y,
-                       const double *__restrict__ Z, const double *__restrict__ Cel,
-                       const double *__restrict__ perm,
+                       const double *__restrict__ Z, const double *__restrict__ coef,
                        const int *__restrict__ ecnt, int eo0, int eo1, int eo2,
                        const uint8_t *__restrict__ mask, const double *__restrict__ Xneu,
                        double sigma, double *poolS, double *Bloc) {
-  const int j = blockIdx.y;
-  const SubDesc &S = subs[j];
-  const int nn = S.nbox.count();
-  long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (long long)nn * 27) return;
-  const int l = (int)(t / 27), s = (int)(t % 27);
-  int gi, gj, gk;
-  S.nbox.global(l, gi, gj, gk);
-  const int i2 = gi + s % 3 - 1, j2 = gj + (s / 3) % 3 - 1, k2 = gk + s / 9 - 1;
-  const int l2 = S.nbox.local(i2, j2, k2);
-  const int nc = S.nc, nc2 = nc * nc;
-  double *bl = Bloc + (S.b_neu + (long long)l * 27 + s) * nc2;
-  if (l2 < 0) {
-    for (int q = 0; q < nc2; ++q) bl[q] = 0.0;
-    return;
+  constexpr int N = kNeuNodes<NC>, NC2 = NC * NC, kT = kNeuThreads<NC>;
+  const SubDesc &S = subs[blockIdx.y];
+  const int nn = S.nbox.count(), l0 = blockIdx.x * N, tid = threadIdx.x;
+  if (l0 >= nn) return;
+  extern __shared__ __align__(16) double sv[];               // [N][27][NC2]
+  int *nb = reinterpret_cast<int *>(sv + N * 27 * NC2);      // [N][27] local neighbour node, or -1
+  uint8_t *mk = reinterpret_cast<uint8_t *>(nb + N * 27);    // [N][27] its Dirichlet bits
+  const int nnx = nx + 1, nny = ny + 1;
+  for (int e = tid; e < N * 27; e += kT) {
+    const int t = e / 27, s = e - 27 * t, l = l0 + t;
+    int l2 = -1;
+    uint8_t m = 0;
+    if (l < nn) {
+      int i, j, k;
+      S.nbox.global(l, i, j, k);
+      i += s % 3 - 1, j += (s / 3) % 3 - 1, k += s / 9 - 1;
+      l2 = S.nbox.local(i, j, k);
+      if (l2 >= 0)
+        for (int c = 0; c < NC; ++c)
+          m |= (uint8_t)((mask[(size_t)NC * (i + nnx * (j + nny * k)) + c] != 0) << c);
+    }
+    nb[e] = l2;
+    mk[e] = m;
   }
-  double KA[9], KO[9];
-  for (int q = 0; q < 9; ++q) KA[q] = KO[q] = 0.0;
-  for (int ez = max(max(gk, k2) - 1, S.elo[2]); ez <= min(min(gk, k2), S.ehi[2] - 1); ++ez)
-    for (int ey = max(max(gj, j2) - 1, S.elo[1]); ey <= min(min(gj, j2), S.ehi[1] - 1); ++ey)
-      for (int ex = max(max(gi, i2) - 1, S.elo[0]); ex <= min(min(gi, i2), S.ehi[0] - 1); ++ex) {
-        int e = ex + nx * (ey + ny * ez);
-        int a = (gi - ex) + 2 * (gj - ey) + 4 * (gk - ez);
-        int b = (i2 - ex) + 2 * (j2 - ey) + 4 * (k2 - ez);
-        double Kb[9];
-        if (nc == 3)
-          element_block(Cel + 36 * (size_t)e, X[ex + 1] - X[ex], Y[ey + 1] - Y[ey],
-                        Z[ez + 1] - Z[ez], a, b, Kb);
-        else
-          Kb[0] = darcy_entry(perm + 3 * (size_t)e, X[ex + 1] - X[ex], Y[ey + 1] - Y[ey],
-                              Z[ez + 1] - Z[ez], a, b);
-        bool ov = ecnt[eo0 + ex] * ecnt[eo1 + ey] * ecnt[eo2 + ez] >= 2;
-        for (int q = 0; q < nc2; ++q) {
-          KA[q] += Kb[q];
-          if (ov) KO[q] += Kb[q];
+  const int t = NC == 3 ? (tid & 31) : tid, l = l0 + t;
+  const bool live = l < nn;
+  int gi = 0, gj = 0, gk = 0;
+  if (live) S.nbox.global(l, gi, gj, gk);
+  NodeAxis ax, ay, az;
+  bool touch = false;                      // the node has an overlap element
+  auto ov = [&](int ex, int ey, int ez) { return ecnt[eo0 + ex] * ecnt[eo1 + ey] * ecnt[eo2 + ez] >= 2; };
+  if (live) {
+    ax = node_axis(X, gi, S.elo[0], S.ehi[0]);
+    ay = node_axis(Y, gj, S.elo[1], S.ehi[1]);
+    az = node_axis(Z, gk, S.elo[2], S.ehi[2]);
+#pragma unroll
+    for (int A = 0; A < 8; ++A)
+      if (ax.in[A & 1] && ay.in[(A >> 1) & 1] && az.in[A >> 2])
+        touch = touch || ov(gi - (A & 1), gj - ((A >> 1) & 1), gk - (A >> 2));
+  }
+  int ci = 0, ck = 0, off[9];
+  if constexpr (NC == 3) component_pair(tid >> 5, ci, ck, off);
+  // this thread's rows over the elements `take` picks, added to the stage
+  auto rows = [&](auto take, bool add) {
+    double acc[27];
+#pragma unroll
+    for (int s = 0; s < 27; ++s) acc[s] = 0.0;
+    double *out = sv + t * 27 * NC2;
+    if constexpr (NC == 3) {
+      double acct[27];
+      if (ci != ck) {
+#pragma unroll
+        for (int s = 0; s < 27; ++s) acct[s] = 0.0;
+        elastic_rows<true>(coef, off, ax, ay, az, gi, gj, gk, nx, ny, take, acc, acct);
+#pragma unroll
+        for (int s = 0; s < 27; ++s) {
+          double *o = out + 9 * s + 3 * ci + ck, *ot = out + 9 * s + 3 * ck + ci;
+          *o = add ? acc[s] + *o : acc[s];
+          *ot = add ? acct[s] + *ot : acct[s];
+        }
+      } else {
+        elastic_rows<false>(coef, off, ax, ay, az, gi, gj, gk, nx, ny, take, acc, acct);
+#pragma unroll
+        for (int s = 0; s < 27; ++s) {
+          double *o = out + 9 * s + 4 * ci;
+          *o = add ? acc[s] + *o : acc[s];
         }
       }
-  const int nnx = nx + 1, nny = ny + 1;
-  const int g = gi + nnx * (gj + nny * gk), g2 = i2 + nnx * (j2 + nny * k2);
-  const BandLayout L = lay[j];
-  for (int r = 0; r < nc; ++r)
-    for (int c = 0; c < nc; ++c) {
-      int rd = nc * g + r, cd = nc * g2 + c;
-      double a = KA[nc * r + c], o = KO[nc * r + c];
-      if (mask[rd] || mask[cd]) {
-        a = (rd == cd) ? 1.0 : 0.0;
-        o = 0.0;
-      }
-      double bv = Xneu[S.x_neu + nc * l + r] * o * Xneu[S.x_neu + nc * l2 + c];
-      bl[nc * r + c] = bv;
-      int R = nc * l + r, C = nc * l2 + c;
-      if (R >= C) tile_at(poolS, L, R >> 5, (R >> 5) - (C >> 5))[(C & 31) * 32 + (R & 31)] = a - sigma * bv;
+    } else {
+      darcy_rows(coef, ax, ay, az, gi, gj, gk, nx, ny, take, acc);
+#pragma unroll
+      for (int s = 0; s < 27; ++s) out[s] = add ? acc[s] + out[s] : acc[s];
     }
+  };
+  const bool any = __syncthreads_or(touch);
+  if (any) {
+    if (live) rows(ov, false);
+    __syncthreads();
+  }
+  double *bl = Bloc + (S.b_neu + (long long)l0 * 27) * NC2;
+  for (int e = tid; e < N * 27 * NC2; e += kT) {
+    const int b = e / NC2, q = e - NC2 * b, t2 = b / 27, r = q / NC, c = q - NC * r, l2 = nb[b];
+    if (l0 + t2 >= nn) break;
+    double bv = 0.0;
+    if (any && l2 >= 0 && !((mk[27 * t2 + 13] >> r & 1) || (mk[b] >> c & 1)))
+      bv = Xneu[S.x_neu + NC * (l0 + t2) + r] * sv[e] * Xneu[S.x_neu + NC * l2 + c];
+    bl[e] = bv;
+    sv[e] = -sigma * bv;
+  }
+  __syncthreads();
+  if (live) rows([](int, int, int) { return true; }, true);
+  __syncthreads();
+  // column C = NC l + c of S: rows R = NC l2 + r >= C (S is symmetric)
+  const BandLayout L = lay[blockIdx.y];
+  for (int e = tid; e < N * 27 * NC2; e += kT) {
+    const int r = e % NC, s = (e / NC) % 27, c = (e / (27 * NC)) % NC, t2 = e / (27 * NC2);
+    const int b = 27 * t2 + s, l2 = nb[b];
+    const int C = NC * (l0 + t2) + c, R = NC * l2 + r;
+    if (l2 < 0 || R < C) continue;
+    const bool drop = (mk[27 * t2 + 13] >> c & 1) || (mk[b] >> r & 1);
+    const int I = R >> 5, J = C >> 5;
+    tile_at(poolS, L, I, I - J)[(C & 31) * 32 + (R & 31)] =
+        drop ? (R == C ? 1.0 : 0.0) : sv[b * NC2 + NC * c + r];
+  }
 }
 
 __global__ void k_bloc_mv(const SubDesc *subs, const double *__restrict__ Bloc,
@@ -897,6 +962,20 @@ void launch_pou_interior(const SubDesc *d_subs, int nsub, int max_nodes, const i
                                    nnx, nny, nnz, px, py, kind, wloc); GENEO_COUNT_LAUNCH();
 }
 
+template <int NC>
+static void launch_neumann(const SubDesc *d_subs, const BandLayout *d_lay, int nsub,
+                           int max_nodes, int nx, int ny, int nz, const double *X, const double *Y,
+                           const double *Z, const double *coef, const int *ecnt,
+                           const int ecnt_off[3], const uint8_t *mask, const double *Xneu,
+                           double sigma, double *poolS, double *Bloc, cudaStream_t s) {
+  (void)ensure_smem(k_neumann_assemble<NC>, kNeuSmem<NC>);   // a failure surfaces as a launch error
+  const dim3 g((unsigned)((max_nodes + kNeuNodes<NC> - 1) / kNeuNodes<NC>), nsub);
+  k_neumann_assemble<NC><<<g, kNeuThreads<NC>, kNeuSmem<NC>, s>>>(
+      d_subs, d_lay, nx, ny, nz, X, Y, Z, coef, ecnt, ecnt_off[0], ecnt_off[1], ecnt_off[2], mask,
+      Xneu, sigma, poolS, Bloc); GENEO_COUNT_LAUNCH();
+}
+
+// Exactly one of Cel (elasticity) and perm (Darcy) is set.
 void launch_neumann_assemble(const SubDesc *d_subs, const BandLayout *d_lay, int nsub,
                              int max_nodes, int nx, int ny, int nz, const double *X,
                              const double *Y, const double *Z, const double *Cel,
@@ -904,11 +983,12 @@ void launch_neumann_assemble(const SubDesc *d_subs, const BandLayout *d_lay, int
                              const int *ecnt, const int ecnt_off[3], const uint8_t *mask,
                              const double *Xneu, double sigma, double *poolS, double *Bloc,
                              cudaStream_t s) {
-  long long tot = (long long)max_nodes * 27;
-  dim3 g((unsigned)((tot + 127) / 128), nsub);
-  k_neumann_assemble<<<g, 128, 0, s>>>(d_subs, d_lay, nx, ny, nz, X, Y, Z, Cel, perm, ecnt,
-                                       ecnt_off[0], ecnt_off[1], ecnt_off[2], mask, Xneu, sigma,
-                                       poolS, Bloc); GENEO_COUNT_LAUNCH();
+  if (Cel)
+    launch_neumann<3>(d_subs, d_lay, nsub, max_nodes, nx, ny, nz, X, Y, Z, Cel, ecnt, ecnt_off,
+                      mask, Xneu, sigma, poolS, Bloc, s);
+  else
+    launch_neumann<1>(d_subs, d_lay, nsub, max_nodes, nx, ny, nz, X, Y, Z, perm, ecnt, ecnt_off,
+                      mask, Xneu, sigma, poolS, Bloc, s);
 }
 
 void launch_bloc_mv(const SubDesc *d_subs, int nsub, int max_nodes, const double *Bloc,

@@ -18,7 +18,7 @@ struct AssemblyArgs {
   const double *nodal;              // device (may be null)
   double top_pressure;              // elasticity: top traction; Darcy: the uniform source f
   double *C0, *Cel;                 // per-material / per-element Voigt stiffness
-  int32_t *cnt, *row_ptr, *col;
+  int32_t *row_ptr, *col;
   double *val, *b, *g;
   double *lift;                     // Dirichlet lifting: g on Dirichlet rows, -A_FD g on free rows
   uint8_t *mask;
