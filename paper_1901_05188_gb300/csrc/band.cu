@@ -1,10 +1,8 @@
-// Band-tiled Cholesky factors of the one-level additive Schwarz term
-// sum_j R_j^T D_j A_j^-1 R_j  (Sec. 3.1, eqn:onelevelAS) and of the GenEO
-// shift-invert operators (whose multi-right-hand-side solves run the local
-// solves' look-ahead sweep), and the extraction of A_j from the global
-// matrix.  The coarse correction and the
-// gather are in coarse.cu, the cluster sweeps of the local solves in
-// schwarz.cu.
+// FP32 band-tiled Cholesky factors of the one-level additive Schwarz term
+// sum_j R_j^T D_j A_j^-1 R_j  (Sec. 3.1, eqn:onelevelAS) and the extraction of
+// A_j from the global matrix.  The FP64 factorisation is in bandchol.cu, the
+// coarse correction and the gather in coarse.cu, the cluster sweeps of the
+// local solves in schwarz.cu.
 //
 // The paper factors A_j with a sparse direct solver (UMFPack).  Here each
 // A_j is a band matrix in a box numbering whose longest axis runs slowest, held
@@ -42,49 +40,37 @@ __global__ void k_band_pad(const BandLayout *lay, int nsys, T *pool) {
 
 // ---- tile Cholesky ---------------------------------------------------------
 
-// 1/sqrt(d) for d > 0: single-precision estimate refined by Newton's iteration
-// for f(y) = 1/y^2 - d, y <- y (3 - d y^2) / 2, which doubles the number of
-// correct bits per step (24 -> 48 -> full double).  The pivot is on the serial
-// path of the diagonal-block factorisation, where a few dependent FP64
-// operations are much cheaper than a correctly rounded square root and
-// division; the factor only needs the pivot to working precision.
-__device__ __forceinline__ double inv_sqrt_pos(double d) {
-  double y = (double)rsqrtf((float)d);
-  if (!(d >= 1e-30 && d <= 1e30)) return 1.0 / sqrt(d);   // outside float range: exact path
-  y = y * (1.5 - 0.5 * d * y * y);
-  y = y * (1.5 - 0.5 * d * y * y);
-  return y;
-}
+// 1/sqrt(d) for d > 0: estimate and one Newton step y (3 - d y^2) / 2.  The
+// pivot is on the serial path of the diagonal-block factorisation.
 __device__ __forceinline__ float inv_sqrt_pos(float d) {
   float y = rsqrtf(d);
   return y * (1.5f - 0.5f * d * y * y);
 }
 
-template <typename T>
 __global__ void __launch_bounds__(1024) k_chol_diag(const BandLayout *lay, int nsys, int J,
-                                                    T *poolL, T *poolU, DevStatus *st) {
+                                                    float *poolL, float *poolU, DevStatus *st) {
   int j = blockIdx.x;
   BandLayout L = lay[j];
   if (J >= L.nt) return;
-  __shared__ T A[32][33];
-  __shared__ T X[32][33];
-  __shared__ T Y[32][33];
-  __shared__ T piv[2];
+  __shared__ float A[32][33];
+  __shared__ float X[32][33];
+  __shared__ float Y[32][33];
+  __shared__ float piv[2];
   __shared__ int bad;
   const int tid = threadIdx.x, r = tid & 31, cc = tid >> 5;   // thread (r, cc) owns entry (r, cc)
-  T *t = tile_ptr(poolL, L, J, 0);
+  float *t = tile_ptr(poolL, L, J, 0);
   A[r][cc] = t[cc * 32 + r];
   if (tid == 0) bad = -1;
   __syncthreads();
   // right-looking Cholesky, one entry per thread: three barriers per column
   for (int k = 0; k < 32; ++k) {
     if (tid == 0) {
-      T d = A[k][k];
-      if (!(d > T(0))) {
+      float d = A[k][k];
+      if (!(d > float(0))) {
         if (bad < 0) bad = J * 32 + k;
-        d = T(1);
+        d = float(1);
       }
-      const T y = inv_sqrt_pos(d);
+      const float y = inv_sqrt_pos(d);
       piv[0] = d * y;          // sqrt(d)
       piv[1] = y;              // 1 / sqrt(d)
     }
@@ -96,26 +82,26 @@ __global__ void __launch_bounds__(1024) k_chol_diag(const BandLayout *lay, int n
   }
   // inverse of the lower-triangular factor by recursive doubling:
   // inv([[P, 0], [Q, R]]) = [[iP, 0], [-iR Q iP, iR]]
-  X[r][cc] = (r == cc) ? T(1) / A[r][r] : T(0);
+  X[r][cc] = (r == cc) ? float(1) / A[r][r] : float(0);
   __syncthreads();
   for (int b = 1; b < 32; b <<= 1) {
     // pairs of b x b diagonal blocks at s and s + b, s = multiple of 2b
     const int s = (r / (2 * b)) * (2 * b);
     const bool lower = (r >= s + b) && (cc >= s) && (cc < s + b);   // block (R-row, P-col)
-    T v = T(0);
+    float v = float(0);
     if (lower) {   // Y = Q iP  (Q = A[s+b.., s..s+b), iP = X[s.., s..])
       for (int k = cc; k < s + b; ++k) v += A[r][k] * X[k][cc];
     }
     Y[r][cc] = v;
     __syncthreads();
     if (lower) {   // X_lower = -iR Y
-      T w = T(0);
+      float w = float(0);
       for (int k = s + b; k <= r; ++k) w += X[r][k] * Y[k][cc];
       X[r][cc] = -w;
     }
     __syncthreads();
   }
-  T *u = tile_ptr(poolU, L, J, 0);
+  float *u = tile_ptr(poolU, L, J, 0);
   t[cc * 32 + r] = X[r][cc];    // inv(L_JJ), column-major
   u[cc * 32 + r] = X[cc][r];    // inv(L_JJ)^T
   if (tid == 0 && bad >= 0) {
@@ -126,26 +112,25 @@ __global__ void __launch_bounds__(1024) k_chol_diag(const BandLayout *lay, int n
   }
 }
 
-// L(J+d, J) = A(J+d, J) inv(L_JJ)^T for d = 1..w (blockIdx.y = d - 1).
-template <typename T>
+// L(J+d, J) = A(J+d, J) inv(L_JJ)^float for d = 1..w (blockIdx.y = d - 1).
 __global__ void __launch_bounds__(256) k_chol_trsm(const BandLayout *lay, int nsys, int J,
-                                                   T *poolL, T *poolU) {
+                                                   float *poolL, float *poolU) {
   int j = blockIdx.x, d = blockIdx.y + 1;
   BandLayout L = lay[j];
   if (J >= L.nt || d > L.w || J + d >= L.nt) return;
-  __shared__ T Aa[32][33];
-  __shared__ T D[32][33];
-  T *ta = tile_ptr(poolL, L, J + d, d);
-  const T *td = tile_ptr(poolL, L, J, 0);
+  __shared__ float Aa[32][33];
+  __shared__ float D[32][33];
+  float *ta = tile_ptr(poolL, L, J + d, d);
+  const float *td = tile_ptr(poolL, L, J, 0);
   for (int e = threadIdx.x; e < 1024; e += 256) {
     Aa[e & 31][e >> 5] = ta[e];
     D[e & 31][e >> 5] = td[e];
   }
   __syncthreads();
-  T *tu = tile_ptr(poolU, L, J, d);
+  float *tu = tile_ptr(poolU, L, J, d);
   for (int e = threadIdx.x; e < 1024; e += 256) {
     int r = e & 31, c = e >> 5;
-    T s = T(0);
+    float s = float(0);
     for (int k = 0; k <= c; ++k) s += Aa[r][k] * D[c][k];
     ta[e] = s;                 // (r, c) column-major
     tu[r * 32 + c] = s;        // transposed: U(J, d)(c, r) = L(J+d, J)(r, c)
@@ -155,9 +140,8 @@ __global__ void __launch_bounds__(256) k_chol_trsm(const BandLayout *lay, int ns
 // A(J+d1, J+d2) -= L(J+d1, J) L(J+d2, J)^T, 1 <= d2 <= d1 <= w.
 // part 0: every pair; part 1: the next tile column only (d2 = 1, blockIdx.y =
 // d1 - 1); part 2: the rest (d2 >= 2).
-template <typename T>
 __global__ void __launch_bounds__(256) k_chol_update(const BandLayout *lay, int nsys, int J,
-                                                     T *poolL, int part) {
+                                                     float *poolL, int part) {
   int j = blockIdx.x;
   BandLayout L = lay[j];
   int p = blockIdx.y;
@@ -175,19 +159,19 @@ __global__ void __launch_bounds__(256) k_chol_update(const BandLayout *lay, int 
     d2 = p - d1 * (d1 - 1) / 2 + 1;
   }
   if (J >= L.nt || d1 > L.w || J + d1 >= L.nt) return;
-  __shared__ T Aa[32][33];
-  __shared__ T Bb[32][33];
-  const T *ta = tile_ptr(poolL, L, J + d1, d1);
-  const T *tb = tile_ptr(poolL, L, J + d2, d2);
+  __shared__ float Aa[32][33];
+  __shared__ float Bb[32][33];
+  const float *ta = tile_ptr(poolL, L, J + d1, d1);
+  const float *tb = tile_ptr(poolL, L, J + d2, d2);
   for (int e = threadIdx.x; e < 1024; e += 256) {
     Aa[e & 31][e >> 5] = ta[e];
     Bb[e & 31][e >> 5] = tb[e];
   }
   __syncthreads();
-  T *tc = tile_ptr(poolL, L, J + d1, d1 - d2);
+  float *tc = tile_ptr(poolL, L, J + d1, d1 - d2);
   for (int e = threadIdx.x; e < 1024; e += 256) {
     int r = e & 31, c = e >> 5;
-    T s = T(0);
+    float s = float(0);
 #pragma unroll 8
     for (int k = 0; k < 32; ++k) s += Aa[r][k] * Bb[c][k];
     tc[e] -= s;
@@ -245,34 +229,28 @@ int launch_band_clear(const BandLayout *d_lay, int nsys, T *pool, long long pool
 }
 
 // Trailing update of tile column J (part 0 all pairs, 1 the next tile column,
-// 2 the rest): FP32 factors on the tensor cores (3xTF32), FP64 on the FMA units.
-template <typename T>
-int launch_update(const BandLayout *d_lay, int nsys, int J, int w_max, T *poolL, int part,
-                  DevStatus *st, cudaStream_t s) {
+// 2 the rest) on the tensor cores (3xTF32) or the FMA units.
+static int launch_update(const BandLayout *d_lay, int nsys, int J, int w_max, float *poolL, int part,
+                         DevStatus *st, cudaStream_t s) {
   const int npairs = w_max * (w_max + 1) / 2;
-  if constexpr (sizeof(T) == 4) {
-    if (use_tensor_cores()) return launch_chol_update_tc(d_lay, nsys, J, w_max, poolL, part, st, s);
-  }
+  if (use_tensor_cores()) return launch_chol_update_tc(d_lay, nsys, J, w_max, poolL, part, st, s);
   const int ny = part == 1 ? w_max : (part == 2 ? npairs - w_max : npairs);
   if (ny > 0) {
-    k_chol_update<T><<<dim3(nsys, ny), 256, 0, s>>>(d_lay, nsys, J, poolL, part); GENEO_COUNT_LAUNCH();
+    k_chol_update<<<dim3(nsys, ny), 256, 0, s>>>(d_lay, nsys, J, poolL, part); GENEO_COUNT_LAUNCH();
   }
   return GENEO_OK;
 }
 
-template <typename T>
-int launch_band_cholesky(const BandLayout *d_lay, int nsys, int nt_max, int w_max, T *poolL,
-                         T *poolU, DevStatus *st, cudaStream_t s, cudaStream_t side) {
+int launch_band_cholesky32(const BandLayout *d_lay, int nsys, int nt_max, int w_max, float *poolL,
+                           float *poolU, DevStatus *st, cudaStream_t s, cudaStream_t side) {
   int rc;
-  if constexpr (sizeof(T) == 4) {
-    if (use_tensor_cores() && (rc = prepare_chol_update_tc())) return rc;
-  }
+  if (use_tensor_cores() && (rc = prepare_chol_update_tc())) return rc;
   if (!side || w_max == 0) {
     for (int J = 0; J < nt_max; ++J) {
-      k_chol_diag<T><<<nsys, 1024, 0, s>>>(d_lay, nsys, J, poolL, poolU, st); GENEO_COUNT_LAUNCH();
+      k_chol_diag<<<nsys, 1024, 0, s>>>(d_lay, nsys, J, poolL, poolU, st); GENEO_COUNT_LAUNCH();
       if (w_max > 0) {
-        k_chol_trsm<T><<<dim3(nsys, w_max), 256, 0, s>>>(d_lay, nsys, J, poolL, poolU); GENEO_COUNT_LAUNCH();
-        if ((rc = launch_update<T>(d_lay, nsys, J, w_max, poolL, 0, st, s))) return rc;
+        k_chol_trsm<<<dim3(nsys, w_max), 256, 0, s>>>(d_lay, nsys, J, poolL, poolU); GENEO_COUNT_LAUNCH();
+        if ((rc = launch_update(d_lay, nsys, J, w_max, poolL, 0, st, s))) return rc;
       }
     }
     GENEO_CUDA_TRY(cudaGetLastError());
@@ -284,15 +262,15 @@ int launch_band_cholesky(const BandLayout *d_lay, int nsys, int nt_max, int w_ma
   cudaEvent_t e_main, e_side;
   GENEO_CUDA_TRY(cudaEventCreateWithFlags(&e_main, cudaEventDisableTiming));
   GENEO_CUDA_TRY(cudaEventCreateWithFlags(&e_side, cudaEventDisableTiming));
-  k_chol_diag<T><<<nsys, 1024, 0, s>>>(d_lay, nsys, 0, poolL, poolU, st); GENEO_COUNT_LAUNCH();
-  k_chol_trsm<T><<<dim3(nsys, w_max), 256, 0, s>>>(d_lay, nsys, 0, poolL, poolU); GENEO_COUNT_LAUNCH();
+  k_chol_diag<<<nsys, 1024, 0, s>>>(d_lay, nsys, 0, poolL, poolU, st); GENEO_COUNT_LAUNCH();
+  k_chol_trsm<<<dim3(nsys, w_max), 256, 0, s>>>(d_lay, nsys, 0, poolL, poolU); GENEO_COUNT_LAUNCH();
   for (int J = 0; J + 1 < nt_max; ++J) {
-    if ((rc = launch_update<T>(d_lay, nsys, J, w_max, poolL, 1, st, s))) return rc;
+    if ((rc = launch_update(d_lay, nsys, J, w_max, poolL, 1, st, s))) return rc;
     GENEO_CUDA_TRY(cudaEventRecord(e_main, s));
     GENEO_CUDA_TRY(cudaStreamWaitEvent(side, e_main, 0));
-    k_chol_diag<T><<<nsys, 1024, 0, side>>>(d_lay, nsys, J + 1, poolL, poolU, st); GENEO_COUNT_LAUNCH();
-    k_chol_trsm<T><<<dim3(nsys, w_max), 256, 0, side>>>(d_lay, nsys, J + 1, poolL, poolU); GENEO_COUNT_LAUNCH();
-    if ((rc = launch_update<T>(d_lay, nsys, J, w_max, poolL, 2, st, s))) return rc;
+    k_chol_diag<<<nsys, 1024, 0, side>>>(d_lay, nsys, J + 1, poolL, poolU, st); GENEO_COUNT_LAUNCH();
+    k_chol_trsm<<<dim3(nsys, w_max), 256, 0, side>>>(d_lay, nsys, J + 1, poolL, poolU); GENEO_COUNT_LAUNCH();
+    if ((rc = launch_update(d_lay, nsys, J, w_max, poolL, 2, st, s))) return rc;
     GENEO_CUDA_TRY(cudaEventRecord(e_side, side));
     GENEO_CUDA_TRY(cudaStreamWaitEvent(s, e_side, 0));
   }
@@ -300,18 +278,6 @@ int launch_band_cholesky(const BandLayout *d_lay, int nsys, int nt_max, int w_ma
   cudaEventDestroy(e_side);
   GENEO_CUDA_TRY(cudaGetLastError());
   return GENEO_OK;
-}
-
-// The GenEO eigensolver's multi-right-hand-side solves run the one-CTA
-// look-ahead sweep of the local solves (schwarz.cu), one CTA per (system,
-// right-hand side), the column in shared memory, or streamed through a ring
-// of tile rows when it does not fit.
-int launch_band_solve_dense(const BandLayout *d_lay, int nsys, int npad_max, int w_max,
-                            int ring, const double *poolL, const double *poolU, const double *in,
-                            long long in_sys, int in_row, double *out, long long out_sys,
-                            int out_row, int ncols, int mode, cudaStream_t s) {
-  return launch_band_solve_la(d_lay, nsys, npad_max, w_max, ring, poolL, poolU, in, in_sys,
-                              in_row, out, out_sys, out_row, ncols, mode, s);
 }
 
 template <typename T>
@@ -327,10 +293,6 @@ int launch_extract_interior(const SubDesc *d_subs, const BandLayout *d_lay, int 
 
 template int launch_band_clear<double>(const BandLayout *, int, double *, long long, cudaStream_t);
 template int launch_band_clear<float>(const BandLayout *, int, float *, long long, cudaStream_t);
-template int launch_band_cholesky<double>(const BandLayout *, int, int, int, double *, double *,
-                                          DevStatus *, cudaStream_t, cudaStream_t);
-template int launch_band_cholesky<float>(const BandLayout *, int, int, int, float *, float *,
-                                         DevStatus *, cudaStream_t, cudaStream_t);
 template int launch_extract_interior<double>(const SubDesc *, const BandLayout *, int, int, int,
                                              int, int, const int32_t *, const double *,
                                              double *, cudaStream_t);

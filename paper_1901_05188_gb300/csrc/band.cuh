@@ -12,33 +12,34 @@ template <typename T>
 int launch_band_clear(const BandLayout *d_lay, int nsys, T *pool, long long pool_elems,
                       cudaStream_t s);
 
-// Right-looking tile Cholesky of nsys band systems held in poolL (lower
+// FP32 right-looking tile Cholesky of nsys band systems held in poolL (lower
 // triangle of each tile row as input).  On exit poolL/poolU hold the forward
 // and backward tile streams described in precond.cuh.  With a side stream the
 // next tile column is factored there while `s` applies the trailing update
 // (the work is ordered by events and complete on `s` at return).
-template <typename T>
-int launch_band_cholesky(const BandLayout *d_lay, int nsys, int nt_max, int w_max, T *poolL,
-                         T *poolU, DevStatus *st, cudaStream_t s, cudaStream_t side = nullptr);
+int launch_band_cholesky32(const BandLayout *d_lay, int nsys, int nt_max, int w_max, float *poolL,
+                           float *poolU, DevStatus *st, cudaStream_t s, cudaStream_t side = nullptr);
 
-// Solve with ncols right-hand sides per system.  Column c of system j lives at
-// in[j*in_sys + l*in_row + c] (l = 0..n-1); the result goes to
-// out[j*out_sys + l*out_row + c] for l < n (padding rows are not written).
-// In-place use (in == out with equal strides) is allowed.
+// FP64 left-looking tile Cholesky on the tensor cores (digits.cuh): the same
+// result in poolL and, unless it is null, poolU, and the factor's digits in D
+// (in the whole-band form, what launch_band_solve64 reads).  With a side
+// stream the two halves of the systems are factored concurrently.
+int launch_band_cholesky64(const BandLayout *d_lay, int nsys, int nt_max, int w_max, double *poolL,
+                           double *poolU, const DigitBand &D, DevStatus *st, cudaStream_t s,
+                           cudaStream_t side = nullptr);
+
+// Solve with ncols right-hand sides per system from the digits of the factor.
+// Column c of system j lives at in[j*in_sys + l*in_row + c] (l = 0..n-1); the
+// result goes to out[j*out_sys + l*out_row + c] for l < n (padding rows are not
+// written).  In-place use (in == out with equal strides) is allowed.
 // mode: 1 forward (L), 2 backward (L^T), 3 both.  w_max: the largest tile
-// half-bandwidth; ring = 1 streams every column through a ring of max(w + 2, 3)
-// tile rows in shared memory (chosen anyway when a whole column does not fit).
-int launch_band_solve_dense(const BandLayout *d_lay, int nsys, int npad_max, int w_max,
-                            int ring, const double *poolL, const double *poolU, const double *in,
-                            long long in_sys, int in_row, double *out, long long out_sys,
-                            int out_row, int ncols, int mode, cudaStream_t s);
-
-// The same solve with the one-CTA look-ahead sweep of the local solves.
-int launch_band_solve_la(const BandLayout *d_lay, int nsys, int npad_max, int w_max, int ring,
-                         const double *poolL, const double *poolU, const double *in,
-                         long long in_sys, int in_row, double *out, long long out_sys,
-                         int out_row, int ncols, int mode, cudaStream_t s);
-// Whether the ring form of the band solve fits for tile half-bandwidth w_max.
+// half-bandwidth; scratch: band_solve_scratch(nsys, w_max, ncols) bytes.
+size_t band_solve_scratch(int nsys, int w_max, int ncols);
+int launch_band_solve64(const BandLayout *d_lay, int nsys, int w_max, const DigitBand &D,
+                        void *scratch, const double *in, long long in_sys, int in_row, double *out,
+                        long long out_sys, int out_row, int ncols, int mode, DevStatus *st,
+                        cudaStream_t s);
+// Widest half-bandwidth (in tiles) the set-up accepts for the eigensolver.
 bool band_solve_fits(int w_max);
 
 // FP32 trailing update of tile column J on the tensor cores (3xTF32 tcgen05

@@ -1,0 +1,791 @@
+// FP64 band Cholesky and the band solves with several right-hand sides, on the
+// tensor cores by exact digit products (digits.cuh):
+// the shift-invert operators of the GenEO eigenproblems (Sec. 3.3.2), the
+// FP64 subdomain factors (Sec. 3.1) and the coarse matrix (Sec. 3.3.3).  The paper
+// factors with a sparse direct solver (UMFPack); here every matrix is a band in
+// a box numbering whose longest axis runs slowest, held as dense 32 x 32 tiles,
+// with the diagonal blocks stored inverted so that triangular sweeps are
+// streams of small products.
+//
+// Both were bound by the FP64 pipe (128 shifted Neumann matrices of
+// about 16,000 unknowns and half-bandwidth 905: 1.31 s per factorisation, 32 ms
+// per sweep with eight right-hand sides).
+#include <algorithm>
+
+#include "band.cuh"
+#include "digits.cuh"
+
+namespace geneo {
+
+namespace {
+
+__device__ __forceinline__ double *tile_ptr(double *base, const BandLayout &L, int I, int d) {
+  return base + L.off + (((long long)I * (L.w + 1) + d) << 10);
+}
+
+// Tile (I, d) of system j in the digit pool: the whole band, or only the w + 1
+// tile rows the factorisation can still touch (row I in slot I mod (w + 1)).
+__device__ __forceinline__ __half *dig_tile(const DigitBand &D, const BandLayout &L, int j, int I,
+                                            int d) {
+  const long long t = D.window ? (long long)j * D.window + (long long)(I % (L.w + 1)) * (L.w + 1) + d
+                               : (L.off >> 10) + (long long)I * (L.w + 1) + d;
+  return static_cast<__half *>(D.pool) + t * kDigTile;
+}
+
+// Scale of row i of the factor: |L_ik| <= sqrt(a_ii) < 2^E.
+__global__ void k_row_exps(const BandLayout *lay, int sys0, double *poolL, DigitBand D) {
+  const int j = sys0 + blockIdx.y;
+  const BandLayout L = lay[j];
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= L.nt * 32) return;
+  const double a = tile_ptr(poolL, L, i >> 5, 0)[(i & 31) * 33];
+  const int e = a > 0.0 ? exp_above(a) : 0;
+  D.rexp[(long long)j * D.npad + i] = e == kNoExp ? 0 : (e + 1) >> 1;
+}
+
+// Adds the products of one K tile to the integer sums of a 16 x 16 block: rows
+// m0 of tile a times rows n0 of tile b (both in shared memory, [row][k] digit
+// slices), eight columns at a time to stay within 128 registers.
+__device__ __forceinline__ void block_product(long long (&hi)[8], long long (&lo)[8], uint32_t a,
+                                              uint32_t b, int m0, int n0, int lane) {
+  __syncwarp();
+#pragma unroll
+  for (int nb = 0; nb < 2; ++nb) {
+    float S[kDig][4];
+#pragma unroll
+    for (int l = 0; l < kDig; ++l)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) S[l][e] = 0.f;
+#pragma unroll
+    for (int kb = 0; kb < 2; ++kb) {
+      uint32_t br[kDig][2];
+      const uint32_t ab = a + ldsm_a(m0, 16 * kb, lane), bb = b + ldsm_b(n0 + 8 * nb, 16 * kb, lane);
+#pragma unroll
+      for (int t = 0; t < kDig; ++t) ldsm2(br[t], bb + t * 2048);
+#pragma unroll
+      for (int s = 0; s < kDig; ++s) {
+        uint32_t ar[4];
+        ldsm4(ar, ab + s * 2048);
+#pragma unroll
+        for (int t = 0; t < kDig - s; ++t) mma_f16(S[s + t], ar, br[t][0], br[t][1]);
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      long long h, l;
+      level_parts(S, e, h, l);
+      hi[4 * nb + e] += h;
+      lo[4 * nb + e] += l;
+    }
+  }
+}
+// Row and column of entry e (0..7) of a lane's 16 x 16 block.
+__device__ __forceinline__ int blk_row(int e, int lane) { return (lane >> 2) + 8 * ((e >> 1) & 1); }
+__device__ __forceinline__ int blk_col(int e, int lane) { return 2 * (lane & 3) + (e & 1) + 8 * (e >> 2); }
+
+// Digits of a row-major 32 x 32 block in shared memory (row stride 33), rows
+// [r0, r0 + n): one warp, lane = column; scale 2^G per row, its own maximum
+// (G written to rowexp) or the given one.
+template <bool kOwn>
+__device__ __forceinline__ bool slice_rows(const double *v, int r0, int n, int *rowexp, __half *dst,
+                                           int lane) {
+  bool finite = true;
+  for (int r = r0; r < r0 + n; ++r) {
+    const double x = v[r * 33 + lane];
+    const int ex = exp_above(x);
+    finite = finite && ex < 1025;
+    int G;
+    if (kOwn) {
+      G = __reduce_max_sync(0xffffffffu, ex);
+      if (lane == 0) rowexp[r] = G;
+    } else {
+      G = rowexp[r];
+    }
+    const long long xb = fixed62(x, G) + kDigBias;
+    __half *o = dst + dig_index(r, lane);
+#pragma unroll
+    for (int s = 0; s < kDig; ++s) o[s * 1024] = digit_half(xb, s);
+  }
+  return finite;
+}
+
+__device__ __forceinline__ void not_spd(DevStatus *st, int j, int detail) {
+  if (atomicCAS(&st->code, 0, GENEO_ERR_NOT_SPD) == 0) {
+    st->where = j;
+    st->detail = detail;
+  }
+}
+
+// 1 / d for d > 0 (single-precision estimate, one third-order step: the error
+// of the estimate, 2^-23, to the third power).
+__device__ __forceinline__ double inv_pos(double d) {
+  if (!(d >= 1e-30 && d <= 1e30)) return 1.0 / d;     // outside float range: exact path
+  const double r = (double)__frcp_rn((float)d);
+  const double e = fma(-d, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+// 1 / sqrt(d), d > 0: Newton's iteration for 1 / y^2 - d from a single-precision estimate.
+__device__ __forceinline__ double inv_sqrt(double d) {
+  if (!(d >= 1e-30 && d <= 1e30)) return 1.0 / sqrt(d);
+  double y = (double)rsqrtf((float)d);
+  y = y * (1.5 - 0.5 * d * y * y);
+  return y * (1.5 - 0.5 * d * y * y);
+}
+
+// Diagonal tile J of every system: the last update (K = J - 1; the earlier ones
+// were applied by the previous panel launch), then L D L^T and the inverse of
+// the unit factor together, one elimination step per column.  Four warps, one
+// per SM sub-partition; lane = row, warp w owns columns 4 q + w.  The FP64
+// pipe takes 64 cycles per warp instruction, so a step costs its eight updates
+// (the entries of L right of the pivot and of the inverse left of it); the
+// warp that owns the next column publishes it and its reciprocal pivot before
+// its other updates.  The
+// kernel that stood here before (one entry per thread, three barriers per
+// column, the inverse afterwards) took 44 us a launch.
+__global__ void __launch_bounds__(128)
+    k_dchol_diag(const BandLayout *lay, int sys0, int J, double *poolL, double *poolU, DigitBand D,
+                 DevStatus *st) {
+  const int j = sys0 + blockIdx.x;
+  const BandLayout L = lay[j];
+  if (J >= L.nt) return;
+  __shared__ __align__(16) __half dg[kDigTile];
+  __shared__ double A[32 * 33];
+  __shared__ double colv[32][32];
+  __shared__ double rinv[32];
+  __shared__ int ex[32];
+  __shared__ int bad;
+  const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+  double *t = tile_ptr(poolL, L, J, 0);
+  for (int e = tid; e < 1024; e += 128) A[(e & 31) * 33 + (e >> 5)] = t[e];
+  if (tid == 0) bad = -1;
+  const bool upd = J > 0 && L.w > 0;
+  if (upd) {
+    const uint4 *src = reinterpret_cast<const uint4 *>(dig_tile(D, L, j, J, 1));
+    for (int e = tid; e < kDigTile / 8; e += 128) reinterpret_cast<uint4 *>(dg)[e] = src[e];
+    if (tid < 32) ex[tid] = D.rexp[(long long)j * D.npad + J * 32 + tid];
+  }
+  __syncthreads();
+  if (upd) {
+    const int m0 = 16 * (w >> 1), n0 = 16 * (w & 1);
+    if (m0 >= n0) {                         // the lower triangle
+      long long hi[8], lo[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) hi[e] = lo[e] = 0;
+      block_product(hi, lo, dig_smem(dg), dig_smem(dg), m0, n0, lane);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const int r = m0 + blk_row(e, lane), c = n0 + blk_col(e, lane);
+        A[r * 33 + c] -= parts_value(hi[e], lo[e], ex[r] + ex[c]);
+      }
+    }
+    __syncthreads();
+  }
+  double a[8], x[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    a[q] = A[lane * 33 + 4 * q + w];
+    x[q] = lane == 4 * q + w ? 1.0 : 0.0;
+  }
+  auto publish = [&](int k, double v) {     // column k, final, and its reciprocal pivot
+    colv[k][lane] = v;
+    if (lane == k) {
+      double d = v;
+      if (!(d > 0.0)) {
+        if (bad < 0) bad = J * 32 + k;
+        d = 1.0;
+        colv[k][lane] = d;
+      }
+      rinv[k] = inv_pos(d);
+    }
+  };
+  if (w == 0) publish(0, a[0]);
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < 32; ++k) {
+    const int kq = k >> 2, kw = k & 3;
+    const double li = lane > k ? colv[k][lane] * rinv[k] : 0.0;
+    const bool own = k + 1 < 32 && w == ((k + 1) & 3);
+    if (own) {
+      const int q = (k + 1) >> 2;
+      a[q] = fma(-li, colv[k][k + 1], a[q]);
+      publish(k + 1, a[q]);
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      if (q > kq || (q == kq && w > kw)) {
+        if (!(own && q == ((k + 1) >> 2))) a[q] = fma(-li, colv[k][4 * q + w], a[q]);
+      } else {
+        x[q] = fma(-li, __shfl_sync(0xffffffffu, x[q], k), x[q]);
+      }
+    }
+    __syncthreads();
+  }
+  const double rs = inv_sqrt(colv[lane][lane]);
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 8; ++q) A[lane * 33 + 4 * q + w] = x[q] * rs;      // inv(L_JJ)
+  __syncthreads();
+  for (int e = tid; e < 1024; e += 128) t[e] = A[(e & 31) * 33 + (e >> 5)];
+  if (poolU) {
+    double *u = tile_ptr(poolU, L, J, 0);
+    for (int e = tid; e < 1024; e += 128) u[e] = A[(e >> 5) * 33 + (e & 31)];
+  }
+  const bool finite = slice_rows<true>(A, 8 * w, 8, ex, dg, lane);
+  if (!finite) bad = J * 32;
+  __syncthreads();
+  uint4 *dst = reinterpret_cast<uint4 *>(dig_tile(D, L, j, J, 0));
+  for (int e = tid; e < kDigTile / 8; e += 128) dst[e] = reinterpret_cast<const uint4 *>(dg)[e];
+  if (tid < 32) D.dexp[(long long)j * D.npad + J * 32 + tid] = ex[tid];
+  if (tid == 0 && bad >= 0) not_spd(st, j, bad);
+}
+
+// Panel of tile column J, left-looking: blockIdx.y = p takes the tiles (I, J),
+// I = J + 2p + 1 and the next, subtracts sum_K L_IK L_JK^double over the band's
+// columns K < J, multiplies by inv(L_JJ)^T (digits again) and writes the
+// factor's FP64 tiles and digits.  The last block row instead applies the
+// columns K < J to the diagonal tile J + 1, so that the next diagonal launch
+// has one tile product left.  Eight warps, 16 x 16 entries each; the K tiles
+// come through two shared-memory stages, one copied while the other is used.  Left-looking: the
+// products of all K are summed as integers in registers, and each tile of A
+// is read and written once (the right-looking FP64 update read and wrote the
+// whole trailing triangle for every tile column).
+constexpr int kPanStages = 2;
+constexpr int kPanSmem = (3 * kPanStages + 1) * (int)kDigBytes;
+
+__global__ void __launch_bounds__(256, 2)
+    k_dchol_panel(const BandLayout *lay, int sys0, int J, double *poolL, double *poolU, DigitBand D,
+                  DevStatus *st) {
+  const int j = sys0 + blockIdx.x;
+  const BandLayout L = lay[j];
+  if (J >= L.nt || L.w == 0) return;
+  const bool ahead = blockIdx.y == gridDim.y - 1;
+  const int I0 = ahead ? J + 1 : J + 2 * blockIdx.y + 1;
+  if (I0 >= L.nt || I0 - J > L.w) return;
+  const bool two = !ahead && I0 + 1 < L.nt && I0 + 1 - J <= L.w;
+  extern __shared__ __align__(128) unsigned char smraw[];
+  __shared__ int rexp_s[64], rowe[64], cexp_s[32], dexp_s[32];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tt = warp >> 2, m0 = 16 * ((warp >> 1) & 1), n0 = 16 * (warp & 1);
+  const int K0 = max(0, I0 - L.w), nK = J - K0;
+  // steps: one K each, or two for the look-ahead tile (each half of the warps takes one)
+  const int nstep = ahead ? (nK + 1) / 2 : nK;
+  const uint32_t sm = dig_smem(smraw);
+  __half *dinv = reinterpret_cast<__half *>(smraw + 3 * kPanStages * kDigBytes);
+  auto tile_in = [&](uint32_t dst, const __half *src) {
+    for (int e = tid; e < kDigTile / 8; e += 256) cp16(dst + 16 * e, src + 8 * e);
+  };
+  auto prefetch = [&](int it) {
+    const uint32_t sp = sm + (it % kPanStages) * 3 * kDigBytes;
+    if (ahead) {
+      const int K = K0 + 2 * it;
+      tile_in(sp, dig_tile(D, L, j, I0, I0 - K));
+      if (K + 1 < J) tile_in(sp + kDigBytes, dig_tile(D, L, j, I0, I0 - K - 1));
+    } else {
+      const int K = K0 + it;
+      tile_in(sp, dig_tile(D, L, j, I0, I0 - K));
+      if (two && I0 + 1 - K <= L.w) tile_in(sp + kDigBytes, dig_tile(D, L, j, I0 + 1, I0 + 1 - K));
+      tile_in(sp + 2 * kDigBytes, dig_tile(D, L, j, J, J - K));
+    }
+  };
+  if (!ahead) tile_in(dig_smem(dinv), dig_tile(D, L, j, J, 0));
+  if (nstep > 0) prefetch(0);
+  cp_commit();
+  const long long eb = (long long)j * D.npad;
+  if (tid < 64) rexp_s[tid] = (tid < 32 || two) ? D.rexp[eb + I0 * 32 + tid] : 0;
+  if (tid < 32) {
+    cexp_s[tid] = D.rexp[eb + (ahead ? I0 : J) * 32 + tid];
+    dexp_s[tid] = D.dexp[eb + J * 32 + tid];
+  }
+  long long hi[8], lo[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) hi[e] = lo[e] = 0;
+  for (int it = 0; it < nstep; ++it) {
+    if (it + 1 < nstep) prefetch(it + 1);
+    cp_commit();
+    cp_wait<1>();
+    __syncthreads();                        // the stage has landed
+    const uint32_t sp = sm + (it % kPanStages) * 3 * kDigBytes;
+    if (ahead) {
+      if (K0 + 2 * it + tt < J && m0 >= n0)
+        block_product(hi, lo, sp + tt * kDigBytes, sp + tt * kDigBytes, m0, n0, lane);
+    } else if (tt == 0 || (two && I0 + 1 - (K0 + it) <= L.w)) {
+      block_product(hi, lo, sp + tt * kDigBytes, sp + 2 * kDigBytes, m0, n0, lane);
+    }
+    __syncthreads();                        // the stage is free
+  }
+  cp_wait<0>();
+  __syncthreads();
+  if (ahead) {
+    // the two halves' sums, then A(J+1, J+1) -= U
+    long long *sh = reinterpret_cast<long long *>(smraw);
+    if (tt == 1)
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        sh[(2 * e) * 128 + (tid & 127)] = hi[e];
+        sh[(2 * e + 1) * 128 + (tid & 127)] = lo[e];
+      }
+    __syncthreads();
+    if (tt == 0 && m0 >= n0) {
+      double *t = tile_ptr(poolL, L, I0, 0);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const int r = m0 + blk_row(e, lane), c = n0 + blk_col(e, lane);
+        t[c * 32 + r] -= parts_value(hi[e] + sh[(2 * e) * 128 + tid], lo[e] + sh[(2 * e + 1) * 128 + tid],
+                                     rexp_s[r] + cexp_s[c]);
+      }
+    }
+  } else {
+    double *R = reinterpret_cast<double *>(smraw);                              // [2][32][33]
+    __half *dg = reinterpret_cast<__half *>(smraw + 2 * 32 * 33 * 8);           // [2] digit tiles
+    double *Rt = R + tt * 32 * 33;
+    const bool mine = tt == 0 || two;
+    const int I = I0 + tt;
+    if (mine) {
+      const double *t = tile_ptr(poolL, L, I, I - J);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const int r = m0 + blk_row(e, lane), c = n0 + blk_col(e, lane);
+        Rt[r * 33 + c] = t[c * 32 + r] - parts_value(hi[e], lo[e], rexp_s[32 * tt + r] + cexp_s[c]);
+      }
+    }
+    __syncthreads();
+    bool finite = true;
+    if (mine) finite = slice_rows<true>(Rt, 8 * (warp & 3), 8, rowe + 32 * tt, dg + tt * kDigTile, lane);
+    __syncthreads();
+    if (mine) {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) hi[e] = lo[e] = 0;
+      block_product(hi, lo, dig_smem(dg + tt * kDigTile), dig_smem(dinv), m0, n0, lane);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const int r = m0 + blk_row(e, lane), c = n0 + blk_col(e, lane);
+        Rt[r * 33 + c] = parts_value(hi[e], lo[e], rowe[32 * tt + r] + dexp_s[c]);
+      }
+    }
+    __syncthreads();
+    if (mine) {
+      const int t4 = tid & 127;
+      double *tl = tile_ptr(poolL, L, I, I - J);
+      for (int e = t4; e < 1024; e += 128) tl[e] = Rt[(e & 31) * 33 + (e >> 5)];
+      if (poolU) {
+        double *tu = tile_ptr(poolU, L, J, I - J);
+        for (int e = t4; e < 1024; e += 128) tu[e] = Rt[(e >> 5) * 33 + (e & 31)];
+      }
+      finite = slice_rows<false>(Rt, 8 * (warp & 3), 8, rexp_s + 32 * tt, dg + tt * kDigTile, lane) && finite;
+      if (!finite) not_spd(st, j, J * 32);
+    }
+    __syncthreads();
+    if (mine) {
+      uint4 *dst = reinterpret_cast<uint4 *>(dig_tile(D, L, j, I, I - J));
+      const uint4 *src = reinterpret_cast<const uint4 *>(dg + tt * kDigTile);
+      for (int e = tid & 127; e < kDigTile / 8; e += 128) dst[e] = src[e];
+    }
+  }
+}
+
+// ---- band solves with up to eight right-hand sides per CTA --------------------
+// One CTA per (system, group of eight columns).  Row I needs
+// s = b_I - sum_{d=1..w} L(I, I-d) y_{I-d} and y_I = inv(L_II) s; backward the
+// transposes.  While the four chain warps finish row I (the coupling d = 1, the
+// inverse diagonal block), the eight far warps multiply the tiles d >= 2 of the
+// next row, which need only rows solved before; a pair of them takes one tile,
+// 16 rows each, with the digits of L read by ldmatrix (transposed for the
+// backward sweep, so one copy of the factor serves both) and those of y in
+// fragment order.  Every row block of y has one scale per column; sums over
+// tiles of different scales are aligned by shifting the integers.  Each far
+// warp copies its halves of the tiles into two private stages, the next one in
+// flight while one is multiplied, across rows; the chain warps refill their two
+// tiles as soon as they have been read.  The window of y digits (w + 2 row
+// blocks) lives in global scratch, read through L1.
+// Bound: streaming the digit tiles (14 KB each) once per sweep for many
+// systems, the chain (about 1.3 us a row) for few or narrow ones.
+constexpr int kSwChain = 4, kSwFar = 8;
+constexpr int kSwThreads = (kSwChain + kSwFar) * 32;
+constexpr int kSwHalf = kDigBytes / 2;      // a far warp's half of a tile
+constexpr int kSwCol = 36;                  // row stride of a column of partial sums
+constexpr int kSwPart = 8 * kSwCol;         // one 32 x 8 block of them
+constexpr int kSwY = kDig * 128;            // words of one row block of y digits
+__host__ __device__ constexpr int sweep_smem(int w) {
+  return 2 * (int)kDigBytes + kSwFar * 2 * kSwHalf + (2 * 4 + 2) * kSwPart * 16 + 3 * kSwY * 4 +
+         (w + 2) * 32 + (2 * 4 * 8 + 2 * 8) * 4;
+}
+
+__device__ __forceinline__ void sw_bar_all() {
+  __syncwarp();                             // bar.sync is .aligned: converge first
+  asm volatile("bar.sync 1, %0;" ::"n"((kSwChain + kSwFar) * 32) : "memory");
+}
+__device__ __forceinline__ void sw_bar_chain() {
+  __syncwarp();
+  asm volatile("bar.sync 2, %0;" ::"n"(kSwChain * 32) : "memory");
+}
+
+// hi 2^27 + lo, divided by 2^sh, added to the pair (hs, ls).
+__device__ __forceinline__ void add_shifted(long long hi, long long lo, int sh, long long &hs,
+                                            long long &ls) {
+  const int s = min(sh, 62);
+  const long long a = hi >> s, rem = hi - (a << s);          // 0 <= rem < 2^s
+  hs += a;
+  ls += s <= 30 ? ((rem << 27) + lo) >> s : (rem >> (s - 27)) + (lo >> s);
+}
+
+struct SweepArgs {
+  const BandLayout *lay;
+  DigitBand D;
+  uint4 *ring;                              // y digits: [CTA][w_max + 2][kSwY / 4]
+  int w_max;
+  const double *in;
+  long long in_sys;
+  int in_row;
+  double *out;
+  long long out_sys;
+  int out_row, ncols, mode;
+  DevStatus *st;
+};
+
+__global__ void __launch_bounds__(kSwThreads, 1) k_band_sweep(const SweepArgs P) {
+  extern __shared__ __align__(128) unsigned char smraw[];
+  const int j = blockIdx.x, grp = blockIdx.y;
+  const BandLayout L = P.lay[j];
+  const int nt = L.nt, w = L.w, slots = w + 2;
+  unsigned char *chain_t = smraw;                                   // [near, diagonal]
+  unsigned char *far_t = chain_t + 2 * kDigBytes;                   // [warp][2] half tiles
+  long long *part = reinterpret_cast<long long *>(far_t + kSwFar * 2 * kSwHalf);  // [2][4][hi, lo]
+  long long *nearp = part + 2 * 4 * 2 * kSwPart;                    // [2][hi, lo]
+  uint32_t *sdig = reinterpret_cast<uint32_t *>(nearp + 2 * 2 * kSwPart);
+  uint32_t *ydig = sdig + kSwY;                                     // [2]
+  int *fexp = reinterpret_cast<int *>(ydig + 2 * kSwY);             // [w + 2][8]
+  int *cmax = fexp + (P.w_max + 2) * 8;                             // [2][4][8]
+  int *fref = cmax + 2 * 4 * 8;                                     // [2][8]
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  uint4 *yring = P.ring + ((long long)grp * gridDim.x + j) * (P.w_max + 2) * (kSwY / 4);
+  for (int back = 0; back < 2; ++back) {
+    if (!(P.mode & (1 << back))) continue;
+    auto row = [&](int q) { return back ? nt - 1 - q : q; };
+    auto dmax = [&](int I) { return back ? min(w, nt - 1 - I) : min(w, I); };
+    if (warp >= kSwChain) {
+      // ---- far warps
+      const int fw = warp - kSwChain, p = fw >> 1, m0 = 16 * (fw & 1), g = lane >> 2, t2 = 2 * (lane & 3);
+      const uint32_t st0 = dig_smem(far_t) + fw * 2 * kSwHalf;
+      // This warp's half of a tile: rows m0.. (forward; 1 KB of every slice), or
+      // columns m0.. (backward; two 16-byte chunks of every row, kept at
+      // 32 bytes a row: chunk c of row r at (c ^ (r >> 2)) & 1, against bank
+      // conflicts in ldmatrix).
+      auto load = [&](int stage, int I, int d) {
+        const char *src = reinterpret_cast<const char *>(dig_tile(P.D, L, j, back ? I + d : I, d));
+        const uint32_t dst = st0 + stage * kSwHalf;
+#pragma unroll
+        for (int k = 0; k < 14; ++k) {
+          const int e = k * 32 + lane, s = e >> 6, i = e & 63;
+          if (back) {
+            const int r = i >> 1, c = i & 1;
+            cp16(dst + s * 1024 + r * 32 + ((c ^ (r >> 2)) & 1) * 16,
+                 src + s * 2048 + r * 64 + (((((m0 >> 3) + c) ^ (r >> 1)) & 3) << 4));
+          } else {
+            cp16(dst + s * 1024 + i * 16, src + s * 2048 + m0 * 64 + i * 16);
+          }
+        }
+      };
+      // the warp's tiles in order: rows 1.. of the sweep, u = p, p + 4, ... of each
+      int pq = 0, pu = p, pn = 0;             // next tile to load: row q = pq, index pu of pn
+      auto advance = [&]() {                  // to the next row that has one; false at the end
+        while (pu >= pn) {
+          if (++pq >= nt) return false;
+          pn = max(dmax(row(pq)) - 1, 0);
+          pu = p;
+        }
+        return true;
+      };
+      int stage = 0;
+      if (advance()) {
+        load(0, row(pq), 2 + pu);
+        pu += 4;
+      }
+      cp_commit();
+      for (int q = 0; q < nt; ++q) {
+        if (q + 1 < nt) {
+          const int In = row(q + 1), n = max(dmax(In) - 1, 0);
+          // the largest scale of the window, per column
+          int fr = kNoExp;
+          for (int u = lane >> 3; u < n; u += 4) {
+            const int K = back ? In + 2 + u : In - 2 - u;
+            fr = max(fr, fexp[(K % slots) * 8 + (lane & 7)]);
+          }
+          fr = max(fr, __shfl_xor_sync(0xffffffffu, fr, 8));
+          fr = max(fr, __shfl_xor_sync(0xffffffffu, fr, 16));
+          const int fr0 = __shfl_sync(0xffffffffu, fr, t2), fr1 = __shfl_sync(0xffffffffu, fr, t2 + 1);
+          long long hs[4] = {0, 0, 0, 0}, ls[4] = {0, 0, 0, 0};
+          for (int u = p; u < n; u += 4) {
+            const int K = back ? In + 2 + u : In - 2 - u, slot = K % slots;
+            uint4 yb[kDig];
+            const uint4 *yp = yring + (long long)slot * (kSwY / 4) + lane;
+#pragma unroll
+            for (int t = 0; t < kDig; ++t) yb[t] = yp[t * 32];
+            const int2 fk = *reinterpret_cast<const int2 *>(fexp + slot * 8 + t2);
+            if (advance()) {
+              load(stage ^ 1, row(pq), 2 + pu);
+              pu += 4;
+            }
+            cp_commit();
+            cp_wait<1>();
+            __syncwarp();                     // this tile has landed, for every lane
+            const uint32_t at = st0 + stage * kSwHalf;
+            float S[kDig][4];
+#pragma unroll
+            for (int l = 0; l < kDig; ++l)
+#pragma unroll
+              for (int e = 0; e < 4; ++e) S[l][e] = 0.f;
+#pragma unroll
+            for (int kb = 0; kb < 2; ++kb) {
+              const int r = 16 * kb + (lane & 7) + 8 * (lane >> 4);
+              const uint32_t ab = at + (back ? r * 32 + (((lane >> 3) ^ (r >> 2)) & 1) * 16
+                                             : ldsm_a(0, 16 * kb, lane));
+#pragma unroll
+              for (int s = 0; s < kDig; ++s) {
+                uint32_t ar[4];
+                if (back) ldsm4_trans(ar, ab + s * 1024);
+                else ldsm4(ar, ab + s * 1024);
+#pragma unroll
+                for (int t = 0; t < kDig - s; ++t)
+                  mma_f16(S[s + t], ar, kb ? yb[t].z : yb[t].x, kb ? yb[t].w : yb[t].y);
+              }
+            }
+            __syncwarp();                     // every lane has read the stage
+            stage ^= 1;
+            const int sh0 = fr0 - fk.x, sh1 = fr1 - fk.y;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              long long hi, lo;
+              level_parts(S, e, hi, lo);
+              add_shifted(hi, lo, (e & 1) ? sh1 : sh0, hs[e], ls[e]);
+            }
+          }
+          long long *po = part + (((q + 1) & 1) * 4 + p) * 2 * kSwPart;
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int o = (t2 + (e & 1)) * kSwCol + m0 + g + 8 * (e >> 1);
+            po[o] = hs[e];
+            po[kSwPart + o] = ls[e];
+          }
+          if (fw == 0 && lane < 8) fref[((q + 1) & 1) * 8 + lane] = fr;
+        }
+        sw_bar_all();
+      }
+    } else {
+      // ---- chain warps: thread (rho, c) owns rows 2 rho, 2 rho + 1 of column c
+      const int kb = warp & 1, m0 = 16 * (warp >> 1), c = tid & 7, r0 = 2 * (tid >> 3);
+      const int t2 = 2 * (lane & 3), g = lane >> 2;
+      const int col = grp * 8 + c;
+      const bool live = col < P.ncols;
+      const bool fresh = !(back && (P.mode & 1));
+      const double *src = fresh ? P.in + j * P.in_sys + col : P.out + j * P.out_sys + col;
+      const long long sst = fresh ? P.in_row : P.out_row;
+      double *dst = P.out + j * P.out_sys + col;
+      const int *re = P.D.rexp + (long long)j * P.D.npad, *de = P.D.dexp + (long long)j * P.D.npad;
+      // word of rows (r0, r0 + 1), column c in a row block of digits
+      const int word = (c * 4 + ((r0 & 7) >> 1)) * 4 + 2 * (r0 >> 4) + ((r0 >> 3) & 1);
+      double b0 = 0.0, b1 = 0.0, n0 = 0.0, n1 = 0.0;
+      int2 eR{0, 0}, eD{0, 0};
+      auto fetch = [&](int q, double &v0, double &v1, int2 &er, int2 &ed) {
+        const int l = row(q) * 32 + r0;
+        v0 = live && l < L.n ? src[l * sst] : 0.0;
+        v1 = live && l + 1 < L.n ? src[(l + 1) * sst] : 0.0;
+        er = *reinterpret_cast<const int2 *>(re + l);
+        ed = *reinterpret_cast<const int2 *>(de + l);
+      };
+      fetch(0, b0, b1, eR, eD);
+      const uint32_t tiles = dig_smem(chain_t);
+      auto tile_in = [&](uint32_t dst, int I, int d) {       // a chain tile, by the chain warps
+        const __half *src = dig_tile(P.D, L, j, back ? I + d : I, d);
+#pragma unroll
+        for (int k = 0; k < 7; ++k) cp16(dst + 16 * (k * 128 + tid), src + 8 * (k * 128 + tid));
+      };
+      tile_in(tiles + kDigBytes, row(0), 0);
+      cp_commit();
+      // product of this warp's quarter of a chain tile with a digit block, to nearp[kb]
+      auto product = [&](uint32_t tile, const uint32_t *dig) {
+        __syncwarp();
+        float S[kDig][4];
+        uint2 yb[kDig];
+#pragma unroll
+        for (int l = 0; l < kDig; ++l) {
+          yb[l] = *reinterpret_cast<const uint2 *>(dig + l * 128 + lane * 4 + 2 * kb);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) S[l][e] = 0.f;
+        }
+        const uint32_t ab = tile + (back ? ldsm_at(m0, 16 * kb, lane) : ldsm_a(m0, 16 * kb, lane));
+#pragma unroll
+        for (int s = 0; s < kDig; ++s) {
+          uint32_t ar[4];
+          if (back) ldsm4_trans(ar, ab + s * 2048);
+          else ldsm4(ar, ab + s * 2048);
+#pragma unroll
+          for (int t = 0; t < kDig - s; ++t) mma_f16(S[s + t], ar, yb[t].x, yb[t].y);
+        }
+        long long *po = nearp + kb * 2 * kSwPart;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          long long hi, lo;
+          level_parts(S, e, hi, lo);
+          const int o = (t2 + (e & 1)) * kSwCol + m0 + g + 8 * (e >> 1);
+          po[o] = hi;
+          po[kSwPart + o] = lo;
+        }
+      };
+      // largest exponent of a column over the 32 rows
+      auto col_max = [&](int v, int buf) {
+        v = max(v, __shfl_xor_sync(0xffffffffu, v, 8));
+        v = max(v, __shfl_xor_sync(0xffffffffu, v, 16));
+        int *cm = cmax + buf * 32;
+        if (lane < 8) cm[warp * 8 + lane] = v;
+        sw_bar_chain();
+        return max(max(cm[c], cm[8 + c]), max(cm[16 + c], cm[24 + c]));
+      };
+      const int o = c * kSwCol + r0;
+      for (int q = 0; q < nt; ++q) {
+        const int I = row(q);
+        const bool has1 = dmax(I) >= 1;
+        cp_wait<0>();                         // both tiles, copied during the previous row
+        sw_bar_chain();
+        if (has1) product(tiles, ydig + ((q + 1) & 1) * kSwY);
+        int2 nR{0, 0}, nD{0, 0};
+        if (q + 1 < nt) fetch(q + 1, n0, n1, nR, nD);
+        double s0 = b0, s1 = b1;
+        if (q > 0) {
+          const int ff = fref[(q & 1) * 8 + c];
+          longlong2 h{0, 0}, l{0, 0};
+#pragma unroll
+          for (int p = 0; p < 4; ++p) {
+            const long long *po = part + ((q & 1) * 4 + p) * 2 * kSwPart + o;
+            const longlong2 a = *reinterpret_cast<const longlong2 *>(po);
+            const longlong2 z = *reinterpret_cast<const longlong2 *>(po + kSwPart);
+            h.x += a.x;
+            h.y += a.y;
+            l.x += z.x;
+            l.y += z.y;
+          }
+          s0 -= parts_value(h.x, l.x, ff + (back ? 0 : eR.x));
+          s1 -= parts_value(h.y, l.y, ff + (back ? 0 : eR.y));
+        }
+        sw_bar_chain();
+        // the coupling tile has been read by every chain warp: refill it
+        if (q + 1 < nt && dmax(row(q + 1)) >= 1) tile_in(tiles, row(q + 1), 1);
+        cp_commit();
+        if (has1) {
+          const int fp = fexp[((back ? I + 1 : I - 1) % slots) * 8 + c];
+          const longlong2 ha = *reinterpret_cast<const longlong2 *>(nearp + o),
+                          la = *reinterpret_cast<const longlong2 *>(nearp + kSwPart + o),
+                          hb = *reinterpret_cast<const longlong2 *>(nearp + 2 * kSwPart + o),
+                          lb = *reinterpret_cast<const longlong2 *>(nearp + 3 * kSwPart + o);
+          s0 -= parts_value(ha.x + hb.x, la.x + lb.x, fp + (back ? 0 : eR.x));
+          s1 -= parts_value(ha.y + hb.y, la.y + lb.y, fp + (back ? 0 : eR.y));
+        }
+        // digits of s (backward: the rows of inv(L_II) carry their scales, folded into s)
+        {
+          const int f0 = back ? eD.x : 0, f1 = back ? eD.y : 0;
+          const int G = col_max(max(exp_above(s0) + f0, exp_above(s1) + f1), 0);
+          const long long x0 = fixed62(s0, G - f0) + kDigBias, x1 = fixed62(s1, G - f1) + kDigBias;
+#pragma unroll
+          for (int s = 0; s < kDig; ++s) sdig[s * 128 + word] = digit_pair(x0, x1, s);
+          sw_bar_chain();
+          product(tiles + kDigBytes, sdig);
+          sw_bar_chain();
+          if (q + 1 < nt) tile_in(tiles + kDigBytes, row(q + 1), 0);
+          cp_commit();
+          const longlong2 ha = *reinterpret_cast<const longlong2 *>(nearp + o),
+                          la = *reinterpret_cast<const longlong2 *>(nearp + kSwPart + o),
+                          hb = *reinterpret_cast<const longlong2 *>(nearp + 2 * kSwPart + o),
+                          lb = *reinterpret_cast<const longlong2 *>(nearp + 3 * kSwPart + o);
+          s0 = parts_value(ha.x + hb.x, la.x + lb.x, G + (back ? 0 : eD.x));
+          s1 = parts_value(ha.y + hb.y, la.y + lb.y, G + (back ? 0 : eD.y));
+        }
+        const int l = I * 32 + r0;
+        if (live && l < L.n) dst[(long long)l * P.out_row] = s0;
+        if (live && l + 1 < L.n) dst[(long long)(l + 1) * P.out_row] = s1;
+        // digits of the solved row (backward: scaled by the factor's row scales)
+        {
+          const int f0 = back ? eR.x : 0, f1 = back ? eR.y : 0;
+          const int F = col_max(max(exp_above(s0) + f0, exp_above(s1) + f1), 1);
+          const long long x0 = fixed62(s0, F - f0) + kDigBias, x1 = fixed62(s1, F - f1) + kDigBias;
+          uint32_t *ys = ydig + (q & 1) * kSwY + word;
+          uint32_t *yg = reinterpret_cast<uint32_t *>(yring + (long long)(I % slots) * (kSwY / 4)) + word;
+#pragma unroll
+          for (int s = 0; s < kDig; ++s) {
+            const uint32_t v = digit_pair(x0, x1, s);
+            ys[s * 128] = v;
+            yg[s * 128] = v;
+          }
+          if (r0 == 0) fexp[(I % slots) * 8 + c] = F;
+        }
+        b0 = n0;
+        b1 = n1;
+        eR = nR;
+        eD = nD;
+        sw_bar_all();
+      }
+    }
+  }
+}
+
+}  // namespace
+
+int launch_band_cholesky64(const BandLayout *d_lay, int nsys, int nt_max, int w_max, double *poolL,
+                           double *poolU, const DigitBand &D, DevStatus *st, cudaStream_t s,
+                           cudaStream_t side) {
+  if (int rc = ensure_smem(k_dchol_panel, kPanSmem)) return rc;
+  // Two halves of the systems on two streams: one half's diagonal tiles (a
+  // serial chain on a few warps) run under the other half's panels.
+  const int half = side && nsys >= 2 ? (nsys + 1) / 2 : nsys;
+  struct Events {
+    cudaEvent_t fork = nullptr, join = nullptr;
+    ~Events() {
+      if (fork) cudaEventDestroy(fork);
+      if (join) cudaEventDestroy(join);
+    }
+  } ev;
+  if (half < nsys) {
+    GENEO_CUDA_TRY(cudaEventCreateWithFlags(&ev.fork, cudaEventDisableTiming));
+    GENEO_CUDA_TRY(cudaEventCreateWithFlags(&ev.join, cudaEventDisableTiming));
+    GENEO_CUDA_TRY(cudaEventRecord(ev.fork, s));
+    GENEO_CUDA_TRY(cudaStreamWaitEvent(side, ev.fork, 0));
+  }
+  for (int J = -1; J < nt_max; ++J)
+    for (int h = 0; h < (half < nsys ? 2 : 1); ++h) {
+      const int j0 = h ? half : 0, n = h ? nsys - half : half;
+      cudaStream_t q = h ? side : s;
+      if (J < 0) {
+        k_row_exps<<<dim3((nt_max * 32 + 255) / 256, n), 256, 0, q>>>(d_lay, j0, poolL, D); GENEO_COUNT_LAUNCH();
+        continue;
+      }
+      k_dchol_diag<<<n, 128, 0, q>>>(d_lay, j0, J, poolL, poolU, D, st); GENEO_COUNT_LAUNCH();
+      if (w_max > 0 && J + 1 < nt_max) {
+        const int d = std::min(w_max, nt_max - 1 - J);
+        k_dchol_panel<<<dim3(n, (d + 1) / 2 + 1), 256, kPanSmem, q>>>(d_lay, j0, J, poolL, poolU, D, st); GENEO_COUNT_LAUNCH();
+      }
+    }
+  if (half < nsys) {
+    GENEO_CUDA_TRY(cudaEventRecord(ev.join, side));
+    GENEO_CUDA_TRY(cudaStreamWaitEvent(s, ev.join, 0));
+  }
+  GENEO_CUDA_TRY(cudaGetLastError());
+  return GENEO_OK;
+}
+
+size_t band_solve_scratch(int nsys, int w_max, int ncols) {
+  return (size_t)nsys * ((ncols + 7) / 8) * (w_max + 2) * kSwY * 4;
+}
+
+int launch_band_solve64(const BandLayout *d_lay, int nsys, int w_max, const DigitBand &D,
+                        void *scratch, const double *in, long long in_sys, int in_row, double *out,
+                        long long out_sys, int out_row, int ncols, int mode, DevStatus *st,
+                        cudaStream_t s) {
+  const int sm = sweep_smem(w_max);
+  if (sm > 227 * 1024 || D.window) return GENEO_ERR_INVALID_ARG;
+  if (int rc = ensure_smem(k_band_sweep, sm)) return rc;
+  const SweepArgs P{d_lay, D, static_cast<uint4 *>(scratch), w_max, in, in_sys, in_row, out, out_sys,
+                    out_row, ncols, mode, st};
+  k_band_sweep<<<dim3(nsys, (ncols + 7) / 8), kSwThreads, sm, s>>>(P); GENEO_COUNT_LAUNCH();
+  GENEO_CUDA_TRY(cudaGetLastError());
+  return GENEO_OK;
+}
+
+}  // namespace geneo

@@ -727,6 +727,16 @@ void take_cg_vectors(Arena &A, geneo_ctx *c) {
   c->cg = A.take<CGScalars>(1);
 }
 
+DigitBand take_digits(Arena &A, int nsys, int npad, long long tiles, long long window) {
+  DigitBand D;
+  D.pool = A.take<uint16_t>((size_t)tiles * kDigHalves);
+  D.rexp = A.take<int>((size_t)nsys * npad);
+  D.dexp = A.take<int>((size_t)nsys * npad);
+  D.npad = npad;
+  D.window = window;
+  return D;
+}
+
 void plan_setup(Arena &A, geneo_ctx *c, const SetupPlan &P) {
   Precond &pc = c->pc;
   const int nsub = P.nsub, p = kLanczosBlock;
@@ -747,6 +757,8 @@ void plan_setup(Arena &A, geneo_ctx *c, const SetupPlan &P) {
   pc.xloc = A.take<char>(pc.xloc_elems * esz);
   pc.yloc = A.take<char>(pc.xloc_elems * esz);   // forward-sweep scratch of the ring form
   pc.wloc = A.take<double>(pc.xloc_elems);     // Sarkis weights (filled for that PoU only)
+  const long long win = (long long)(pc.w_int_max + 1) * (pc.w_int_max + 1);
+  pc.dig_int = f32 ? DigitBand{} : take_digits(A, nsub, pc.npad_int_max, win * nsub, win);
   int cap = pc.modes.fixed_modes > 0 ? pc.modes.fixed_modes : pc.modes.max_modes;
   if (pc.coarse == GENEO_COARSE_NONE) cap = 0;
   if (pc.coarse == GENEO_COARSE_ZEM) cap = 6;     // the rigid displacements
@@ -756,12 +768,13 @@ void plan_setup(Arena &A, geneo_ctx *c, const SetupPlan &P) {
   if (cap > 0) {
     const int npad = pc.npad_neu_max;
     const bool eig = pc.coarse == GENEO_COARSE_GENEO;
-    pc.neuL = pc.neuU = pc.Bloc = pc.V = pc.Vt = pc.W = pc.T1 = pc.Hm = nullptr;
+    pc.neuL = pc.Bloc = pc.V = pc.Vt = pc.W = pc.T1 = pc.Hm = nullptr;
+    pc.dig_neu = DigitBand{};
     pc.Racc = pc.Rblk = pc.Evec = pc.Eval = pc.Eres = nullptr;
     pc.gate = nullptr;
     if (eig) {   // shift-invert block Lanczos of the GenEO eigenproblems
       pc.neuL = A.take<double>(pc.fac_neu_elems);
-      pc.neuU = A.take<double>(pc.fac_neu_elems);
+      pc.dig_neu = take_digits(A, nsub, npad, pc.fac_neu_elems / 1024, 0);
       pc.Bloc = A.take<double>((size_t)c->nc * c->nc * pc.bloc_blocks);
       pc.V = A.take<double>((size_t)nsub * npad * (pc.kdim + p));
       pc.Vt = A.take<double>((size_t)nsub * npad * pc.kkeep);
@@ -796,7 +809,10 @@ void plan_setup(Arena &A, geneo_ctx *c, const SetupPlan &P) {
     pc.AH = A.take<double>((size_t)pc.nH_cap * pc.nH_cap);
     pc.AHinv = A.take<double>((size_t)pc.nH_cap * pc.nH_cap);
     pc.AHL = A.take<double>((size_t)ntH * ntH * 1024);
-    pc.AHU = A.take<double>((size_t)ntH * ntH * 1024);
+    pc.dig_H = take_digits(A, 1, ntH * 32, (long long)ntH * ntH, 0);
+    size_t scr = band_solve_scratch(1, ntH - 1, pc.nH_cap);
+    if (eig) scr = std::max(scr, band_solve_scratch(nsub, pc.w_neu_max, std::max(pc.mcap, p)));
+    pc.solve_scr = A.take<char>(scr);
     pc.wpart = A.take<double>((size_t)nsub * restrict_chunks(P.max_nint) * pc.mcap);
     pc.wH = A.take<double>(pc.nH_cap);
     pc.yH = A.take<double>(pc.nH_cap);
@@ -809,11 +825,13 @@ void plan_setup(Arena &A, geneo_ctx *c, const SetupPlan &P) {
     pc.BJ = pc.cwork = nullptr;
     pc.cbar = nullptr;
     pc.c_inner = nullptr;
-    pc.neuL = pc.neuU = pc.Bloc = pc.Xneu = pc.V = pc.Vt = pc.W = pc.T1 = pc.Hm = pc.Hpart = nullptr;
+    pc.neuL = pc.Bloc = pc.Xneu = pc.V = pc.Vt = pc.W = pc.T1 = pc.Hm = pc.Hpart = nullptr;
     pc.Hs = pc.G = pc.Racc = nullptr;
     pc.Rblk = pc.Evec = pc.Eval = pc.Eres = pc.P = pc.Zp = pc.Yp = nullptr;
     pc.gate = nullptr;
-    pc.AH = pc.AHinv = pc.AHL = pc.AHU = pc.wpart = pc.wH = pc.yH = pc.zy = nullptr;
+    pc.AH = pc.AHinv = pc.AHL = pc.wpart = pc.wH = pc.yH = pc.zy = nullptr;
+    pc.dig_neu = pc.dig_H = DigitBand{};
+    pc.solve_scr = nullptr;
     pc.nH_cap = 0;
     pc.z_elems = 0;
   }
@@ -960,8 +978,8 @@ static int setup_coarse(geneo_ctx *c, SetupPlan &P, cudaStream_t s) {
   launch_neumann_assemble(pc.d_subs, pc.d_lay_neu, nsub, P.max_nodes_neu, c->nx, c->ny, c->nz,
                           c->X, c->Y, c->Z, c->Cel, c->perm, pc.d_ecnt, pc.ecnt_off, c->mask,
                           pc.Xneu, sigma, pc.neuL, pc.Bloc, s);
-  if ((st = launch_band_cholesky<double>(pc.d_lay_neu, nsub, pc.nt_neu_max, pc.w_neu_max,
-                                         pc.neuL, pc.neuU, c->status, s, c->side_stream)))
+  if ((st = launch_band_cholesky64(pc.d_lay_neu, nsub, pc.nt_neu_max, pc.w_neu_max, pc.neuL,
+                                   nullptr, pc.dig_neu, c->status, s, c->side_stream)))
     return st;
   // Thick-restart block Lanczos on C = L^-1 B L^-T with full re-orthogonalisation.
   const int ldv = kdim + p;
@@ -1019,13 +1037,17 @@ static int setup_coarse(geneo_ctx *c, SetupPlan &P, cudaStream_t s) {
     double *Racc = pc.Racc + j0 * p * p, *Ri = Rinv + j0 * p * p, *Rblk = pc.Rblk + j0 * p * p;
     int *gate = pc.gate + j0;
     int r;
+    DigitBand D = pc.dig_neu;
+    D.rexp += j0 * D.npad;
+    D.dexp += j0 * D.npad;
+    char *scr = (char *)pc.solve_scr + band_solve_scratch((int)j0, pc.w_neu_max, p);
     // W = L^-1 B L^-T V_k
-    if ((r = launch_band_solve_dense(lay, n, npad, pc.w_neu_max, pc.eig_ring, pc.neuL, pc.neuU,
-                                     V + k * p, sV, ldv, T1, sW, p, p, 2, gs)))
+    if ((r = launch_band_solve64(lay, n, pc.w_neu_max, D, scr, V + k * p, sV, ldv, T1, sW, p, p, 2,
+                                 c->status, gs)))
       return r;
     launch_bloc_mv(subs, n, P.max_nodes_neu, pc.Bloc, T1, W, sW, p, gs);
-    if ((r = launch_band_solve_dense(lay, n, npad, pc.w_neu_max, pc.eig_ring, pc.neuL, pc.neuU, W,
-                                     sW, p, W, sW, p, p, 1, gs)))
+    if ((r = launch_band_solve64(lay, n, pc.w_neu_max, D, scr, W, sW, p, W, sW, p, p, 1, c->status,
+                                 gs)))
       return r;
     const int na = (k + 1) * p;
     // full re-orthogonalisation against V: a second pass only for the
@@ -1124,8 +1146,8 @@ static int setup_coarse(geneo_ctx *c, SetupPlan &P, cudaStream_t s) {
   const long long sP = (long long)npad * mcap;
   launch_tsgemm(pc.d_subs, nsub, npad, pc.V, ldv, sV, kdim, pc.Evec, kdim, (long long)kdim * kdim,
                 pc.P, mcap, sP, mcap, 1.0, 0.0, s);
-  if ((st = launch_band_solve_dense(pc.d_lay_neu, nsub, npad, pc.w_neu_max, pc.eig_ring, pc.neuL,
-                                    pc.neuU, pc.P, sP, mcap, pc.P, sP, mcap, mcap, 2, s)))
+  if ((st = launch_band_solve64(pc.d_lay_neu, nsub, pc.w_neu_max, pc.dig_neu, pc.solve_scr, pc.P, sP,
+                                mcap, pc.P, sP, mcap, mcap, 2, c->status, s)))
     return st;
   launch_tsdots(pc.d_subs, nsub, npad, pc.P, mcap, sP, mcap, pc.P, mcap, sP, mcap, pc.Hpart,
                 kDotChunks, pc.G, (long long)mcap * mcap, s);
@@ -1225,11 +1247,11 @@ static int build_coarse_operator(geneo_ctx *c, SetupPlan &P, const std::vector<l
   GENEO_CUDA_TRY(cudaMemcpyAsync(pc.d_lay_H, &LH, sizeof(LH), cudaMemcpyHostToDevice, s));
   if ((st = launch_band_clear<double>(pc.d_lay_H, 1, pc.AHL, (long long)LH.nt * LH.nt * 1024, s))) return st;
   launch_dense_to_tiles(pc.AH, nH, pc.d_lay_H, pc.AHL, s);
-  if ((st = launch_band_cholesky<double>(pc.d_lay_H, 1, LH.nt, LH.w, pc.AHL, pc.AHU, c->status, s)))
+  if ((st = launch_band_cholesky64(pc.d_lay_H, 1, LH.nt, LH.w, pc.AHL, nullptr, pc.dig_H, c->status, s)))
     return st;
   launch_identity(pc.AHinv, nH, s);
-  if ((st = launch_band_solve_dense(pc.d_lay_H, 1, LH.nt * 32, LH.w, 0, pc.AHL, pc.AHU, pc.AHinv,
-                                    0, nH, pc.AHinv, 0, nH, nH, 3, s)))
+  if ((st = launch_band_solve64(pc.d_lay_H, 1, LH.w, pc.dig_H, pc.solve_scr, pc.AHinv, 0, nH, pc.AHinv,
+                                0, nH, nH, 3, c->status, s)))
     return st;
   launch_symmetrize(pc.AHinv, nH, s);
   GENEO_CUDA_TRY(cudaGetLastError());
@@ -1572,7 +1594,6 @@ int geneo_setup(geneo_ctx *c, const geneo_partition *part, const geneo_modes *mo
   }
   if (pc.coarse == GENEO_COARSE_GENEO && pc.mcap > 1 && !band_solve_fits(pc.w_neu_max))
     return fail(GENEO_ERR_INVALID_ARG, "band too wide for the eigensolver's shared memory");
-  pc.eig_ring = env_choice("GENEO_BAND_SOLVE_RING", {0, 1}) == 1;
   cudaEvent_t ev[4];
   for (auto &e : ev) GENEO_CUDA_TRY(cudaEventCreate(&e));
   GENEO_CUDA_TRY(cudaEventRecord(ev[0], s));
@@ -1613,8 +1634,8 @@ int geneo_setup(geneo_ctx *c, const geneo_partition *part, const geneo_modes *mo
                                              nny, nnz, c->row_ptr, c->val, L, fs)))
       return st;
     GENEO_CUDA_TRY(cudaEventRecord(e_extracted, fs));
-    if ((st = launch_band_cholesky<float>(pc.d_lay_int, P.nsub, pc.nt_int_max, pc.w_int_max, L, U,
-                                          c->status, fs, c->fac_side)))
+    if ((st = launch_band_cholesky32(pc.d_lay_int, P.nsub, pc.nt_int_max, pc.w_int_max, L, U,
+                                     c->status, fs, c->fac_side)))
       return st;
   } else {
     double *L = (double *)pc.facL, *U = (double *)pc.facU;
@@ -1623,8 +1644,8 @@ int geneo_setup(geneo_ctx *c, const geneo_partition *part, const geneo_modes *mo
                                               nnx, nny, nnz, c->row_ptr, c->val, L, fs)))
       return st;
     GENEO_CUDA_TRY(cudaEventRecord(e_extracted, fs));
-    if ((st = launch_band_cholesky<double>(pc.d_lay_int, P.nsub, pc.nt_int_max, pc.w_int_max, L,
-                                           U, c->status, fs, c->fac_side)))
+    if ((st = launch_band_cholesky64(pc.d_lay_int, P.nsub, pc.nt_int_max, pc.w_int_max, L, U,
+                                     pc.dig_int, c->status, fs, c->fac_side)))
       return st;
   }
   GENEO_CUDA_TRY(cudaEventRecord(ev[2], fs));
@@ -2006,8 +2027,14 @@ extern "C" int geneo_debug_local_matrix(geneo_ctx *c, int sub, int kind, double 
     GENEO_CUDA_TRY(cudaMallocAsync(&tmp, el * sizeof(double), s));
     GENEO_CUDA_TRY(cudaMallocAsync(&dl, sizeof(BandLayout), s));
     GENEO_CUDA_TRY(cudaMemcpyAsync(dl, &L, sizeof(L), cudaMemcpyHostToDevice, s));
-    double *tmpU = nullptr;
-    if (factor) GENEO_CUDA_TRY(cudaMallocAsync(&tmpU, el * sizeof(double), s));
+    DigitBand D;                           // digit window of the factorisation
+    if (factor) {
+      D.npad = L.nt * 32;
+      D.window = (long long)(L.w + 1) * (L.w + 1);
+      GENEO_CUDA_TRY(cudaMallocAsync(&D.pool, (size_t)D.window * kDigHalves * 2, s));
+      GENEO_CUDA_TRY(cudaMallocAsync((void **)&D.rexp, 2 * (size_t)D.npad * sizeof(int), s));
+      D.dexp = D.rexp + D.npad;
+    }
     int st = launch_band_clear<double>(dl, 1, tmp, el, s);
     if (!st) {
       if (base_kind == 0)
@@ -2020,13 +2047,16 @@ extern "C" int geneo_debug_local_matrix(geneo_ctx *c, int sub, int kind, double 
     }
     if (!st && factor) {
       GENEO_CUDA_TRY(cudaMemsetAsync(c->status, 0, sizeof(DevStatus), s));
-      st = launch_band_cholesky<double>(dl, 1, L.nt, L.w, tmp, tmpU, c->status, s);
+      st = launch_band_cholesky64(dl, 1, L.nt, L.w, tmp, nullptr, D, c->status, s);
     }
     std::vector<double> tiles(el);
     GENEO_CUDA_TRY(cudaMemcpyAsync(tiles.data(), tmp, el * sizeof(double), cudaMemcpyDeviceToHost, s));
     GENEO_CUDA_TRY(cudaFreeAsync(tmp, s));
     GENEO_CUDA_TRY(cudaFreeAsync(dl, s));
-    if (tmpU) GENEO_CUDA_TRY(cudaFreeAsync(tmpU, s));
+    if (factor) {
+      GENEO_CUDA_TRY(cudaFreeAsync(D.pool, s));
+      GENEO_CUDA_TRY(cudaFreeAsync(D.rexp, s));
+    }
     GENEO_CUDA_TRY(cudaStreamSynchronize(s));
     if (st) return st;
     if (factor && (st = check_status(c))) return st;
@@ -2132,17 +2162,17 @@ extern "C" int geneo_profile(geneo_ctx *c, int what, int reps, double *ms_per_la
         launch_spmv(A, c->r, c->q, s);
       } else if (what == 3) {
         const int p = kLanczosBlock, ldv = pc.kdim + p, npad = pc.npad_neu_max;
-        st = launch_band_solve_dense(pc.d_lay_neu, pc.nsub, npad, pc.w_neu_max, pc.eig_ring,
-                                     pc.neuL, pc.neuU, pc.V, (long long)npad * ldv, ldv, pc.T1,
-                                     (long long)npad * p, p, p, 2, s);
+        st = launch_band_solve64(pc.d_lay_neu, pc.nsub, pc.w_neu_max, pc.dig_neu, pc.solve_scr, pc.V,
+                                 (long long)npad * ldv, ldv, pc.T1, (long long)npad * p, p, p, 2,
+                                 c->status, s);
       } else if (what == 4) {
         // re-assemble S_j = A_j - sigma B_j and factor it again (same result)
         if (!(st = launch_band_clear<double>(pc.d_lay_neu, pc.nsub, pc.neuL, pc.fac_neu_elems, s))) {
           launch_neumann_assemble(pc.d_subs, pc.d_lay_neu, pc.nsub, pc.max_nodes_neu, c->nx, c->ny,
                                   c->nz, c->X, c->Y, c->Z, c->Cel, c->perm, pc.d_ecnt, pc.ecnt_off,
                                   c->mask, pc.Xneu, pc.modes.shift, pc.neuL, pc.Bloc, s);
-          st = launch_band_cholesky<double>(pc.d_lay_neu, pc.nsub, pc.nt_neu_max, pc.w_neu_max,
-                                            pc.neuL, pc.neuU, c->status, s, c->side_stream);
+          st = launch_band_cholesky64(pc.d_lay_neu, pc.nsub, pc.nt_neu_max, pc.w_neu_max, pc.neuL,
+                                      nullptr, pc.dig_neu, c->status, s, c->side_stream);
         }
       } else if (what == 5) {
         // re-extract A_j and factor it again in the set-up's precision
@@ -2153,16 +2183,16 @@ extern "C" int geneo_profile(geneo_ctx *c, int what, int reps, double *ms_per_la
               !(st = launch_extract_interior<float>(pc.d_subs, pc.d_lay_int, pc.nsub,
                                                     pc.max_nodes_int, nnx, nny, nnz, c->row_ptr,
                                                     c->val, L, s)))
-            st = launch_band_cholesky<float>(pc.d_lay_int, pc.nsub, pc.nt_int_max, pc.w_int_max, L,
-                                             U, c->status, s, c->side_stream);
+            st = launch_band_cholesky32(pc.d_lay_int, pc.nsub, pc.nt_int_max, pc.w_int_max, L, U,
+                                        c->status, s, c->side_stream);
         } else {
           double *L = (double *)pc.facL, *U = (double *)pc.facU;
           if (!(st = launch_band_clear<double>(pc.d_lay_int, pc.nsub, L, pc.fac_int_elems, s)) &&
               !(st = launch_extract_interior<double>(pc.d_subs, pc.d_lay_int, pc.nsub,
                                                      pc.max_nodes_int, nnx, nny, nnz, c->row_ptr,
                                                      c->val, L, s)))
-            st = launch_band_cholesky<double>(pc.d_lay_int, pc.nsub, pc.nt_int_max, pc.w_int_max,
-                                              L, U, c->status, s, c->side_stream);
+            st = launch_band_cholesky64(pc.d_lay_int, pc.nsub, pc.nt_int_max, pc.w_int_max, L, U,
+                                        pc.dig_int, c->status, s, c->side_stream);
         }
       } else {
         st = precond_apply(c, c->r, c->z, nullptr, s);

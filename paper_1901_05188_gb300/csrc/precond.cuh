@@ -18,6 +18,18 @@ struct BandLayout {
   long long off;       // element offset of tile (0, 0) in its pool
 };
 
+// Digits of an FP64 band factor (digits.cuh): kDigHalves 16-bit values per tile
+// and two scale exponents per row.  window = 0: the tiles of the whole band, in
+// the order of the FP64 tiles; window > 0: only the w + 1 tile rows the
+// factorisation can still touch, `window` tiles per system.
+constexpr int kDigHalves = 7 * 1024;
+struct DigitBand {
+  void *pool = nullptr;
+  int *rexp = nullptr, *dexp = nullptr;   // [system][npad]: rows of L, rows of the inverted diagonal blocks
+  int npad = 0;
+  long long window = 0;
+};
+
 struct Precond {
   geneo_partition part{};
   geneo_modes modes{};
@@ -43,7 +55,6 @@ struct Precond {
   int cand_off[3] = {0, 0, 0}, ecnt_off[3] = {0, 0, 0};
   int nt_int_max = 0, w_int_max = 0, npad_int_max = 0;
   int nt_neu_max = 0, w_neu_max = 0, npad_neu_max = 0;
-  int eig_ring = 0;               // the eigensolver's band solves stream their columns through a ring
   long long fac_int_elems = 0, xloc_elems = 0;
   long long fac_neu_elems = 0, bloc_blocks = 0, xneu_elems = 0;
   // interior factors (T = double or float), L and U copies
@@ -53,7 +64,9 @@ struct Precond {
   int pou = 0;                    // partition of unity: GENEO_POU_MULTIPLICITY or _SARKIS
   double *wloc = nullptr;         // Sarkis weights X_j on interior dofs (like xloc), or null
   // GenEO eigenproblem data (FP64)
-  double *neuL = nullptr, *neuU = nullptr;   // factor of S = A - sigma B
+  double *neuL = nullptr;         // factor of S = A - sigma B
+  DigitBand dig_neu, dig_int, dig_H;   // digits of it, of the FP64 interior factors, of A_H's factor
+  void *solve_scr = nullptr;      // scratch of the band solves
   double *Bloc = nullptr;         // 27-slot local BSR of B (9 doubles per block)
   double *Xneu = nullptr;         // PoU on Neumann dofs
   int ksteps = 12;                // Lanczos block steps per cycle (basis size kdim = p * ksteps)
@@ -83,7 +96,7 @@ struct Precond {
   double *Zp = nullptr;           // Z_j, row-major n_int x m_j per subdomain
   double *Yp = nullptr;           // A Z_j on Neumann dofs, [nsub] x n_neu x m_j
   double *AH = nullptr, *AHinv = nullptr;   // dense nH x nH
-  double *AHL = nullptr, *AHU = nullptr;    // tiles of the coarse factor
+  double *AHL = nullptr;          // tiles of the coarse factor
   double *wpart = nullptr;        // restriction partials [nsub][row blocks][mcap]
   double *wH = nullptr, *yH = nullptr;
   double *zy = nullptr;           // coarse correction Z_j y_j per interior dof [sum n_int]

@@ -928,17 +928,6 @@ struct ArrayDst {
   T *p;
   __device__ void operator()(int l, T v) const { p[l] = v; }
 };
-// Column of a row-major block of right-hand sides (row stride `ld`).
-struct StridedSrc {
-  const double *p;
-  long long ld;
-  __device__ double operator()(int l) const { return __ldcg(p + l * ld); }
-};
-struct StridedDst {
-  double *p;
-  long long ld;
-  __device__ void operator()(int l, double v) const { p[l * ld] = v; }
-};
 // R_j r: the subdomain's interior unknowns gathered from the global vector.
 template <typename T>
 struct GatherSrc {
@@ -1255,40 +1244,10 @@ __global__ void __launch_bounds__(kClWarps * 32, 1)
   cluster.sync();                          // no CTA leaves while others may still write to it
 }
 
-// ---- the GenEO eigensolver's band solves in the look-ahead form ------------------
-// One CTA per (system, right-hand side): the column is loaded into shared
-// memory (row stride in_row), swept forward and/or backward with the
-// one-CTA look-ahead sweep above (far warps multiply row I+1 while the chain
-// warps finish row I), and written back (row stride out_row).
-__global__ void __launch_bounds__(kClWarps * 32)
-    k_band_solve_la(const BandLayout *lay, const double *poolL, const double *poolU,
-                    const double *__restrict__ in, long long in_sys, int in_row,
-                    double *__restrict__ out, long long out_sys, int out_row, int mode) {
-  cg::cluster_group cluster = cg::this_cluster();
-  extern __shared__ __align__(16) unsigned char smraw[];
-  double *red = reinterpret_cast<double *>(smraw);   // [2][kClWarps - kChain][32]
-  double *chn = red + 2 * (kClWarps - kChain) * 32;   // [2][kChain][32]
-  double *part = chn + 2 * kChain * 32;               // [2][1][32]
-  double *y = part + 2 * 32;                          // [npad]
-  const int j = blockIdx.x, c = blockIdx.y;
-  const BandLayout L = lay[j];
-  const int n = L.n, npad = L.nt * 32;
-  const double *src = in + j * in_sys + c;
-  for (int l = threadIdx.x; l < npad; l += blockDim.x) y[l] = l < n ? src[(long long)l * in_row] : 0.0;
-  cluster.sync();
-  if (mode & 1) cluster_sweep_la<double, 1>(cluster, poolL, L, y, red, chn, part, false);
-  cluster.sync();
-  if (mode & 2) cluster_sweep_la<double, 1>(cluster, poolU, L, y, red, chn, part, true);
-  cluster.sync();
-  double *dst = out + j * out_sys + c;
-  for (int l = threadIdx.x; l < n; l += blockDim.x) dst[(long long)l * out_row] = y[l];
-}
-
 // ---- the same sweeps with the local vector streamed through a ring ----------
 // For subdomains whose local vector does not fit in shared memory: the
-// look-ahead sweep (one cluster of C CTAs per subdomain, or one CTA per
-// (system, right-hand side)) with the vector in a ring of max(w + 2, 3) tile
-// rows in every CTA.  The forward sweep writes y to a scratch vector as it
+// look-ahead sweep (one cluster of C CTAs per subdomain) with the vector in a
+// ring of max(w + 2, 3) tile rows in every CTA.  The forward sweep writes y to a scratch vector as it
 // goes (rank 0) and the backward sweep reads it back from there: two more
 // passes over the n unknowns than the shared-memory form, beside the 32 (w + 1)
 // factor elements per unknown that each sweep streams.  Reading y from a
@@ -1320,32 +1279,6 @@ __global__ void __launch_bounds__(kClWarps * 32)
                                                  {xloc + S->v_int}};
   cluster_sweep_la<T, C>(cluster, poolU, L, y, red, chn, part, true, bwd);
   cluster.sync();                          // no CTA leaves while others may still write to it
-}
-
-__global__ void __launch_bounds__(kClWarps * 32)
-    k_band_solve_ring(const BandLayout *lay, const double *poolL, const double *poolU,
-                      const double *in, long long in_sys, int in_row, double *out,
-                      long long out_sys, int out_row, int mode) {
-  cg::cluster_group cluster = cg::this_cluster();
-  extern __shared__ __align__(16) unsigned char smraw[];
-  double *red = reinterpret_cast<double *>(smraw);   // [2][kClWarps - kChain][32]
-  double *chn = red + 2 * (kClWarps - kChain) * 32;   // [2][kChain][32]
-  double *part = chn + 2 * kChain * 32;               // [2][1][32]
-  double *y = part + 2 * 32;                          // [ring_rows(w)][32]
-  const int j = blockIdx.x, c = blockIdx.y;
-  const BandLayout L = lay[j];
-  const double *src = in + j * in_sys + c;
-  double *dst = out + j * out_sys + c;
-  if (mode & 1) {
-    const RingVec<double, StridedSrc, StridedDst> fwd{ring_rows(L.w), L.n, {src, in_row}, {dst, out_row}};
-    cluster_sweep_la<double, 1>(cluster, poolL, L, y, red, chn, part, false, fwd);
-    cluster.sync();
-  }
-  if (mode & 2) {
-    const StridedSrc b = (mode & 1) ? StridedSrc{dst, out_row} : StridedSrc{src, in_row};
-    const RingVec<double, StridedSrc, StridedDst> bwd{ring_rows(L.w), L.n, b, {dst, out_row}};
-    cluster_sweep_la<double, 1>(cluster, poolU, L, y, red, chn, part, true, bwd);
-  }
 }
 
 // ---- local solves of a batch of instances: one persistent launch ---------------
@@ -1656,38 +1589,6 @@ int launch_schwarz_solve(const SubDesc *d_subs, const BandLayout *d_lay, int nsu
 }
 
 bool band_solve_fits(int w_max) { return smem_bytes_ring<double>(w_max) <= kSmemMax; }
-
-int launch_band_solve_la(const BandLayout *d_lay, int nsys, int npad_max, int w_max, int ring,
-                         const double *poolL, const double *poolU, const double *in,
-                         long long in_sys, int in_row, double *out, long long out_sys,
-                         int out_row, int ncols, int mode, cudaStream_t s) {
-  const bool use_ring = ring || smem_bytes<double>(npad_max, 1, 0) > kSmemMax;
-  const long long sm = use_ring ? smem_bytes_ring<double>(w_max) : smem_bytes<double>(npad_max, 1, 0);
-  if (sm > kSmemMax) return GENEO_ERR_INVALID_ARG;
-  if (int st = use_ring ? ensure_smem(k_band_solve_ring, (int)sm) : ensure_smem(k_band_solve_la, (int)sm))
-    return st;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(nsys, ncols);
-  cfg.blockDim = dim3(kClWarps * 32);
-  cfg.dynamicSmemBytes = (size_t)sm;
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = 1;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  if (use_ring) {
-    GENEO_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_band_solve_ring, d_lay, poolL, poolU, in, in_sys,
-                                      in_row, out, out_sys, out_row, mode));
-  } else {
-    GENEO_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_band_solve_la, d_lay, poolL, poolU, in, in_sys,
-                                      in_row, out, out_sys, out_row, mode));
-  }
-  GENEO_COUNT_LAUNCH();
-  return GENEO_OK;
-}
 
 // ---- batch launchers -----------------------------------------------------------
 template <typename T>
