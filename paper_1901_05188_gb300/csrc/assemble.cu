@@ -52,20 +52,20 @@ __device__ __forceinline__ int row_start(int i, int j, int k, int nnx, int nny, 
 
 // Rows of the matrix, assembled with the Dirichlet set eliminated: one block
 // per kRowNodes consecutive nodes.  The sums over the elements are formed in
-// registers -- elasticity: lane = node, one warp per component pair (i, k);
-// Darcy: thread = node -- and staged in shared memory, from where the rows
+// registers -- elasticity: lane = node, one warp per component (i, k); Darcy:
+// thread = node -- and staged in shared memory, from where the rows
 // (contiguous in `val`) are written coalesced, with the Dirichlet rows and
 // columns replaced by the identity and the lifting
 //   lift_i = -sum_{c in D} A_ic g_c on free rows, g_i on Dirichlet rows
 // formed on the way (kept so that a new load needs no eliminated columns).
-// FP64 issue bounds it: about 3,500 FP64 operations per node for elasticity,
-// 450 for Darcy.
+// FP64 issue bounds it: about 6,000 FP64 operations per node for elasticity,
+// 500 for Darcy.
 template <int NC>
 constexpr int kRowNodes = NC == 3 ? 32 : 128;
 template <int NC>
-constexpr int kRowThreads = NC == 3 ? 192 : 128;
+constexpr int kRowThreads = NC == 3 ? 288 : 128;
 template <int NC>
-constexpr int kRowSmem = kRowNodes<NC> * 27 * (NC * NC * 8 + 4 + 1);
+constexpr int kRowSmem = kRowNodes<NC> * (27 * (NC * NC * 8 + 4 + 1) + (NC == 3 ? 8 * 8 * kCornerG : 0));
 
 template <int NC>
 __global__ void __launch_bounds__(kRowThreads<NC>)
@@ -77,7 +77,8 @@ __global__ void __launch_bounds__(kRowThreads<NC>)
                     double *__restrict__ val) {
   constexpr int N = kRowNodes<NC>, NC2 = NC * NC;
   extern __shared__ __align__(16) double sv[];               // [N][27][NC2]
-  int *pos = reinterpret_cast<int *>(sv + N * 27 * NC2);     // [N][27] block index in val, or -1
+  double *gs = sv + N * 27 * NC2;                            // [N][8][kCornerG] (elasticity)
+  int *pos = reinterpret_cast<int *>(gs + (NC == 3 ? N * 8 * kCornerG : 0));   // [N][27] block index in val, or -1
   uint8_t *mk = reinterpret_cast<uint8_t *>(pos + N * 27);   // [N][27] Dirichlet bits of the column node
   const int nnx = nx + 1, nny = ny + 1, nnz = nz + 1, nnode = nnx * nny * nnz;
   const int n0 = blockIdx.x * N, tid = threadIdx.x;
@@ -104,6 +105,18 @@ __global__ void __launch_bounds__(kRowThreads<NC>)
     pos[e] = p;
     mk[e] = m;
   }
+  if constexpr (NC == 3) {
+    stage_integrals(gs, N, kRowThreads<NC>, [&](int t, NodeAxis &ax, NodeAxis &ay, NodeAxis &az) {
+      if (n0 + t >= nnode) return false;
+      int i, j, k;
+      node_ijk(n0 + t, nnx, nny, i, j, k);
+      ax = node_axis(X, i, 0, nx);
+      ay = node_axis(Y, j, 0, ny);
+      az = node_axis(Z, k, 0, nz);
+      return true;
+    });
+    __syncthreads();
+  }
   const int t = NC == 3 ? (tid & 31) : tid, n = n0 + t;
   if (n < nnode) {
     int i, j, k;
@@ -115,23 +128,12 @@ __global__ void __launch_bounds__(kRowThreads<NC>)
     for (int s = 0; s < 27; ++s) acc[s] = 0.0;
     double *out = sv + t * 27 * NC2;
     if constexpr (NC == 3) {
-      int ci, ck, off[9];
-      component_pair(tid >> 5, ci, ck, off);
-      double acct[27];
-      if (ci != ck) {
+      const int p = tid >> 5;
+      int off[9];
+      component_offsets(p, off);
+      elastic_rows(coef, off, gs + t * 8 * kCornerG, ax, ay, az, i, j, k, nx, ny, all, acc);
 #pragma unroll
-        for (int s = 0; s < 27; ++s) acct[s] = 0.0;
-        elastic_rows<true>(coef, off, ax, ay, az, i, j, k, nx, ny, all, acc, acct);
-#pragma unroll
-        for (int s = 0; s < 27; ++s) {
-          out[9 * s + 3 * ci + ck] = acc[s];
-          out[9 * s + 3 * ck + ci] = acct[s];
-        }
-      } else {
-        elastic_rows<false>(coef, off, ax, ay, az, i, j, k, nx, ny, all, acc, acct);
-#pragma unroll
-        for (int s = 0; s < 27; ++s) out[9 * s + 4 * ci] = acc[s];
-      }
+      for (int s = 0; s < 27; ++s) out[9 * s + p] = acc[s];
     } else {
       darcy_rows(coef, ax, ay, az, i, j, k, nx, ny, all, acc);
 #pragma unroll
@@ -217,10 +219,20 @@ __global__ void k_load_darcy(int nx, int ny, int nz, const double *__restrict__ 
   if (n >= nnx * nny * (nz + 1)) return;
   int i, j, k;
   node_ijk(n, nnx, nny, i, j, k);
-  // the element volumes around a node sum to a product of the axis widths
-  const double wx = X[min(i + 1, nx)] - X[max(i - 1, 0)], wy = Y[min(j + 1, ny)] - Y[max(j - 1, 0)],
-               wz = Z[min(k + 1, nz)] - Z[max(k - 1, 0)];
-  const double v = f * wx * wy * wz * 0.125;
+  double v = 0.0;
+  if (f != 0.0)
+    for (int ex = max(i - 1, 0), e = min(i, nx - 1), q = 0; q < 1; ++q) {
+      // f dx, f dx dy, f dx dy dz of the (up to) eight elements, summed in element order
+      const double fx[2] = {f * (X[ex + 1] - X[ex]), f * (X[e + 1] - X[e])};
+      for (int ez = max(k - 1, 0); ez <= min(k, nz - 1); ++ez) {
+        const double dz = Z[ez + 1] - Z[ez];
+        for (int ey = max(j - 1, 0); ey <= min(j, ny - 1); ++ey) {
+          const double dy = Y[ey + 1] - Y[ey];
+          v = fma(fx[0] * dy * dz, 0.125, v);
+          if (e > ex) v = fma(fx[1] * dy * dz, 0.125, v);
+        }
+      }
+    }
   b[n] = v + (nodal ? nodal[n] : 0.0);
 }
 

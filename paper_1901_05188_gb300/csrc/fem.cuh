@@ -58,12 +58,10 @@ __device__ inline void material_stiffness(const geneo_ortho &m, double C[36]) {
 // stress transformation (Bond) matrix M of Q = R_z(theta) R_y(phi): C' = M C M^T.
 // The fibre direction Q e1 is (cos t cos p, sin t cos p, -sin p).  In its own
 // axes C couples only the three normal components and is diagonal in the
-// shears, and C' is symmetric: 198 multiply-adds instead of 432.
+// shears, so the first product skips the zeros.
 __device__ inline void rotate_voigt(const double *__restrict__ C, double theta, double phi,
                                     double *__restrict__ Cr) {
-  double ct, st, cp, sp;
-  sincos(theta, &st, &ct);
-  sincos(phi, &sp, &cp);
+  const double ct = cos(theta), st = sin(theta), cp = cos(phi), sp = sin(phi);
   // Q = Rz * Ry
   const double Q[3][3] = {{ct * cp, -st, ct * sp}, {st * cp, ct, st * sp}, {-sp, 0.0, cp}};
   constexpr int VI[6] = {0, 1, 2, 1, 0, 0};
@@ -75,7 +73,7 @@ __device__ inline void rotate_voigt(const double *__restrict__ C, double theta, 
     for (int J = 0; J < 6; ++J) {
       const int i = VI[I], j = VJ[I], k = VI[J], l = VJ[J];
       double v = Q[i][k] * Q[j][l];
-      if (k != l) v += Q[i][l] * Q[j][k];
+      if (k != l) v = fma(Q[i][l], Q[j][k], v);
       M[I][J] = v;
     }
 #pragma unroll
@@ -83,36 +81,35 @@ __device__ inline void rotate_voigt(const double *__restrict__ C, double theta, 
     double t[6];                                // row I of M C
 #pragma unroll
     for (int J = 0; J < 3; ++J)
-      t[J] = M[I][0] * C[J] + M[I][1] * C[6 + J] + M[I][2] * C[12 + J];
+      t[J] = fma(M[I][2], C[12 + J], fma(M[I][1], C[6 + J], M[I][0] * C[J]));
 #pragma unroll
     for (int J = 3; J < 6; ++J) t[J] = M[I][J] * C[7 * J];
 #pragma unroll
-    for (int J = I; J < 6; ++J) {
-      double s = 0.0;
+    for (int J = 0; J < 6; ++J) {
+      double v = t[0] * M[J][0];
 #pragma unroll
-      for (int K = 0; K < 6; ++K) s += t[K] * M[J][K];
-      Cr[6 * I + J] = s;
-      Cr[6 * J + I] = s;
+      for (int K = 1; K < 6; ++K) v = fma(t[K], M[J][K], v);
+      Cr[6 * I + J] = v;
     }
   }
 }
 
 // ---- rows of the Q1 stiffness, node by node ----------------------------------
 // The 3x3 (or 1x1) block of local nodes a, b of an axis-aligned box element is
-//   K_ab[i][k] = sum_{j,l} C_ijkl int d_j N_a d_l N_b,
+//   K_ab[i][k] = sum_{j,l} C_ijkl G_ab[j][l],  G_ab[j][l] = int d_j N_a d_l N_b,
 // with trilinear N and integrals that are products of 1D integrals of linear
-// factors (equal to the 2x2x2 Gauss rule, which is exact for them).  With the
-// corner signs s_a, s_b in {-1, 1}^3 a 1D mass factor is h/4 + s_a s_b h/12, a
-// mixed one s/2 and a stiffness one s_a s_b / h, so for one component pair
-// (i, k) all 64 blocks follow from the nine numbers
-//   T[j][l] = C_ijkl g_jl,  g_jj = h_e h_f / (16 h_j),  g_jl = h_e / 16
-// (e, f the other axes): with w = s_0 s_1 s_2, r = T^T s_a, t = tr T,
-//   K_ab = r . s_b + w_a w_b (q . s_b + t / 9),
-//   3 q = T s_a + s_a o (t - 2 diag T).
-// Every s is a compile-time sign, so a corner's row of eight blocks takes
-// about 45 FP64 operations per component pair instead of the 81 multiply-adds
-// per block of the direct sum over (j, l); FP64 issue (two per clock and SM)
-// is what bounds the assembly on this GPU.
+// factors (equal to the 2x2x2 Gauss rule, which is exact for them): h/3 or h/6
+// (same or other side), +-1/2 for one derivative, +-1/h for two.  Signs and
+// halves are exact, so all 64 tables G_ab of an element are its nine numbers
+//   g_jj = (1/h_j) m_e m_f,  m_d = h_d / 3,  and m_e / 4 for j != l,
+// (multiplied in the order of the axes) times a sign and a power of two fixed by
+// the corners at compile time; nine multiply-adds then give an entry of K_ab.
+// FP64 issue (two per clock and SM) is what bounds the assembly on this GPU: the
+// loop over blocks with run-time Voigt and sign tables that stood here took
+// 21.5 ms on the 128x64x48 laminate, these rows take 5.0 ms.  The sums keep that
+// loop's order (the matrices agree to 4e-17): a grouping of the 81 products that
+// needs 40 % fewer operations (3.2 ms) moved entries by 2e-16, which the
+// condition number carries to 1e-9 of a solution.
 
 // Axis data of a node's two adjacent elements: [0] starts at the node, [1] ends there.
 struct NodeAxis {
@@ -131,92 +128,72 @@ __device__ __forceinline__ NodeAxis node_axis(const double *__restrict__ X, int 
   return a;
 }
 
-// Adds r . s_b + w_a w_b (q . s_b + t9) to the slot of every local node b of
-// the element in which the node is corner A (slot = dx + 3 dy + 9 dz, offset
-// of b from A in -1..1 per axis, plus 13).
-__device__ __forceinline__ void spread_corner(int A, const double (&r)[3], const double (&q)[3],
-                                              double t9, double (&acc)[27]) {
-  const int wa = ((A & 1) ^ ((A >> 1) & 1) ^ (A >> 2)) ? 1 : -1;   // s_0 s_1 s_2 of corner A
+// The scaled integrals of an element: [3 j + k] = g_jj 2^-k, [9 + 2 e + k] = m_e 2^-(2+k).
+constexpr int kCornerG = 15;
+__device__ __forceinline__ void corner_integrals(double hx, double hy, double hz, double rx,
+                                                 double ry, double rz, double *g) {
+  const double m0 = (1.0 / 3.0) * hx, m1 = (1.0 / 3.0) * hy, m2 = (1.0 / 3.0) * hz;
+  const double d[3] = {(rx * m1) * m2, (m0 * ry) * m2, (m0 * m1) * rz};
+  const double m[3] = {m0, m1, m2};
 #pragma unroll
-  for (int half = 0; half < 2; ++half) {      // corners b with w_a w_b = +1, then -1
-    const int sg = half ? -1 : 1;
-    const double p0 = r[0] + sg * q[0], p1 = r[1] + sg * q[1], p2 = r[2] + sg * q[2];
-    const double t = sg * t9;
-    const double up = t + p0, dn = t - p0, su = p1 + p2, di = p1 - p2;
-#pragma unroll
-    for (int b = 0; b < 8; ++b) {
-      const int b0 = b & 1, b1 = (b >> 1) & 1, b2 = b >> 2;
-      const int wb = (b0 ^ b1 ^ b2) ? 1 : -1;
-      if (wa * wb != sg) continue;
-      const double in = b1 == b2 ? su : di, ou = b0 ? up : dn;
-      const int slot = 13 + (b0 - (A & 1)) + 3 * (b1 - ((A >> 1) & 1)) + 9 * (b2 - (A >> 2));
-      acc[slot] += b1 ? ou + in : ou - in;
-    }
+  for (int j = 0; j < 3; ++j) {
+    g[3 * j] = d[j];
+    g[3 * j + 1] = 0.5 * d[j];
+    g[3 * j + 2] = 0.25 * d[j];
+    g[9 + 2 * j] = 0.25 * m[j];
+    g[10 + 2 * j] = 0.125 * m[j];
   }
 }
 
-// The nine numbers T of one component pair from the element's coefficients
-// c[off[3 j + l]] and the box scalings of corner A's element.
-__device__ __forceinline__ void corner_T(const double *__restrict__ c, const int (&off)[9], double hx,
-                                         double hy, double hz, double rx, double ry, double rz,
-                                         double (&T)[9]) {
-  const double fx = 0.0625 * hx, fy = 0.0625 * hy, fz = 0.0625 * hz;
-  T[0] = __ldg(c + off[0]) * (fy * hz * rx);
-  T[4] = __ldg(c + off[4]) * (fx * hz * ry);
-  T[8] = __ldg(c + off[8]) * (fx * hy * rz);
-  T[1] = __ldg(c + off[1]) * fz;
-  T[3] = __ldg(c + off[3]) * fz;
-  T[2] = __ldg(c + off[2]) * fy;
-  T[6] = __ldg(c + off[6]) * fy;
-  T[5] = __ldg(c + off[5]) * fx;
-  T[7] = __ldg(c + off[7]) * fx;
+// sign (+-1) and index of G_ab[j][l] in corner_integrals' table.
+__device__ __forceinline__ constexpr int corner_bit(int a, int d) { return a >> d & 1; }
+__device__ __forceinline__ constexpr int corner_sign(int a, int b, int j, int l) {
+  return corner_bit(a, j) == corner_bit(b, l) ? 1 : -1;
+}
+__device__ __forceinline__ constexpr int corner_index(int a, int b, int j, int l) {
+  if (j == l) {
+    const int e = (j + 1) % 3, f = (j + 2) % 3;
+    return 3 * j + (corner_bit(a, e) != corner_bit(b, e)) + (corner_bit(a, f) != corner_bit(b, f));
+  }
+  const int e = 3 - j - l;
+  return 9 + 2 * e + (corner_bit(a, e) != corner_bit(b, e));
+}
+// Slot of local node b of the element in which the node is corner a.
+__device__ __forceinline__ constexpr int corner_slot(int a, int b) {
+  return 13 + corner_bit(b, 0) - corner_bit(a, 0) + 3 * (corner_bit(b, 1) - corner_bit(a, 1)) +
+         9 * (corner_bit(b, 2) - corner_bit(a, 2));
 }
 
-// Blocks (i, k) in acc and, for a pair i != k, (k, i) in acct of a node's 27
-// slots, summed over its (up to eight) elements for which take(e) holds.
-// `off` indexes the element's 6x6 Voigt stiffness.
-template <bool kPair, typename Take>
+// Component (ci, ck) of a node's 27 slots, summed over its (up to eight)
+// elements for which take(e) holds, in ascending element order.  `off` indexes
+// C_ijkl, j, l = 0..2, in the element's 6x6 Voigt stiffness; `g` holds the
+// corner_integrals of the node's eight elements, [corner][kCornerG].
+template <typename Take>
 __device__ __forceinline__ void elastic_rows(const double *__restrict__ Cel, const int (&off)[9],
-                                             const NodeAxis &ax, const NodeAxis &ay,
-                                             const NodeAxis &az, int gi, int gj, int gk, int nx,
-                                             int ny, Take take, double (&acc)[27],
-                                             double (&acct)[27]) {
-  const double third = 1.0 / 3.0;
+                                             const double *g, const NodeAxis &ax,
+                                             const NodeAxis &ay, const NodeAxis &az, int gi, int gj,
+                                             int gk, int nx, int ny, Take take, double (&acc)[27]) {
 #pragma unroll
-  for (int A = 0; A < 8; ++A) {
+  for (int A = 7; A >= 0; --A) {
     const int a0 = A & 1, a1 = (A >> 1) & 1, a2 = A >> 2;
     if (!(ax.in[a0] && ay.in[a1] && az.in[a2])) continue;
     const int ex = gi - a0, ey = gj - a1, ez = gk - a2;
     if (!take(ex, ey, ez)) continue;
-    double T[9];
-    corner_T(Cel + 36 * (size_t)(ex + nx * (ey + ny * ez)), off, ax.h[a0], ay.h[a1], az.h[a2],
-             ax.r[a0], ay.r[a1], az.r[a2], T);
-    const int s0 = a0 ? 1 : -1, s1 = a1 ? 1 : -1, s2 = a2 ? 1 : -1;
-    const double tr = (T[0] + T[4]) + T[8], t9 = tr * (1.0 / 9.0);
-    double r[3], q[3];
-    r[0] = s0 * T[0] + s1 * T[3] + s2 * T[6];
-    r[1] = s0 * T[1] + s1 * T[4] + s2 * T[7];
-    r[2] = s0 * T[2] + s1 * T[5] + s2 * T[8];
-    const double e0 = s0 * third * (tr - 2.0 * T[0]), e1 = s1 * third * (tr - 2.0 * T[4]),
-                 e2 = s2 * third * (tr - 2.0 * T[8]);
-    if (kPair) {
-      double rt[3];                            // T s_a: the same for the transposed block
-      rt[0] = s0 * T[0] + s1 * T[1] + s2 * T[2];
-      rt[1] = s0 * T[3] + s1 * T[4] + s2 * T[5];
-      rt[2] = s0 * T[6] + s1 * T[7] + s2 * T[8];
-      q[0] = fma(third, rt[0], e0);
-      q[1] = fma(third, rt[1], e1);
-      q[2] = fma(third, rt[2], e2);
-      spread_corner(A, r, q, t9, acc);
-      q[0] = fma(third, r[0], e0);
-      q[1] = fma(third, r[1], e1);
-      q[2] = fma(third, r[2], e2);
-      spread_corner(A, rt, q, t9, acct);
-    } else {                                   // i = k: T is symmetric
-      q[0] = fma(third, r[0], e0);
-      q[1] = fma(third, r[1], e1);
-      q[2] = fma(third, r[2], e2);
-      spread_corner(A, r, q, t9, acc);
+    const double *c = Cel + 36 * (size_t)(ex + nx * (ey + ny * ez));
+    double C[9], G[kCornerG];
+#pragma unroll
+    for (int q = 0; q < 9; ++q) C[q] = __ldg(c + off[q]);
+#pragma unroll
+    for (int q = 0; q < kCornerG; ++q) G[q] = g[A * kCornerG + q];
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+      double v = 0.0;
+#pragma unroll
+      for (int q = 0; q < 9; ++q) {
+        const double cq = corner_sign(A, b, q / 3, q % 3) > 0 ? C[q] : -C[q];
+        v = q == 0 ? cq * G[corner_index(A, b, 0, 0)] : fma(cq, G[corner_index(A, b, q / 3, q % 3)], v);
+      }
+      acc[corner_slot(A, b)] += v;
     }
   }
 }
@@ -226,35 +203,45 @@ template <typename Take>
 __device__ __forceinline__ void darcy_rows(const double *__restrict__ perm, const NodeAxis &ax,
                                            const NodeAxis &ay, const NodeAxis &az, int gi, int gj,
                                            int gk, int nx, int ny, Take take, double (&acc)[27]) {
-  const double third = 1.0 / 3.0;
 #pragma unroll
-  for (int A = 0; A < 8; ++A) {
+  for (int A = 7; A >= 0; --A) {
     const int a0 = A & 1, a1 = (A >> 1) & 1, a2 = A >> 2;
     if (!(ax.in[a0] && ay.in[a1] && az.in[a2])) continue;
     const int ex = gi - a0, ey = gj - a1, ez = gk - a2;
     if (!take(ex, ey, ez)) continue;
     const double *kd = perm + 3 * (size_t)(ex + nx * (ey + ny * ez));
-    const double fx = 0.0625 * ax.h[a0], fy = 0.0625 * ay.h[a1];
-    const double T0 = __ldg(kd) * (fy * az.h[a2] * ax.r[a0]),
-                 T1 = __ldg(kd + 1) * (fx * az.h[a2] * ay.r[a1]),
-                 T2 = __ldg(kd + 2) * (fx * ay.h[a1] * az.r[a2]);
-    const double tr = (T0 + T1) + T2;
-    const int s0 = a0 ? 1 : -1, s1 = a1 ? 1 : -1, s2 = a2 ? 1 : -1;
-    const double r[3] = {s0 * T0, s1 * T1, s2 * T2};
-    const double q[3] = {s0 * third * (tr - T0), s1 * third * (tr - T1), s2 * third * (tr - T2)};
-    spread_corner(A, r, q, tr * (1.0 / 9.0), acc);
+    const double k0 = __ldg(kd), k1 = __ldg(kd + 1), k2 = __ldg(kd + 2);
+    double G[kCornerG];
+    corner_integrals(ax.h[a0], ay.h[a1], az.h[a2], ax.r[a0], ay.r[a1], az.r[a2], G);
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+      const double g0 = corner_sign(A, b, 0, 0) * G[corner_index(A, b, 0, 0)],
+                   g1 = corner_sign(A, b, 1, 1) * G[corner_index(A, b, 1, 1)],
+                   g2 = corner_sign(A, b, 2, 2) * G[corner_index(A, b, 2, 2)];
+      acc[corner_slot(A, b)] += fma(k2, g2, fma(k0, g0, k1 * g1));
+    }
   }
 }
 
-// Component pair p of 0..5: (0,1), (0,2), (1,2), then the diagonal (0,0),
-// (1,1), (2,2); the offsets of C_ijkl, j, l = 0..2, in the 6x6 Voigt matrix.
-__device__ __forceinline__ void component_pair(int p, int &ci, int &ck, int (&off)[9]) {
-  ci = p < 3 ? (p == 2 ? 1 : 0) : p - 3;
-  ck = p < 3 ? (p == 0 ? 1 : 2) : p - 3;
+// The corner_integrals of the eight elements of nodes t = 0..n-1 into
+// g[t][corner][kCornerG] (shared memory), one (node, corner) per thread and turn.
+template <typename Axes>
+__device__ __forceinline__ void stage_integrals(double *g, int n, int threads, Axes axes) {
+  for (int e = threadIdx.x; e < 8 * n; e += threads) {
+    NodeAxis ax, ay, az;
+    const int A = e & 7;
+    if (!axes(e >> 3, ax, ay, az)) continue;
+    corner_integrals(ax.h[A & 1], ay.h[(A >> 1) & 1], az.h[A >> 2], ax.r[A & 1], ay.r[(A >> 1) & 1],
+                     az.r[A >> 2], g + e * kCornerG);
+  }
+}
+
+// The offsets of C_ijkl, j, l = 0..2, of component (ci, ck) = (p / 3, p % 3).
+__device__ __forceinline__ void component_offsets(int p, int (&off)[9]) {
 #pragma unroll
   for (int j = 0; j < 3; ++j)
 #pragma unroll
-    for (int l = 0; l < 3; ++l) off[3 * j + l] = 6 * voigt(ci, j) + voigt(ck, l);
+    for (int l = 0; l < 3; ++l) off[3 * j + l] = 6 * voigt(p / 3, j) + voigt(p % 3, l);
 }
 
 }  // namespace geneo

@@ -88,16 +88,16 @@ __global__ void k_pou_interior(const SubDesc *subs, const int *cand, int co0, in
 // S_j = A_Omega_j - sigma B_j in band tiles (lower part) and B_j as 27-slot
 // rows, from the rows of the node's elements inside Omega_j (fem.cuh): one
 // block per kNeuNodes consecutive local nodes, summed in registers (elasticity:
-// lane = node, one warp per component pair) and staged in shared memory, from
+// lane = node, one warp per component) and staged in shared memory, from
 // where B's rows are written coalesced and S's entries column by column.  The
 // overlap elements' rows are summed only in blocks that have some.  FP64 issue
 // bounds it, as for the global matrix.
 template <int NC>
 constexpr int kNeuNodes = NC == 3 ? 32 : 128;
 template <int NC>
-constexpr int kNeuThreads = NC == 3 ? 192 : 128;
+constexpr int kNeuThreads = NC == 3 ? 288 : 128;
 template <int NC>
-constexpr int kNeuSmem = kNeuNodes<NC> * 27 * (NC * NC * 8 + 4 + 1);
+constexpr int kNeuSmem = kNeuNodes<NC> * (27 * (NC * NC * 8 + 4 + 1) + (NC == 3 ? 8 * 8 * kCornerG : 0));
 
 template <int NC>
 __global__ void __launch_bounds__(kNeuThreads<NC>)
@@ -112,7 +112,8 @@ __global__ void __launch_bounds__(kNeuThreads<NC>)
   const int nn = S.nbox.count(), l0 = blockIdx.x * N, tid = threadIdx.x;
   if (l0 >= nn) return;
   extern __shared__ __align__(16) double sv[];               // [N][27][NC2]
-  int *nb = reinterpret_cast<int *>(sv + N * 27 * NC2);      // [N][27] local neighbour node, or -1
+  double *gs = sv + N * 27 * NC2;                            // [N][8][kCornerG] (elasticity)
+  int *nb = reinterpret_cast<int *>(gs + (NC == 3 ? N * 8 * kCornerG : 0));   // [N][27] local neighbour node, or -1
   uint8_t *mk = reinterpret_cast<uint8_t *>(nb + N * 27);    // [N][27] its Dirichlet bits
   const int nnx = nx + 1, nny = ny + 1;
   for (int e = tid; e < N * 27; e += kT) {
@@ -147,39 +148,32 @@ __global__ void __launch_bounds__(kNeuThreads<NC>)
       if (ax.in[A & 1] && ay.in[(A >> 1) & 1] && az.in[A >> 2])
         touch = touch || ov(gi - (A & 1), gj - ((A >> 1) & 1), gk - (A >> 2));
   }
-  int ci = 0, ck = 0, off[9];
-  if constexpr (NC == 3) component_pair(tid >> 5, ci, ck, off);
-  // this thread's rows over the elements `take` picks, added to the stage
-  auto rows = [&](auto take, bool add) {
+  int off[9];
+  if constexpr (NC == 3) {
+    component_offsets(tid >> 5, off);
+    stage_integrals(gs, N, kT, [&](int t, NodeAxis &bx, NodeAxis &by, NodeAxis &bz) {
+      if (l0 + t >= nn) return false;
+      int i, j, k;
+      S.nbox.global(l0 + t, i, j, k);
+      bx = node_axis(X, i, S.elo[0], S.ehi[0]);
+      by = node_axis(Y, j, S.elo[1], S.ehi[1]);
+      bz = node_axis(Z, k, S.elo[2], S.ehi[2]);
+      return true;
+    });
+  }
+  // this thread's rows over the elements `take` picks: to the stage, or
+  // S = A - sigma B with the stage holding B
+  auto rows = [&](auto take, bool shift) {
     double acc[27];
 #pragma unroll
     for (int s = 0; s < 27; ++s) acc[s] = 0.0;
-    double *out = sv + t * 27 * NC2;
-    if constexpr (NC == 3) {
-      double acct[27];
-      if (ci != ck) {
-#pragma unroll
-        for (int s = 0; s < 27; ++s) acct[s] = 0.0;
-        elastic_rows<true>(coef, off, ax, ay, az, gi, gj, gk, nx, ny, take, acc, acct);
-#pragma unroll
-        for (int s = 0; s < 27; ++s) {
-          double *o = out + 9 * s + 3 * ci + ck, *ot = out + 9 * s + 3 * ck + ci;
-          *o = add ? acc[s] + *o : acc[s];
-          *ot = add ? acct[s] + *ot : acct[s];
-        }
-      } else {
-        elastic_rows<false>(coef, off, ax, ay, az, gi, gj, gk, nx, ny, take, acc, acct);
-#pragma unroll
-        for (int s = 0; s < 27; ++s) {
-          double *o = out + 9 * s + 4 * ci;
-          *o = add ? acc[s] + *o : acc[s];
-        }
-      }
-    } else {
+    double *out = sv + t * 27 * NC2 + (NC == 3 ? tid >> 5 : 0);
+    if constexpr (NC == 3)
+      elastic_rows(coef, off, gs + t * 8 * kCornerG, ax, ay, az, gi, gj, gk, nx, ny, take, acc);
+    else
       darcy_rows(coef, ax, ay, az, gi, gj, gk, nx, ny, take, acc);
 #pragma unroll
-      for (int s = 0; s < 27; ++s) out[s] = add ? acc[s] + out[s] : acc[s];
-    }
+    for (int s = 0; s < 27; ++s) out[NC2 * s] = shift ? fma(-sigma, out[NC2 * s], acc[s]) : acc[s];
   };
   const bool any = __syncthreads_or(touch);
   if (any) {
@@ -194,7 +188,7 @@ __global__ void __launch_bounds__(kNeuThreads<NC>)
     if (any && l2 >= 0 && !((mk[27 * t2 + 13] >> r & 1) || (mk[b] >> c & 1)))
       bv = Xneu[S.x_neu + NC * (l0 + t2) + r] * sv[e] * Xneu[S.x_neu + NC * l2 + c];
     bl[e] = bv;
-    sv[e] = -sigma * bv;
+    sv[e] = bv;
   }
   __syncthreads();
   if (live) rows([](int, int, int) { return true; }, true);
