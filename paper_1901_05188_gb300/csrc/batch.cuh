@@ -91,13 +91,15 @@ void launch_batch_coarse(const BatchInst *inst, const BatchTables &T, const CGSc
 void launch_batch_gather(const BatchInst *inst, const BatchTables &T, const CGScalars *cg,
                          bool precision_f32, double *z, cudaStream_t s);
 // One-level local solves of every (instance, subdomain) item in one persistent
-// launch of `blocks` CTAs pulling items from *head (zero it before).
+// launch of `clusters` clusters of `cluster` CTAs (1, 2 or 4) pulling items from
+// *head (zero it before).
 template <typename T>
 int launch_batch_schwarz(const BatchInst *inst, const CGScalars *cg, const int2 *items,
                          int nitems, int *head, const double *r, int npad_max, int w_max,
-                         int rows, int staged, int blocks, DevStatus *status, cudaStream_t s);
+                         int cluster, int rows, int staged, int clusters, DevStatus *status,
+                         cudaStream_t s);
 template <typename T>
-bool batch_schwarz_fits(int npad_max, int w_max, int rows, int staged);
+bool batch_schwarz_fits(int npad_max, int w_max, int cluster, int rows, int staged);
 template <typename T>
 int prepare_batch_schwarz(int npad_max, int w_max);
 

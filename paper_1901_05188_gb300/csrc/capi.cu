@@ -2232,7 +2232,8 @@ struct geneo_batch {
   CGScalars *cg = nullptr, *cg_host = nullptr;
   int *heads = nullptr;
   DevStatus *status = nullptr;
-  int npad_max = 0, w_max = 0, rows = 0, staged = 0, blocks = 0;
+  int npad_max = 0, w_max = 0, sms = 0;
+  int cluster = 1, rows = 0, staged = 0;      // launch shape of the local solves
   bool any_coarse = false;
   cudaGraphExec_t graph = nullptr;
   long long graph_kernels = 0;
@@ -2248,14 +2249,15 @@ int batch_precond(geneo_batch *B, const double *r, double *z, int head, cudaStre
   int st;
   if (B->any_coarse) launch_batch_coarse(B->d_inst, B->T, B->cg, r, s);
   GENEO_CUDA_TRY(cudaMemsetAsync(B->heads + head, 0, sizeof(int), s));
+  const int clusters = std::max(1, std::min(B->sms / B->cluster, B->T.nsub_items));
   if (B->f32)
     st = launch_batch_schwarz<float>(B->d_inst, B->cg, B->T.sub_items, B->T.nsub_items,
-                                     B->heads + head, r, B->npad_max, B->w_max, B->rows,
-                                     B->staged, B->blocks, B->status, s);
+                                     B->heads + head, r, B->npad_max, B->w_max, B->cluster,
+                                     B->rows, B->staged, clusters, B->status, s);
   else
     st = launch_batch_schwarz<double>(B->d_inst, B->cg, B->T.sub_items, B->T.nsub_items,
-                                      B->heads + head, r, B->npad_max, B->w_max, B->rows,
-                                      B->staged, B->blocks, B->status, s);
+                                      B->heads + head, r, B->npad_max, B->w_max, B->cluster,
+                                      B->rows, B->staged, clusters, B->status, s);
   if (st) return st;
   launch_batch_gather(B->d_inst, B->T, B->cg, B->f32, z, s);
   GENEO_CUDA_TRY(cudaGetLastError());
@@ -2476,32 +2478,42 @@ extern "C" int geneo_batch_create(geneo_batch **out, geneo_ctx *const *ctxs, int
   } else {
     if ((st = prepare_batch_schwarz<double>(B->npad_max, B->w_max))) return st;
   }
-  int sms = 0;
-  GENEO_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  B->blocks = std::max(1, std::min(sms, B->T.nsub_items));
-  // batch autotuner: the one-CTA launch shapes of the local solves, timed on
-  // the batch's own items (rhs = b, every instance running); GENEO_SCHWARZ_ROWS
-  // and GENEO_SCHWARZ_STAGED pin a dimension
+  GENEO_CUDA_TRY(cudaDeviceGetAttribute(&B->sms, cudaDevAttrMultiProcessorCount, dev));
+  // batch autotuner: the launch shapes of the local solves, timed on the
+  // batch's own items (rhs = b, every instance running).  Clusters of more than
+  // one CTA are tried while the items make at most two rounds of them: with more
+  // the queue keeps the SMs busy, and a cluster only adds its exchange.
+  // GENEO_SCHWARZ_CLUSTER, GENEO_SCHWARZ_ROWS and GENEO_SCHWARZ_STAGED pin a
+  // dimension (a cluster of 8, which the batch has not, leaves it open).
+  const int fc = env_choice("GENEO_SCHWARZ_CLUSTER", {1, 2, 4});
   const int fr = env_choice("GENEO_SCHWARZ_ROWS", {0, 1});
   const int fs = env_choice("GENEO_SCHWARZ_STAGED", {0, 1});
-  std::vector<std::pair<int, int>> cand;
-  for (int R : {0, 1})
-    for (int Sg : {1, 0}) {
-      if ((fr >= 0 && R != fr) || (fs >= 0 && Sg != fs)) continue;
-      const bool fits = f32 ? batch_schwarz_fits<float>(B->npad_max, B->w_max, R, Sg)
-                            : batch_schwarz_fits<double>(B->npad_max, B->w_max, R, Sg);
-      if (fits) cand.push_back({R, Sg});
-    }
+  struct Shape {
+    int cluster, rows, staged;
+  };
+  std::vector<Shape> cand;
+  for (int Cl : {1, 2, 4})
+    for (int R : {0, 1})
+      for (int Sg : {1, 0}) {
+        if (fc >= 0 ? Cl != fc : (Cl > 1 && B->T.nsub_items * Cl > 2 * B->sms)) continue;
+        if ((fr >= 0 && R != fr) || (fs >= 0 && Sg != fs)) continue;
+        const bool fits = f32 ? batch_schwarz_fits<float>(B->npad_max, B->w_max, Cl, R, Sg)
+                              : batch_schwarz_fits<double>(B->npad_max, B->w_max, Cl, R, Sg);
+        if (fits) cand.push_back({Cl, R, Sg});
+      }
   if (cand.empty()) return fail(GENEO_ERR_INVALID_ARG, "no batched local-solve shape fits");
-  B->rows = cand[0].first;
-  B->staged = cand[0].second;
+  auto use = [&](const Shape &c) {
+    B->cluster = c.cluster;
+    B->rows = c.rows;
+    B->staged = c.staged;
+  };
+  use(cand[0]);
   if (cand.size() > 1) {
     cudaEvent_t e0 = B->ev0, e1 = B->ev1;
     float best = 1e30f;
-    std::pair<int, int> pick = cand[0];
-    for (const auto &cd : cand) {
-      B->rows = cd.first;
-      B->staged = cd.second;
+    Shape pick = cand[0];
+    for (const Shape &cd : cand) {
+      use(cd);
       for (int rep = 0; rep < 3; ++rep) {         // one warm-up, two timed applications
         if (rep == 1) GENEO_CUDA_TRY(cudaEventRecord(e0, s));
         if ((st = batch_precond(B, B->b, B->z, kGraphIters, s))) return st;
@@ -2516,8 +2528,7 @@ extern "C" int geneo_batch_create(geneo_batch **out, geneo_ctx *const *ctxs, int
         pick = cd;
       }
     }
-    B->rows = pick.first;
-    B->staged = pick.second;
+    use(pick);
     if ((st = batch_check_status(B))) return st;
   }
   guard.b = nullptr;
@@ -2614,7 +2625,7 @@ extern "C" int geneo_batch_solve(geneo_batch *B, double tol, int max_it, double 
     o.flexible = B->inst[i].flexible;
     o.eig_cycles = c->pc.eig_cycles;
     o.lanczos_steps = c->pc.lanczos_steps;
-    o.schwarz_cluster = 1;
+    o.schwarz_cluster = B->cluster;
     o.schwarz_rows = B->rows;
     o.schwarz_staged = B->staged;
     if (!o.flexible && h.it > 0) {
