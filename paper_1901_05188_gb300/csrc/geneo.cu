@@ -821,34 +821,82 @@ __global__ void k_AZ(const SubDesc *subs, int nnx, int nny, int nnz, const int32
     if (q < m) yr[q] = acc[q];
 }
 
-__global__ void __launch_bounds__(256)
+// A_H block of a pair of meeting subdomains, Z_j^T (A Z_k) over the nodes of
+// V_{h,0}(Omega_j) inside Omega_k's box.  The rows are staged 32 at a time; a
+// thread keeps one or two 2 x 2 blocks of the m_j x m_k products.  FP64 issue
+// bounds it: the previous form (one entry per thread, its rows in a serial
+// loop with index arithmetic per row) took 11.5 ms for 72 subdomains of 13,600
+// unknowns and 28 ms for 108 Darcy ones.  Every entry is still one chain of
+// multiply-adds over the rows: splitting the rows over the idle threads saved
+// nothing more and made the coarse correction two to eight times less accurate
+// (the entries cancel against each other along the rigid displacements).
+constexpr int kCbRows = 32, kCbLd = kMaxModes + 2, kCbThreads = 128;
+constexpr int kCbGroups = kMaxModes / 2 * kMaxModes / 2 / kCbThreads;
+__global__ void __launch_bounds__(kCbThreads)
     k_coarse_blocks(const SubDesc *subs, const int2 *pairs, const double *__restrict__ Zp,
                     const double *__restrict__ Yp, const long long *yoff, double *AH, int nH) {
   const int2 pr = pairs[blockIdx.x];
   const SubDesc &Sj = subs[pr.x];
   const SubDesc &Sk = subs[pr.y];
-  const int mj = Sj.m, mk = Sk.m;
-  int lo[3], hi[3];
+  const int mj = Sj.m, mk = Sk.m, nc = Sj.nc, tid = threadIdx.x;
+  __shared__ __align__(16) double zs[kCbRows][kCbLd], ys[kCbRows][kCbLd];
+  __shared__ int zrow[kCbRows], yrow[kCbRows];
+  int lo[3], ext[3];
   for (int d = 0; d < 3; ++d) {
     lo[d] = max(Sj.ibox.lo[d], Sk.nbox.lo[d]);
-    hi[d] = min(Sj.ibox.lo[d] + Sj.ibox.n[d], Sk.nbox.lo[d] + Sk.nbox.n[d]);
+    ext[d] = max(0, min(Sj.ibox.lo[d] + Sj.ibox.n[d], Sk.nbox.lo[d] + Sk.nbox.n[d]) - lo[d]);
   }
-  const int ex = hi[0] - lo[0], ey = hi[1] - lo[1], ez = hi[2] - lo[2];
-  const int nout = mj * mk;
-  for (int o = threadIdx.x; o < nout; o += blockDim.x) {
-    int a = o / mk, b = o - a * mk;
-    double s = 0.0;
-    if (ex > 0 && ey > 0 && ez > 0) {
-      for (int q = 0; q < ex * ey * ez; ++q) {
-        int ii = lo[0] + q % ex, rr = q / ex, jj = lo[1] + rr % ey, kk = lo[2] + rr / ey;
-        int lj = Sj.ibox.local(ii, jj, kk), lk = Sk.nbox.local(ii, jj, kk);
-        for (int c = 0; c < Sj.nc; ++c)
-          s += Zp[Sj.z_off + (long long)(Sj.nc * lj + c) * mj + a] *
-               Yp[yoff[pr.y] + (long long)(Sj.nc * lk + c) * mk + b];
+  const int nrow = nc * ext[0] * ext[1] * ext[2];
+  const int gk = (mk + 1) / 2, groups = (mj + 1) / 2 * gk;
+  double acc[kCbGroups][2][2] = {};
+  // odd counts: the last column of a 2 x 2 block multiplies zeros
+  for (int e = tid; e < kCbRows * kCbLd; e += kCbThreads) zs[e / kCbLd][e % kCbLd] = ys[e / kCbLd][e % kCbLd] = 0.0;
+  for (int r0 = 0; r0 < nrow; r0 += kCbRows) {
+    const int rows = min(kCbRows, nrow - r0);
+    __syncthreads();                       // the stage has been read
+    if (tid < rows) {
+      const int q = (r0 + tid) / nc, c = r0 + tid - nc * q;
+      const int i = lo[0] + q % ext[0], t = q / ext[0], jj = lo[1] + t % ext[1], k = lo[2] + t / ext[1];
+      zrow[tid] = nc * Sj.ibox.local(i, jj, k) + c;
+      yrow[tid] = nc * Sk.nbox.local(i, jj, k) + c;
+    }
+    __syncthreads();
+    for (int e = tid; e < rows * mj; e += kCbThreads) {
+      const int r = e / mj, a = e - r * mj;
+      zs[r][a] = __ldg(Zp + Sj.z_off + (long long)zrow[r] * mj + a);
+    }
+    for (int e = tid; e < rows * mk; e += kCbThreads) {
+      const int r = e / mk, b = e - r * mk;
+      ys[r][b] = __ldg(Yp + yoff[pr.y] + (long long)yrow[r] * mk + b);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < kCbGroups; ++q) {
+      const int g = tid + q * kCbThreads;
+      if (g >= groups) break;
+      const int a0 = 2 * (g / gk), b0 = 2 * (g % gk);
+      for (int r = 0; r < rows; ++r) {
+        const double2 z = *reinterpret_cast<const double2 *>(&zs[r][a0]);
+        const double2 y = *reinterpret_cast<const double2 *>(&ys[r][b0]);
+        acc[q][0][0] = fma(z.x, y.x, acc[q][0][0]);
+        acc[q][0][1] = fma(z.x, y.y, acc[q][0][1]);
+        acc[q][1][0] = fma(z.y, y.x, acc[q][1][0]);
+        acc[q][1][1] = fma(z.y, y.y, acc[q][1][1]);
       }
     }
-    AH[(long long)(Sj.coff + a) * nH + Sk.coff + b] = s;
-    if (pr.x != pr.y) AH[(long long)(Sk.coff + b) * nH + Sj.coff + a] = s;
+  }
+#pragma unroll
+  for (int q = 0; q < kCbGroups; ++q) {
+    const int g = tid + q * kCbThreads;
+    if (g >= groups) break;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int a = 2 * (g / gk) + (e >> 1), b = 2 * (g % gk) + (e & 1);
+      if (a >= mj || b >= mk) continue;
+      const double s = acc[q][e >> 1][e & 1];
+      AH[(long long)(Sj.coff + a) * nH + Sk.coff + b] = s;
+      if (pr.x != pr.y) AH[(long long)(Sk.coff + b) * nH + Sj.coff + a] = s;
+    }
   }
 }
 
@@ -1082,7 +1130,7 @@ void launch_coarse_blocks(const SubDesc *d_subs, const int2 *pairs, int npairs, 
                           const double *Yp, const long long *yoff, double *AH, int nH,
                           cudaStream_t s) {
   if (npairs > 0) {
-    k_coarse_blocks<<<npairs, 256, 0, s>>>(d_subs, pairs, Zp, Yp, yoff, AH, nH);
+    k_coarse_blocks<<<npairs, kCbThreads, 0, s>>>(d_subs, pairs, Zp, Yp, yoff, AH, nH);
     GENEO_COUNT_LAUNCH();
   }
 }
