@@ -10,12 +10,16 @@
 // Both were bound by the FP64 pipe (128 shifted Neumann matrices of
 // about 16,000 unknowns and half-bandwidth 905: 1.31 s per factorisation, 32 ms
 // per sweep with eight right-hand sides).
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 #include "band.cuh"
 #include "digits.cuh"
 
 namespace geneo {
+
+namespace cg = cooperative_groups;
 
 namespace {
 
@@ -383,36 +387,60 @@ __global__ void __launch_bounds__(256, 2)
   }
 }
 
-// ---- band solves with up to eight right-hand sides per CTA --------------------
-// One CTA per (system, group of eight columns).  Row I needs
+// ---- band solves with up to eight right-hand sides per cluster -----------------
+// One cluster of one or two CTAs per (system, group of eight columns).  Row I needs
 // s = b_I - sum_{d=1..w} L(I, I-d) y_{I-d} and y_I = inv(L_II) s; backward the
-// transposes.  While the four chain warps finish row I (the coupling d = 1, the
-// inverse diagonal block), the eight far warps multiply the tiles d >= 2 of the
-// next row, which need only rows solved before; a pair of them takes one tile,
-// 16 rows each, with the digits of L read by ldmatrix (transposed for the
-// backward sweep, so one copy of the factor serves both) and those of y in
-// fragment order.  Every row block of y has one scale per column; sums over
-// tiles of different scales are aligned by shifting the integers.  Each far
-// warp copies its halves of the tiles into two private stages, the next one in
-// flight while one is multiplied, across rows; the chain warps refill their two
-// tiles as soon as they have been read.  The window of y digits (w + 2 row
-// blocks) lives in global scratch, read through L1.
-// Bound: streaming the digit tiles (14 KB each) once per sweep for many
-// systems, the chain (about 1.3 us a row) for few or narrow ones.
-constexpr int kSwChain = 4, kSwFar = 8;
+// transposes.  While the chain warps finish row I (the coupling d = 1, the
+// inverse diagonal block), the eight far warps of every CTA multiply the tiles
+// d >= 2 of the next row, which need only rows solved before; a pair of them
+// takes one tile, 16 rows each, with the digits of L read by ldmatrix
+// (transposed for the backward sweep, so one copy of the factor serves both) and
+// those of y in fragment order.  Every row block of y has one scale per column,
+// kept from row to row while it is at most four bits too large, so that the far
+// warps can add the level sums of successive tiles as 32-bit integers; sums of
+// different scales are aligned by shifting.  Each far warp copies its halves of
+// the tiles into two private stages, the next one in flight while one is
+// multiplied, across rows.  The window of y digits (w + 2 row blocks) lives in
+// global scratch.
+// The chain is a sequence of dependent integer instructions, at four to five
+// cycles each, so it is spread wide and kept in integers: thread (c, r) of eight
+// warps owns row r of column c.  Warps 0..3 multiply the chain's two tiles, a
+// quarter each; meanwhile warps 4..7 form t = b - far sum and copy the next
+// tiles.  s and y are cut into digits straight from the 128-bit sums; only the
+// output becomes FP64, after the row's barrier.
+// In a cluster the chain runs on the first CTA.  The second one only adds far
+// warps: its other warps sum the CTA's partials of a row into the first CTA's
+// buffer (integers: the result does not depend on the cluster), and one
+// cluster barrier ends the row.
+// Bound: the larger of the chain (six barriers and two products, about 3 us a
+// row) and a CTA's share of the tiles, where issuing the copies counts for as
+// much as the matrix instructions.  Per launch of half the subdomains (forward
+// or backward, eight right-hand sides): 36 of 14,500
+// unknowns and 27 tiles half-bandwidth 1.4 ms, 54 Darcy ones of 16,000 and 7
+// tiles 2.0 ms, 16 of 7,600 and 15 tiles 1.0 ms.  With four chain warps, FP64
+// row values and one CTA per system they took 4.0, 2.3 and 1.7 ms.
+constexpr int kSwChain = 8, kSwFar = 8;
 constexpr int kSwThreads = (kSwChain + kSwFar) * 32;
 constexpr int kSwHalf = kDigBytes / 2;      // a far warp's half of a tile
-constexpr int kSwCol = 36;                  // row stride of a column of partial sums
+constexpr int kSwCol = 34;                  // row stride of a column of partial sums
 constexpr int kSwPart = 8 * kSwCol;         // one 32 x 8 block of them
 constexpr int kSwY = kDig * 128;            // words of one row block of y digits
-__host__ __device__ constexpr int sweep_smem(int w) {
-  return 2 * (int)kDigBytes + kSwFar * 2 * kSwHalf + (2 * 4 + 2) * kSwPart * 16 + 3 * kSwY * 4 +
-         (w + 2) * 32 + (2 * 4 * 8 + 2 * 8) * 4;
+constexpr int kSwSlack = 4;                 // bits a column's scale may be too large
+constexpr int kSwFlush = 64;                // tiles added in 32 bits: 64 * 7 * 2^21 < 2^31
+__host__ __device__ constexpr int sweep_smem(int w, int cl, int nbuf) {
+  return (2 + nbuf) * (int)kDigBytes + kSwFar * 2 * kSwHalf + (2 * (3 + cl) + 2) * kSwPart * 16 +
+         kSwY * 4 + 8 * 32 * 4 + 2 * 8 * 4 + (w + 2) * 16;
 }
 
-__device__ __forceinline__ void sw_bar_all() {
+__device__ __forceinline__ void sw_bar_cta() {
   __syncwarp();                             // bar.sync is .aligned: converge first
-  asm volatile("bar.sync 1, %0;" ::"n"((kSwChain + kSwFar) * 32) : "memory");
+  asm volatile("bar.sync 1, %0;" ::"n"(kSwThreads) : "memory");
+}
+// All CTAs of the cluster; their writes to shared and global memory are visible after it.
+__device__ __forceinline__ void sw_bar_all(int cl) {
+  if (cl == 1) return sw_bar_cta();
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void sw_bar_chain() {
   __syncwarp();
@@ -431,61 +459,62 @@ __device__ __forceinline__ void add_shifted(long long hi, long long lo, int sh, 
 struct SweepArgs {
   const BandLayout *lay;
   DigitBand D;
-  uint4 *ring;                              // y digits: [CTA][w_max + 2][kSwY / 4]
+  uint4 *ring;                              // y digits: [cluster][w_max + 2][kSwY / 4]
   int w_max;
   const double *in;
   long long in_sys;
   int in_row;
   double *out;
   long long out_sys;
-  int out_row, ncols, mode;
-  DevStatus *st;
+  int out_row, ncols, mode, cl, nbuf;
 };
 
 __global__ void __launch_bounds__(kSwThreads, 1) k_band_sweep(const SweepArgs P) {
   extern __shared__ __align__(128) unsigned char smraw[];
-  const int j = blockIdx.x, grp = blockIdx.y;
+  const int cl = P.cl, rank = blockIdx.x % cl, j = blockIdx.x / cl, grp = blockIdx.y;
   const BandLayout L = P.lay[j];
-  const int nt = L.nt, w = L.w, slots = w + 2;
-  unsigned char *chain_t = smraw;                                   // [near, diagonal]
-  unsigned char *far_t = chain_t + 2 * kDigBytes;                   // [warp][2] half tiles
-  long long *part = reinterpret_cast<long long *>(far_t + kSwFar * 2 * kSwHalf);  // [2][4][hi, lo]
-  long long *nearp = part + 2 * 4 * 2 * kSwPart;                    // [2][hi, lo]
-  uint32_t *sdig = reinterpret_cast<uint32_t *>(nearp + 2 * 2 * kSwPart);
-  uint32_t *ydig = sdig + kSwY;                                     // [2]
-  int *fexp = reinterpret_cast<int *>(ydig + 2 * kSwY);             // [w + 2][8]
-  int *cmax = fexp + (P.w_max + 2) * 8;                             // [2][4][8]
-  int *fref = cmax + 2 * 4 * 8;                                     // [2][8]
+  const int nt = L.nt, w = L.w, slots = w + 2, np = 3 + cl;
+  unsigned char *chain_t = smraw;                                   // [diagonal x 2, near x nbuf]
+  unsigned char *far_t = chain_t + (2 + P.nbuf) * kDigBytes;        // [warp][2] half tiles
+  long long *part = reinterpret_cast<long long *>(far_t + kSwFar * 2 * kSwHalf);  // [2][np][hi, lo]
+  long long *nearp = part + 2 * np * 2 * kSwPart;                   // [2][hi, lo]
+  uint32_t *dig = reinterpret_cast<uint32_t *>(nearp + 2 * 2 * kSwPart);   // digits of s or y
+  int *tf = reinterpret_cast<int *>(dig + kSwY);                    // [8][32] exponents of t
+  int *fref = tf + 8 * 32;                                          // [2][8] scale of the far sums
+  short *fexp = reinterpret_cast<short *>(fref + 2 * 8);            // [w + 2][8]
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  uint4 *yring = P.ring + ((long long)grp * gridDim.x + j) * (P.w_max + 2) * (kSwY / 4);
+  const cg::cluster_group cluster = cg::this_cluster();
+  const char *tiles = static_cast<const char *>(P.D.pool) + (L.off >> 10) * (int)kDigBytes;
+  uint4 *yring = P.ring + ((long long)grp * (gridDim.x / cl) + j) * (P.w_max + 2) * (kSwY / 4);
+  if (cl > 1) sw_bar_all(cl);               // every CTA is there before its memory is written
   for (int back = 0; back < 2; ++back) {
     if (!(P.mode & (1 << back))) continue;
     auto row = [&](int q) { return back ? nt - 1 - q : q; };
     auto dmax = [&](int I) { return back ? min(w, nt - 1 - I) : min(w, I); };
+    auto tile_at = [&](int I, int d) {        // byte offset of the tile that couples row I to I -+ d
+      return (long long)((back ? I + d : I) * (w + 1) + d) * (int)kDigBytes;
+    };
     if (warp >= kSwChain) {
       // ---- far warps
-      const int fw = warp - kSwChain, p = fw >> 1, m0 = 16 * (fw & 1), g = lane >> 2, t2 = 2 * (lane & 3);
+      const int fw = warp - kSwChain, pl = fw >> 1, p = 4 * rank + pl, step = 4 * cl;
+      const int m0 = 16 * (fw & 1), g = lane >> 2, t2 = 2 * (lane & 3);
       const uint32_t st0 = dig_smem(far_t) + fw * 2 * kSwHalf;
-      // This warp's half of a tile: rows m0.. (forward; 1 KB of every slice), or
-      // columns m0.. (backward; two 16-byte chunks of every row, kept at
-      // 32 bytes a row: chunk c of row r at (c ^ (r >> 2)) & 1, against bank
-      // conflicts in ldmatrix).
+      // This warp's half of a tile, two 16 x 16 blocks of every slice: rows m0..
+      // (forward) or columns m0.. (backward), the block of k = 16 kb.. at 512 kb.
+      const char *lsrc = tiles + (back ? m0 * 32 : m0 * 64) + lane * 16;
+      const int lnext = back ? 1024 : 512;
       auto load = [&](int stage, int I, int d) {
-        const char *src = reinterpret_cast<const char *>(dig_tile(P.D, L, j, back ? I + d : I, d));
-        const uint32_t dst = st0 + stage * kSwHalf;
+        const char *from = lsrc + tile_at(I, d);
+        const uint32_t dst = st0 + stage * kSwHalf + lane * 16;
 #pragma unroll
-        for (int k = 0; k < 14; ++k) {
-          const int e = k * 32 + lane, s = e >> 6, i = e & 63;
-          if (back) {
-            const int r = i >> 1, c = i & 1;
-            cp16(dst + s * 1024 + r * 32 + ((c ^ (r >> 2)) & 1) * 16,
-                 src + s * 2048 + r * 64 + (((((m0 >> 3) + c) ^ (r >> 1)) & 3) << 4));
-          } else {
-            cp16(dst + s * 1024 + i * 16, src + s * 2048 + m0 * 64 + i * 16);
-          }
+        for (int s = 0; s < kDig; ++s) {
+          cp16(dst + s * 1024, from + s * 2048);
+          cp16(dst + s * 1024 + 512, from + s * 2048 + lnext);
         }
       };
-      // the warp's tiles in order: rows 1.. of the sweep, u = p, p + 4, ... of each
+      const int ar0 = back ? (lane & 7) + 8 * (lane >> 4) : lane & 15;
+      const uint32_t aoff = ar0 * 32 + (((back ? lane >> 3 : lane >> 4) ^ (ar0 >> 2)) & 1) * 16;
+      // the warp's tiles in order: rows 1.. of the sweep, u = p, p + step, ... of each
       int pq = 0, pu = p, pn = 0;             // next tile to load: row q = pq, index pu of pn
       auto advance = [&]() {                  // to the next row that has one; false at the end
         while (pu >= pn) {
@@ -498,230 +527,291 @@ __global__ void __launch_bounds__(kSwThreads, 1) k_band_sweep(const SweepArgs P)
       int stage = 0;
       if (advance()) {
         load(0, row(pq), 2 + pu);
-        pu += 4;
+        pu += step;
       }
       cp_commit();
       for (int q = 0; q < nt; ++q) {
         if (q + 1 < nt) {
           const int In = row(q + 1), n = max(dmax(In) - 1, 0);
-          // the largest scale of the window, per column
-          int fr = kNoExp;
-          for (int u = lane >> 3; u < n; u += 4) {
-            const int K = back ? In + 2 + u : In - 2 - u;
-            fr = max(fr, fexp[(K % slots) * 8 + (lane & 7)]);
-          }
-          fr = max(fr, __shfl_xor_sync(0xffffffffu, fr, 8));
-          fr = max(fr, __shfl_xor_sync(0xffffffffu, fr, 16));
-          const int fr0 = __shfl_sync(0xffffffffu, fr, t2), fr1 = __shfl_sync(0xffffffffu, fr, t2 + 1);
-          long long hs[4] = {0, 0, 0, 0}, ls[4] = {0, 0, 0, 0};
-          for (int u = p; u < n; u += 4) {
-            const int K = back ? In + 2 + u : In - 2 - u, slot = K % slots;
-            uint4 yb[kDig];
-            const uint4 *yp = yring + (long long)slot * (kSwY / 4) + lane;
+          uint4 yb[kDig];
+          auto y_in = [&](int slot) {
+            const uint4 *yp = yring + slot * (kSwY / 4) + lane;
 #pragma unroll
-            for (int t = 0; t < kDig; ++t) yb[t] = yp[t * 32];
-            const int2 fk = *reinterpret_cast<const int2 *>(fexp + slot * 8 + t2);
+            for (int t = 0; t < kDig; ++t) yb[t] = rank ? __ldcg(yp + t * 32) : yp[t * 32];
+          };
+          int slot = (back ? In + 2 + p : In - 2 - p + slots) % slots;   // p <= w - 2 where it is used
+          if (p < n) y_in(slot);
+          const int fr0 = fref[((q + 1) & 1) * 8 + t2], fr1 = fref[((q + 1) & 1) * 8 + t2 + 1];
+          long long *po = part + (((q + 1) & 1) * np + pl) * 2 * kSwPart;
+          unsigned A[kDig][4];                // level sums of the tiles with scales (k0, k1)
+          int k0 = 0, k1 = 0, cnt = 0;
+          bool first = true;
+#pragma unroll
+          for (int l = 0; l < kDig; ++l)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) A[l][e] = 0;
+          auto flush = [&]() {                // A into this warp's partials
+            const bool aligned = __all_sync(0xffffffffu, cnt == 0 || (k0 == fr0 && k1 == fr1));
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const int o = (t2 + (e & 1)) * kSwCol + m0 + g + 8 * (e >> 1);
+              const unsigned z = cnt * 0x4b400000u;   // the start value of levels 0 and 1
+              auto lev = [&](int l) { return (long long)(int)(l < 2 ? A[l][e] - z : A[l][e]); };
+              const long long hi = lev(0) * 134217728 + lev(1) * 262144 + (lev(2) * 512 + lev(3)),
+                              lo = lev(4) * 262144 + (lev(5) * 512 + lev(6));
+              long long hs = first ? 0 : po[o], ls = first ? 0 : po[kSwPart + o];
+              if (aligned) {
+                hs += hi;
+                ls += lo;
+              } else {
+                add_shifted(hi, lo, (e & 1) ? fr1 - k1 : fr0 - k0, hs, ls);
+              }
+              po[o] = hs;
+              po[kSwPart + o] = ls;
+#pragma unroll
+              for (int l = 0; l < kDig; ++l) A[l][e] = 0u;
+            }
+            first = false;
+            cnt = 0;
+          };
+          for (int u = p; u < n; u += step) {
+            const short2 fk = *reinterpret_cast<const short2 *>(fexp + slot * 8 + t2);
+            if (__any_sync(0xffffffffu, cnt == kSwFlush || (cnt > 0 && (fk.x != k0 || fk.y != k1)))) flush();
+            k0 = fk.x;
+            k1 = fk.y;
             if (advance()) {
               load(stage ^ 1, row(pq), 2 + pu);
-              pu += 4;
+              pu += step;
             }
             cp_commit();
             cp_wait<1>();
             __syncwarp();                     // this tile has landed, for every lane
-            const uint32_t at = st0 + stage * kSwHalf;
             float S[kDig][4];
-#pragma unroll
-            for (int l = 0; l < kDig; ++l)
-#pragma unroll
-              for (int e = 0; e < 4; ++e) S[l][e] = 0.f;
+            level_start<2>(S);
 #pragma unroll
             for (int kb = 0; kb < 2; ++kb) {
-              const int r = 16 * kb + (lane & 7) + 8 * (lane >> 4);
-              const uint32_t ab = at + (back ? r * 32 + (((lane >> 3) ^ (r >> 2)) & 1) * 16
-                                             : ldsm_a(0, 16 * kb, lane));
+              const uint32_t ab = st0 + stage * kSwHalf + aoff + kb * 512;
+              uint32_t ar[2][4];
+              auto a_in = [&](int s) {
+                if (back) ldsm4_trans(ar[s & 1], ab + s * 1024);
+                else ldsm4(ar[s & 1], ab + s * 1024);
+              };
+              a_in(0);
 #pragma unroll
               for (int s = 0; s < kDig; ++s) {
-                uint32_t ar[4];
-                if (back) ldsm4_trans(ar, ab + s * 1024);
-                else ldsm4(ar, ab + s * 1024);
+                if (s + 1 < kDig) a_in(s + 1);
 #pragma unroll
                 for (int t = 0; t < kDig - s; ++t)
-                  mma_f16(S[s + t], ar, kb ? yb[t].z : yb[t].x, kb ? yb[t].w : yb[t].y);
+                  mma_f16(S[s + t], ar[s & 1], kb ? yb[t].z : yb[t].x, kb ? yb[t].w : yb[t].y);
               }
             }
             __syncwarp();                     // every lane has read the stage
             stage ^= 1;
-            const int sh0 = fr0 - fk.x, sh1 = fr1 - fk.y;
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              long long hi, lo;
-              level_parts(S, e, hi, lo);
-              add_shifted(hi, lo, (e & 1) ? sh1 : sh0, hs[e], ls[e]);
+            if (u + step < n) {               // the next digits, in flight under the integer work
+              slot += back ? step : -step;
+              slot += slot < 0 ? slots : slot >= slots ? -slots : 0;
+              y_in(slot);
             }
-          }
-          long long *po = part + (((q + 1) & 1) * 4 + p) * 2 * kSwPart;
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const int o = (t2 + (e & 1)) * kSwCol + m0 + g + 8 * (e >> 1);
-            po[o] = hs[e];
-            po[kSwPart + o] = ls[e];
+            for (int e = 0; e < 4; ++e)
+#pragma unroll
+              for (int l = 0; l < kDig; ++l)
+                A[l][e] += l < 2 ? __float_as_int(S[l][e]) : __float2int_rn(S[l][e]);
+            ++cnt;
           }
-          if (fw == 0 && lane < 8) fref[((q + 1) & 1) * 8 + lane] = fr;
+          if (cnt > 0 || first) flush();      // zeros if there was no tile
         }
-        sw_bar_all();
+        if (rank) sw_bar_cta();               // to this CTA's summing warps
+        sw_bar_all(cl);
+      }
+    } else if (rank) {
+      // ---- summing warps of the second CTA
+      const int o = warp * kSwCol + lane;
+      for (int q = 0; q < nt; ++q) {
+        sw_bar_cta();
+        if (q + 1 < nt) {
+          const int buf = ((q + 1) & 1) * np;
+          long long h = 0, l = 0;
+#pragma unroll
+          for (int p = 0; p < 4; ++p) {
+            h += part[(buf + p) * 2 * kSwPart + o];
+            l += part[(buf + p) * 2 * kSwPart + kSwPart + o];
+          }
+          long long *po = cluster.map_shared_rank(part, 0) + (buf + 3 + rank) * 2 * kSwPart + o;
+          po[0] = h;
+          po[kSwPart] = l;
+        }
+        sw_bar_all(cl);
       }
     } else {
-      // ---- chain warps: thread (rho, c) owns rows 2 rho, 2 rho + 1 of column c
-      const int kb = warp & 1, m0 = 16 * (warp >> 1), c = tid & 7, r0 = 2 * (tid >> 3);
-      const int t2 = 2 * (lane & 3), g = lane >> 2;
-      const int col = grp * 8 + c;
-      const bool live = col < P.ncols;
+      // ---- chain warps: thread (c, r) = (warp, lane) owns row r of column c
+      const bool mult = warp < 4;             // the others: t = b - far sum, copies
+      const int kb = warp & 1, m0 = 16 * ((warp >> 1) & 1), t2 = 2 * (lane & 3), g = lane >> 2;
+      const int c = warp, o = c * kSwCol + lane, c2 = 2 * (warp & 3);
       const bool fresh = !(back && (P.mode & 1));
-      const double *src = fresh ? P.in + j * P.in_sys + col : P.out + j * P.out_sys + col;
+      const double *src = (fresh ? P.in + j * P.in_sys : P.out + j * P.out_sys) + grp * 8 + c2;
       const long long sst = fresh ? P.in_row : P.out_row;
-      double *dst = P.out + j * P.out_sys + col;
-      const int *re = P.D.rexp + (long long)j * P.D.npad, *de = P.D.dexp + (long long)j * P.D.npad;
-      // word of rows (r0, r0 + 1), column c in a row block of digits
-      const int word = (c * 4 + ((r0 & 7) >> 1)) * 4 + 2 * (r0 >> 4) + ((r0 >> 3) & 1);
+      double *dst = P.out + j * P.out_sys + grp * 8 + c;
+      const bool live0 = !mult && grp * 8 + c2 < P.ncols, live1 = !mult && grp * 8 + c2 + 1 < P.ncols;
+      const int *re = P.D.rexp + (long long)j * P.D.npad + lane, *de = P.D.dexp + (long long)j * P.D.npad + lane;
+      // half of row `lane`, column c in a row block of digits
+      const int half = 2 * ((c * 4 + ((lane & 7) >> 1)) * 4 + 2 * (lane >> 4) + ((lane >> 3) & 1)) + (lane & 1);
       double b0 = 0.0, b1 = 0.0, n0 = 0.0, n1 = 0.0;
-      int2 eR{0, 0}, eD{0, 0};
-      auto fetch = [&](int q, double &v0, double &v1, int2 &er, int2 &ed) {
-        const int l = row(q) * 32 + r0;
-        v0 = live && l < L.n ? src[l * sst] : 0.0;
-        v1 = live && l + 1 < L.n ? src[(l + 1) * sst] : 0.0;
-        er = *reinterpret_cast<const int2 *>(re + l);
-        ed = *reinterpret_cast<const int2 *>(de + l);
+      int eR = 0, eD = 0, nR = 0, nD = 0;
+      auto fetch = [&](int q) {
+        const int i = row(q) * 32 + lane;
+        n0 = live0 && i < L.n ? src[i * sst] : 0.0;
+        n1 = live1 && i < L.n ? src[i * sst + 1] : 0.0;
+        nR = re[row(q) * 32];
+        nD = de[row(q) * 32];
       };
-      fetch(0, b0, b1, eR, eD);
-      const uint32_t tiles = dig_smem(chain_t);
-      auto tile_in = [&](uint32_t dst, int I, int d) {       // a chain tile, by the chain warps
-        const __half *src = dig_tile(P.D, L, j, back ? I + d : I, d);
+      const uint32_t diag_t = dig_smem(chain_t), near_t = diag_t + 2 * kDigBytes;
+      const int nmask = P.nbuf - 1, ct = tid & 127;
+      auto tile_in = [&](uint32_t to, int I, int d) {        // a chain tile, by four warps
+        const char *from = tiles + tile_at(I, d) + ct * 16;
 #pragma unroll
-        for (int k = 0; k < 7; ++k) cp16(dst + 16 * (k * 128 + tid), src + 8 * (k * 128 + tid));
+        for (int k = 0; k < 7; ++k) cp16(to + 16 * (k * 128 + ct), from + k * 2048);
       };
-      tile_in(tiles + kDigBytes, row(0), 0);
-      cp_commit();
-      // product of this warp's quarter of a chain tile with a digit block, to nearp[kb]
-      auto product = [&](uint32_t tile, const uint32_t *dig) {
+      auto near_in = [&](int q) {
+        if (q < nt && dmax(row(q)) >= 1) tile_in(near_t + (q & nmask) * kDigBytes, row(q), 1);
+      };
+      // product of this warp's quarter of a chain tile with the digit block, to nearp[kb]
+      auto product = [&](uint32_t tile) {
         __syncwarp();
         float S[kDig][4];
         uint2 yb[kDig];
-#pragma unroll
-        for (int l = 0; l < kDig; ++l) {
-          yb[l] = *reinterpret_cast<const uint2 *>(dig + l * 128 + lane * 4 + 2 * kb);
-#pragma unroll
-          for (int e = 0; e < 4; ++e) S[l][e] = 0.f;
-        }
+        uint32_t ar[kDig][4];
         const uint32_t ab = tile + (back ? ldsm_at(m0, 16 * kb, lane) : ldsm_a(m0, 16 * kb, lane));
 #pragma unroll
         for (int s = 0; s < kDig; ++s) {
-          uint32_t ar[4];
-          if (back) ldsm4_trans(ar, ab + s * 2048);
-          else ldsm4(ar, ab + s * 2048);
-#pragma unroll
-          for (int t = 0; t < kDig - s; ++t) mma_f16(S[s + t], ar, yb[t].x, yb[t].y);
+          yb[s] = *reinterpret_cast<const uint2 *>(dig + s * 128 + lane * 4 + 2 * kb);
+          if (back) ldsm4_trans(ar[s], ab + s * 2048);
+          else ldsm4(ar[s], ab + s * 2048);
         }
+        level_start<4>(S);
+#pragma unroll
+        for (int s = 0; s < kDig; ++s)
+#pragma unroll
+          for (int t = 0; t < kDig - s; ++t) mma_f16(S[s + t], ar[s], yb[t].x, yb[t].y);
         long long *po = nearp + kb * 2 * kSwPart;
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           long long hi, lo;
-          level_parts(S, e, hi, lo);
-          const int o = (t2 + (e & 1)) * kSwCol + m0 + g + 8 * (e >> 1);
-          po[o] = hi;
-          po[kSwPart + o] = lo;
+          level_parts<4>(S, e, hi, lo);
+          const int oe = (t2 + (e & 1)) * kSwCol + m0 + g + 8 * (e >> 1);
+          po[oe] = hi;
+          po[kSwPart + oe] = lo;
         }
       };
-      // largest exponent of a column over the 32 rows
-      auto col_max = [&](int v, int buf) {
-        v = max(v, __shfl_xor_sync(0xffffffffu, v, 8));
-        v = max(v, __shfl_xor_sync(0xffffffffu, v, 16));
-        int *cm = cmax + buf * 32;
-        if (lane < 8) cm[warp * 8 + lane] = v;
-        sw_bar_chain();
-        return max(max(cm[c], cm[8 + c]), max(cm[16 + c], cm[24 + c]));
+      auto store_digits = [&](const Fixed &v, int G, __half *a, __half *z) {
+        const long long xb = v.at(G) + kDigBias;
+#pragma unroll
+        for (int s = 0; s < kDig; ++s) {
+          const __half d = digit_half(xb, s);
+          a[s * 256] = d;
+          if (z) z[s * 256] = d;
+        }
       };
-      const int o = c * kSwCol + r0;
+      __half *dh = reinterpret_cast<__half *>(dig) + half;
+      fetch(0);
+      for (int z = lane; z < slots; z += 32) fexp[z * 8 + c] = kNoExp;   // the first CTA's copy
+      if (lane < 2) fref[lane * 8 + c] = kNoExp;
+      if (!mult) tile_in(diag_t, row(0), 0);
+      cp_commit();
+      cp_wait<0>();
+      sw_bar_chain();
+      int F = kNoExp;                         // scale of the last solved row, this column
+      Fixed y{0, kNoExp, false};
+      int yi = L.n;                           // its unknown, not yet stored
+      int slot = row(0) % slots;              // of row I
       for (int q = 0; q < nt; ++q) {
         const int I = row(q);
         const bool has1 = dmax(I) >= 1;
-        cp_wait<0>();                         // both tiles, copied during the previous row
-        sw_bar_chain();
-        if (has1) product(tiles, ydig + ((q + 1) & 1) * kSwY);
-        int2 nR{0, 0}, nD{0, 0};
-        if (q + 1 < nt) fetch(q + 1, n0, n1, nR, nD);
-        double s0 = b0, s1 = b1;
-        if (q > 0) {
-          const int ff = fref[(q & 1) * 8 + c];
-          longlong2 h{0, 0}, l{0, 0};
-#pragma unroll
-          for (int p = 0; p < 4; ++p) {
-            const long long *po = part + ((q & 1) * 4 + p) * 2 * kSwPart + o;
-            const longlong2 a = *reinterpret_cast<const longlong2 *>(po);
-            const longlong2 z = *reinterpret_cast<const longlong2 *>(po + kSwPart);
-            h.x += a.x;
-            h.y += a.y;
-            l.x += z.x;
-            l.y += z.y;
-          }
-          s0 -= parts_value(h.x, l.x, ff + (back ? 0 : eR.x));
-          s1 -= parts_value(h.y, l.y, ff + (back ? 0 : eR.y));
-        }
-        sw_bar_chain();
-        // the coupling tile has been read by every chain warp: refill it
-        if (q + 1 < nt && dmax(row(q + 1)) >= 1) tile_in(tiles, row(q + 1), 1);
-        cp_commit();
-        if (has1) {
-          const int fp = fexp[((back ? I + 1 : I - 1) % slots) * 8 + c];
-          const longlong2 ha = *reinterpret_cast<const longlong2 *>(nearp + o),
-                          la = *reinterpret_cast<const longlong2 *>(nearp + kSwPart + o),
-                          hb = *reinterpret_cast<const longlong2 *>(nearp + 2 * kSwPart + o),
-                          lb = *reinterpret_cast<const longlong2 *>(nearp + 3 * kSwPart + o);
-          s0 -= parts_value(ha.x + hb.x, la.x + lb.x, fp + (back ? 0 : eR.x));
-          s1 -= parts_value(ha.y + hb.y, la.y + lb.y, fp + (back ? 0 : eR.y));
-        }
-        // digits of s (backward: the rows of inv(L_II) carry their scales, folded into s)
-        {
-          const int f0 = back ? eD.x : 0, f1 = back ? eD.y : 0;
-          const int G = col_max(max(exp_above(s0) + f0, exp_above(s1) + f1), 0);
-          const long long x0 = fixed62(s0, G - f0) + kDigBias, x1 = fixed62(s1, G - f1) + kDigBias;
-#pragma unroll
-          for (int s = 0; s < kDig; ++s) sdig[s * 128 + word] = digit_pair(x0, x1, s);
-          sw_bar_chain();
-          product(tiles + kDigBytes, sdig);
-          sw_bar_chain();
-          if (q + 1 < nt) tile_in(tiles + kDigBytes, row(q + 1), 0);
-          cp_commit();
-          const longlong2 ha = *reinterpret_cast<const longlong2 *>(nearp + o),
-                          la = *reinterpret_cast<const longlong2 *>(nearp + kSwPart + o),
-                          hb = *reinterpret_cast<const longlong2 *>(nearp + 2 * kSwPart + o),
-                          lb = *reinterpret_cast<const longlong2 *>(nearp + 3 * kSwPart + o);
-          s0 = parts_value(ha.x + hb.x, la.x + lb.x, G + (back ? 0 : eD.x));
-          s1 = parts_value(ha.y + hb.y, la.y + lb.y, G + (back ? 0 : eD.y));
-        }
-        const int l = I * 32 + r0;
-        if (live && l < L.n) dst[(long long)l * P.out_row] = s0;
-        if (live && l + 1 < L.n) dst[(long long)(l + 1) * P.out_row] = s1;
-        // digits of the solved row (backward: scaled by the factor's row scales)
-        {
-          const int f0 = back ? eR.x : 0, f1 = back ? eR.y : 0;
-          const int F = col_max(max(exp_above(s0) + f0, exp_above(s1) + f1), 1);
-          const long long x0 = fixed62(s0, F - f0) + kDigBias, x1 = fixed62(s1, F - f1) + kDigBias;
-          uint32_t *ys = ydig + (q & 1) * kSwY + word;
-          uint32_t *yg = reinterpret_cast<uint32_t *>(yring + (long long)(I % slots) * (kSwY / 4)) + word;
-#pragma unroll
-          for (int s = 0; s < kDig; ++s) {
-            const uint32_t v = digit_pair(x0, x1, s);
-            ys[s * 128] = v;
-            yg[s * 128] = v;
-          }
-          if (r0 == 0) fexp[(I % slots) * 8 + c] = F;
-        }
         b0 = n0;
         b1 = n1;
         eR = nR;
         eD = nD;
-        sw_bar_all();
+        const int sR = back ? 0 : eR, sD = back ? 0 : eD, fR = back ? eR : 0, fD = back ? eD : 0;
+        if (mult) {
+          if (has1) product(near_t + (q & nmask) * kDigBytes);
+          if (nmask) near_in(q + 1);
+        } else {
+          // t = b - far sum, two entries, to the first block of partials
+          long long *po = part + (q & 1) * np * 2 * kSwPart + c2 * kSwCol + lane;
+#pragma unroll
+          for (int x = 0; x < 2; ++x, po += kSwCol) {
+            long long h = 0, l = 0;
+            int ef = kNoExp;
+            if (q > 0) {
+              ef = fref[(q & 1) * 8 + c2 + x] + sR;
+#pragma unroll 4
+              for (int p = 0; p < np; ++p) {
+                h += po[p * 2 * kSwPart];
+                l += po[p * 2 * kSwPart + kSwPart];
+              }
+            }
+            const double b = x ? b1 : b0;
+            const int eb = exp_above(b) - 10, ft = max(ef, eb);
+            long long ht = 0, lt = 0;
+            add_shifted(mantissa53(b), 0, ft - eb, ht, lt);
+            add_shifted(-h, -l, ft - ef, ht, lt);
+            po[0] = ht;
+            po[kSwPart] = lt;
+            tf[(c2 + x) * 32 + lane] = ft;
+          }
+          if (q + 1 < nt) tile_in(diag_t + ((q + 1) & 1) * kDigBytes, row(q + 1), 0);
+        }
+        cp_commit();
+        if (yi < L.n && grp * 8 + c < P.ncols) dst[(long long)yi * P.out_row] = y.value();
+        if (q + 1 < nt) fetch(q + 1);
+        sw_bar_chain();
+        int G;
+        {
+          const long long *tp = part + (q & 1) * np * 2 * kSwPart + o;
+          const int ft = tf[c * 32 + lane], en = has1 ? F + sR : kNoExp, fs = max(ft, en);
+          long long hs = 0, ls = 0;
+          add_shifted(tp[0], tp[kSwPart], fs - ft, hs, ls);
+          if (has1)
+            add_shifted(-(nearp[o] + nearp[2 * kSwPart + o]), -(nearp[kSwPart + o] + nearp[3 * kSwPart + o]),
+                        fs - en, hs, ls);
+          // digits of s (backward: the rows of inv(L_II) carry their scales, folded into s)
+          Fixed s = fixed_of(hs, ls, fs);
+          s.ex += fD;
+          G = __reduce_max_sync(0xffffffffu, s.ex);
+          store_digits(s, G, dh, nullptr);
+        }
+        sw_bar_chain();
+        int fm = kNoExp;                      // the largest scale of the window so far
+        for (int z = lane; z < slots; z += 32) fm = max(fm, (int)fexp[z * 8 + c]);
+        if (mult) {
+          product(diag_t + (q & 1) * kDigBytes);
+        } else if (!nmask) {
+          near_in(q + 1);
+          cp_commit();
+        }
+        fm = __reduce_max_sync(0xffffffffu, fm);
+        sw_bar_chain();
+        {
+          y = fixed_of(nearp[o] + nearp[2 * kSwPart + o], nearp[kSwPart + o] + nearp[3 * kSwPart + o], G + sD);
+          yi = I * 32 + lane;
+          // digits of the solved row (backward: scaled by the factor's row scales)
+          Fixed v = y;
+          v.ex += fR;
+          const int need = __reduce_max_sync(0xffffffffu, v.ex);
+          if (need > F || (need > kNoExp / 2 && F - need > kSwSlack)) F = need + 1;
+          store_digits(v, F, dh, reinterpret_cast<__half *>(yring + slot * (kSwY / 4)) + half);
+          if (lane < cl) {                    // the far warps of every CTA read these
+            cluster.map_shared_rank(fexp, lane)[slot * 8 + c] = (short)F;
+            cluster.map_shared_rank(fref, lane)[(q & 1) * 8 + c] = max(fm, F);
+          }
+          slot += back ? -1 : 1;
+          slot = slot < 0 ? slots - 1 : slot == slots ? 0 : slot;
+        }
+        cp_wait<0>();                         // the next row's tiles, before the barrier
+        sw_bar_all(cl);
       }
+      if (yi < L.n && grp * 8 + c < P.ncols) dst[(long long)yi * P.out_row] = y.value();
+      sw_bar_chain();                         // before the backward sweep fetches them
     }
   }
 }
@@ -777,13 +867,33 @@ size_t band_solve_scratch(int nsys, int w_max, int ncols) {
 int launch_band_solve64(const BandLayout *d_lay, int nsys, int w_max, const DigitBand &D,
                         void *scratch, const double *in, long long in_sys, int in_row, double *out,
                         long long out_sys, int out_row, int ncols, int mode, DevStatus *st,
-                        cudaStream_t s) {
-  const int sm = sweep_smem(w_max);
-  if (sm > 227 * 1024 || D.window) return GENEO_ERR_INVALID_ARG;
+                        cudaStream_t s, int alongside) {
+  if (D.window) return GENEO_ERR_INVALID_ARG;
+  int dev = 0, sms = 0;
+  GENEO_CUDA_TRY(cudaGetDevice(&dev));
+  GENEO_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  // A second CTA for the far tiles while every CTA of the launches in flight
+  // still has an SM of its own and a full row has a tile for each pair of warps.
+  const int groups = (ncols + 7) / 8;
+  const int cl = 2 * groups * (nsys + alongside) <= sms && w_max - 1 > 4 &&
+                         sweep_smem(w_max, 2, 1) <= 227 * 1024 ? 2 : 1;
+  const int nbuf = sweep_smem(w_max, cl, 2) <= 227 * 1024 ? 2 : 1;   // coupling tiles in flight
+  const int sm = sweep_smem(w_max, cl, nbuf);
+  if (sm > 227 * 1024) return GENEO_ERR_INVALID_ARG;
   if (int rc = ensure_smem(k_band_sweep, sm)) return rc;
   const SweepArgs P{d_lay, D, static_cast<uint4 *>(scratch), w_max, in, in_sys, in_row, out, out_sys,
-                    out_row, ncols, mode, st};
-  k_band_sweep<<<dim3(nsys, (ncols + 7) / 8), kSwThreads, sm, s>>>(P); GENEO_COUNT_LAUNCH();
+                    out_row, ncols, mode, cl, nbuf};
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(nsys * cl, groups);
+  cfg.blockDim = dim3(kSwThreads);
+  cfg.dynamicSmemBytes = sm;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim = {(unsigned)cl, 1, 1};
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  GENEO_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_band_sweep, P)); GENEO_COUNT_LAUNCH();
   GENEO_CUDA_TRY(cudaGetLastError());
   return GENEO_OK;
 }

@@ -1027,7 +1027,7 @@ static int setup_coarse(geneo_ctx *c, SetupPlan &P, cudaStream_t s) {
   if (ngrp == 2) GENEO_CUDA_TRY(cudaStreamWaitEvent(grp[1].st, e_fork, 0));
   auto lanczos_step = [&](const Group &g, int k) -> int {
     const long long j0 = g.j0;
-    const int n = g.n;
+    const int n = g.n, other = nsub - n;
     cudaStream_t gs = g.st;
     const SubDesc *subs = pc.d_subs + j0;
     const BandLayout *lay = pc.d_lay_neu + j0;
@@ -1043,11 +1043,11 @@ static int setup_coarse(geneo_ctx *c, SetupPlan &P, cudaStream_t s) {
     char *scr = (char *)pc.solve_scr + band_solve_scratch((int)j0, pc.w_neu_max, p);
     // W = L^-1 B L^-T V_k
     if ((r = launch_band_solve64(lay, n, pc.w_neu_max, D, scr, V + k * p, sV, ldv, T1, sW, p, p, 2,
-                                 c->status, gs)))
+                                 c->status, gs, other)))
       return r;
     launch_bloc_mv(subs, n, P.max_nodes_neu, pc.Bloc, T1, W, sW, p, gs);
     if ((r = launch_band_solve64(lay, n, pc.w_neu_max, D, scr, W, sW, p, W, sW, p, p, 1, c->status,
-                                 gs)))
+                                 gs, other)))
       return r;
     const int na = (k + 1) * p;
     // full re-orthogonalisation against V: a second pass only for the

@@ -65,10 +65,12 @@ __device__ __forceinline__ __half digit_half(long long xb, int s) {
   return __hsub(__ushort_as_half((unsigned short)(0x6400u | digit_bits(xb, s))), __ushort_as_half(0x6500));
 }
 
-// Element (r, k) of a digit slice of a 32 x 32 tile: rows of 64 bytes whose
-// 16-byte chunks are permuted so that ldmatrix reads without bank conflicts.
+// Element (r, k) of a digit slice of a 32 x 32 tile: four 16 x 16 blocks, so
+// that sixteen rows or sixteen columns of the tile are whole 512-byte pieces
+// for a warp's copy, with rows of 32 bytes whose two 16-byte chunks change
+// places every four rows: ldmatrix reads them without bank conflicts.
 __device__ __forceinline__ int dig_index(int r, int k) {
-  return r * 32 + ((((k >> 3) ^ (r >> 1)) & 3) << 3) + (k & 7);
+  return (r >> 4) * 512 + (k >> 4) * 256 + (r & 15) * 16 + ((((k >> 3) ^ (r >> 2)) & 1) << 3) + (k & 7);
 }
 
 __device__ __forceinline__ uint32_t dig_smem(const void *p) {
@@ -107,20 +109,79 @@ __device__ __forceinline__ uint32_t ldsm_b(int n0, int k0, int lane) {
   return 2 * dig_index(n0 + (lane & 7), k0 + 8 * ((lane >> 3) & 1));
 }
 
-// The two integer parts of one product entry from its level sums.
+// The two integer parts of one product entry from its level sums.  Levels below
+// M, whose sums stay within 2^22 (over 16 terms the first four, over 32 the first
+// two), start at 1.5 2^23 (level_start) and are read from the bits: conversions
+// issue at an eighth of the rate of integer instructions.
+constexpr float kLevelOne = 12582912.f;          // 1.5 2^23: unit spacing, 2^22 either way
+template <int M>
+__device__ __forceinline__ void level_start(float (&S)[kDig][4]) {
+#pragma unroll
+  for (int l = 0; l < kDig; ++l)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) S[l][e] = l < M ? kLevelOne : 0.f;
+}
+template <int M = 0>
 __device__ __forceinline__ void level_parts(const float (&S)[kDig][4], int e, long long &hi,
                                             long long &lo) {
-  const int s0 = __float2int_rn(S[0][e]), s1 = __float2int_rn(S[1][e]), s2 = __float2int_rn(S[2][e]),
-            s3 = __float2int_rn(S[3][e]), s4 = __float2int_rn(S[4][e]), s5 = __float2int_rn(S[5][e]),
-            s6 = __float2int_rn(S[6][e]);
-  hi = (long long)(s0 * 512 + s1) * 262144 + ((long long)s2 * 512 + s3);
-  lo = (long long)s4 * 262144 + ((long long)s5 * 512 + s6);
+  int s[kDig];
+#pragma unroll
+  for (int l = 0; l < kDig; ++l)
+    s[l] = l < M ? __float_as_int(S[l][e]) - 0x4b400000 : __float2int_rn(S[l][e]);
+  hi = (long long)(s[0] * 512 + s[1]) * 262144 + ((long long)s[2] * 512 + s[3]);
+  lo = (long long)s[4] * 262144 + ((long long)s[5] * 512 + s[6]);
 }
 
 // (hi 2^27 + lo) 2^(e - 70)
 __device__ __forceinline__ double parts_value(long long hi, long long lo, int e) {
   const int k = min(max(e - 70, -1022), 1023);
   return fma((double)hi, 134217728.0, (double)lo) * __hiloint2double((k + 1023) << 20, 0);
+}
+
+// m 2^(ex - 64) with 2^63 <= m < 2^64, or zero (m = 0, ex <= kNoExp), and a sign.
+struct Fixed {
+  unsigned long long m;
+  int ex;
+  bool neg;
+  // The number times 2^(62 - G), rounded to an integer (ex <= G).
+  __device__ __forceinline__ long long at(int G) const {
+    const int sh = 2 + G - ex;
+    const long long x = m == 0 || sh > 64 ? 0 : (long long)((m >> (sh - 1)) + 1) >> 1;
+    return neg ? -x : x;
+  }
+  // As a double, rounded to nearest; zero below the normal range.
+  __device__ __forceinline__ double value() const {
+    const int be = ex + 1022;
+    if (m == 0 || be < 1) return 0.0;
+    const unsigned long long b = be > 2046 ? 0x7ff0000000000000ULL
+                                           : ((unsigned long long)(be - 1) << 52) + (m >> 11) + ((m >> 10) & 1);
+    return __longlong_as_double((long long)(b | (neg ? 0x8000000000000000ULL : 0)));
+  }
+};
+
+// (hi 2^27 + lo) 2^(f - 70), to 64 bits.
+__device__ __forceinline__ Fixed fixed_of(long long hi, long long lo, int f) {
+  unsigned long long l = ((unsigned long long)hi << 27) + (unsigned long long)lo;
+  unsigned long long h = (unsigned long long)((hi >> 37) + (lo >> 63)) + (l < (unsigned long long)lo);
+  const bool neg = (long long)h < 0;
+  if (neg) {
+    l = 0 - l;
+    h = ~h + (l == 0);
+  }
+  const bool wide = h != 0;
+  const unsigned long long t = wide ? h : l;
+  const int z = __clzll(t);                      // 64 if zero
+  unsigned long long m = t << (z & 63);
+  if (wide && z) m |= l >> (64 - z);
+  return t ? Fixed{m, (wide ? 58 : -6) - z + f, neg} : Fixed{0, kNoExp, false};
+}
+
+// The integer M with v = M 2^(exp_above(v) - 53), |M| < 2^53 (zero for subnormal v).
+__device__ __forceinline__ long long mantissa53(double v) {
+  const long long b = __double_as_longlong(v);
+  if (!((b >> 52) & 0x7ff)) return 0;
+  const long long m = (b & 0xfffffffffffffLL) | 0x10000000000000LL;
+  return b < 0 ? -m : m;
 }
 
 // 16-byte asynchronous copies into shared memory, in groups of the issuing thread.
