@@ -73,8 +73,11 @@ __device__ __forceinline__ double spmv_lane_row(const int32_t *__restrict__ rp,
   return s;
 }
 
-template <int NC>
-__global__ void __launch_bounds__(256, 8) k_spmv(int nnode, const int32_t *__restrict__ rp,
+// U: blocks of a row loaded together.  1 for large systems (above); 9 when the
+// rows are too few to fill the chip, where a row is a chain of 27 dependent
+// gathers (8x8x8 elements: 16 us a product).  The sums are the same.
+template <int NC, int U>
+__global__ void __launch_bounds__(256, U == 1 ? 8 : 2) k_spmv(int nnode, const int32_t *__restrict__ rp,
                                               const int32_t *__restrict__ col,
                                               const double *__restrict__ val,
                                               const double *__restrict__ x,
@@ -87,13 +90,13 @@ __global__ void __launch_bounds__(256, 8) k_spmv(int nnode, const int32_t *__res
     const int row = g * 32 + lane;
     if (row < nrow) {
       const int node = row / NC;
-      y[row] = spmv_lane_row<NC>(rp, col, val, x, node, row - NC * node);
+      y[row] = spmv_lane_row<NC, U>(rp, col, val, x, node, row - NC * node);
     }
   }
 }
 
-template <int NC>
-__global__ void __launch_bounds__(NT, 8) k_cg_spmv_pq(int nnode, const int32_t *__restrict__ rp,
+template <int NC, int U>
+__global__ void __launch_bounds__(NT, U == 1 ? 8 : 2) k_cg_spmv_pq(int nnode, const int32_t *__restrict__ rp,
                                                    const int32_t *__restrict__ col,
                                                    const double *__restrict__ val,
                                                    const double *__restrict__ p,
@@ -110,7 +113,7 @@ __global__ void __launch_bounds__(NT, 8) k_cg_spmv_pq(int nnode, const int32_t *
     const int row = g * 32 + lane;
     if (row < nrow) {
       const int node = row / NC;
-      const double yv = spmv_lane_row<NC>(rp, col, val, p, node, row - NC * node);
+      const double yv = spmv_lane_row<NC, U>(rp, col, val, p, node, row - NC * node);
       q[row] = yv;
       acc = fma(p[row], yv, acc);
     }
@@ -530,50 +533,56 @@ void launch_batch_reduce(const BatchInst *inst, const BatchTables &T, CGScalars 
   k_batch_reduce<<<T.n, NT, 0, s>>>(T.task_off, cg, tpart, kind, alphas, betas, hist, out); GENEO_COUNT_LAUNCH();
 }
 
+// Blocks with a row to work on, NB (x 4) at most: with fewer than that every
+// thread has the row it would have in the full grid and the blocks left out
+// have no part in the sums, so results do not change, but the last block waits
+// for fewer tickets (2,187 unknowns: 9 blocks, not 304).
+static unsigned row_grid(int n, int most) { return std::max(1, std::min(most, (n + NT - 1) / NT)); }
+// At most eight warps of rows per SM: latency, not the loads in flight, decides.
+static bool few_rows(int n) { return n <= 152 * 8 * 32; }
+
 void launch_spmv(const BSR &A, const double *x, double *y, cudaStream_t s) {
-  if (A.nc == 1) {
-    k_spmv<1><<<NB * 4, 256, 0, s>>>(A.nnode, A.row_ptr, A.col, A.val, x, y); GENEO_COUNT_LAUNCH();
-  } else {
-    k_spmv<3><<<NB * 4, 256, 0, s>>>(A.nnode, A.row_ptr, A.col, A.val, x, y); GENEO_COUNT_LAUNCH();
-  }
+  const int n = A.nc * A.nnode;
+  auto k = A.nc == 1 ? (few_rows(n) ? k_spmv<1, 9> : k_spmv<1, 1>)
+                     : (few_rows(n) ? k_spmv<3, 9> : k_spmv<3, 1>);
+  k<<<row_grid(n, NB * 4), NT, 0, s>>>(A.nnode, A.row_ptr, A.col, A.val, x, y); GENEO_COUNT_LAUNCH();
 }
 void launch_cg_init(int n, const double *b, double *x, double *r, CGScalars *cg, double *part,
                     cudaStream_t s) {
-  k_cg_init<<<NB, NT, 0, s>>>(n, b, x, r, cg, part); GENEO_COUNT_LAUNCH();
+  k_cg_init<<<row_grid(n, NB), NT, 0, s>>>(n, b, x, r, cg, part); GENEO_COUNT_LAUNCH();
 }
 void launch_cg_init2(int n, const double *r, const double *z, double *p, CGScalars *cg,
                      double *part, cudaStream_t s) {
-  k_cg_init2<<<NB, NT, 0, s>>>(n, r, z, p, cg, part); GENEO_COUNT_LAUNCH();
+  k_cg_init2<<<row_grid(n, NB), NT, 0, s>>>(n, r, z, p, cg, part); GENEO_COUNT_LAUNCH();
 }
 void launch_cg_spmv_pq(const BSR &A, const double *p, double *q, CGScalars *cg, double *part,
                        cudaStream_t s) {
-  if (A.nc == 1) {
-    k_cg_spmv_pq<1><<<NB * 4, NT, 0, s>>>(A.nnode, A.row_ptr, A.col, A.val, p, q, cg, part); GENEO_COUNT_LAUNCH();
-  } else {
-    k_cg_spmv_pq<3><<<NB * 4, NT, 0, s>>>(A.nnode, A.row_ptr, A.col, A.val, p, q, cg, part); GENEO_COUNT_LAUNCH();
-  }
+  const int n = A.nc * A.nnode;
+  auto k = A.nc == 1 ? (few_rows(n) ? k_cg_spmv_pq<1, 9> : k_cg_spmv_pq<1, 1>)
+                     : (few_rows(n) ? k_cg_spmv_pq<3, 9> : k_cg_spmv_pq<3, 1>);
+  k<<<row_grid(n, NB * 4), NT, 0, s>>>(A.nnode, A.row_ptr, A.col, A.val, p, q, cg, part); GENEO_COUNT_LAUNCH();
 }
 void launch_cg_update_xr(int n, const double *p, const double *q, double *x, double *r,
                          CGScalars *cg, double *part, double *alphas, cudaStream_t s) {
-  k_cg_update_xr<<<NB, NT, 0, s>>>(n, p, q, x, r, cg, part, alphas); GENEO_COUNT_LAUNCH();
+  k_cg_update_xr<<<row_grid(n, NB), NT, 0, s>>>(n, p, q, x, r, cg, part, alphas); GENEO_COUNT_LAUNCH();
 }
 void launch_cg_dots(int n, const double *r, const double *z, const double *q, CGScalars *cg,
                     double *part, double *betas, cudaStream_t s) {
-  k_cg_dots<<<NB, NT, 0, s>>>(n, r, z, q, cg, part, betas); GENEO_COUNT_LAUNCH();
+  k_cg_dots<<<row_grid(n, NB), NT, 0, s>>>(n, r, z, q, cg, part, betas); GENEO_COUNT_LAUNCH();
 }
 void launch_cg_update_p(int n, const double *z, double *p, CGScalars *cg, cudaStream_t s) {
-  k_cg_update_p<<<NB, NT, 0, s>>>(n, z, p, cg); GENEO_COUNT_LAUNCH();
+  k_cg_update_p<<<row_grid(n, NB), NT, 0, s>>>(n, z, p, cg); GENEO_COUNT_LAUNCH();
 }
 void launch_copy_if_running(int n, const double *src, double *dst, const CGScalars *cg,
                             cudaStream_t s) {
-  k_copy_if_running<<<NB, NT, 0, s>>>(n, src, dst, cg); GENEO_COUNT_LAUNCH();
+  k_copy_if_running<<<row_grid(n, NB), NT, 0, s>>>(n, src, dst, cg); GENEO_COUNT_LAUNCH();
 }
 void launch_norm2(int n, const double *v, double *out, double *part, unsigned *counter,
                   cudaStream_t s) {
-  k_norm2<<<NB, NT, 0, s>>>(n, v, out, part, counter); GENEO_COUNT_LAUNCH();
+  k_norm2<<<row_grid(n, NB), NT, 0, s>>>(n, v, out, part, counter); GENEO_COUNT_LAUNCH();
 }
 void launch_sub(int n, const double *a, const double *b, double *out, cudaStream_t s) {
-  k_sub<<<NB, NT, 0, s>>>(n, a, b, out); GENEO_COUNT_LAUNCH();
+  k_sub<<<row_grid(n, NB), NT, 0, s>>>(n, a, b, out); GENEO_COUNT_LAUNCH();
 }
 
 }  // namespace geneo
