@@ -427,8 +427,8 @@ constexpr int kSwPart = 8 * kSwCol;         // one 32 x 8 block of them
 constexpr int kSwY = kDig * 128;            // words of one row block of y digits
 constexpr int kSwSlack = 4;                 // bits a column's scale may be too large
 constexpr int kSwFlush = 64;                // tiles added in 32 bits: 64 * 7 * 2^21 < 2^31
-__host__ __device__ constexpr int sweep_smem(int w, int cl, int nbuf) {
-  return (2 + nbuf) * (int)kDigBytes + kSwFar * 2 * kSwHalf + (2 * (3 + cl) + 2) * kSwPart * 16 +
+__host__ __device__ constexpr int sweep_smem(int w, int cl) {
+  return 3 * (int)kDigBytes + kSwFar * 2 * kSwHalf + (2 * (3 + cl) + 2) * kSwPart * 16 +
          kSwY * 4 + 8 * 32 * 4 + 2 * 8 * 4 + (w + 2) * 16;
 }
 
@@ -466,7 +466,7 @@ struct SweepArgs {
   int in_row;
   double *out;
   long long out_sys;
-  int out_row, ncols, mode, cl, nbuf;
+  int out_row, ncols, mode, cl;
 };
 
 __global__ void __launch_bounds__(kSwThreads, 1) k_band_sweep(const SweepArgs P) {
@@ -474,8 +474,8 @@ __global__ void __launch_bounds__(kSwThreads, 1) k_band_sweep(const SweepArgs P)
   const int cl = P.cl, rank = blockIdx.x % cl, j = blockIdx.x / cl, grp = blockIdx.y;
   const BandLayout L = P.lay[j];
   const int nt = L.nt, w = L.w, slots = w + 2, np = 3 + cl;
-  unsigned char *chain_t = smraw;                                   // [diagonal x 2, near x nbuf]
-  unsigned char *far_t = chain_t + (2 + P.nbuf) * kDigBytes;        // [warp][2] half tiles
+  unsigned char *chain_t = smraw;                                   // [diagonal x 2, coupling]
+  unsigned char *far_t = chain_t + 3 * kDigBytes;                  // [warp][2] half tiles
   long long *part = reinterpret_cast<long long *>(far_t + kSwFar * 2 * kSwHalf);  // [2][np][hi, lo]
   long long *nearp = part + 2 * np * 2 * kSwPart;                   // [2][hi, lo]
   uint32_t *dig = reinterpret_cast<uint32_t *>(nearp + 2 * 2 * kSwPart);   // digits of s or y
@@ -666,14 +666,14 @@ __global__ void __launch_bounds__(kSwThreads, 1) k_band_sweep(const SweepArgs P)
         nD = de[row(q) * 32];
       };
       const uint32_t diag_t = dig_smem(chain_t), near_t = diag_t + 2 * kDigBytes;
-      const int nmask = P.nbuf - 1, ct = tid & 127;
+      const int ct = tid & 127;
       auto tile_in = [&](uint32_t to, int I, int d) {        // a chain tile, by four warps
         const char *from = tiles + tile_at(I, d) + ct * 16;
 #pragma unroll
         for (int k = 0; k < 7; ++k) cp16(to + 16 * (k * 128 + ct), from + k * 2048);
       };
       auto near_in = [&](int q) {
-        if (q < nt && dmax(row(q)) >= 1) tile_in(near_t + (q & nmask) * kDigBytes, row(q), 1);
+        if (q < nt && dmax(row(q)) >= 1) tile_in(near_t, row(q), 1);
       };
       // product of this warp's quarter of a chain tile with the digit block, to nearp[kb]
       auto product = [&](uint32_t tile) {
@@ -733,8 +733,7 @@ __global__ void __launch_bounds__(kSwThreads, 1) k_band_sweep(const SweepArgs P)
         eD = nD;
         const int sR = back ? 0 : eR, sD = back ? 0 : eD, fR = back ? eR : 0, fD = back ? eD : 0;
         if (mult) {
-          if (has1) product(near_t + (q & nmask) * kDigBytes);
-          if (nmask) near_in(q + 1);
+          if (has1) product(near_t);
         } else {
           // t = b - far sum, two entries, to the first block of partials
           long long *po = part + (q & 1) * np * 2 * kSwPart + c2 * kSwCol + lane;
@@ -785,8 +784,8 @@ __global__ void __launch_bounds__(kSwThreads, 1) k_band_sweep(const SweepArgs P)
         for (int z = lane; z < slots; z += 32) fm = max(fm, (int)fexp[z * 8 + c]);
         if (mult) {
           product(diag_t + (q & 1) * kDigBytes);
-        } else if (!nmask) {
-          near_in(q + 1);
+        } else {
+          near_in(q + 1);                     // the coupling tile has been read
           cp_commit();
         }
         fm = __reduce_max_sync(0xffffffffu, fm);
@@ -876,13 +875,12 @@ int launch_band_solve64(const BandLayout *d_lay, int nsys, int w_max, const Digi
   // still has an SM of its own and a full row has a tile for each pair of warps.
   const int groups = (ncols + 7) / 8;
   const int cl = 2 * groups * (nsys + alongside) <= sms && w_max - 1 > 4 &&
-                         sweep_smem(w_max, 2, 1) <= 227 * 1024 ? 2 : 1;
-  const int nbuf = sweep_smem(w_max, cl, 2) <= 227 * 1024 ? 2 : 1;   // coupling tiles in flight
-  const int sm = sweep_smem(w_max, cl, nbuf);
+                         sweep_smem(w_max, 2) <= 227 * 1024 ? 2 : 1;
+  const int sm = sweep_smem(w_max, cl);
   if (sm > 227 * 1024) return GENEO_ERR_INVALID_ARG;
   if (int rc = ensure_smem(k_band_sweep, sm)) return rc;
   const SweepArgs P{d_lay, D, static_cast<uint4 *>(scratch), w_max, in, in_sys, in_row, out, out_sys,
-                    out_row, ncols, mode, cl, nbuf};
+                    out_row, ncols, mode, cl};
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(nsys * cl, groups);
   cfg.blockDim = dim3(kSwThreads);
