@@ -263,65 +263,6 @@ __global__ void k_random_block(const SubDesc *subs, int npad, double *V, int ld,
   V[j * stride + (long long)row * ld + c] = v;
 }
 
-// partial dot products over a chunk of rows, staged 16 rows at a time
-__global__ void __launch_bounds__(256)
-    k_tsdots(const SubDesc *subs, const double *__restrict__ A, int lda, long long sa, int na,
-             const double *__restrict__ B, int ldb, long long sb, int nb, double *Hpart,
-             int chunks, const int *gate) {
-  const int j = blockIdx.y, ch = blockIdx.x;
-  if (gate && !gate[j]) return;                       // the reduction writes zeros
-  const int n = subs[j].n_neu;
-  const int per = (n + chunks - 1) / chunks;
-  const int r0 = ch * per, r1 = min(n, r0 + per);
-  const int nout = na * nb;
-  extern __shared__ __align__(16) unsigned char smraw[];
-  double *sA = reinterpret_cast<double *>(smraw);     // [16][na]
-  double *sB = sA + 16 * na;                          // [16][nb]
-  double acc[5] = {0, 0, 0, 0, 0};
-  const double *Aj = A + j * sa;
-  const double *Bj = B + j * sb;
-  for (int rb = r0; rb < r1; rb += 16) {
-    int nr = min(16, r1 - rb);
-    for (int e = threadIdx.x; e < 16 * na; e += 256) {
-      int rr = e / na, c = e - rr * na;
-      sA[e] = rr < nr ? Aj[(long long)(rb + rr) * lda + c] : 0.0;
-    }
-    for (int e = threadIdx.x; e < 16 * nb; e += 256) {
-      int rr = e / nb, c = e - rr * nb;
-      sB[e] = rr < nr ? Bj[(long long)(rb + rr) * ldb + c] : 0.0;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < 5; ++q) {
-      int o = threadIdx.x + 256 * q;
-      if (o < nout) {
-        int a = o / nb, b = o - a * nb;
-        double s = 0.0;
-        for (int rr = 0; rr < 16; ++rr) s += sA[rr * na + a] * sB[rr * nb + b];
-        acc[q] += s;
-      }
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int q = 0; q < 5; ++q) {
-    int o = threadIdx.x + 256 * q;
-    if (o < nout) Hpart[((long long)j * chunks + ch) * nout + o] = acc[q];
-  }
-}
-
-__global__ void k_tsdots_reduce(const double *Hpart, int chunks, int nout, double *H, long long hs,
-                                const int *gate) {
-  const int j = blockIdx.x;
-  const bool skip = gate && !gate[j];
-  for (int o = threadIdx.x; o < nout; o += blockDim.x) {
-    double s = 0.0;
-    if (!skip)
-      for (int ch = 0; ch < chunks; ++ch) s += Hpart[((long long)j * chunks + ch) * nout + o];
-    H[j * hs + o] = s;
-  }
-}
-
 // Second re-orthogonalisation pass needed?  After one projection W -= V H,
 // column b of W has squared norm G_bb and lost sum_a H_ab^2; the pass is
 // repeated where more than half of the column's squared norm was removed,
@@ -344,34 +285,6 @@ __global__ void k_reorth_gate(const double *G, int p, const double *H, int na, l
   }
   __syncthreads();
   if (threadIdx.x == 0) gate[j] = need;
-}
-
-__global__ void __launch_bounds__(256)
-    k_tsgemm(const SubDesc *subs, int npad, const double *__restrict__ A, int lda, long long sa,
-             int na, const double *__restrict__ H, int ldh, long long hs, double *C, int ldc,
-             long long sc, int nb, double alpha, double beta, const int *gate) {
-  const int j = blockIdx.y;
-  if (gate && !gate[j]) return;
-  extern __shared__ __align__(16) unsigned char smraw[];
-  double *sH = reinterpret_cast<double *>(smraw);   // [na][nb]
-  for (int e = threadIdx.x; e < na * nb; e += blockDim.x) {
-    int a = e / nb, b = e - a * nb;
-    sH[e] = H[j * hs + (long long)a * ldh + b];
-  }
-  __syncthreads();
-  const int n = subs[j].n_neu;
-  long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (long long)npad * nb) return;
-  int row = (int)(t / nb), b = (int)(t - (long long)row * nb);
-  double *cp = C + j * sc + (long long)row * ldc + b;
-  if (row >= n) {
-    if (beta == 0.0) *cp = 0.0;
-    return;
-  }
-  const double *ar = A + j * sa + (long long)row * lda;
-  double s = 0.0;
-  for (int a = 0; a < na; ++a) s += ar[a] * sH[a * nb + b];
-  *cp = (beta == 0.0 ? 0.0 : beta * *cp) + alpha * s;
 }
 
 // Cholesky of the p x p Gram matrix, inverse, and Racc update (one block per subdomain)
@@ -1045,35 +958,10 @@ void launch_random_block(const SubDesc *d_subs, int nsub, int npad, double *V, i
   k_random_block<<<g, 256, 0, s>>>(d_subs, npad, V, ld, sys_stride, p, seed); GENEO_COUNT_LAUNCH();
 }
 
-void launch_tsdots(const SubDesc *d_subs, int nsub, int npad, const double *A, int lda,
-                   long long sa, int na, const double *B, int ldb, long long sb, int nb,
-                   double *Hpart, int chunks, double *H, long long hs, cudaStream_t s,
-                   const int *gate) {
-  (void)npad;
-  int sm = 16 * (na + nb) * (int)sizeof(double);
-  (void)ensure_smem(k_tsdots, sm);   // a failure surfaces as a launch error
-  k_tsdots<<<dim3(chunks, nsub), 256, sm, s>>>(d_subs, A, lda, sa, na, B, ldb, sb, nb, Hpart,
-                                               chunks, gate); GENEO_COUNT_LAUNCH();
-  k_tsdots_reduce<<<nsub, 256, 0, s>>>(Hpart, chunks, na * nb, H, hs, gate); GENEO_COUNT_LAUNCH();
-}
-
 void launch_reorth_gate(int nsub, const double *G, int p, const double *H, int na, long long hs,
                         int *gate, cudaStream_t s) {
   k_reorth_gate<<<nsub, 32, 0, s>>>(G, p, H, na, hs, gate); GENEO_COUNT_LAUNCH();
 }
-
-void launch_tsgemm(const SubDesc *d_subs, int nsub, int npad, const double *A, int lda,
-                   long long sa, int na, const double *H, int ldh, long long hs, double *C,
-                   int ldc, long long sc, int nb, double alpha, double beta, cudaStream_t s,
-                   const int *gate) {
-  int sm = na * nb * (int)sizeof(double);
-  (void)ensure_smem(k_tsgemm, sm);
-  long long tot = (long long)npad * nb;
-  dim3 g((unsigned)((tot + 255) / 256), nsub);
-  k_tsgemm<<<g, 256, sm, s>>>(d_subs, npad, A, lda, sa, na, H, ldh, hs, C, ldc, sc, nb, alpha,
-                              beta, gate); GENEO_COUNT_LAUNCH();
-}
-
 void launch_cholqr(const SubDesc *d_subs, int nsub, int npad, const double *G, double *W,
                    int p, double *Racc, double *Rinv, int first, double abs_tiny, cudaStream_t s) {
   k_cholqr_small<<<nsub, 32, 0, s>>>(G, p, Rinv, Racc, first, abs_tiny); GENEO_COUNT_LAUNCH();
