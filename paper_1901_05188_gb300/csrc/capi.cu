@@ -252,6 +252,8 @@ int geneo_create(geneo_ctx **out, void *cuda_stream) {
   GENEO_CUDA_TRY(cudaStreamCreateWithPriority(&c->side_stream, cudaStreamNonBlocking, greatest));
   GENEO_CUDA_TRY(cudaStreamCreateWithFlags(&c->fac_stream, cudaStreamNonBlocking));
   GENEO_CUDA_TRY(cudaStreamCreateWithFlags(&c->fac_side, cudaStreamNonBlocking));
+  GENEO_CUDA_TRY(cudaEventCreateWithFlags(&c->coarse_fork, cudaEventDisableTiming));
+  GENEO_CUDA_TRY(cudaEventCreateWithFlags(&c->coarse_join, cudaEventDisableTiming));
   *out = c;
   return GENEO_OK;
 }
@@ -280,6 +282,8 @@ int geneo_destroy(geneo_ctx *c) {
   if (c->side_stream) cudaStreamDestroy(c->side_stream);
   if (c->fac_stream) cudaStreamDestroy(c->fac_stream);
   if (c->fac_side) cudaStreamDestroy(c->fac_side);
+  if (c->coarse_fork) cudaEventDestroy(c->coarse_fork);
+  if (c->coarse_join) cudaEventDestroy(c->coarse_join);
   delete c;
   return GENEO_OK;
 }
@@ -890,11 +894,21 @@ static int precond_apply(geneo_ctx *c, const double *r, double *z, const CGScala
                                             c->status, pc.c_inner, s)))
       return st;
   } else if (coarse) {
+    // The coarse correction needs only r, like the local solves, and runs beside
+    // them: these leave SMs free (one cluster per subdomain) and wait on their
+    // serial chains.  The side stream's priority lets the restriction start
+    // first.  60x220x85 Darcy: 175 us of 860 an iteration, one after the other.
+    GENEO_CUDA_TRY(cudaEventRecord(c->coarse_fork, s));
+    GENEO_CUDA_TRY(cudaStreamWaitEvent(c->side_stream, c->coarse_fork, 0));
     launch_coarse_apply(pc.d_subs, pc.nsub, pc.max_nint, nnx, nny, pc.Zp, r, pc.wpart, pc.wH,
-                        pc.yH, pc.zy, pc.AHinv, pc.nH, pc.mcap, cg, s);
+                        pc.yH, pc.zy, pc.AHinv, pc.nH, pc.mcap, cg, c->side_stream);
+    GENEO_CUDA_TRY(cudaEventRecord(c->coarse_join, c->side_stream));
   }
   const int pou = pc.schwarz == GENEO_AS_POU;
-  if ((st = schwarz_local_solves(c, r, cg, pc.cluster, pc.rows, pc.staged, s))) return st;
+  st = schwarz_local_solves(c, r, cg, pc.cluster, pc.rows, pc.staged, s);
+  if (coarse && pc.csolver != GENEO_COARSE_ITERATIVE)
+    GENEO_CUDA_TRY(cudaStreamWaitEvent(s, c->coarse_join, 0));
+  if (st) return st;
   if (pc.prec == GENEO_MIXED_FP32) {
     launch_schwarz_gather<float>(c->nx, c->ny, c->nz, pc.part.px, pc.part.py, pc.d_cand,
                                  pc.cand_off, pc.d_subs, pc.gmap, pc.gcnt,
@@ -2239,6 +2253,8 @@ struct geneo_batch {
   long long graph_kernels = 0;
   float ms_tune = 0.f;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;   // timing of a batched solve
+  cudaStream_t side = nullptr;                // the coarse corrections, beside the local solves
+  cudaEvent_t fork = nullptr, join = nullptr;
 };
 
 namespace {
@@ -2247,7 +2263,12 @@ constexpr int kBatchHist = 4096;   // Krylov coefficients kept per instance (con
 
 int batch_precond(geneo_batch *B, const double *r, double *z, int head, cudaStream_t s) {
   int st;
-  if (B->any_coarse) launch_batch_coarse(B->d_inst, B->T, B->cg, r, s);
+  if (B->any_coarse) {
+    GENEO_CUDA_TRY(cudaEventRecord(B->fork, s));
+    GENEO_CUDA_TRY(cudaStreamWaitEvent(B->side, B->fork, 0));
+    launch_batch_coarse(B->d_inst, B->T, B->cg, r, B->side);
+    GENEO_CUDA_TRY(cudaEventRecord(B->join, B->side));
+  }
   GENEO_CUDA_TRY(cudaMemsetAsync(B->heads + head, 0, sizeof(int), s));
   const int clusters = std::max(1, std::min(B->sms / B->cluster, B->T.nsub_items));
   if (B->f32)
@@ -2258,6 +2279,7 @@ int batch_precond(geneo_batch *B, const double *r, double *z, int head, cudaStre
     st = launch_batch_schwarz<double>(B->d_inst, B->cg, B->T.sub_items, B->T.nsub_items,
                                       B->heads + head, r, B->npad_max, B->w_max, B->cluster,
                                       B->rows, B->staged, clusters, B->status, s);
+  if (B->any_coarse) GENEO_CUDA_TRY(cudaStreamWaitEvent(s, B->join, 0));
   if (st) return st;
   launch_batch_gather(B->d_inst, B->T, B->cg, B->f32, z, s);
   GENEO_CUDA_TRY(cudaGetLastError());
@@ -2303,6 +2325,9 @@ void batch_free(geneo_batch *B) {
   if (B->mem) cudaFree(B->mem);
   if (B->cg_host) cudaFreeHost(B->cg_host);
   if (B->cap) cudaStreamDestroy(B->cap);
+  if (B->side) cudaStreamDestroy(B->side);
+  if (B->fork) cudaEventDestroy(B->fork);
+  if (B->join) cudaEventDestroy(B->join);
   delete B;
 }
 
@@ -2349,6 +2374,11 @@ extern "C" int geneo_batch_create(geneo_batch **out, geneo_ctx *const *ctxs, int
   GENEO_CUDA_TRY(cudaStreamCreateWithFlags(&B->cap, cudaStreamNonBlocking));
   GENEO_CUDA_TRY(cudaEventCreate(&B->ev0));
   GENEO_CUDA_TRY(cudaEventCreate(&B->ev1));
+  int least = 0, greatest = 0;
+  GENEO_CUDA_TRY(cudaDeviceGetStreamPriorityRange(&least, &greatest));
+  GENEO_CUDA_TRY(cudaStreamCreateWithPriority(&B->side, cudaStreamNonBlocking, greatest));
+  GENEO_CUDA_TRY(cudaEventCreateWithFlags(&B->fork, cudaEventDisableTiming));
+  GENEO_CUDA_TRY(cudaEventCreateWithFlags(&B->join, cudaEventDisableTiming));
   for (geneo_ctx *c : B->ctx) GENEO_CUDA_TRY(cudaStreamSynchronize(c->stream));
   // instances and work tables (host)
   std::vector<long long> task_off(n + 1, 0), node_off(n + 1, 0);

@@ -12,7 +12,8 @@ struct geneo_ctx {
   cudaStream_t cap_stream = nullptr;        // private stream used only to capture graphs
   cudaStream_t eig_stream = nullptr;        // GenEO eigensolve and coarse space (highest priority)
   cudaStream_t eig_stream2 = nullptr;       // second group of the Lanczos iterations (same)
-  cudaStream_t side_stream = nullptr;       // its look-ahead factorisation (highest priority)
+  cudaStream_t side_stream = nullptr;       // half of its factorisation; coarse corrections (highest priority)
+  cudaEvent_t coarse_fork = nullptr, coarse_join = nullptr;   // beside the local solves
   cudaStream_t fac_stream = nullptr;        // subdomain factorisation, overlapping the eigensolve
   cudaStream_t fac_side = nullptr;          // its look-ahead stream
   int device = 0;
