@@ -136,54 +136,37 @@ __device__ __forceinline__ double inv_sqrt(double d) {
   return y * (1.5 - 0.5 * d * y * y);
 }
 
-// Diagonal tile J of every system: the last update (K = J - 1; the earlier ones
-// were applied by the previous panel launch), then L D L^T and the inverse of
-// the unit factor together, one elimination step per column.  Four warps, one
-// per SM sub-partition; lane = row, warp w owns columns 4 q + w.  The FP64
-// pipe takes 64 cycles per warp instruction, so a step costs its eight updates
-// (the entries of L right of the pivot and of the inverse left of it); the
-// warp that owns the next column publishes it and its reciprocal pivot before
-// its other updates.  The
-// kernel that stood here before (one entry per thread, three barriers per
-// column, the inverse afterwards) took 44 us a launch.
-__global__ void __launch_bounds__(128)
-    k_dchol_diag(const BandLayout *lay, int sys0, int J, double *poolL, double *poolU, DigitBand D,
-                 DevStatus *st) {
-  const int j = sys0 + blockIdx.x;
-  const BandLayout L = lay[j];
-  if (J >= L.nt) return;
-  __shared__ __align__(16) __half dg[kDigTile];
-  __shared__ double A[32 * 33];
-  __shared__ double colv[32][32];
-  __shared__ double rinv[32];
-  __shared__ int ex[32];
-  __shared__ int bad;
+__device__ __forceinline__ void diag_bar() {
+  __syncwarp();
+  asm volatile("bar.sync 1, 128;" ::: "memory");
+}
+
+// Shared memory of a diagonal tile's factorisation.
+struct DiagSmem {
+  double A[32 * 33];
+  double colv[32][32];
+  double rinv[32];
+  int ex[32], bad;
+  __align__(16) __half dg[kDigTile];
+};
+
+// L D L^T of the diagonal tile J in Sm.A (updates applied) and the inverse of the
+// unit factor together, one elimination step per column; the inverse of the
+// Cholesky factor goes to the pools.  Four warps, one per SM sub-partition;
+// lane = row, warp w owns columns 4 q + w.  The FP64 pipe takes 64 cycles per
+// warp instruction, so a step costs its eight updates (the entries of L right
+// of the pivot and of the inverse left of it); the warp that owns the next
+// column publishes it and its reciprocal pivot before its other updates.  One
+// entry per thread with three barriers per column and the inverse afterwards
+// took 44 us.
+__device__ __forceinline__ void diag_factor(DiagSmem &Sm, const BandLayout &L, int j, int J,
+                                            double *poolL, double *poolU, const DigitBand &D,
+                                            DevStatus *st) {
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
-  double *t = tile_ptr(poolL, L, J, 0);
-  for (int e = tid; e < 1024; e += 128) A[(e & 31) * 33 + (e >> 5)] = t[e];
-  if (tid == 0) bad = -1;
-  const bool upd = J > 0 && L.w > 0;
-  if (upd) {
-    const uint4 *src = reinterpret_cast<const uint4 *>(dig_tile(D, L, j, J, 1));
-    for (int e = tid; e < kDigTile / 8; e += 128) reinterpret_cast<uint4 *>(dg)[e] = src[e];
-    if (tid < 32) ex[tid] = D.rexp[(long long)j * D.npad + J * 32 + tid];
-  }
-  __syncthreads();
-  if (upd) {
-    const int m0 = 16 * (w >> 1), n0 = 16 * (w & 1);
-    if (m0 >= n0) {                         // the lower triangle
-      long long hi[8], lo[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) hi[e] = lo[e] = 0;
-      block_product(hi, lo, dig_smem(dg), dig_smem(dg), m0, n0, lane);
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const int r = m0 + blk_row(e, lane), c = n0 + blk_col(e, lane);
-        A[r * 33 + c] -= parts_value(hi[e], lo[e], ex[r] + ex[c]);
-      }
-    }
-    __syncthreads();
-  }
+  double *t = tile_ptr(poolL, L, J, 0), *A = Sm.A, *rinv = Sm.rinv;
+  double (*colv)[32] = Sm.colv;
+  int *ex = Sm.ex, *bad = &Sm.bad;
+  __half *dg = Sm.dg;
   double a[8], x[8];
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
@@ -195,7 +178,7 @@ __global__ void __launch_bounds__(128)
     if (lane == k) {
       double d = v;
       if (!(d > 0.0)) {
-        if (bad < 0) bad = J * 32 + k;
+        if (*bad < 0) *bad = J * 32 + k;
         d = 1.0;
         colv[k][lane] = d;
       }
@@ -203,7 +186,7 @@ __global__ void __launch_bounds__(128)
     }
   };
   if (w == 0) publish(0, a[0]);
-  __syncthreads();
+  diag_bar();
 #pragma unroll
   for (int k = 0; k < 32; ++k) {
     const int kq = k >> 2, kw = k & 3;
@@ -222,37 +205,58 @@ __global__ void __launch_bounds__(128)
         x[q] = fma(-li, __shfl_sync(0xffffffffu, x[q], k), x[q]);
       }
     }
-    __syncthreads();
+    diag_bar();
   }
   const double rs = inv_sqrt(colv[lane][lane]);
-  __syncthreads();
+  diag_bar();
 #pragma unroll
   for (int q = 0; q < 8; ++q) A[lane * 33 + 4 * q + w] = x[q] * rs;      // inv(L_JJ)
-  __syncthreads();
+  diag_bar();
   for (int e = tid; e < 1024; e += 128) t[e] = A[(e & 31) * 33 + (e >> 5)];
   if (poolU) {
     double *u = tile_ptr(poolU, L, J, 0);
     for (int e = tid; e < 1024; e += 128) u[e] = A[(e >> 5) * 33 + (e & 31)];
   }
   const bool finite = slice_rows<true>(A, 8 * w, 8, ex, dg, lane);
-  if (!finite) bad = J * 32;
-  __syncthreads();
+  if (!finite) *bad = J * 32;
+  diag_bar();
   uint4 *dst = reinterpret_cast<uint4 *>(dig_tile(D, L, j, J, 0));
   for (int e = tid; e < kDigTile / 8; e += 128) dst[e] = reinterpret_cast<const uint4 *>(dg)[e];
   if (tid < 32) D.dexp[(long long)j * D.npad + J * 32 + tid] = ex[tid];
-  if (tid == 0 && bad >= 0) not_spd(st, j, bad);
+  if (tid == 0 && *bad >= 0) not_spd(st, j, *bad);
 }
 
-// Panel of tile column J, left-looking: blockIdx.y = p takes the tiles (I, J),
-// I = J + 2p + 1 and the next, subtracts sum_K L_IK L_JK^double over the band's
+// The first diagonal tile of every system (all of them if no tiles couple); the
+// others are factored by the panel launch before.
+__global__ void __launch_bounds__(128)
+    k_dchol_diag(const BandLayout *lay, int sys0, int J, double *poolL, double *poolU, DigitBand D,
+                 DevStatus *st) {
+  const int j = sys0 + blockIdx.x;
+  const BandLayout L = lay[j];
+  if (J >= L.nt) return;
+  __shared__ DiagSmem Sm;
+  const double *t = tile_ptr(poolL, L, J, 0);
+  for (int e = threadIdx.x; e < 1024; e += 128) Sm.A[(e & 31) * 33 + (e >> 5)] = t[e];
+  if (threadIdx.x == 0) Sm.bad = -1;
+  __syncthreads();
+  diag_factor(Sm, L, j, J, poolL, poolU, D, st);
+}
+
+// Panel of tile column J, left-looking.  blockIdx.y = 2 + p takes the tiles (I, J),
+// I = J + 2p + 2 and the next, subtracts sum_K L_IK L_JK^T over the band's
 // columns K < J, multiplies by inv(L_JJ)^T (digits again) and writes the
-// factor's FP64 tiles and digits.  The last block row instead applies the
-// columns K < J to the diagonal tile J + 1, so that the next diagonal launch
-// has one tile product left.  Eight warps, 16 x 16 entries each; the K tiles
-// come through two shared-memory stages, one copied while the other is used.  Left-looking: the
-// products of all K are summed as integers in registers, and each tile of A
-// is read and written once (the right-looking FP64 update read and wrote the
-// whole trailing triangle for every tile column).
+// factor's FP64 tiles and digits.  The serial part of a column hides behind
+// these: y = 0 finishes tile (J + 1, J), to which only column J - 1 is left to
+// apply, then the diagonal tile J + 1 (columns J - 1 and J) and factors it, while
+// y = 1 applies the columns K < J to the tiles (J + 2, J + 1) and (J + 2, J + 2),
+// for y = 0 of the next launch.  With the diagonal tile in a launch of its own a
+// column took 39 + 49 us on 16 systems of 7,600 unknowns, 53 + 119 us on 36 of
+// 14,500 and 43 + 36 us on 54 Darcy ones (two such sets in flight); now 57, 115
+// and 59 us, of which the serial part is 42.  Eight warps, 16 x 16 entries each; the K tiles
+// come through two shared-memory stages, one copied while the other is used.
+// Left-looking: the products of all K are summed as integers in registers, and
+// each tile of A is read and written once (the right-looking FP64 update read
+// and wrote the whole trailing triangle for every tile column).
 constexpr int kPanStages = 2;
 constexpr int kPanSmem = (3 * kPanStages + 1) * (int)kDigBytes;
 
@@ -261,43 +265,113 @@ __global__ void __launch_bounds__(256, 2)
                   DevStatus *st) {
   const int j = sys0 + blockIdx.x;
   const BandLayout L = lay[j];
-  if (J >= L.nt || L.w == 0) return;
-  const bool ahead = blockIdx.y == gridDim.y - 1;
-  const int I0 = ahead ? J + 1 : J + 2 * blockIdx.y + 1;
-  if (I0 >= L.nt || I0 - J > L.w) return;
+  if (J + 1 >= L.nt) return;
+  const bool ahead = blockIdx.y == 1;
+  const int I0 = ahead ? J + 2 : J + 2 * ((int)blockIdx.y - 1);
+  if (blockIdx.y > 0 && (I0 >= L.nt || (ahead ? 1 : I0 - J) > L.w)) return;
   const bool two = !ahead && I0 + 1 < L.nt && I0 + 1 - J <= L.w;
   extern __shared__ __align__(128) unsigned char smraw[];
   __shared__ int rexp_s[64], rowe[64], cexp_s[32], dexp_s[32];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int tt = warp >> 2, m0 = 16 * ((warp >> 1) & 1), n0 = 16 * (warp & 1);
-  const int K0 = max(0, I0 - L.w), nK = J - K0;
-  // steps: one K each, or two for the look-ahead tile (each half of the warps takes one)
-  const int nstep = ahead ? (nK + 1) / 2 : nK;
+  const int K0 = max(0, I0 - L.w), nstep = max(0, J - K0);
   const uint32_t sm = dig_smem(smraw);
   __half *dinv = reinterpret_cast<__half *>(smraw + 3 * kPanStages * kDigBytes);
   auto tile_in = [&](uint32_t dst, const __half *src) {
     for (int e = tid; e < kDigTile / 8; e += 256) cp16(dst + 16 * e, src + 8 * e);
   };
+  const long long eb = (long long)j * D.npad;
+  if (blockIdx.y == 0) {
+    // ---- tile (J + 1, J) and the diagonal tile J + 1
+    const int I = J + 1;
+    const bool tile = L.w >= 1, last = J >= 1 && L.w >= 2;
+    double *R = reinterpret_cast<double *>(smraw + 2 * kDigBytes);      // [32][33]
+    __half *dg = reinterpret_cast<__half *>(R + 32 * 33);
+    DiagSmem &Sm = *reinterpret_cast<DiagSmem *>(dg + kDigTile);
+    static_assert(2 * kDigBytes + 32 * 33 * 8 + kDigBytes + sizeof(DiagSmem) <= 3 * kPanStages * kDigBytes,
+                  "the inverse of the diagonal tile follows the stages");
+    if (tile) tile_in(dig_smem(dinv), dig_tile(D, L, j, J, 0));
+    if (last) {
+      tile_in(sm, dig_tile(D, L, j, I, 2));
+      tile_in(sm + kDigBytes, dig_tile(D, L, j, J, 1));
+    }
+    cp_commit();
+    if (tid < 32) {
+      rexp_s[tid] = D.rexp[eb + I * 32 + tid];
+      cexp_s[tid] = D.rexp[eb + J * 32 + tid];
+      dexp_s[tid] = D.dexp[eb + J * 32 + tid];
+    }
+    const double *ta = tile_ptr(poolL, L, I, 0);
+    double *tr = tile ? tile_ptr(poolL, L, I, 1) : nullptr;
+    for (int e = tid; e < 1024; e += 256) {
+      Sm.A[(e & 31) * 33 + (e >> 5)] = ta[e];
+      if (tile) R[(e & 31) * 33 + (e >> 5)] = tr[e];
+    }
+    if (tid == 0) Sm.bad = -1;
+    cp_wait<0>();
+    __syncthreads();
+    // warps 0..3 update the tile (J + 1, J), warps 4..7 the lower triangle of the diagonal tile
+    auto update = [&](bool mine, uint32_t a, uint32_t b, double *T, const int *ec) {
+      if (!mine) return;
+      long long hi[8], lo[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) hi[e] = lo[e] = 0;
+      block_product(hi, lo, a, b, m0, n0, lane);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const int r = m0 + blk_row(e, lane), c = n0 + blk_col(e, lane);
+        T[r * 33 + c] -= parts_value(hi[e], lo[e], rexp_s[r] + ec[c]);
+      }
+    };
+    if (last)
+      update(tt == 0 || m0 >= n0, sm, tt == 0 ? sm + kDigBytes : sm, tt == 0 ? R : Sm.A,
+             tt == 0 ? cexp_s : rexp_s);
+    __syncthreads();
+    if (tile) {
+      bool finite = slice_rows<true>(R, 4 * warp, 4, rowe, dg, lane);
+      __syncthreads();
+      if (tt == 0) {
+        long long hi[8], lo[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) hi[e] = lo[e] = 0;
+        block_product(hi, lo, dig_smem(dg), dig_smem(dinv), m0, n0, lane);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          const int r = m0 + blk_row(e, lane), c = n0 + blk_col(e, lane);
+          R[r * 33 + c] = parts_value(hi[e], lo[e], rowe[r] + dexp_s[c]);
+        }
+      }
+      __syncthreads();
+      finite = slice_rows<false>(R, 4 * warp, 4, rexp_s, dg, lane) && finite;
+      if (!finite) not_spd(st, j, J * 32);
+      __syncthreads();
+      update(tt == 1 && m0 >= n0, dig_smem(dg), dig_smem(dg), Sm.A, rexp_s);
+      uint4 *dst = reinterpret_cast<uint4 *>(dig_tile(D, L, j, I, 1));
+      const uint4 *src = reinterpret_cast<const uint4 *>(dg);
+      for (int e = tid; e < kDigTile / 8; e += 256) dst[e] = src[e];
+      double *tu = poolU ? tile_ptr(poolU, L, J, 1) : nullptr;
+      for (int e = tid; e < 1024; e += 256) {
+        tr[e] = R[(e & 31) * 33 + (e >> 5)];
+        if (tu) tu[e] = R[(e >> 5) * 33 + (e & 31)];
+      }
+      __syncthreads();
+    }
+    if (warp < 4) diag_factor(Sm, L, j, I, poolL, poolU, D, st);
+    return;
+  }
   auto prefetch = [&](int it) {
     const uint32_t sp = sm + (it % kPanStages) * 3 * kDigBytes;
-    if (ahead) {
-      const int K = K0 + 2 * it;
-      tile_in(sp, dig_tile(D, L, j, I0, I0 - K));
-      if (K + 1 < J) tile_in(sp + kDigBytes, dig_tile(D, L, j, I0, I0 - K - 1));
-    } else {
-      const int K = K0 + it;
-      tile_in(sp, dig_tile(D, L, j, I0, I0 - K));
-      if (two && I0 + 1 - K <= L.w) tile_in(sp + kDigBytes, dig_tile(D, L, j, I0 + 1, I0 + 1 - K));
-      tile_in(sp + 2 * kDigBytes, dig_tile(D, L, j, J, J - K));
-    }
+    const int K = K0 + it, C = ahead ? J + 1 : J;
+    tile_in(sp, dig_tile(D, L, j, I0, I0 - K));
+    if (two && I0 + 1 - K <= L.w) tile_in(sp + kDigBytes, dig_tile(D, L, j, I0 + 1, I0 + 1 - K));
+    tile_in(sp + 2 * kDigBytes, dig_tile(D, L, j, C, C - K));
   };
   if (!ahead) tile_in(dig_smem(dinv), dig_tile(D, L, j, J, 0));
   if (nstep > 0) prefetch(0);
   cp_commit();
-  const long long eb = (long long)j * D.npad;
   if (tid < 64) rexp_s[tid] = (tid < 32 || two) ? D.rexp[eb + I0 * 32 + tid] : 0;
   if (tid < 32) {
-    cexp_s[tid] = D.rexp[eb + (ahead ? I0 : J) * 32 + tid];
+    cexp_s[tid] = D.rexp[eb + (ahead ? J + 1 : J) * 32 + tid];
     dexp_s[tid] = D.dexp[eb + J * 32 + tid];
   }
   long long hi[8], lo[8];
@@ -309,9 +383,8 @@ __global__ void __launch_bounds__(256, 2)
     cp_wait<1>();
     __syncthreads();                        // the stage has landed
     const uint32_t sp = sm + (it % kPanStages) * 3 * kDigBytes;
-    if (ahead) {
-      if (K0 + 2 * it + tt < J && m0 >= n0)
-        block_product(hi, lo, sp + tt * kDigBytes, sp + tt * kDigBytes, m0, n0, lane);
+    if (ahead) {                            // warps 0..3: (J + 2, J + 1), 4..7: (J + 2, J + 2)
+      if (tt == 0 || m0 >= n0) block_product(hi, lo, sp, tt == 0 ? sp + 2 * kDigBytes : sp, m0, n0, lane);
     } else if (tt == 0 || (two && I0 + 1 - (K0 + it) <= L.w)) {
       block_product(hi, lo, sp + tt * kDigBytes, sp + 2 * kDigBytes, m0, n0, lane);
     }
@@ -320,22 +393,13 @@ __global__ void __launch_bounds__(256, 2)
   cp_wait<0>();
   __syncthreads();
   if (ahead) {
-    // the two halves' sums, then A(J+1, J+1) -= U
-    long long *sh = reinterpret_cast<long long *>(smraw);
-    if (tt == 1)
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        sh[(2 * e) * 128 + (tid & 127)] = hi[e];
-        sh[(2 * e + 1) * 128 + (tid & 127)] = lo[e];
-      }
-    __syncthreads();
-    if (tt == 0 && m0 >= n0) {
-      double *t = tile_ptr(poolL, L, I0, 0);
+    if (nstep > 0 && (tt == 0 || m0 >= n0)) {
+      double *t = tile_ptr(poolL, L, I0, tt == 0 ? 1 : 0);
+      const int *ec = tt == 0 ? cexp_s : rexp_s;
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
         const int r = m0 + blk_row(e, lane), c = n0 + blk_col(e, lane);
-        t[c * 32 + r] -= parts_value(hi[e] + sh[(2 * e) * 128 + tid], lo[e] + sh[(2 * e + 1) * 128 + tid],
-                                     rexp_s[r] + cexp_s[c]);
+        t[c * 32 + r] -= parts_value(hi[e], lo[e], rexp_s[r] + ec[c]);
       }
     }
   } else {
@@ -837,18 +901,18 @@ int launch_band_cholesky64(const BandLayout *d_lay, int nsys, int nt_max, int w_
     GENEO_CUDA_TRY(cudaEventRecord(ev.fork, s));
     GENEO_CUDA_TRY(cudaStreamWaitEvent(side, ev.fork, 0));
   }
-  for (int J = -1; J < nt_max; ++J)
+  for (int J = -1; J + 1 < nt_max; ++J)
     for (int h = 0; h < (half < nsys ? 2 : 1); ++h) {
       const int j0 = h ? half : 0, n = h ? nsys - half : half;
       cudaStream_t q = h ? side : s;
       if (J < 0) {
         k_row_exps<<<dim3((nt_max * 32 + 255) / 256, n), 256, 0, q>>>(d_lay, j0, poolL, D); GENEO_COUNT_LAUNCH();
-        continue;
-      }
-      k_dchol_diag<<<n, 128, 0, q>>>(d_lay, j0, J, poolL, poolU, D, st); GENEO_COUNT_LAUNCH();
-      if (w_max > 0 && J + 1 < nt_max) {
-        const int d = std::min(w_max, nt_max - 1 - J);
-        k_dchol_panel<<<dim3(n, (d + 1) / 2 + 1), 256, kPanSmem, q>>>(d_lay, j0, J, poolL, poolU, D, st); GENEO_COUNT_LAUNCH();
+        k_dchol_diag<<<n, 128, 0, q>>>(d_lay, j0, 0, poolL, poolU, D, st); GENEO_COUNT_LAUNCH();
+      } else if (w_max == 0) {
+        k_dchol_diag<<<n, 128, 0, q>>>(d_lay, j0, J + 1, poolL, poolU, D, st); GENEO_COUNT_LAUNCH();
+      } else {
+        const int d = std::min(w_max, nt_max - 1 - J);      // tiles (J + 2 .. J + d, J) in pairs
+        k_dchol_panel<<<dim3(n, d / 2 + 2), 256, kPanSmem, q>>>(d_lay, j0, J, poolL, poolU, D, st); GENEO_COUNT_LAUNCH();
       }
     }
   if (half < nsys) {
@@ -873,6 +937,8 @@ int launch_band_solve64(const BandLayout *d_lay, int nsys, int w_max, const Digi
   GENEO_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   // A second CTA for the far tiles while every CTA of the launches in flight
   // still has an SM of its own and a full row has a tile for each pair of warps.
+  // All sweeps of one solve with and without: 93 and 135 ms (32 systems, 15 tiles),
+  // 200 and 283 ms (72 systems, 27 tiles).
   const int groups = (ncols + 7) / 8;
   const int cl = 2 * groups * (nsys + alongside) <= sms && w_max - 1 > 4 &&
                          sweep_smem(w_max, 2) <= 227 * 1024 ? 2 : 1;
