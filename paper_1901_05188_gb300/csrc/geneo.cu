@@ -287,65 +287,60 @@ __global__ void k_reorth_gate(const double *G, int p, const double *H, int na, l
   if (threadIdx.x == 0) gate[j] = need;
 }
 
-// Cholesky of the p x p Gram matrix, inverse, and Racc update (one block per subdomain)
+// Cholesky of the p x p Gram matrix, inverse, and Racc update: one warp per
+// subdomain, lane = column.  A chain of square roots and divisions bounds it;
+// one thread for everything took 57 us a launch.
 __global__ void k_cholqr_small(const double *G, int p, double *Rinv, double *Racc, int first,
                                double abs_tiny) {
-  const int j = blockIdx.x;
+  const int j = blockIdx.x, c = threadIdx.x;
   __shared__ double R[kLanczosBlock][kLanczosBlock];
   __shared__ double Ri[kLanczosBlock][kLanczosBlock];
-  __shared__ double Ra[kLanczosBlock][kLanczosBlock];
-  if (threadIdx.x == 0) {
-    const double *g = G + (long long)j * p * p;
-    for (int a = 0; a < p; ++a)
-      for (int b = 0; b < p; ++b) R[a][b] = 0.0;
-    // upper factor R with G = R^T R; dead columns get R[k][k] = 0
-    for (int k = 0; k < p; ++k) {
-      double d = g[k * p + k];
-      for (int i = 0; i < k; ++i) d -= R[i][k] * R[i][k];
-      // numerically dependent (angle to the block's span below 1e-7) or
-      // negligible against the operator scale: deflate the column
-      bool dead = !(d > 1e-14 * g[k * p + k]) || !(d > abs_tiny);
-      double rk = dead ? 0.0 : sqrt(d);
+  const double *g = G + (long long)j * p * p;
+  if (c < p)
+    for (int a = 0; a < p; ++a) R[a][c] = 0.0;
+  __syncwarp();
+  // upper factor R with G = R^T R; dead columns get R[k][k] = 0
+  for (int k = 0; k < p; ++k) {
+    double d = g[k * p + k];
+    for (int i = 0; i < k; ++i) d -= R[i][k] * R[i][k];
+    // numerically dependent (angle to the block's span below 1e-7) or
+    // negligible against the operator scale: deflate the column
+    const bool dead = !(d > 1e-14 * g[k * p + k]) || !(d > abs_tiny);
+    const double rk = dead ? 0.0 : sqrt(d);
+    if (c > k && c < p) {
+      double v = g[k * p + c];
+      for (int i = 0; i < k; ++i) v -= R[i][k] * R[i][c];
+      R[k][c] = dead ? 0.0 : v / rk;
+    } else if (c == k) {
       R[k][k] = rk;
-      for (int c = k + 1; c < p; ++c) {
-        double v = g[k * p + c];
-        for (int i = 0; i < k; ++i) v -= R[i][k] * R[i][c];
-        R[k][c] = dead ? 0.0 : v / rk;
-      }
     }
-    // Rinv (upper); a dead column maps to zero
-    for (int c = 0; c < p; ++c) {
-      for (int a = p - 1; a >= 0; --a) {
-        if (a > c) {
-          Ri[a][c] = 0.0;
-          continue;
-        }
-        if (R[a][a] == 0.0) {
-          Ri[a][c] = 0.0;
-          continue;
-        }
-        double s = (a == c) ? 1.0 : 0.0;
-        for (int k = a + 1; k <= c; ++k) s -= R[a][k] * Ri[k][c];
-        Ri[a][c] = s / R[a][a];
+    __syncwarp();
+  }
+  // Rinv (upper); a dead column maps to zero
+  if (c < p)
+    for (int a = p - 1; a >= 0; --a) {
+      if (a > c || R[a][a] == 0.0) {
+        Ri[a][c] = 0.0;
+        continue;
       }
+      double s = (a == c) ? 1.0 : 0.0;
+      for (int k = a + 1; k <= c; ++k) s -= R[a][k] * Ri[k][c];
+      Ri[a][c] = s / R[a][a];
     }
-    double *racc = Racc + (long long)j * p * p;
-    for (int a = 0; a < p; ++a)
-      for (int b = 0; b < p; ++b) {
-        double s;
-        if (first) {
-          s = R[a][b];
-        } else {
-          s = 0.0;
-          for (int k = 0; k < p; ++k) s += R[a][k] * racc[k * p + b];
-        }
-        Ra[a][b] = s;
+  double *racc = Racc + (long long)j * p * p;
+  if (c < p) {
+    double in[kLanczosBlock];
+    for (int k = 0; k < p; ++k) in[k] = first ? 0.0 : racc[k * p + c];
+    for (int a = 0; a < p; ++a) {
+      double s = 0.0;
+      if (first) {
+        s = R[a][c];
+      } else {
+        for (int k = 0; k < p; ++k) s += R[a][k] * in[k];
       }
-    for (int a = 0; a < p; ++a)
-      for (int b = 0; b < p; ++b) {
-        racc[a * p + b] = Ra[a][b];
-        Rinv[(long long)j * p * p + a * p + b] = Ri[a][b];
-      }
+      racc[a * p + c] = s;
+      Rinv[(long long)j * p * p + a * p + c] = Ri[a][c];
+    }
   }
 }
 
