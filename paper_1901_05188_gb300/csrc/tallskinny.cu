@@ -39,7 +39,8 @@ __device__ __forceinline__ void ts_b(uint32_t (&b)[4], uint32_t tile, int n0, in
 }
 
 // ---- H = A^T B over a chunk of rows ----------------------------------------------
-// One CTA per (chunk, subdomain).  Rows are taken 32 at a time: each thread reads
+// One CTA per (chunk, subdomain, `width` columns of B: as many as leave at most
+// sixteen blocks and halves).  Rows are taken 32 at a time: each thread reads
 // its entries (lane = column), the running largest exponent of every column is
 // kept, and the digits go to shared memory at a scale that may be up to two bits
 // too large; only when a column outgrows its scale are the sums so far turned
@@ -53,8 +54,8 @@ __host__ __device__ constexpr int tsdots_smem() {
 template <int NCG, int WARPS>
 __global__ void __launch_bounds__(32 * WARPS, 16 / WARPS)
     k_tsdots(const SubDesc *subs, const double *__restrict__ A, int lda, long long sa, int na,
-             const double *__restrict__ B, int ldb, long long sb, int nb, double *Hpart, int chunks,
-             const int *gate) {
+             const double *__restrict__ B, int ldb, long long sb, int nball, int width, double *Hpart,
+             int chunks, const int *gate) {
   const int j = blockIdx.y, ch = blockIdx.x;
   if (gate && !gate[j]) return;                       // the reduction writes zeros
   const int n = subs[j].n_neu;
@@ -68,8 +69,9 @@ __global__ void __launch_bounds__(32 * WARPS, 16 / WARPS)
   int *mx = reinterpret_cast<int *>(sum + 2 * 1024);  // largest exponents: A's, then B's columns
   int *G = mx + 32 * NCG + 32;                        // their scales
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int b0 = blockIdx.z * width, nb = min(width, nball - b0);     // this CTA's columns of B
   const int mt = (na + 15) / 16, jobs = 2 * mt * ((nb + 7) / 8);
-  const double *Aj = A + j * sa, *Bj = B + j * sb;
+  const double *Aj = A + j * sa, *Bj = B + j * sb + b0;
   for (int e = tid; e < 32 * NCG + 32; e += T) mx[e] = G[e] = kNoExp;
   for (int e = tid; e < 2 * 1024; e += T) sum[e] = 0.0;
   double x[NCG + 1][R];                               // rows R warp .. + R - 1
@@ -165,11 +167,11 @@ __global__ void __launch_bounds__(32 * WARPS, 16 / WARPS)
   }
   if (cnt > 0) flush();
   __syncthreads();
-  double *out = Hpart + ((long long)j * chunks + ch) * na * nb;
+  double *out = Hpart + ((long long)j * chunks + ch) * na * nball + b0;
   for (int o = tid; o < na * nb; o += T) {
     const int a = o / nb, b = o - a * nb, e = ((b >> 3) * mt + (a >> 4)) * 128 + (a & 15) * 8 + (b & 7);
     const bool finite = mx[a] < 1025 && mx[32 * NCG + b] < 1025;
-    out[o] = finite ? sum[e] + sum[1024 + e] : __longlong_as_double(0x7ff8000000000000LL);
+    out[a * nball + b] = finite ? sum[e] + sum[1024 + e] : __longlong_as_double(0x7ff8000000000000LL);
   }
 }
 
@@ -412,9 +414,13 @@ void launch_tsdots(const SubDesc *d_subs, int nsub, int npad, const double *A, i
                    double *Hpart, int chunks, double *H, long long hs, cudaStream_t s,
                    const int *gate) {
   (void)npad;
+  // One warp for each half of a 16 x 8 block of H, sixteen at most: all 32
+  // columns a CTA can stage for up to 32 of A, 16 for up to 64, else eight.
+  const int width = na <= 32 ? 32 : na <= 64 ? 16 : 8, groups = (nb + width - 1) / width;
+  const bool small = 2 * ((na + 15) / 16) * ((std::min(nb, width) + 7) / 8) <= 8;
   auto run = [&](auto k, int warps, int sm) {
     (void)ensure_smem(k, sm);                // a failure surfaces as a launch error
-    k<<<dim3(chunks, nsub), 32 * warps, sm, s>>>(d_subs, A, lda, sa, na, B, ldb, sb, nb, Hpart, chunks, gate); GENEO_COUNT_LAUNCH();
+    k<<<dim3(chunks, nsub, groups), 32 * warps, sm, s>>>(d_subs, A, lda, sa, na, B, ldb, sb, nb, width, Hpart, chunks, gate); GENEO_COUNT_LAUNCH();
   };
   if (A == B && lda == ldb && sa == sb && na == nb && na <= 8) {
     (void)ensure_smem(k_tsgram, kTgSmem);
@@ -422,8 +428,6 @@ void launch_tsdots(const SubDesc *d_subs, int nsub, int npad, const double *A, i
     k_tsdots_reduce<<<nsub, 256, 0, s>>>(Hpart, chunks, na * nb, H, hs, gate); GENEO_COUNT_LAUNCH();
     return;
   }
-  // one warp for each half of a 16 x 8 block: eight, or sixteen (up to 128 columns with 8, 32 with 32)
-  const bool small = 2 * ((na + 15) / 16) * ((nb + 7) / 8) <= 8;
   if (na <= 32) small ? run(k_tsdots<1, 8>, 8, tsdots_smem<1>()) : run(k_tsdots<1, 16>, 16, tsdots_smem<1>());
   else if (na <= 64) small ? run(k_tsdots<2, 8>, 8, tsdots_smem<2>()) : run(k_tsdots<2, 16>, 16, tsdots_smem<2>());
   else if (na <= 96) run(k_tsdots<3, 16>, 16, tsdots_smem<3>());
