@@ -8,7 +8,8 @@
 // so the wanted smallest lambda are the largest mu.  Instead of ARPACK's
 // implicitly restarted Lanczos, a block Lanczos process (block size 8, full
 // re-orthogonalisation, Cholesky-QR) runs batched over all subdomains and the
-// projected matrix is diagonalised by a cyclic Jacobi method; p = L^-T y.
+// projected matrix is diagonalised by tridiagonalisation, bisection and inverse
+// iteration; p = L^-T y.
 #include "geneo.cuh"
 #include "fem.cuh"
 
@@ -288,8 +289,8 @@ __global__ void k_reorth_gate(const double *G, int p, const double *H, int na, l
 }
 
 // Cholesky of the p x p Gram matrix, inverse, and Racc update: one warp per
-// subdomain, lane = column.  A chain of square roots and divisions bounds it;
-// one thread for everything took 57 us a launch.
+// subdomain, lane = column.  A chain of square roots and divisions bounds it:
+// 25 us a launch, with one thread for everything 57 us.
 __global__ void k_cholqr_small(const double *G, int p, double *Rinv, double *Racc, int first,
                                double abs_tiny) {
   const int j = blockIdx.x, c = threadIdx.x;
@@ -411,25 +412,40 @@ __global__ void k_copy_block(const SubDesc *subs, int npad, const double *W, int
 
 // Ritz pairs of the symmetrised projected matrix H (n x n, n <= kMaxKdim):
 // Householder reduction to tridiagonal form (H = Q T Q^T), the nw largest
-// eigenvalues of T by Sturm-sequence bisection, their eigenvectors by inverse
+// eigenvalues of T by Sturm-sequence multisection, their eigenvectors by inverse
 // iteration (re-orthogonalised inside clusters of close eigenvalues), and the
 // back-transformation y = Q x.  One block per subdomain; eigenvalues are
 // returned in descending order, columns nw..n-1 of Evec are zero.
 constexpr int kMaxKdim = 128;
 
-__device__ __forceinline__ int sturm_count(const double *d, const double *e2, int n, double x,
-                                           double pivmin) {
-  // number of eigenvalues of T smaller than x
+// Number of eigenvalues of T smaller than x: sign changes of the leading
+// principal minors of T - x, p_i = (d_i - x) p_{i-1} - e_{i-1}^2 p_{i-2}: three
+// instructions of the FP64 pipe a step (64 cycles each) where the quotients
+// p_i / p_{i-1} take a division and comparisons, about fourteen; signs and
+// sizes are read from the bits.  T is scaled to norm <= 1, so |p| grows at most
+// threefold a step (n <= 128: below 2^203); pairs below 2^-303 are scaled up.
+__device__ __forceinline__ int sturm_count(const double *d, const double *e2, int n, double x) {
   int cnt = 0;
-  double q = d[0] - x;
-  if (fabs(q) < pivmin) q = -pivmin;
-  if (q < 0) ++cnt;
-  for (int i = 1; i < n; ++i) {
-    q = d[i] - x - e2[i - 1] / q;
-    if (fabs(q) < pivmin) q = -pivmin;
-    if (q < 0) ++cnt;
+  double p0 = 1.0, p1 = d[0] - x;
+  int h0 = __double2hiint(p0), h1 = __double2hiint(p1);
+  for (int i = 0;; ++i) {
+    if (((h1 & 0x7fffffff) | __double2loint(p1)) == 0) {     // as a small negative quotient
+      p1 = p0 * -1e-30;
+      h1 = __double2hiint(p1);
+    }
+    cnt += (unsigned)(h0 ^ h1) >> 31;
+    if (i + 1 == n) return cnt;
+    if (max(h0 & 0x7fffffff, h1 & 0x7fffffff) < 0x2d000000) {
+      const double up = __hiloint2double(0x52b00000, 0);     // 2^300
+      p0 *= up;
+      p1 *= up;
+    }
+    const double p2 = fma(d[i + 1] - x, p1, -(e2[i] * p0));
+    p0 = p1;
+    p1 = p2;
+    h0 = __double2hiint(p0);
+    h1 = __double2hiint(p1);
   }
-  return cnt;
 }
 
 __global__ void __launch_bounds__(256)
@@ -541,21 +557,39 @@ __global__ void __launch_bounds__(256)
     red[0] = mx;
   }
   __syncthreads();
-  for (int i = tid; i < n; i += blockDim.x) e2[i] = e[i] * e[i];
-  __syncthreads();
   const double tnorm = red[0];
-  const double pivmin = fmax(1e-290, 1e-30 * tnorm * tnorm) / fmax(tnorm, 1e-300);
-  // ---- bisection: thread q finds the q-th largest eigenvalue
-  for (int q = tid; q < nw; q += blockDim.x) {
+  // T times a power of two, norm at most one: vs = diagonal, e2 = squares
+  const int tex = tnorm > 0.0 ? ilogb(tnorm) + 1 : 0;
+  const double down = ldexp(1.0, -tex);
+  for (int i = tid; i < n; i += blockDim.x) {
+    vs[i] = d[i] * down;
+    e2[i] = (e[i] * down) * (e[i] * down);
+  }
+  __syncthreads();
+  // ---- multisection on four warps, one per SM sub-partition: G lanes cut the
+  // interval of an eigenvalue into G + 1, as many lanes as nw leaves (80 columns,
+  // 40 wanted: G = 3, 27 evaluations; the kernel takes 2.06 ms, bisection by one
+  // thread with the quotients took 2.3 of its 3.65 ms)
+  if (warp < 4) {
+    const int G = nw <= 16 ? 8 : nw <= 20 ? 6 : nw <= 24 ? 5 : nw <= 32 ? 4 : nw <= 40 ? 3 : nw <= 64 ? 2 : 1;
+    const int per = 32 / G, grp = lane / G, sub = lane - grp * G, q = warp * per + grp;
     const int target = n - 1 - q;          // index from the bottom
-    double a = bounds[0], bnd = bounds[1];
+    double a = bounds[0] * down, bnd = bounds[1] * down;
+    const double cut = 1.0 / (G + 1);
+    bool open = grp < per && q < nw;
     for (int it = 0; it < 200; ++it) {
-      double mid = 0.5 * (a + bnd);
-      if (sturm_count(d, e2, n, mid, pivmin) > target) bnd = mid;
-      else a = mid;
-      if (bnd - a <= 2.2e-16 * (fabs(a) + fabs(bnd)) + 1e-300) break;
+      open = open && bnd - a > 2.2e-16 * (fabs(a) + fabs(bnd)) + 1e-300;
+      if (!__any_sync(0xffffffffu, open)) break;
+      const double h = (bnd - a) * cut;
+      const bool above = open && sturm_count(vs, e2, n, fma(h, (double)(sub + 1), a)) > target;
+      const unsigned m = (__ballot_sync(0xffffffffu, above) >> (grp * G)) & ((1u << G) - 1u);
+      if (!open) continue;
+      const int f = m ? __ffs(m) : G + 1;  // the first point above
+      const double lo = f > 1 ? fma(h, (double)(f - 1), a) : a;
+      if (f <= G) bnd = fma(h, (double)f, a);
+      a = lo;
     }
-    lam[q] = 0.5 * (a + bnd);
+    if (grp < per && q < nw && sub == 0) lam[q] = ldexp(0.5 * (a + bnd), tex);
   }
   __syncthreads();
   // ---- inverse iteration on T - lam I (partial pivoting), vectors to Evec columns
