@@ -355,6 +355,18 @@ int geneo_get_coarse(geneo_ctx *ctx, double *Phi, double *AH);
  * coarse space.  Allocates scratch with cudaMallocAsync. */
 int geneo_debug_local_matrix(geneo_ctx *ctx, int sub, int kind, double *dense, int32_t *gdof);
 
+/* Inspection of the set-up's FP64 band factorisation and band solves (Sec. 3.1,
+ * Sec. 3.3.2) on a matrix of the caller's: a is n x n row-major, symmetric, with
+ * a_ij = 0 for |i - j| > half_band (its lower triangle is read).  factor (n x n,
+ * may be NULL) receives the factor as in kind 3 of geneo_debug_local_matrix.
+ * With ncols > 0, x (n x ncols, row-major) receives the solutions for the
+ * right-hand sides b: mode 1 L x = b, 2 L^T x = b, 3 both; ctas 1 or 2 CTAs per
+ * eight columns, 0 as in the set-up (2 is refused where it does not fit).
+ * Returns GENEO_ERR_NOT_SPD if the matrix has no Cholesky factor.  Needs no
+ * set-up; allocates scratch with cudaMallocAsync. */
+int geneo_debug_band(geneo_ctx *ctx, int n, int half_band, const double *a, double *factor,
+                     int ncols, int mode, int ctas, const double *b, double *x);
+
 /* Time `reps` back-to-back launches of one hot kernel on the context stream
  * with CUDA events (after one warm-up launch) and report its algorithmic
  * traffic: what 0 = the one-level Schwarz local solves (Sec. 3.1,

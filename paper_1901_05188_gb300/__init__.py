@@ -115,6 +115,7 @@ _SIGS = {
     "geneo_get_coarse": [_P, _P, _P],
     "geneo_solve": [_P, C.c_double, C.c_int, _P, C.POINTER(geneo_stats)],
     "geneo_debug_local_matrix": [_P, C.c_int, C.c_int, _P, _P],
+    "geneo_debug_band": [_P, C.c_int, C.c_int, _P, _P, C.c_int, C.c_int, C.c_int, _P, _P],
     "geneo_spmv_dot_noalloc": [C.c_int, _P, _P, _P, _P, _P, _P, _P],
     "geneo_set_partition_of_unity": [_P, C.c_int],
     "geneo_set_coarse_solver": [_P, C.c_int, C.c_double, C.c_int],
@@ -321,6 +322,13 @@ def geneo_get_coarse(ctx, Phi=None, AH=None):
 
 def geneo_debug_local_matrix(ctx, sub, kind, dense=None, gdof=None):
     _check(load().geneo_debug_local_matrix(ctx, sub, kind, _ptr(dense), _ptr(gdof)))
+
+
+def geneo_debug_band(ctx, a, half_band, factor=None, b=None, x=None, mode=3, ctas=0):
+    """FP64 band factor of the symmetric n x n array a, and solves with the columns of b."""
+    _check(load().geneo_debug_band(ctx, a.shape[0], int(half_band), _ptr(a), _ptr(factor),
+                                   0 if b is None else b.shape[1], int(mode), int(ctas),
+                                   _ptr(b), _ptr(x)))
 
 
 def geneo_set_partition_of_unity(ctx, kind):

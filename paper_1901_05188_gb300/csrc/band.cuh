@@ -34,12 +34,13 @@ int launch_band_cholesky64(const BandLayout *d_lay, int nsys, int nt_max, int w_
 // written).  In-place use (in == out with equal strides) is allowed.
 // mode: 1 forward (L), 2 backward (L^T), 3 both.  w_max: the largest tile
 // half-bandwidth; scratch: band_solve_scratch(nsys, w_max, ncols) bytes;
-// alongside: systems of a launch that runs at the same time on another stream.
+// alongside: systems of a launch that runs at the same time on another stream;
+// ctas: CTAs per system and eight columns, 1 or 2, or 0 for the rule's choice.
 size_t band_solve_scratch(int nsys, int w_max, int ncols);
 int launch_band_solve64(const BandLayout *d_lay, int nsys, int w_max, const DigitBand &D,
                         void *scratch, const double *in, long long in_sys, int in_row, double *out,
                         long long out_sys, int out_row, int ncols, int mode, DevStatus *st,
-                        cudaStream_t s, int alongside = 0);
+                        cudaStream_t s, int alongside = 0, int ctas = 0);
 // Widest half-bandwidth (in tiles) the set-up accepts for the eigensolver.
 bool band_solve_fits(int w_max);
 

@@ -474,8 +474,9 @@ __global__ void __launch_bounds__(256, 2)
 // output becomes FP64, after the row's barrier.
 // In a cluster the chain runs on the first CTA.  The second one only adds far
 // warps: its other warps sum the CTA's partials of a row into the first CTA's
-// buffer (integers: the result does not depend on the cluster), and one
-// cluster barrier ends the row.
+// buffer (integers: the result depends on the cluster only through the bits
+// dropped when sums of different scales are aligned, below 2^-57 of the
+// largest), and one cluster barrier ends the row.
 // Bound: the larger of the chain (six barriers and two products, about 3 us a
 // row) and a CTA's share of the tiles, where issuing the copies counts for as
 // much as the matrix instructions.  Per launch of half the subdomains (forward
@@ -930,8 +931,8 @@ size_t band_solve_scratch(int nsys, int w_max, int ncols) {
 int launch_band_solve64(const BandLayout *d_lay, int nsys, int w_max, const DigitBand &D,
                         void *scratch, const double *in, long long in_sys, int in_row, double *out,
                         long long out_sys, int out_row, int ncols, int mode, DevStatus *st,
-                        cudaStream_t s, int alongside) {
-  if (D.window) return GENEO_ERR_INVALID_ARG;
+                        cudaStream_t s, int alongside, int ctas) {
+  if (D.window || ctas < 0 || ctas > 2) return GENEO_ERR_INVALID_ARG;
   int dev = 0, sms = 0;
   GENEO_CUDA_TRY(cudaGetDevice(&dev));
   GENEO_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -940,7 +941,8 @@ int launch_band_solve64(const BandLayout *d_lay, int nsys, int w_max, const Digi
   // All sweeps of one solve with and without: 93 and 135 ms (32 systems, 15 tiles),
   // 200 and 283 ms (72 systems, 27 tiles).
   const int groups = (ncols + 7) / 8;
-  const int cl = 2 * groups * (nsys + alongside) <= sms && w_max - 1 > 4 &&
+  const int cl = ctas ? ctas
+                 : 2 * groups * (nsys + alongside) <= sms && w_max - 1 > 4 &&
                          sweep_smem(w_max, 2) <= 227 * 1024 ? 2 : 1;
   const int sm = sweep_smem(w_max, cl);
   if (sm > 227 * 1024) return GENEO_ERR_INVALID_ARG;

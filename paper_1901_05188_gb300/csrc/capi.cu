@@ -2096,6 +2096,73 @@ extern "C" int geneo_debug_local_matrix(geneo_ctx *c, int sub, int kind, double 
   return GENEO_OK;
 }
 
+extern "C" int geneo_debug_band(geneo_ctx *c, int n, int half_band, const double *a, double *factor,
+                                int ncols, int mode, int ctas, const double *b, double *x) try {
+  if (!c) return fail(GENEO_ERR_INVALID_ARG, "null context");
+  if (n < 1 || half_band < 0 || !a || ncols < 0 || mode < 1 || mode > 3 || ctas < 0 || ctas > 2 ||
+      (ncols > 0 && (!b || !x)))
+    return fail(GENEO_ERR_INVALID_ARG, "bad matrix, mode or right-hand sides");
+  half_band = std::min(half_band, n - 1);
+  cudaStream_t s = c->stream;
+  const BandLayout L = make_layout(n, half_band, 0);
+  const size_t el = layout_elems(L), nn = (size_t)n * n, nb = (size_t)n * ncols;
+  std::vector<double> dense(nn), tiles(el, 0.0);
+  GENEO_CUDA_TRY(copy_sync(c, dense.data(), a, nn * sizeof(double), cudaMemcpyDefault));
+  auto tile = [&](int R, int C) -> double & {
+    const int I = R >> 5, d = I - (C >> 5);
+    return tiles[((size_t)I * (L.w + 1) + d) * 1024 + (C & 31) * 32 + (R & 31)];
+  };
+  for (int R = 0; R < n; ++R)
+    for (int C = std::max(0, R - half_band); C <= R; ++C) tile(R, C) = dense[(size_t)R * n + C];
+  for (int R = n; R < L.nt * 32; ++R) tile(R, R) = 1.0;
+  struct Scratch {                         // freed on every way out
+    cudaStream_t s;
+    void *p[7] = {};
+    ~Scratch() {
+      for (void *q : p)
+        if (q) cudaFreeAsync(q, s);
+    }
+  } m{s};
+  const size_t exps = 2 * (size_t)L.nt * 32 * sizeof(int);
+  const size_t want[7] = {el * sizeof(double), sizeof(BandLayout), sizeof(DevStatus), exps,
+                          el / 1024 * kDigHalves * 2, nb * sizeof(double),
+                          ncols > 0 ? band_solve_scratch(1, L.w, ncols) : 0};
+  for (int i = 0; i < 7; ++i)
+    if (want[i]) GENEO_CUDA_TRY(cudaMallocAsync(&m.p[i], want[i], s));
+  double *pool = (double *)m.p[0], *rhs = (double *)m.p[5];
+  BandLayout *dl = (BandLayout *)m.p[1];
+  DevStatus *status = (DevStatus *)m.p[2], h{};
+  DigitBand D;
+  D.pool = m.p[4];
+  D.rexp = (int *)m.p[3];
+  D.dexp = D.rexp + L.nt * 32;
+  D.npad = L.nt * 32;
+  GENEO_CUDA_TRY(cudaMemcpyAsync(pool, tiles.data(), el * sizeof(double), cudaMemcpyHostToDevice, s));
+  GENEO_CUDA_TRY(cudaMemcpyAsync(dl, &L, sizeof(L), cudaMemcpyHostToDevice, s));
+  GENEO_CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(DevStatus), s));
+  if (int st = launch_band_cholesky64(dl, 1, L.nt, L.w, pool, nullptr, D, status, s)) return st;
+  if (ncols > 0) {
+    GENEO_CUDA_TRY(cudaMemcpyAsync(rhs, b, nb * sizeof(double), cudaMemcpyDefault, s));
+    if (int st = launch_band_solve64(dl, 1, L.w, D, m.p[6], rhs, 0, ncols, rhs, 0, ncols, ncols, mode,
+                                     status, s, 0, ctas))
+      return st;
+  }
+  GENEO_CUDA_TRY(copy_sync(c, &h, status, sizeof(h), cudaMemcpyDeviceToHost));
+  if (h.code) return fail(h.code, ("no positive pivot in row " + std::to_string(h.detail)).c_str());
+  if (ncols > 0) GENEO_CUDA_TRY(copy_sync(c, x, rhs, nb * sizeof(double), cudaMemcpyDefault));
+  if (factor) {
+    GENEO_CUDA_TRY(copy_sync(c, tiles.data(), pool, el * sizeof(double), cudaMemcpyDeviceToHost));
+    std::fill(dense.begin(), dense.end(), 0.0);
+    for (int R = 0; R < n; ++R)
+      for (int C = std::max(0, (R >> 5) - L.w) * 32; C < std::min(n, ((R >> 5) + 1) * 32); ++C)
+        dense[(size_t)R * n + C] = tile(R, C);
+    GENEO_CUDA_TRY(copy_sync(c, factor, dense.data(), nn * sizeof(double), cudaMemcpyDefault));
+  }
+  return GENEO_OK;
+} catch (const std::exception &) {
+  return fail(GENEO_ERR_INVALID_ARG, "out of host memory");
+}
+
 // ============================================================================
 // Kernel timing for the benchmark: `reps` back-to-back launches of one hot
 // kernel on the context stream between CUDA events, with its algorithmic
