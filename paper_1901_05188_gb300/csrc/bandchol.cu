@@ -88,11 +88,15 @@ __device__ __forceinline__ int blk_row(int e, int lane) { return (lane >> 2) + 8
 __device__ __forceinline__ int blk_col(int e, int lane) { return 2 * (lane & 3) + (e & 1) + 8 * (e >> 2); }
 
 // Digits of a row-major 32 x 32 block in shared memory (row stride 33), rows
-// [r0, r0 + n): one warp, lane = column; scale 2^G per row, its own maximum
-// (G written to rowexp) or the given one.
+// [r0, r0 + n), with this lane's column taken times 2^cs: one warp, lane =
+// column; scale 2^G per row, its own maximum (G written to rowexp) or the given
+// one.  A row has one scale, so its entries have to be of one natural size:
+// column k of R = L_IJ L_JJ^T is taken divided by the row scale of L at k, about
+// sqrt(a_kk), and column k of inv(L_JJ) times it.  Without, a coefficient that
+// jumps by 1e12 inside a tile cost the factor 2e-13 of sqrt(a_ii a_jj).
 template <bool kOwn>
-__device__ __forceinline__ bool slice_rows(const double *v, int r0, int n, int *rowexp, __half *dst,
-                                           int lane) {
+__device__ __forceinline__ bool slice_rows(const double *v, int r0, int n, int cs, int *rowexp,
+                                           __half *dst, int lane) {
   bool finite = true;
   for (int r = r0; r < r0 + n; ++r) {
     const double x = v[r * 33 + lane];
@@ -100,12 +104,12 @@ __device__ __forceinline__ bool slice_rows(const double *v, int r0, int n, int *
     finite = finite && ex < 1025;
     int G;
     if (kOwn) {
-      G = __reduce_max_sync(0xffffffffu, ex);
+      G = __reduce_max_sync(0xffffffffu, ex == kNoExp ? ex : ex + cs);
       if (lane == 0) rowexp[r] = G;
     } else {
       G = rowexp[r];
     }
-    const long long xb = fixed62(x, G) + kDigBias;
+    const long long xb = fixed62(x, G - cs) + kDigBias;
     __half *o = dst + dig_index(r, lane);
 #pragma unroll
     for (int s = 0; s < kDig; ++s) o[s * 1024] = digit_half(xb, s);
@@ -168,6 +172,7 @@ __device__ __forceinline__ void diag_factor(DiagSmem &Sm, const BandLayout &L, i
   int *ex = Sm.ex, *bad = &Sm.bad;
   __half *dg = Sm.dg;
   double a[8], x[8];
+  const int cs = D.rexp[(long long)j * D.npad + J * 32 + lane];
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
     a[q] = A[lane * 33 + 4 * q + w];
@@ -217,7 +222,7 @@ __device__ __forceinline__ void diag_factor(DiagSmem &Sm, const BandLayout &L, i
     double *u = tile_ptr(poolU, L, J, 0);
     for (int e = tid; e < 1024; e += 128) u[e] = A[(e >> 5) * 33 + (e & 31)];
   }
-  const bool finite = slice_rows<true>(A, 8 * w, 8, ex, dg, lane);
+  const bool finite = slice_rows<true>(A, 8 * w, 8, cs, ex, dg, lane);
   if (!finite) *bad = J * 32;
   diag_bar();
   uint4 *dst = reinterpret_cast<uint4 *>(dig_tile(D, L, j, J, 0));
@@ -328,7 +333,7 @@ __global__ void __launch_bounds__(256, 2)
              tt == 0 ? cexp_s : rexp_s);
     __syncthreads();
     if (tile) {
-      bool finite = slice_rows<true>(R, 4 * warp, 4, rowe, dg, lane);
+      bool finite = slice_rows<true>(R, 4 * warp, 4, -cexp_s[lane], rowe, dg, lane);
       __syncthreads();
       if (tt == 0) {
         long long hi[8], lo[8];
@@ -342,7 +347,7 @@ __global__ void __launch_bounds__(256, 2)
         }
       }
       __syncthreads();
-      finite = slice_rows<false>(R, 4 * warp, 4, rexp_s, dg, lane) && finite;
+      finite = slice_rows<false>(R, 4 * warp, 4, 0, rexp_s, dg, lane) && finite;
       if (!finite) not_spd(st, j, J * 32);
       __syncthreads();
       update(tt == 1 && m0 >= n0, dig_smem(dg), dig_smem(dg), Sm.A, rexp_s);
@@ -418,7 +423,8 @@ __global__ void __launch_bounds__(256, 2)
     }
     __syncthreads();
     bool finite = true;
-    if (mine) finite = slice_rows<true>(Rt, 8 * (warp & 3), 8, rowe + 32 * tt, dg + tt * kDigTile, lane);
+    if (mine)
+      finite = slice_rows<true>(Rt, 8 * (warp & 3), 8, -cexp_s[lane], rowe + 32 * tt, dg + tt * kDigTile, lane);
     __syncthreads();
     if (mine) {
 #pragma unroll
@@ -439,7 +445,7 @@ __global__ void __launch_bounds__(256, 2)
         double *tu = tile_ptr(poolU, L, J, I - J);
         for (int e = t4; e < 1024; e += 128) tu[e] = Rt[(e >> 5) * 33 + (e & 31)];
       }
-      finite = slice_rows<false>(Rt, 8 * (warp & 3), 8, rexp_s + 32 * tt, dg + tt * kDigTile, lane) && finite;
+      finite = slice_rows<false>(Rt, 8 * (warp & 3), 8, 0, rexp_s + 32 * tt, dg + tt * kDigTile, lane) && finite;
       if (!finite) not_spd(st, j, J * 32);
     }
     __syncthreads();
@@ -796,7 +802,9 @@ __global__ void __launch_bounds__(kSwThreads, 1) k_band_sweep(const SweepArgs P)
         b1 = n1;
         eR = nR;
         eD = nD;
-        const int sR = back ? 0 : eR, sD = back ? 0 : eD, fR = back ? eR : 0, fD = back ? eD : 0;
+        // powers of two: of the sums with L's rows and with inv(L_II), into the solved
+        // row and into s (the digits of inv(L_II) carry the row scales of L in its columns)
+        const int sR = back ? 0 : eR, sD = back ? -eR : eD, fR = back ? eR : 0, fD = back ? eD : -eR;
         if (mult) {
           if (has1) product(near_t);
         } else {
@@ -838,7 +846,7 @@ __global__ void __launch_bounds__(kSwThreads, 1) k_band_sweep(const SweepArgs P)
           if (has1)
             add_shifted(-(nearp[o] + nearp[2 * kSwPart + o]), -(nearp[kSwPart + o] + nearp[3 * kSwPart + o]),
                         fs - en, hs, ls);
-          // digits of s (backward: the rows of inv(L_II) carry their scales, folded into s)
+          // digits of s, its entries of one natural size
           Fixed s = fixed_of(hs, ls, fs);
           s.ex += fD;
           G = __reduce_max_sync(0xffffffffu, s.ex);

@@ -1,4 +1,6 @@
-// FP64 products on the tensor cores, by exact digits.
+// FP64 products on the tensor cores, by exact digits (an error-free splitting
+// in the manner of Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 2012,
+// with fixed instead of floating point slices).
 //
 // On this GPU the FP64 pipe issues two multiply-adds per clock and SM, 1/64 of
 // the FP32 rate, so FP64 matrix products (the GenEO band factorisations and
@@ -18,7 +20,12 @@
 // entry, |L_ik| <= sqrt(a_ii), so that is its scale, known before the
 // factorisation: the error of a product is relative to sqrt(a_ii a_jj), as in
 // the backward error bound of Cholesky itself, and smaller than FP64's by the
-// guard bits.  Results are independent of the order of summation.
+// guard bits.  Operands without such a bound of their own (a tile before its
+// triangular solve, the inverse of a diagonal tile, right-hand sides) are
+// scaled by those powers of two first, so that what shares a scale is of one
+// natural size: multiplying the matrix by powers of four from row to row (and
+// column to column) changes no digit.  Results are independent of the order of
+// summation.
 #pragma once
 
 #include <cuda_fp16.h>

@@ -54,3 +54,51 @@ def test_solves_match_dense_with_one_and_two_ctas(ctx, n, hb, ncols):
         one = _solve(ctx, A, hb, b, mode, 1)
         assert np.linalg.norm(one - ref) <= 24 * n * U * np.linalg.norm(ref), mode
         assert np.max(np.abs(one - _solve(ctx, A, hb, b, mode, 2))) <= 8 * U * np.abs(one).max(), mode
+
+
+def _lower(F):
+    """L from the tile storage: the 32 x 32 diagonal blocks hold the inverses."""
+    L = np.tril(F).astype(np.longdouble)
+    for r in range(0, F.shape[0], 32):
+        D = np.tril(F[r:r + 32, r:r + 32]).astype(np.longdouble)
+        X = np.zeros_like(D)
+        for i in range(D.shape[0]):
+            X[i, i] = 1 / D[i, i]
+            X[i, :i] = -(D[i, :i] @ X[:i, :i]) * X[i, i]
+        L[r:r + 32, r:r + 32] = X
+    return L
+
+
+@pytest.mark.parametrize("bits", [0, 6, 17, 24])
+@pytest.mark.parametrize("n,hb", [(31, 3), (200, 40), (270, 100), (270, 270)])
+def test_coefficients_that_vary_within_a_tile(ctx, n, hb, bits):
+    """A = S M S with S_ii in {1, 2^bits} at random: a contrast of up to 3e14 from row to row.
+
+    Cholesky is invariant under such a scaling, so the errors are M's.  Backward
+    error relative to sqrt(a_ii a_jj): two subtractions and the rounding of L leave
+    at most 8 u outside the diagonal blocks (of which L is taken as the exact inverse of what is
+    stored); inside, 32 eliminations and the inverse 150 u.  L, and
+    the solutions scaled back, equal those of M but for the pivots' reciprocals
+    (a few u, carried by the condition number 3): 100 u of the largest in the row or column.
+    """
+    import paper_1901_05188_gb300 as pkg
+    M = _matrix(n, hb)
+    S = np.where(np.random.default_rng(bits).integers(0, 2, n) == 1, 2.0 ** bits, 1.0)
+    A = S[:, None] * M * S[None, :]
+    F0, F = np.zeros((n, n)), np.zeros((n, n))
+    pkg.geneo_debug_band(ctx, M, hb, F0)
+    pkg.geneo_debug_band(ctx, A, hb, F)
+    L0, L = _lower(F0), _lower(F)
+    d = np.sqrt(np.diag(A))
+    E = np.abs(np.tril((A - L @ L.T) / np.outer(d, d)))
+    tile = np.arange(n) // 32
+    inside = tile[:, None] == tile[None, :]
+    assert E[~inside].max(initial=0) <= 8 * U
+    assert E[inside].max() <= 150 * U
+    top = np.abs(L0).max(axis=1)[:, None]
+    assert np.max(np.abs(L / S[:, None] - L0) / top) <= 100 * U
+    b = np.random.default_rng(5).normal(size=(n, 9))
+    # L x = S b and L^T x = b: the solutions of M, the second divided by S
+    for mode, rhs, back in ((1, S[:, None] * b, 1.0), (2, b, S[:, None]), (3, S[:, None] * b, S[:, None])):
+        x0, x = _solve(ctx, M, hb, b, mode), _solve(ctx, A, hb, rhs, mode) * back
+        assert np.max(np.abs(x - x0)) <= 100 * U * np.abs(x0).max(), mode
