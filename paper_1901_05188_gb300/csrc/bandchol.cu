@@ -93,15 +93,17 @@ __device__ __forceinline__ int blk_col(int e, int lane) { return 2 * (lane & 3) 
 // one.  A row has one scale, so its entries have to be of one natural size:
 // column k of R = L_IJ L_JJ^T is taken divided by the row scale of L at k, about
 // sqrt(a_kk), and column k of inv(L_JJ) times it.  Without, a coefficient that
-// jumps by 1e12 inside a tile cost the factor 2e-13 of sqrt(a_ii a_jj).
+// jumps by 1e12 inside a tile cost the factor 2e-13 of sqrt(a_ii a_jj).  False
+// if an entry is not finite or, at a given scale, not below it: the row scale of L
+// is an upper bound of sqrt(a_ii), so the matrix is not positive definite (and
+// fixed62 would cut the entry short, which can leave a positive pivot).
 template <bool kOwn>
 __device__ __forceinline__ bool slice_rows(const double *v, int r0, int n, int cs, int *rowexp,
                                            __half *dst, int lane) {
-  bool finite = true;
+  bool fits = true;
   for (int r = r0; r < r0 + n; ++r) {
     const double x = v[r * 33 + lane];
     const int ex = exp_above(x);
-    finite = finite && ex < 1025;
     int G;
     if (kOwn) {
       G = __reduce_max_sync(0xffffffffu, ex == kNoExp ? ex : ex + cs);
@@ -109,12 +111,13 @@ __device__ __forceinline__ bool slice_rows(const double *v, int r0, int n, int c
     } else {
       G = rowexp[r];
     }
+    fits = fits && ex < 1025 && (kOwn || ex <= G);
     const long long xb = fixed62(x, G - cs) + kDigBias;
     __half *o = dst + dig_index(r, lane);
 #pragma unroll
     for (int s = 0; s < kDig; ++s) o[s * 1024] = digit_half(xb, s);
   }
-  return finite;
+  return fits;
 }
 
 __device__ __forceinline__ void not_spd(DevStatus *st, int j, int detail) {
@@ -222,8 +225,8 @@ __device__ __forceinline__ void diag_factor(DiagSmem &Sm, const BandLayout &L, i
     double *u = tile_ptr(poolU, L, J, 0);
     for (int e = tid; e < 1024; e += 128) u[e] = A[(e >> 5) * 33 + (e & 31)];
   }
-  const bool finite = slice_rows<true>(A, 8 * w, 8, cs, ex, dg, lane);
-  if (!finite) *bad = J * 32;
+  const bool fits = slice_rows<true>(A, 8 * w, 8, cs, ex, dg, lane);
+  if (!fits) *bad = J * 32;
   diag_bar();
   uint4 *dst = reinterpret_cast<uint4 *>(dig_tile(D, L, j, J, 0));
   for (int e = tid; e < kDigTile / 8; e += 128) dst[e] = reinterpret_cast<const uint4 *>(dg)[e];
@@ -333,7 +336,7 @@ __global__ void __launch_bounds__(256, 2)
              tt == 0 ? cexp_s : rexp_s);
     __syncthreads();
     if (tile) {
-      bool finite = slice_rows<true>(R, 4 * warp, 4, -cexp_s[lane], rowe, dg, lane);
+      bool fits = slice_rows<true>(R, 4 * warp, 4, -cexp_s[lane], rowe, dg, lane);
       __syncthreads();
       if (tt == 0) {
         long long hi[8], lo[8];
@@ -347,8 +350,8 @@ __global__ void __launch_bounds__(256, 2)
         }
       }
       __syncthreads();
-      finite = slice_rows<false>(R, 4 * warp, 4, 0, rexp_s, dg, lane) && finite;
-      if (!finite) not_spd(st, j, J * 32);
+      fits = slice_rows<false>(R, 4 * warp, 4, 0, rexp_s, dg, lane) && fits;
+      if (!fits) not_spd(st, j, J * 32);
       __syncthreads();
       update(tt == 1 && m0 >= n0, dig_smem(dg), dig_smem(dg), Sm.A, rexp_s);
       uint4 *dst = reinterpret_cast<uint4 *>(dig_tile(D, L, j, I, 1));
@@ -422,9 +425,9 @@ __global__ void __launch_bounds__(256, 2)
       }
     }
     __syncthreads();
-    bool finite = true;
+    bool fits = true;
     if (mine)
-      finite = slice_rows<true>(Rt, 8 * (warp & 3), 8, -cexp_s[lane], rowe + 32 * tt, dg + tt * kDigTile, lane);
+      fits = slice_rows<true>(Rt, 8 * (warp & 3), 8, -cexp_s[lane], rowe + 32 * tt, dg + tt * kDigTile, lane);
     __syncthreads();
     if (mine) {
 #pragma unroll
@@ -445,8 +448,8 @@ __global__ void __launch_bounds__(256, 2)
         double *tu = tile_ptr(poolU, L, J, I - J);
         for (int e = t4; e < 1024; e += 128) tu[e] = Rt[(e >> 5) * 33 + (e & 31)];
       }
-      finite = slice_rows<false>(Rt, 8 * (warp & 3), 8, 0, rexp_s + 32 * tt, dg + tt * kDigTile, lane) && finite;
-      if (!finite) not_spd(st, j, J * 32);
+      fits = slice_rows<false>(Rt, 8 * (warp & 3), 8, 0, rexp_s + 32 * tt, dg + tt * kDigTile, lane) && fits;
+      if (!fits) not_spd(st, j, J * 32);
     }
     __syncthreads();
     if (mine) {

@@ -14,6 +14,8 @@ in each sweep, which the condition number carries to 4 u; 8 u.
 import numpy as np
 import pytest
 
+from workloads.darcy import make_darcy
+
 from gpu_common import require_gpu
 
 pytestmark = pytest.mark.gpu
@@ -102,3 +104,35 @@ def test_coefficients_that_vary_within_a_tile(ctx, n, hb, bits):
     for mode, rhs, back in ((1, S[:, None] * b, 1.0), (2, b, S[:, None]), (3, S[:, None] * b, S[:, None])):
         x0, x = _solve(ctx, M, hb, b, mode), _solve(ctx, A, hb, rhs, mode) * back
         assert np.max(np.abs(x - x0)) <= 100 * U * np.abs(x0).max(), mode
+
+
+@pytest.mark.parametrize("entry", [3.95, 8.1, 12.0, 1e3, 1e6, 1e200, np.inf, np.nan])
+@pytest.mark.parametrize("at", [(40, 0), (33, 31), (95, 0), (95, 33)])
+def test_indefinite_matrices_are_refused(ctx, at, entry):
+    """3.9 on the diagonal and one larger entry beside it, in every launch that
+    forms a tile: the tile below the diagonal and those further down."""
+    import paper_1901_05188_gb300 as pkg
+    A = 3.9 * np.eye(96)
+    A[at] = A[at[::-1]] = 3.85
+    F = np.zeros((96, 96))
+    pkg.geneo_debug_band(ctx, A, 96, F)
+    assert abs(F[at] * F[at[1], at[1]] - 3.85 / 3.9) <= 16 * U    # L_ij / L_jj, the inverse stored
+    A[at] = A[at[::-1]] = entry
+    with pytest.raises(pkg.GeneoError) as e:
+        pkg.geneo_debug_band(ctx, A, 96, F)
+    assert e.value.status == 4                                   # GENEO_ERR_NOT_SPD
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("coarse", ["GENEO_COARSE_NONE", "GENEO_COARSE_GENEO"])
+def test_a_negative_permeability_is_refused(prec, coarse):
+    pkg = require_gpu()
+    p = make_darcy(12, 6, 5, seed=2, partition=(2, 1, 1, 1))
+    p["perm"] = p["perm"].copy()
+    p["perm"][72:216] *= -1.0         # two layers: the nodes between them have negative diagonals
+    s = pkg.GeneoSolver()
+    s.assemble(p)
+    with pytest.raises(pkg.GeneoError) as e:
+        s.setup(p, prec, pkg.GENEO_AS, getattr(pkg, coarse))
+    assert e.value.status == 4
+    s.close()
