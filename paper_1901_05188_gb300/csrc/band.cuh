@@ -39,8 +39,8 @@ int launch_band_cholesky64(const BandLayout *d_lay, int nsys, int nt_max, int w_
 size_t band_solve_scratch(int nsys, int w_max, int ncols);
 int launch_band_solve64(const BandLayout *d_lay, int nsys, int w_max, const DigitBand &D,
                         void *scratch, const double *in, long long in_sys, int in_row, double *out,
-                        long long out_sys, int out_row, int ncols, int mode, DevStatus *st,
-                        cudaStream_t s, int alongside = 0, int ctas = 0);
+                        long long out_sys, int out_row, int ncols, int mode, cudaStream_t s,
+                        int alongside = 0, int ctas = 0);
 // Widest half-bandwidth (in tiles) the set-up accepts for the eigensolver.
 bool band_solve_fits(int w_max);
 

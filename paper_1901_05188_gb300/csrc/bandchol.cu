@@ -503,7 +503,7 @@ constexpr int kSwSlack = 4;                 // bits a column's scale may be too 
 constexpr int kSwFlush = 64;                // tiles added in 32 bits: 64 * 7 * 2^21 < 2^31
 __host__ __device__ constexpr int sweep_smem(int w, int cl) {
   return 3 * (int)kDigBytes + kSwFar * 2 * kSwHalf + (2 * (3 + cl) + 2) * kSwPart * 16 +
-         kSwY * 4 + 8 * 32 * 4 + 2 * 8 * 4 + (w + 2) * 16;
+         kSwY * 4 + 8 * 32 * 4 + 3 * 8 * 4 + (w + 2) * 16;
 }
 
 __device__ __forceinline__ void sw_bar_cta() {
@@ -555,7 +555,8 @@ __global__ void __launch_bounds__(kSwThreads, 1) k_band_sweep(const SweepArgs P)
   uint32_t *dig = reinterpret_cast<uint32_t *>(nearp + 2 * 2 * kSwPart);   // digits of s or y
   int *tf = reinterpret_cast<int *>(dig + kSwY);                    // [8][32] exponents of t
   int *fref = tf + 8 * 32;                                          // [2][8] scale of the far sums
-  short *fexp = reinterpret_cast<short *>(fref + 2 * 8);            // [w + 2][8]
+  int *nanb = fref + 2 * 8;                                         // [8] b not finite in this row
+  short *fexp = reinterpret_cast<short *>(nanb + 8);                // [w + 2][8]
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const cg::cluster_group cluster = cg::this_cluster();
   const char *tiles = static_cast<const char *>(P.D.pool) + (L.off >> 10) * (int)kDigBytes;
@@ -797,6 +798,13 @@ __global__ void __launch_bounds__(kSwThreads, 1) k_band_sweep(const SweepArgs P)
       int F = kNoExp;                         // scale of the last solved row, this column
       Fixed y{0, kNoExp, false};
       int yi = L.n;                           // its unknown, not yet stored
+      // A right-hand side that is not finite has no digits: its column is NaN from
+      // that row on, as coupling by dense tiles makes it (w = 0: in that row).
+      bool lost = false;
+      auto store = [&]() {
+        if (yi < L.n && grp * 8 + c < P.ncols)
+          dst[(long long)yi * P.out_row] = lost ? __longlong_as_double(0x7ff8000000000000LL) : y.value();
+      };
       int slot = row(0) % slots;              // of row I
       for (int q = 0; q < nt; ++q) {
         const int I = row(q);
@@ -827,6 +835,8 @@ __global__ void __launch_bounds__(kSwThreads, 1) k_band_sweep(const SweepArgs P)
             }
             const double b = x ? b1 : b0;
             const int eb = exp_above(b) - 10, ft = max(ef, eb);
+            const bool bad = __any_sync(0xffffffffu, eb >= 1015);     // infinite or NaN
+            if (lane == 0) nanb[c2 + x] = bad;
             long long ht = 0, lt = 0;
             add_shifted(mantissa53(b), 0, ft - eb, ht, lt);
             add_shifted(-h, -l, ft - ef, ht, lt);
@@ -837,9 +847,10 @@ __global__ void __launch_bounds__(kSwThreads, 1) k_band_sweep(const SweepArgs P)
           if (q + 1 < nt) tile_in(diag_t + ((q + 1) & 1) * kDigBytes, row(q + 1), 0);
         }
         cp_commit();
-        if (yi < L.n && grp * 8 + c < P.ncols) dst[(long long)yi * P.out_row] = y.value();
+        store();
         if (q + 1 < nt) fetch(q + 1);
         sw_bar_chain();
+        lost = nanb[c] || (lost && w > 0);
         int G;
         {
           const long long *tp = part + (q & 1) * np * 2 * kSwPart + o;
@@ -885,7 +896,7 @@ __global__ void __launch_bounds__(kSwThreads, 1) k_band_sweep(const SweepArgs P)
         cp_wait<0>();                         // the next row's tiles, before the barrier
         sw_bar_all(cl);
       }
-      if (yi < L.n && grp * 8 + c < P.ncols) dst[(long long)yi * P.out_row] = y.value();
+      store();
       sw_bar_chain();                         // before the backward sweep fetches them
     }
   }
@@ -941,8 +952,8 @@ size_t band_solve_scratch(int nsys, int w_max, int ncols) {
 
 int launch_band_solve64(const BandLayout *d_lay, int nsys, int w_max, const DigitBand &D,
                         void *scratch, const double *in, long long in_sys, int in_row, double *out,
-                        long long out_sys, int out_row, int ncols, int mode, DevStatus *st,
-                        cudaStream_t s, int alongside, int ctas) {
+                        long long out_sys, int out_row, int ncols, int mode, cudaStream_t s,
+                        int alongside, int ctas) {
   if (D.window || ctas < 0 || ctas > 2) return GENEO_ERR_INVALID_ARG;
   int dev = 0, sms = 0;
   GENEO_CUDA_TRY(cudaGetDevice(&dev));

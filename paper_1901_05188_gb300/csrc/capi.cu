@@ -1057,11 +1057,11 @@ static int setup_coarse(geneo_ctx *c, SetupPlan &P, cudaStream_t s) {
     char *scr = (char *)pc.solve_scr + band_solve_scratch((int)j0, pc.w_neu_max, p);
     // W = L^-1 B L^-T V_k
     if ((r = launch_band_solve64(lay, n, pc.w_neu_max, D, scr, V + k * p, sV, ldv, T1, sW, p, p, 2,
-                                 c->status, gs, other)))
+                                 gs, other)))
       return r;
     launch_bloc_mv(subs, n, P.max_nodes_neu, pc.Bloc, T1, W, sW, p, gs);
-    if ((r = launch_band_solve64(lay, n, pc.w_neu_max, D, scr, W, sW, p, W, sW, p, p, 1, c->status,
-                                 gs, other)))
+    if ((r = launch_band_solve64(lay, n, pc.w_neu_max, D, scr, W, sW, p, W, sW, p, p, 1, gs,
+                                 other)))
       return r;
     const int na = (k + 1) * p;
     // full re-orthogonalisation against V: a second pass only for the
@@ -1161,7 +1161,7 @@ static int setup_coarse(geneo_ctx *c, SetupPlan &P, cudaStream_t s) {
   launch_tsgemm(pc.d_subs, nsub, npad, pc.V, ldv, sV, kdim, pc.Evec, kdim, (long long)kdim * kdim,
                 pc.P, mcap, sP, mcap, 1.0, 0.0, s);
   if ((st = launch_band_solve64(pc.d_lay_neu, nsub, pc.w_neu_max, pc.dig_neu, pc.solve_scr, pc.P, sP,
-                                mcap, pc.P, sP, mcap, mcap, 2, c->status, s)))
+                                mcap, pc.P, sP, mcap, mcap, 2, s)))
     return st;
   launch_tsdots(pc.d_subs, nsub, npad, pc.P, mcap, sP, mcap, pc.P, mcap, sP, mcap, pc.Hpart,
                 kDotChunks, pc.G, (long long)mcap * mcap, s);
@@ -1265,7 +1265,7 @@ static int build_coarse_operator(geneo_ctx *c, SetupPlan &P, const std::vector<l
     return st;
   launch_identity(pc.AHinv, nH, s);
   if ((st = launch_band_solve64(pc.d_lay_H, 1, LH.w, pc.dig_H, pc.solve_scr, pc.AHinv, 0, nH, pc.AHinv,
-                                0, nH, nH, 3, c->status, s)))
+                                0, nH, nH, 3, s)))
     return st;
   launch_symmetrize(pc.AHinv, nH, s);
   GENEO_CUDA_TRY(cudaGetLastError());
@@ -2144,7 +2144,7 @@ extern "C" int geneo_debug_band(geneo_ctx *c, int n, int half_band, const double
   if (ncols > 0) {
     GENEO_CUDA_TRY(cudaMemcpyAsync(rhs, b, nb * sizeof(double), cudaMemcpyDefault, s));
     if (int st = launch_band_solve64(dl, 1, L.w, D, m.p[6], rhs, 0, ncols, rhs, 0, ncols, ncols, mode,
-                                     status, s, 0, ctas))
+                                     s, 0, ctas))
       return st;
   }
   GENEO_CUDA_TRY(copy_sync(c, &h, status, sizeof(h), cudaMemcpyDeviceToHost));
@@ -2244,8 +2244,7 @@ extern "C" int geneo_profile(geneo_ctx *c, int what, int reps, double *ms_per_la
       } else if (what == 3) {
         const int p = kLanczosBlock, ldv = pc.kdim + p, npad = pc.npad_neu_max;
         st = launch_band_solve64(pc.d_lay_neu, pc.nsub, pc.w_neu_max, pc.dig_neu, pc.solve_scr, pc.V,
-                                 (long long)npad * ldv, ldv, pc.T1, (long long)npad * p, p, p, 2,
-                                 c->status, s);
+                                 (long long)npad * ldv, ldv, pc.T1, (long long)npad * p, p, p, 2, s);
       } else if (what == 4) {
         // re-assemble S_j = A_j - sigma B_j and factor it again (same result)
         if (!(st = launch_band_clear<double>(pc.d_lay_neu, pc.nsub, pc.neuL, pc.fac_neu_elems, s))) {

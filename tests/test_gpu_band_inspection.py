@@ -136,3 +136,24 @@ def test_a_negative_permeability_is_refused(prec, coarse):
         s.setup(p, prec, pkg.GENEO_AS, getattr(pkg, coarse))
     assert e.value.status == 4
     s.close()
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+@pytest.mark.parametrize("n,hb,ctas", [(270, 40, 1), (420, 192, 2), (90, 0, 1), (20, 3, 1)])
+def test_a_right_hand_side_that_is_not_finite_stays_so(ctx, n, hb, ctas, bad):
+    """As with dense tiles: from the tile of the bad row on (backward: up to it; an
+    uncoupled matrix: in it), in its column only."""
+    A = _matrix(n, hb)
+    rng = np.random.default_rng(3)
+    b = rng.normal(size=(n, 11))
+    i, c = n // 2, 9
+    tile, I = np.arange(n) // 32, (n // 2) // 32
+    worse = b.copy()
+    worse[i, c] = bad
+    for mode in (1, 2, 3):
+        good, x = _solve(ctx, A, hb, b, mode, ctas), _solve(ctx, A, hb, worse, mode, ctas)
+        other = np.arange(11) != c
+        assert np.array_equal(good[:, other], x[:, other])
+        hit = tile == I if hb == 0 else tile >= I if mode == 1 else tile <= I if mode == 2 else tile >= 0
+        assert not np.any(np.isfinite(x[hit, c])), mode
+        assert np.array_equal(x[~hit, c], good[~hit, c]), mode
