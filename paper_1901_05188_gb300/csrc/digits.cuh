@@ -139,10 +139,14 @@ __device__ __forceinline__ void level_parts(const float (&S)[kDig][4], int e, lo
   lo = (long long)s[4] * 262144 + ((long long)s[5] * 512 + s[6]);
 }
 
-// (hi 2^27 + lo) 2^(e - 70)
+// (hi 2^27 + lo) 2^(e - 70), zero below the normal range: the integer as a double,
+// whose exponent field is then moved (a factor 2^(e - 70) may itself leave the range).
 __device__ __forceinline__ double parts_value(long long hi, long long lo, int e) {
-  const int k = min(max(e - 70, -1022), 1023);
-  return fma((double)hi, 134217728.0, (double)lo) * __hiloint2double((k + 1023) << 20, 0);
+  const double v = fma((double)hi, 134217728.0, (double)lo);
+  const int h = __double2hiint(v), bv = (h >> 20) & 0x7ff, be = bv + e - 70;
+  if (bv == 0 || be < 1) return 0.0;
+  if (be > 2046) return __hiloint2double((h & 0x80000000) | 0x7ff00000, 0);
+  return __hiloint2double(h + ((e - 70) << 20), __double2loint(v));
 }
 
 // m 2^(ex - 64) with 2^63 <= m < 2^64, or zero (m = 0, ex <= kNoExp), and a sign.

@@ -157,3 +157,26 @@ def test_a_right_hand_side_that_is_not_finite_stays_so(ctx, n, hb, ctas, bad):
         hit = tile == I if hb == 0 else tile >= I if mode == 1 else tile <= I if mode == 2 else tile >= 0
         assert not np.any(np.isfinite(x[hit, c])), mode
         assert np.array_equal(x[~hit, c], good[~hit, c]), mode
+
+
+@pytest.mark.parametrize("power", [-980, -960, -512, 512, 960])
+@pytest.mark.parametrize("n,hb", [(31, 3), (200, 40), (270, 270)])
+def test_small_and_large_matrices(ctx, n, hb, power):
+    """2^power M: products of digits whose scales lie near the ends of the FP64 range.
+
+    The factor and the solutions are M's times powers of two, but for the pivots'
+    reciprocals (a few u, carried by the condition number 3): 100 u of the largest.
+    """
+    import paper_1901_05188_gb300 as pkg
+    M, s = _matrix(n, hb), 2.0 ** (power // 2)
+    F0, F = np.zeros((n, n)), np.zeros((n, n))
+    pkg.geneo_debug_band(ctx, M, hb, F0)
+    pkg.geneo_debug_band(ctx, M * s * s, hb, F)
+    tile = np.arange(n) // 32
+    F = np.where(tile[:, None] == tile[None, :], F * s, F / s)
+    assert np.max(np.abs(F - F0)) <= 100 * U * np.abs(F0).max()
+    b = np.random.default_rng(5).normal(size=(n, 9))
+    for mode, back in ((1, s), (2, s), (3, s)):
+        x0 = _solve(ctx, M, hb, b, mode)
+        x = _solve(ctx, M * s * s, hb, b if mode < 3 else b * s, mode) * back
+        assert np.max(np.abs(x - x0)) <= 100 * U * np.abs(x0).max(), mode
