@@ -1599,6 +1599,8 @@ int launch_schwarz_solve(const SubDesc *d_subs, const BandLayout *d_lay, int nsu
 bool band_solve_fits(int w_max) { return smem_bytes_ring<double>(w_max) <= kSmemMax; }
 
 // ---- batch launchers -----------------------------------------------------------
+constexpr long long kBatchSmemMax = kSmemMax - 16;   // beside the item index, in static memory
+
 template <typename T>
 static long long batch_smem(int npad_max, int w_max, int cluster, int rows, int staged, int *stride,
                             int *stage_chain) {
@@ -1614,7 +1616,7 @@ template <typename T>
 bool batch_schwarz_fits(int npad_max, int w_max, int cluster, int rows, int staged) {
   if (rows < 0 || rows > 1 || (cluster != 1 && cluster != 2 && cluster != 4)) return false;
   int st, sc;
-  return batch_smem<T>(npad_max, w_max, cluster, rows, staged, &st, &sc) <= kSmemMax;
+  return batch_smem<T>(npad_max, w_max, cluster, rows, staged, &st, &sc) <= kBatchSmemMax;
 }
 
 // The kernel of a shape (raised to its shared memory), or null.
@@ -1634,7 +1636,7 @@ int prepare_batch_schwarz(int npad_max, int w_max) {
       for (int staged = 0; staged < 2; ++staged) {
         int st, stride, sc;
         const long long b = batch_smem<T>(npad_max, w_max, cluster, rows, staged, &stride, &sc);
-        if (b > kSmemMax) continue;
+        if (b > kBatchSmemMax) continue;
         auto k = cluster == 1 ? batch_kernel<T, 1>(rows, staged, sc)
                  : cluster == 2 ? batch_kernel<T, 2>(rows, staged, sc) : batch_kernel<T, 4>(rows, staged, sc);
         if ((st = ensure_smem(k, (int)b))) return st;
