@@ -24,6 +24,8 @@
  *    Schwarz pins), fix choices the set-up otherwise makes itself; a value
  *    outside the listed set is ignored:
  *      GENEO_SCHWARZ_CLUSTER  CTAs per subdomain of the local solves: 1, 2, 4, 8
+ *                             (a batch: that, at most 4, halved while it does
+ *                             not fit in shared memory)
  *      GENEO_SCHWARZ_ROWS     tile rows per step: 1, 2, 4, or 0 (look-ahead)
  *      GENEO_SCHWARZ_STAGED   0 tiles from global memory, 1 staged by bulk
  *                             copies, 2 ring form (local vector streamed)
@@ -441,10 +443,10 @@ int geneo_kappa_from_cg(const double *alphas, const double *betas, int k, double
  * and owns only the concatenated Krylov vectors and its work tables.  Every
  * kernel launch of an iteration covers every instance; each instance keeps
  * its own (F)PCG scalars and stops on its own criterion; the one-level local
- * solves of all instances run in one persistent launch whose CTAs take
+ * solves of all instances run in one persistent launch whose clusters take
  * (instance, subdomain) items from a device work queue, largest first, in a
- * launch shape chosen by timing at creation (GENEO_SCHWARZ_ROWS /
- * GENEO_SCHWARZ_STAGED pin it); the iterations are captured in a CUDA graph.
+ * launch shape chosen by timing at creation (GENEO_SCHWARZ_CLUSTER,
+ * GENEO_SCHWARZ_ROWS and GENEO_SCHWARZ_STAGED pin it); the iterations are captured in a CUDA graph.
  * While a batch exists its contexts must not run other work (it uses their
  * buffers).  Work goes to cuda_stream (NULL = legacy default stream).
  * Returns GENEO_ERR_STATE for a context that is not set up,

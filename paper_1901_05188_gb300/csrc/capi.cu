@@ -2580,23 +2580,31 @@ extern "C" int geneo_batch_create(geneo_batch **out, geneo_ctx *const *ctxs, int
   // one CTA are tried while the items make at most two rounds of them: with more
   // the queue keeps the SMs busy, and a cluster only adds its exchange.
   // GENEO_SCHWARZ_CLUSTER, GENEO_SCHWARZ_ROWS and GENEO_SCHWARZ_STAGED pin a
-  // dimension (a cluster of 8, which the batch has not, leaves it open).
-  const int fc = env_choice("GENEO_SCHWARZ_CLUSTER", {1, 2, 4});
+  // dimension; a cluster that the batch has not (8) or that does not fit is
+  // halved until one does, so that the pin neither refuses a batch nor leaves
+  // the choice to the timing.
+  const int fc = env_choice("GENEO_SCHWARZ_CLUSTER", {1, 2, 4, 8});
   const int fr = env_choice("GENEO_SCHWARZ_ROWS", {0, 1});
   const int fs = env_choice("GENEO_SCHWARZ_STAGED", {0, 1});
   struct Shape {
     int cluster, rows, staged;
   };
   std::vector<Shape> cand;
-  for (int Cl : {1, 2, 4})
+  auto shapes = [&](int Cl) {
     for (int R : {0, 1})
       for (int Sg : {1, 0}) {
-        if (fc >= 0 ? Cl != fc : (Cl > 1 && B->T.nsub_items * Cl > 2 * B->sms)) continue;
         if ((fr >= 0 && R != fr) || (fs >= 0 && Sg != fs)) continue;
         const bool fits = f32 ? batch_schwarz_fits<float>(B->npad_max, B->w_max, Cl, R, Sg)
                               : batch_schwarz_fits<double>(B->npad_max, B->w_max, Cl, R, Sg);
         if (fits) cand.push_back({Cl, R, Sg});
       }
+  };
+  if (fc >= 0) {
+    for (int Cl = std::min(fc, 4); Cl >= 1 && cand.empty(); Cl /= 2) shapes(Cl);
+  } else {
+    for (int Cl : {1, 2, 4})
+      if (Cl == 1 || B->T.nsub_items * Cl <= 2 * B->sms) shapes(Cl);
+  }
   if (cand.empty()) return fail(GENEO_ERR_INVALID_ARG, "no batched local-solve shape fits");
   auto use = [&](const Shape &c) {
     B->cluster = c.cluster;
