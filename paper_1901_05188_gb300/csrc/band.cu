@@ -32,9 +32,10 @@ __global__ void k_band_pad(const BandLayout *lay, int nsys, T *pool) {
   if (j >= nsys) return;
   BandLayout L = lay[j];
   int last = L.nt - 1;
+  T *t = pool + L.off + (long long)last * (L.w + 1) * L.slot;
   for (int idx = L.n + threadIdx.x; idx < L.nt * 32; idx += blockDim.x) {
     int r = idx - last * 32;
-    tile_ptr(pool, L, last, 0)[r * 32 + r] = T(1);
+    t[r * 32 + r] = T(1);
   }
 }
 
@@ -221,8 +222,12 @@ __global__ void k_extract_interior(const SubDesc *subs, const BandLayout *lay, i
 
 template <typename T>
 int launch_band_clear(const BandLayout *d_lay, int nsys, T *pool, long long pool_elems,
-                      cudaStream_t s) {
-  GENEO_CUDA_TRY(cudaMemsetAsync(pool, 0, pool_elems * sizeof(T), s));
+                      cudaStream_t s, int slot) {
+  if (slot == 1024) {
+    GENEO_CUDA_TRY(cudaMemsetAsync(pool, 0, pool_elems * sizeof(T), s));
+  } else {                                 // the tiles, not what their digits need beside them
+    GENEO_CUDA_TRY(cudaMemset2DAsync(pool, slot * sizeof(T), 0, 1024 * sizeof(T), pool_elems / slot, s));
+  }
   k_band_pad<T><<<nsys, 32, 0, s>>>(d_lay, nsys, pool); GENEO_COUNT_LAUNCH();
   GENEO_CUDA_TRY(cudaGetLastError());
   return GENEO_OK;
@@ -291,8 +296,8 @@ int launch_extract_interior(const SubDesc *d_subs, const BandLayout *d_lay, int 
   return GENEO_OK;
 }
 
-template int launch_band_clear<double>(const BandLayout *, int, double *, long long, cudaStream_t);
-template int launch_band_clear<float>(const BandLayout *, int, float *, long long, cudaStream_t);
+template int launch_band_clear<double>(const BandLayout *, int, double *, long long, cudaStream_t, int);
+template int launch_band_clear<float>(const BandLayout *, int, float *, long long, cudaStream_t, int);
 template int launch_extract_interior<double>(const SubDesc *, const BandLayout *, int, int, int,
                                              int, int, const int32_t *, const double *,
                                              double *, cudaStream_t);

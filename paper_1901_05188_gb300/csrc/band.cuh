@@ -10,7 +10,7 @@ namespace geneo {
 // Zero a pool of tiles and put ones on the padded diagonal of every system.
 template <typename T>
 int launch_band_clear(const BandLayout *d_lay, int nsys, T *pool, long long pool_elems,
-                      cudaStream_t s);
+                      cudaStream_t s, int slot = 1024);
 
 // FP32 right-looking tile Cholesky of nsys band systems held in poolL (lower
 // triangle of each tile row as input).  On exit poolL/poolU hold the forward
@@ -20,10 +20,11 @@ int launch_band_clear(const BandLayout *d_lay, int nsys, T *pool, long long pool
 int launch_band_cholesky32(const BandLayout *d_lay, int nsys, int nt_max, int w_max, float *poolL,
                            float *poolU, DevStatus *st, cudaStream_t s, cudaStream_t side = nullptr);
 
-// FP64 left-looking tile Cholesky on the tensor cores (digits.cuh): the same
-// result in poolL and, unless it is null, poolU, and the factor's digits in D
-// (in the whole-band form, what launch_band_solve64 reads).  With a side
-// stream the two halves of the systems are factored concurrently.
+// FP64 left-looking tile Cholesky on the tensor cores (digits.cuh).  With a
+// window of digits: the same result in poolL and, unless it is null, poolU.
+// Without (D.window = 0, D.pool = poolL, layouts with slots of kDigSlot): the
+// factor's digits in place of the matrix, what launch_band_solve64 reads.  With
+// a side stream the two halves of the systems are factored concurrently.
 int launch_band_cholesky64(const BandLayout *d_lay, int nsys, int nt_max, int w_max, double *poolL,
                            double *poolU, const DigitBand &D, DevStatus *st, cudaStream_t s,
                            cudaStream_t side = nullptr);

@@ -24,17 +24,18 @@ namespace cg = cooperative_groups;
 namespace {
 
 __device__ __forceinline__ double *tile_ptr(double *base, const BandLayout &L, int I, int d) {
-  return base + L.off + (((long long)I * (L.w + 1) + d) << 10);
+  return base + L.off + ((long long)I * (L.w + 1) + d) * L.slot;
 }
 
-// Tile (I, d) of system j in the digit pool: the whole band, or only the w + 1
-// tile rows the factorisation can still touch (row I in slot I mod (w + 1)).
+// Tile (I, d) of system j in the digit pool: in place of the FP64 tile, or only the
+// w + 1 tile rows the factorisation can still touch (row I in slot I mod (w + 1)).
 __device__ __forceinline__ __half *dig_tile(const DigitBand &D, const BandLayout &L, int j, int I,
                                             int d) {
-  const long long t = D.window ? (long long)j * D.window + (long long)(I % (L.w + 1)) * (L.w + 1) + d
-                               : (L.off >> 10) + (long long)I * (L.w + 1) + d;
-  return static_cast<__half *>(D.pool) + t * kDigTile;
+  if (!D.window) return reinterpret_cast<__half *>(tile_ptr(static_cast<double *>(D.pool), L, I, d));
+  return static_cast<__half *>(D.pool) +
+         ((long long)j * D.window + (long long)(I % (L.w + 1)) * (L.w + 1) + d) * kDigTile;
 }
+static_assert(kDigSlot * 8 == kDigBytes && kDigHalves == kDigTile, "a slot holds a tile's digits");
 
 // Scale of row i of the factor: |L_ik| <= sqrt(a_ii) < 2^E.
 __global__ void k_row_exps(const BandLayout *lay, int sys0, double *poolL, DigitBand D) {
@@ -159,7 +160,7 @@ struct DiagSmem {
 
 // L D L^T of the diagonal tile J in Sm.A (updates applied) and the inverse of the
 // unit factor together, one elimination step per column; the inverse of the
-// Cholesky factor goes to the pools.  Four warps, one per SM sub-partition;
+// Cholesky factor goes to the pools (in place, D.window = 0: only its digits).  Four warps, one per SM sub-partition;
 // lane = row, warp w owns columns 4 q + w.  The FP64 pipe takes 64 cycles per
 // warp instruction, so a step costs its eight updates (the entries of L right
 // of the pivot and of the inverse left of it); the warp that owns the next
@@ -220,7 +221,8 @@ __device__ __forceinline__ void diag_factor(DiagSmem &Sm, const BandLayout &L, i
 #pragma unroll
   for (int q = 0; q < 8; ++q) A[lane * 33 + 4 * q + w] = x[q] * rs;      // inv(L_JJ)
   diag_bar();
-  for (int e = tid; e < 1024; e += 128) t[e] = A[(e & 31) * 33 + (e >> 5)];
+  if (D.window)
+    for (int e = tid; e < 1024; e += 128) t[e] = A[(e & 31) * 33 + (e >> 5)];
   if (poolU) {
     double *u = tile_ptr(poolU, L, J, 0);
     for (int e = tid; e < 1024; e += 128) u[e] = A[(e >> 5) * 33 + (e & 31)];
@@ -359,7 +361,7 @@ __global__ void __launch_bounds__(256, 2)
       for (int e = tid; e < kDigTile / 8; e += 256) dst[e] = src[e];
       double *tu = poolU ? tile_ptr(poolU, L, J, 1) : nullptr;
       for (int e = tid; e < 1024; e += 256) {
-        tr[e] = R[(e & 31) * 33 + (e >> 5)];
+        if (D.window) tr[e] = R[(e & 31) * 33 + (e >> 5)];
         if (tu) tu[e] = R[(e >> 5) * 33 + (e & 31)];
       }
       __syncthreads();
@@ -443,7 +445,8 @@ __global__ void __launch_bounds__(256, 2)
     if (mine) {
       const int t4 = tid & 127;
       double *tl = tile_ptr(poolL, L, I, I - J);
-      for (int e = t4; e < 1024; e += 128) tl[e] = Rt[(e & 31) * 33 + (e >> 5)];
+      if (D.window)
+        for (int e = t4; e < 1024; e += 128) tl[e] = Rt[(e & 31) * 33 + (e >> 5)];
       if (poolU) {
         double *tu = tile_ptr(poolU, L, J, I - J);
         for (int e = t4; e < 1024; e += 128) tu[e] = Rt[(e >> 5) * 33 + (e & 31)];
@@ -559,7 +562,7 @@ __global__ void __launch_bounds__(kSwThreads, 1) k_band_sweep(const SweepArgs P)
   short *fexp = reinterpret_cast<short *>(nanb + 8);                // [w + 2][8]
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const cg::cluster_group cluster = cg::this_cluster();
-  const char *tiles = static_cast<const char *>(P.D.pool) + (L.off >> 10) * (int)kDigBytes;
+  const char *tiles = static_cast<const char *>(P.D.pool) + L.off * 8;
   uint4 *yring = P.ring + ((long long)grp * (gridDim.x / cl) + j) * (P.w_max + 2) * (kSwY / 4);
   if (cl > 1) sw_bar_all(cl);               // every CTA is there before its memory is written
   for (int back = 0; back < 2; ++back) {

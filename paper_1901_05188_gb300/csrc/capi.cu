@@ -167,16 +167,17 @@ int axis_partition(int n, int p, int O, AxisPart &a) {
   return GENEO_OK;
 }
 
-BandLayout make_layout(int n, int hb, long long off) {
+BandLayout make_layout(int n, int hb, long long off, int slot = 1024) {
   BandLayout L;
   L.n = n;
   L.nt = (n + 31) / 32;
   L.w = std::min((hb + 31) / 32, L.nt - 1);
   L.off = off;
+  L.slot = slot;
   return L;
 }
 
-long long layout_elems(const BandLayout &L) { return (long long)L.nt * (L.w + 1) * 1024; }
+long long layout_elems(const BandLayout &L) { return (long long)L.nt * (L.w + 1) * L.slot; }
 
 // Host restatement of the mode-selection rule (Sec. 3.2 threshold with cap and
 // cluster guard): returns m_j given ascending eigenvalues (inf = infinite).
@@ -664,7 +665,7 @@ int build_plan(geneo_ctx *c, const geneo_partition *part, const geneo_modes *mod
         S.n_int = c->nc * S.ibox.count();
         S.n_neu = c->nc * S.nbox.count();
         BandLayout Li = make_layout(S.n_int, S.ibox.half_band_dofs(c->nc), f_int);
-        BandLayout Ln = make_layout(S.n_neu, S.nbox.half_band_dofs(c->nc), f_neu);
+        BandLayout Ln = make_layout(S.n_neu, S.nbox.half_band_dofs(c->nc), f_neu, kDigSlot);
         S.nt_int = Li.nt;
         S.w_int = Li.w;
         S.f_int = f_int;
@@ -731,9 +732,10 @@ void take_cg_vectors(Arena &A, geneo_ctx *c) {
   c->cg = A.take<CGScalars>(1);
 }
 
-DigitBand take_digits(Arena &A, int nsys, int npad, long long tiles, long long window) {
+// Digits in place of the tiles in `pool`, or in windows of their own.
+DigitBand take_digits(Arena &A, int nsys, int npad, double *pool, long long window) {
   DigitBand D;
-  D.pool = A.take<uint16_t>((size_t)tiles * kDigHalves);
+  D.pool = window ? (void *)A.take<uint16_t>((size_t)nsys * window * kDigHalves) : pool;
   D.rexp = A.take<int>((size_t)nsys * npad);
   D.dexp = A.take<int>((size_t)nsys * npad);
   D.npad = npad;
@@ -762,7 +764,7 @@ void plan_setup(Arena &A, geneo_ctx *c, const SetupPlan &P) {
   pc.yloc = A.take<char>(pc.xloc_elems * esz);   // forward-sweep scratch of the ring form
   pc.wloc = A.take<double>(pc.xloc_elems);     // Sarkis weights (filled for that PoU only)
   const long long win = (long long)(pc.w_int_max + 1) * (pc.w_int_max + 1);
-  pc.dig_int = f32 ? DigitBand{} : take_digits(A, nsub, pc.npad_int_max, win * nsub, win);
+  pc.dig_int = f32 ? DigitBand{} : take_digits(A, nsub, pc.npad_int_max, nullptr, win);
   int cap = pc.modes.fixed_modes > 0 ? pc.modes.fixed_modes : pc.modes.max_modes;
   if (pc.coarse == GENEO_COARSE_NONE) cap = 0;
   if (pc.coarse == GENEO_COARSE_ZEM) cap = 6;     // the rigid displacements
@@ -778,7 +780,7 @@ void plan_setup(Arena &A, geneo_ctx *c, const SetupPlan &P) {
     pc.gate = nullptr;
     if (eig) {   // shift-invert block Lanczos of the GenEO eigenproblems
       pc.neuL = A.take<double>(pc.fac_neu_elems);
-      pc.dig_neu = take_digits(A, nsub, npad, pc.fac_neu_elems / 1024, 0);
+      pc.dig_neu = take_digits(A, nsub, npad, pc.neuL, 0);
       pc.Bloc = A.take<double>((size_t)c->nc * c->nc * pc.bloc_blocks);
       pc.V = A.take<double>((size_t)nsub * npad * (pc.kdim + p));
       pc.Vt = A.take<double>((size_t)nsub * npad * pc.kkeep);
@@ -812,8 +814,8 @@ void plan_setup(Arena &A, geneo_ctx *c, const SetupPlan &P) {
     int ntH = (pc.nH_cap + 31) / 32;
     pc.AH = A.take<double>((size_t)pc.nH_cap * pc.nH_cap);
     pc.AHinv = A.take<double>((size_t)pc.nH_cap * pc.nH_cap);
-    pc.AHL = A.take<double>((size_t)ntH * ntH * 1024);
-    pc.dig_H = take_digits(A, 1, ntH * 32, (long long)ntH * ntH, 0);
+    pc.AHL = A.take<double>((size_t)ntH * ntH * kDigSlot);
+    pc.dig_H = take_digits(A, 1, ntH * 32, pc.AHL, 0);
     size_t scr = band_solve_scratch(1, ntH - 1, pc.nH_cap);
     if (eig) scr = std::max(scr, band_solve_scratch(nsub, pc.w_neu_max, std::max(pc.mcap, p)));
     pc.solve_scr = A.take<char>(scr);
@@ -988,7 +990,7 @@ static int setup_coarse(geneo_ctx *c, SetupPlan &P, cudaStream_t s) {
   // PoU, S = A - sigma B into band tiles, B into a local BSR
   launch_pou_neumann(pc.d_subs, nsub, P.max_nodes_neu, pc.d_cand, pc.cand_off, c->mask, nnx, nny,
                      c->nz + 1, pc.part.px, pc.part.py, pc.pou, pc.Xneu, s);
-  if ((st = launch_band_clear<double>(pc.d_lay_neu, nsub, pc.neuL, pc.fac_neu_elems, s))) return st;
+  if ((st = launch_band_clear<double>(pc.d_lay_neu, nsub, pc.neuL, pc.fac_neu_elems, s, kDigSlot))) return st;
   launch_neumann_assemble(pc.d_subs, pc.d_lay_neu, nsub, P.max_nodes_neu, c->nx, c->ny, c->nz,
                           c->X, c->Y, c->Z, c->Cel, c->perm, pc.d_ecnt, pc.ecnt_off, c->mask,
                           pc.Xneu, sigma, pc.neuL, pc.Bloc, s);
@@ -1253,13 +1255,9 @@ static int build_coarse_operator(geneo_ctx *c, SetupPlan &P, const std::vector<l
     return GENEO_OK;
   }
   // dense Cholesky of A_H (a band system of full width) and its inverse
-  BandLayout LH;
-  LH.n = nH;
-  LH.nt = (nH + 31) / 32;
-  LH.w = LH.nt - 1;
-  LH.off = 0;
+  const BandLayout LH = make_layout(nH, nH, 0, kDigSlot);
   GENEO_CUDA_TRY(cudaMemcpyAsync(pc.d_lay_H, &LH, sizeof(LH), cudaMemcpyHostToDevice, s));
-  if ((st = launch_band_clear<double>(pc.d_lay_H, 1, pc.AHL, (long long)LH.nt * LH.nt * 1024, s))) return st;
+  if ((st = launch_band_clear<double>(pc.d_lay_H, 1, pc.AHL, layout_elems(LH), s, kDigSlot))) return st;
   launch_dense_to_tiles(pc.AH, nH, pc.d_lay_H, pc.AHL, s);
   if ((st = launch_band_cholesky64(pc.d_lay_H, 1, LH.nt, LH.w, pc.AHL, nullptr, pc.dig_H, c->status, s)))
     return st;
@@ -2104,17 +2102,13 @@ extern "C" int geneo_debug_band(geneo_ctx *c, int n, int half_band, const double
     return fail(GENEO_ERR_INVALID_ARG, "bad matrix, mode or right-hand sides");
   half_band = std::min(half_band, n - 1);
   cudaStream_t s = c->stream;
-  const BandLayout L = make_layout(n, half_band, 0);
-  const size_t el = layout_elems(L), nn = (size_t)n * n, nb = (size_t)n * ncols;
-  std::vector<double> dense(nn), tiles(el, 0.0);
+  // for the factor beside a window of digits, as the interior factors; for
+  // solves in place, as the eigensolver's
+  const BandLayout L[2] = {make_layout(n, half_band, 0), make_layout(n, half_band, 0, kDigSlot)};
+  const int nt = L[0].nt, w = L[0].w;
+  const size_t nn = (size_t)n * n, nb = (size_t)n * ncols;
+  std::vector<double> dense(nn), tiles;
   GENEO_CUDA_TRY(copy_sync(c, dense.data(), a, nn * sizeof(double), cudaMemcpyDefault));
-  auto tile = [&](int R, int C) -> double & {
-    const int I = R >> 5, d = I - (C >> 5);
-    return tiles[((size_t)I * (L.w + 1) + d) * 1024 + (C & 31) * 32 + (R & 31)];
-  };
-  for (int R = 0; R < n; ++R)
-    for (int C = std::max(0, R - half_band); C <= R; ++C) tile(R, C) = dense[(size_t)R * n + C];
-  for (int R = n; R < L.nt * 32; ++R) tile(R, R) = 1.0;
   struct Scratch {                         // freed on every way out
     cudaStream_t s;
     void *p[7] = {};
@@ -2123,40 +2117,56 @@ extern "C" int geneo_debug_band(geneo_ctx *c, int n, int half_band, const double
         if (q) cudaFreeAsync(q, s);
     }
   } m{s};
-  const size_t exps = 2 * (size_t)L.nt * 32 * sizeof(int);
-  const size_t want[7] = {el * sizeof(double), sizeof(BandLayout), sizeof(DevStatus), exps,
-                          el / 1024 * kDigHalves * 2, nb * sizeof(double),
-                          ncols > 0 ? band_solve_scratch(1, L.w, ncols) : 0};
+  const long long window = (long long)(w + 1) * (w + 1);
+  const size_t want[7] = {layout_elems(L[ncols > 0]) * sizeof(double), sizeof(BandLayout),
+                          sizeof(DevStatus), 2 * (size_t)nt * 32 * sizeof(int),
+                          (ncols > 0 && !factor) ? 0 : (size_t)window * kDigHalves * 2,
+                          nb * sizeof(double), ncols > 0 ? band_solve_scratch(1, w, ncols) : 0};
   for (int i = 0; i < 7; ++i)
     if (want[i]) GENEO_CUDA_TRY(cudaMallocAsync(&m.p[i], want[i], s));
   double *pool = (double *)m.p[0], *rhs = (double *)m.p[5];
   BandLayout *dl = (BandLayout *)m.p[1];
   DevStatus *status = (DevStatus *)m.p[2], h{};
-  DigitBand D;
-  D.pool = m.p[4];
-  D.rexp = (int *)m.p[3];
-  D.dexp = D.rexp + L.nt * 32;
-  D.npad = L.nt * 32;
-  GENEO_CUDA_TRY(cudaMemcpyAsync(pool, tiles.data(), el * sizeof(double), cudaMemcpyHostToDevice, s));
-  GENEO_CUDA_TRY(cudaMemcpyAsync(dl, &L, sizeof(L), cudaMemcpyHostToDevice, s));
-  GENEO_CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(DevStatus), s));
-  if (int st = launch_band_cholesky64(dl, 1, L.nt, L.w, pool, nullptr, D, status, s)) return st;
-  if (ncols > 0) {
-    GENEO_CUDA_TRY(cudaMemcpyAsync(rhs, b, nb * sizeof(double), cudaMemcpyDefault, s));
-    if (int st = launch_band_solve64(dl, 1, L.w, D, m.p[6], rhs, 0, ncols, rhs, 0, ncols, ncols, mode,
-                                     s, 0, ctas))
-      return st;
-  }
-  GENEO_CUDA_TRY(copy_sync(c, &h, status, sizeof(h), cudaMemcpyDeviceToHost));
-  if (h.code) return fail(h.code, ("no positive pivot in row " + std::to_string(h.detail)).c_str());
-  if (ncols > 0) GENEO_CUDA_TRY(copy_sync(c, x, rhs, nb * sizeof(double), cudaMemcpyDefault));
-  if (factor) {
-    GENEO_CUDA_TRY(copy_sync(c, tiles.data(), pool, el * sizeof(double), cudaMemcpyDeviceToHost));
-    std::fill(dense.begin(), dense.end(), 0.0);
+  for (int solve = 0; solve < 2; ++solve) {
+    if (solve ? ncols == 0 : (ncols > 0 && !factor)) continue;
+    const BandLayout &Ls = L[solve];
+    auto tile = [&](int R, int C) -> double & {
+      const int I = R >> 5, d = I - (C >> 5);
+      return tiles[((size_t)I * (w + 1) + d) * Ls.slot + (C & 31) * 32 + (R & 31)];
+    };
+    tiles.assign(layout_elems(Ls), 0.0);
     for (int R = 0; R < n; ++R)
-      for (int C = std::max(0, (R >> 5) - L.w) * 32; C < std::min(n, ((R >> 5) + 1) * 32); ++C)
-        dense[(size_t)R * n + C] = tile(R, C);
-    GENEO_CUDA_TRY(copy_sync(c, factor, dense.data(), nn * sizeof(double), cudaMemcpyDefault));
+      for (int C = std::max(0, R - half_band); C <= R; ++C) tile(R, C) = dense[(size_t)R * n + C];
+    for (int R = n; R < nt * 32; ++R) tile(R, R) = 1.0;
+    DigitBand D;
+    D.pool = solve ? m.p[0] : m.p[4];
+    D.rexp = (int *)m.p[3];
+    D.dexp = D.rexp + nt * 32;
+    D.npad = nt * 32;
+    D.window = solve ? 0 : window;
+    GENEO_CUDA_TRY(cudaMemcpyAsync(pool, tiles.data(), tiles.size() * sizeof(double),
+                                   cudaMemcpyHostToDevice, s));
+    GENEO_CUDA_TRY(cudaMemcpyAsync(dl, &Ls, sizeof(Ls), cudaMemcpyHostToDevice, s));
+    GENEO_CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(DevStatus), s));
+    if (int st = launch_band_cholesky64(dl, 1, nt, w, pool, nullptr, D, status, s)) return st;
+    if (solve) {
+      GENEO_CUDA_TRY(cudaMemcpyAsync(rhs, b, nb * sizeof(double), cudaMemcpyDefault, s));
+      if (int st = launch_band_solve64(dl, 1, w, D, m.p[6], rhs, 0, ncols, rhs, 0, ncols, ncols,
+                                       mode, s, 0, ctas))
+        return st;
+    }
+    GENEO_CUDA_TRY(copy_sync(c, &h, status, sizeof(h), cudaMemcpyDeviceToHost));
+    if (h.code) return fail(h.code, ("no positive pivot in row " + std::to_string(h.detail)).c_str());
+    if (solve) {
+      GENEO_CUDA_TRY(copy_sync(c, x, rhs, nb * sizeof(double), cudaMemcpyDefault));
+    } else if (factor) {
+      GENEO_CUDA_TRY(copy_sync(c, tiles.data(), pool, tiles.size() * sizeof(double), cudaMemcpyDeviceToHost));
+      std::vector<double> out(nn, 0.0);
+      for (int R = 0; R < n; ++R)
+        for (int C = std::max(0, (R >> 5) - w) * 32; C < std::min(n, ((R >> 5) + 1) * 32); ++C)
+          out[(size_t)R * n + C] = tile(R, C);
+      GENEO_CUDA_TRY(copy_sync(c, factor, out.data(), nn * sizeof(double), cudaMemcpyDefault));
+    }
   }
   return GENEO_OK;
 } catch (const std::exception &) {
@@ -2247,7 +2257,7 @@ extern "C" int geneo_profile(geneo_ctx *c, int what, int reps, double *ms_per_la
                                  (long long)npad * ldv, ldv, pc.T1, (long long)npad * p, p, p, 2, s);
       } else if (what == 4) {
         // re-assemble S_j = A_j - sigma B_j and factor it again (same result)
-        if (!(st = launch_band_clear<double>(pc.d_lay_neu, pc.nsub, pc.neuL, pc.fac_neu_elems, s))) {
+        if (!(st = launch_band_clear<double>(pc.d_lay_neu, pc.nsub, pc.neuL, pc.fac_neu_elems, s, kDigSlot))) {
           launch_neumann_assemble(pc.d_subs, pc.d_lay_neu, pc.nsub, pc.max_nodes_neu, c->nx, c->ny,
                                   c->nz, c->X, c->Y, c->Z, c->Cel, c->perm, pc.d_ecnt, pc.ecnt_off,
                                   c->mask, pc.Xneu, pc.modes.shift, pc.neuL, pc.Bloc, s);

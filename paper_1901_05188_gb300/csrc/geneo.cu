@@ -18,7 +18,7 @@ namespace geneo {
 namespace {
 
 __device__ __forceinline__ double *tile_at(double *pool, const BandLayout &L, int I, int d) {
-  return pool + L.off + (((long long)I * (L.w + 1) + d) << 10);
+  return pool + L.off + ((long long)I * (L.w + 1) + d) * L.slot;
 }
 
 __device__ __forceinline__ int cand_count(const int *c) {

@@ -16,13 +16,17 @@ namespace geneo {
 struct BandLayout {
   int n, nt, w;        // dofs, tile rows, tile half-bandwidth
   long long off;       // element offset of tile (0, 0) in its pool
+  int slot;            // elements from a tile to the next (1024, or kDigSlot)
 };
 
 // Digits of an FP64 band factor (digits.cuh): kDigHalves 16-bit values per tile
-// and two scale exponents per row.  window = 0: the tiles of the whole band, in
-// the order of the FP64 tiles; window > 0: only the w + 1 tile rows the
-// factorisation can still touch, `window` tiles per system.
+// and two scale exponents per row.  window = 0: the whole band, each tile's digits
+// in place of its FP64 values (pool is the matrix's own, in slots of kDigSlot):
+// 14 bytes an entry where FP64 tiles in both orders take 16.  window > 0: beside
+// the FP64 tiles, only the w + 1 tile rows the factorisation can still touch,
+// `window` tiles per system.
 constexpr int kDigHalves = 7 * 1024;
+constexpr int kDigSlot = kDigHalves / 4;
 struct DigitBand {
   void *pool = nullptr;
   int *rexp = nullptr, *dexp = nullptr;   // [system][npad]: rows of L, rows of the inverted diagonal blocks
@@ -64,7 +68,7 @@ struct Precond {
   int pou = 0;                    // partition of unity: GENEO_POU_MULTIPLICITY or _SARKIS
   double *wloc = nullptr;         // Sarkis weights X_j on interior dofs (like xloc), or null
   // GenEO eigenproblem data (FP64)
-  double *neuL = nullptr;         // factor of S = A - sigma B
+  double *neuL = nullptr;         // S = A - sigma B, then the digits of its factor
   DigitBand dig_neu, dig_int, dig_H;   // digits of it, of the FP64 interior factors, of A_H's factor
   void *solve_scr = nullptr;      // scratch of the band solves
   double *Bloc = nullptr;         // 27-slot local BSR of B (9 doubles per block)
@@ -96,7 +100,7 @@ struct Precond {
   double *Zp = nullptr;           // Z_j, row-major n_int x m_j per subdomain
   double *Yp = nullptr;           // A Z_j on Neumann dofs, [nsub] x n_neu x m_j
   double *AH = nullptr, *AHinv = nullptr;   // dense nH x nH
-  double *AHL = nullptr;          // tiles of the coarse factor
+  double *AHL = nullptr;          // tiles of A_H, then the digits of its factor
   double *wpart = nullptr;        // restriction partials [nsub][row blocks][mcap]
   double *wH = nullptr, *yH = nullptr;
   double *zy = nullptr;           // coarse correction Z_j y_j per interior dof [sum n_int]
