@@ -21,7 +21,8 @@ int launch_band_cholesky32(const BandLayout *d_lay, int nsys, int nt_max, int w_
                            float *poolU, DevStatus *st, cudaStream_t s, cudaStream_t side = nullptr);
 
 // FP64 left-looking tile Cholesky on the tensor cores (digits.cuh).  With a
-// window of digits: the same result in poolL and, unless it is null, poolU.
+// window of digits: the same result in poolL and, unless it is null, poolU (D.pool
+// may lie there: poolU is written after the last use of the digits).
 // Without (D.window = 0, D.pool = poolL, layouts with slots of kDigSlot): the
 // factor's digits in place of the matrix, what launch_band_solve64 reads.  With
 // a side stream the two halves of the systems are factored concurrently.

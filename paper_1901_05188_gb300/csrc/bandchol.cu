@@ -168,8 +168,7 @@ struct DiagSmem {
 // entry per thread with three barriers per column and the inverse afterwards
 // took 44 us.
 __device__ __forceinline__ void diag_factor(DiagSmem &Sm, const BandLayout &L, int j, int J,
-                                            double *poolL, double *poolU, const DigitBand &D,
-                                            DevStatus *st) {
+                                            double *poolL, const DigitBand &D, DevStatus *st) {
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
   double *t = tile_ptr(poolL, L, J, 0), *A = Sm.A, *rinv = Sm.rinv;
   double (*colv)[32] = Sm.colv;
@@ -223,10 +222,6 @@ __device__ __forceinline__ void diag_factor(DiagSmem &Sm, const BandLayout &L, i
   diag_bar();
   if (D.window)
     for (int e = tid; e < 1024; e += 128) t[e] = A[(e & 31) * 33 + (e >> 5)];
-  if (poolU) {
-    double *u = tile_ptr(poolU, L, J, 0);
-    for (int e = tid; e < 1024; e += 128) u[e] = A[(e >> 5) * 33 + (e & 31)];
-  }
   const bool fits = slice_rows<true>(A, 8 * w, 8, cs, ex, dg, lane);
   if (!fits) *bad = J * 32;
   diag_bar();
@@ -239,8 +234,7 @@ __device__ __forceinline__ void diag_factor(DiagSmem &Sm, const BandLayout &L, i
 // The first diagonal tile of every system (all of them if no tiles couple); the
 // others are factored by the panel launch before.
 __global__ void __launch_bounds__(128)
-    k_dchol_diag(const BandLayout *lay, int sys0, int J, double *poolL, double *poolU, DigitBand D,
-                 DevStatus *st) {
+    k_dchol_diag(const BandLayout *lay, int sys0, int J, double *poolL, DigitBand D, DevStatus *st) {
   const int j = sys0 + blockIdx.x;
   const BandLayout L = lay[j];
   if (J >= L.nt) return;
@@ -249,7 +243,7 @@ __global__ void __launch_bounds__(128)
   for (int e = threadIdx.x; e < 1024; e += 128) Sm.A[(e & 31) * 33 + (e >> 5)] = t[e];
   if (threadIdx.x == 0) Sm.bad = -1;
   __syncthreads();
-  diag_factor(Sm, L, j, J, poolL, poolU, D, st);
+  diag_factor(Sm, L, j, J, poolL, D, st);
 }
 
 // Panel of tile column J, left-looking.  blockIdx.y = 2 + p takes the tiles (I, J),
@@ -271,8 +265,7 @@ constexpr int kPanStages = 2;
 constexpr int kPanSmem = (3 * kPanStages + 1) * (int)kDigBytes;
 
 __global__ void __launch_bounds__(256, 2)
-    k_dchol_panel(const BandLayout *lay, int sys0, int J, double *poolL, double *poolU, DigitBand D,
-                  DevStatus *st) {
+    k_dchol_panel(const BandLayout *lay, int sys0, int J, double *poolL, DigitBand D, DevStatus *st) {
   const int j = sys0 + blockIdx.x;
   const BandLayout L = lay[j];
   if (J + 1 >= L.nt) return;
@@ -359,14 +352,11 @@ __global__ void __launch_bounds__(256, 2)
       uint4 *dst = reinterpret_cast<uint4 *>(dig_tile(D, L, j, I, 1));
       const uint4 *src = reinterpret_cast<const uint4 *>(dg);
       for (int e = tid; e < kDigTile / 8; e += 256) dst[e] = src[e];
-      double *tu = poolU ? tile_ptr(poolU, L, J, 1) : nullptr;
-      for (int e = tid; e < 1024; e += 256) {
-        if (D.window) tr[e] = R[(e & 31) * 33 + (e >> 5)];
-        if (tu) tu[e] = R[(e >> 5) * 33 + (e & 31)];
-      }
+      if (D.window)
+        for (int e = tid; e < 1024; e += 256) tr[e] = R[(e & 31) * 33 + (e >> 5)];
       __syncthreads();
     }
-    if (warp < 4) diag_factor(Sm, L, j, I, poolL, poolU, D, st);
+    if (warp < 4) diag_factor(Sm, L, j, I, poolL, D, st);
     return;
   }
   auto prefetch = [&](int it) {
@@ -447,10 +437,6 @@ __global__ void __launch_bounds__(256, 2)
       double *tl = tile_ptr(poolL, L, I, I - J);
       if (D.window)
         for (int e = t4; e < 1024; e += 128) tl[e] = Rt[(e & 31) * 33 + (e >> 5)];
-      if (poolU) {
-        double *tu = tile_ptr(poolU, L, J, I - J);
-        for (int e = t4; e < 1024; e += 128) tu[e] = Rt[(e >> 5) * 33 + (e & 31)];
-      }
       fits = slice_rows<false>(Rt, 8 * (warp & 3), 8, 0, rexp_s + 32 * tt, dg + tt * kDigTile, lane) && fits;
       if (!fits) not_spd(st, j, J * 32);
     }
@@ -461,6 +447,22 @@ __global__ void __launch_bounds__(256, 2)
       for (int e = tid & 127; e < kDigTile / 8; e += 128) dst[e] = src[e];
     }
   }
+}
+
+// The backward tile stream: U(J, d) = L(J + d, J)^T, one block per tile.  A pass of
+// its own after the factorisation (which then never reads poolU), so that the
+// digit windows can lie in poolU until here.
+__global__ void __launch_bounds__(256)
+    k_band_transpose(const BandLayout *lay, int w_max, const double *poolL, double *poolU) {
+  const BandLayout L = lay[blockIdx.y];
+  const int J = blockIdx.x / (w_max + 1), d = blockIdx.x - J * (w_max + 1);
+  if (J >= L.nt || d > L.w || J + d >= L.nt) return;
+  __shared__ double t[32][33];
+  const double *l = poolL + L.off + ((long long)(J + d) * (L.w + 1) + d) * L.slot;
+  double *u = tile_ptr(poolU, L, J, d);
+  for (int e = threadIdx.x; e < 1024; e += 256) t[e >> 5][e & 31] = l[e];
+  __syncthreads();
+  for (int e = threadIdx.x; e < 1024; e += 256) u[e] = t[e & 31][e >> 5];
 }
 
 // ---- band solves with up to eight right-hand sides per cluster -----------------
@@ -933,17 +935,21 @@ int launch_band_cholesky64(const BandLayout *d_lay, int nsys, int nt_max, int w_
       cudaStream_t q = h ? side : s;
       if (J < 0) {
         k_row_exps<<<dim3((nt_max * 32 + 255) / 256, n), 256, 0, q>>>(d_lay, j0, poolL, D); GENEO_COUNT_LAUNCH();
-        k_dchol_diag<<<n, 128, 0, q>>>(d_lay, j0, 0, poolL, poolU, D, st); GENEO_COUNT_LAUNCH();
+        k_dchol_diag<<<n, 128, 0, q>>>(d_lay, j0, 0, poolL, D, st); GENEO_COUNT_LAUNCH();
       } else if (w_max == 0) {
-        k_dchol_diag<<<n, 128, 0, q>>>(d_lay, j0, J + 1, poolL, poolU, D, st); GENEO_COUNT_LAUNCH();
+        k_dchol_diag<<<n, 128, 0, q>>>(d_lay, j0, J + 1, poolL, D, st); GENEO_COUNT_LAUNCH();
       } else {
         const int d = std::min(w_max, nt_max - 1 - J);      // tiles (J + 2 .. J + d, J) in pairs
-        k_dchol_panel<<<dim3(n, d / 2 + 2), 256, kPanSmem, q>>>(d_lay, j0, J, poolL, poolU, D, st); GENEO_COUNT_LAUNCH();
+        k_dchol_panel<<<dim3(n, d / 2 + 2), 256, kPanSmem, q>>>(d_lay, j0, J, poolL, D, st); GENEO_COUNT_LAUNCH();
       }
     }
   if (half < nsys) {
     GENEO_CUDA_TRY(cudaEventRecord(ev.join, side));
     GENEO_CUDA_TRY(cudaStreamWaitEvent(s, ev.join, 0));
+  }
+  if (poolU) {
+    const dim3 g((unsigned)(nt_max * (w_max + 1)), nsys);
+    k_band_transpose<<<g, 256, 0, s>>>(d_lay, w_max, poolL, poolU); GENEO_COUNT_LAUNCH();
   }
   GENEO_CUDA_TRY(cudaGetLastError());
   return GENEO_OK;

@@ -74,6 +74,9 @@ cudaError_t copy_sync(const geneo_ctx *c, void *dst, const void *src, size_t byt
 constexpr int kHistCap = 20000;
 constexpr int kGraphIters = 8;
 constexpr int kDotChunks = 8;
+// Columns of A_H^-1 solved for in one launch, eight per SM: the sweeps keep a
+// window of digits for every eight columns, 14 bytes per entry of A_H in all.
+constexpr int kInverseCols = 8 * (kRedBlocks / 2);
 
 int fail(int code, const char *msg) {
   g_last_error = msg;
@@ -732,10 +735,12 @@ void take_cg_vectors(Arena &A, geneo_ctx *c) {
   c->cg = A.take<CGScalars>(1);
 }
 
-// Digits in place of the tiles in `pool`, or in windows of their own.
-DigitBand take_digits(Arena &A, int nsys, int npad, double *pool, long long window) {
+// Digits in place of the tiles in `pool` (window = 0), or in windows that lie in
+// `pool` if its `bytes` hold them, else in memory of their own.
+DigitBand take_digits(Arena &A, int nsys, int npad, void *pool, long long window, size_t bytes) {
   DigitBand D;
-  D.pool = window ? (void *)A.take<uint16_t>((size_t)nsys * window * kDigHalves) : pool;
+  const size_t need = (size_t)nsys * window * kDigHalves * 2;
+  D.pool = need <= bytes ? pool : A.take<uint16_t>(need / 2);
   D.rexp = A.take<int>((size_t)nsys * npad);
   D.dexp = A.take<int>((size_t)nsys * npad);
   D.npad = npad;
@@ -764,7 +769,7 @@ void plan_setup(Arena &A, geneo_ctx *c, const SetupPlan &P) {
   pc.yloc = A.take<char>(pc.xloc_elems * esz);   // forward-sweep scratch of the ring form
   pc.wloc = A.take<double>(pc.xloc_elems);     // Sarkis weights (filled for that PoU only)
   const long long win = (long long)(pc.w_int_max + 1) * (pc.w_int_max + 1);
-  pc.dig_int = f32 ? DigitBand{} : take_digits(A, nsub, pc.npad_int_max, nullptr, win);
+  pc.dig_int = f32 ? DigitBand{} : take_digits(A, nsub, pc.npad_int_max, pc.facU, win, pc.fac_int_elems * esz);
   int cap = pc.modes.fixed_modes > 0 ? pc.modes.fixed_modes : pc.modes.max_modes;
   if (pc.coarse == GENEO_COARSE_NONE) cap = 0;
   if (pc.coarse == GENEO_COARSE_ZEM) cap = 6;     // the rigid displacements
@@ -780,7 +785,7 @@ void plan_setup(Arena &A, geneo_ctx *c, const SetupPlan &P) {
     pc.gate = nullptr;
     if (eig) {   // shift-invert block Lanczos of the GenEO eigenproblems
       pc.neuL = A.take<double>(pc.fac_neu_elems);
-      pc.dig_neu = take_digits(A, nsub, npad, pc.neuL, 0);
+      pc.dig_neu = take_digits(A, nsub, npad, pc.neuL, 0, 0);
       pc.Bloc = A.take<double>((size_t)c->nc * c->nc * pc.bloc_blocks);
       pc.V = A.take<double>((size_t)nsub * npad * (pc.kdim + p));
       pc.Vt = A.take<double>((size_t)nsub * npad * pc.kkeep);
@@ -815,8 +820,8 @@ void plan_setup(Arena &A, geneo_ctx *c, const SetupPlan &P) {
     pc.AH = A.take<double>((size_t)pc.nH_cap * pc.nH_cap);
     pc.AHinv = A.take<double>((size_t)pc.nH_cap * pc.nH_cap);
     pc.AHL = A.take<double>((size_t)ntH * ntH * kDigSlot);
-    pc.dig_H = take_digits(A, 1, ntH * 32, pc.AHL, 0);
-    size_t scr = band_solve_scratch(1, ntH - 1, pc.nH_cap);
+    pc.dig_H = take_digits(A, 1, ntH * 32, pc.AHL, 0, 0);
+    size_t scr = band_solve_scratch(1, ntH - 1, std::min(pc.nH_cap, kInverseCols));
     if (eig) scr = std::max(scr, band_solve_scratch(nsub, pc.w_neu_max, std::max(pc.mcap, p)));
     pc.solve_scr = A.take<char>(scr);
     pc.wpart = A.take<double>((size_t)nsub * restrict_chunks(P.max_nint) * pc.mcap);
@@ -1262,9 +1267,12 @@ static int build_coarse_operator(geneo_ctx *c, SetupPlan &P, const std::vector<l
   if ((st = launch_band_cholesky64(pc.d_lay_H, 1, LH.nt, LH.w, pc.AHL, nullptr, pc.dig_H, c->status, s)))
     return st;
   launch_identity(pc.AHinv, nH, s);
-  if ((st = launch_band_solve64(pc.d_lay_H, 1, LH.w, pc.dig_H, pc.solve_scr, pc.AHinv, 0, nH, pc.AHinv,
-                                0, nH, nH, 3, s)))
-    return st;
+  for (int c0 = 0; c0 < nH; c0 += kInverseCols) {
+    double *cols = pc.AHinv + c0;
+    if ((st = launch_band_solve64(pc.d_lay_H, 1, LH.w, pc.dig_H, pc.solve_scr, cols, 0, nH, cols, 0, nH,
+                                  std::min(kInverseCols, nH - c0), 3, s)))
+      return st;
+  }
   launch_symmetrize(pc.AHinv, nH, s);
   GENEO_CUDA_TRY(cudaGetLastError());
   return GENEO_OK;

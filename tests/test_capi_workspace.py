@@ -13,9 +13,9 @@ from workloads.darcy import darcy_config
 
 # (workload, precision): bytes
 BOUND = {("tiny", 1): 2108248, ("small", 0): 35519832, ("small", 1): 32152408,
-         ("c1", 1): 32262488, ("c2", 0): 4139346776, ("c2", 1): 3500547416,
-         ("c3", 0): 50488090200, ("c3", 1): 41593012824, ("d-small", 1): 16745560,
-         ("d-large", 0): 1934177368, ("d-large", 1): 1496039512,
+         ("c1", 0): 35432280, ("c1", 1): 32262488, ("c2", 0): 4139346776, ("c2", 1): 3500547416,
+         ("c3", 0): 50488090200, ("c3", 1): 41593012824, ("d-small", 0): 19386968,
+         ("d-small", 1): 16745560, ("d-large", 0): 1934177368, ("d-large", 1): 1496039512,
          ("d-spe10", 0): 15355705176, ("d-spe10", 1): 13185552216}
 
 
