@@ -180,3 +180,22 @@ def test_small_and_large_matrices(ctx, n, hb, power):
         x0 = _solve(ctx, M, hb, b, mode)
         x = _solve(ctx, M * s * s, hb, b if mode < 3 else b * s, mode) * back
         assert np.max(np.abs(x - x0)) <= 100 * U * np.abs(x0).max(), mode
+
+
+def test_more_tiles_than_one_sum_of_level_sums_holds(ctx):
+    """A full matrix of 264 tile rows: with one CTA a warp adds up to 65 tiles of
+    a row, one more than its 32-bit sums hold; with two CTAs 33.
+
+    A = 2 I + V V^T with ||V V^T|| = 2 (condition number at most 2) has the inverse
+    (I - V (2 I + V^T V)^-1 V^T) / 2; bound as above.
+    """
+    n = 264 * 32 - 5
+    rng = np.random.default_rng(8)
+    V = np.linalg.qr(rng.normal(size=(n, 4)))[0] * np.sqrt([2.0, 1.5, 1.0, 0.5])
+    A = V @ V.T
+    A[np.arange(n), np.arange(n)] += 2.0
+    b = rng.normal(size=(n, 3))
+    ref = 0.5 * (b - V @ np.linalg.solve(2.0 * np.eye(4) + V.T @ V, V.T @ b))
+    one = _solve(ctx, A, n, b, 3, 1)
+    assert np.linalg.norm(one - ref) <= 24 * n * U * np.linalg.norm(ref)
+    assert np.max(np.abs(one - _solve(ctx, A, n, b, 3, 2))) <= 8 * U * np.abs(one).max()
