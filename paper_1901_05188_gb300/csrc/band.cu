@@ -67,9 +67,9 @@ __global__ void __launch_bounds__(1024) k_chol_diag(const BandLayout *lay, int n
   for (int k = 0; k < 32; ++k) {
     if (tid == 0) {
       float d = A[k][k];
-      if (!(d > float(0))) {
+      if (!(d > 0.f)) {
         if (bad < 0) bad = J * 32 + k;
-        d = float(1);
+        d = 1.f;
       }
       const float y = inv_sqrt_pos(d);
       piv[0] = d * y;          // sqrt(d)
@@ -83,20 +83,20 @@ __global__ void __launch_bounds__(1024) k_chol_diag(const BandLayout *lay, int n
   }
   // inverse of the lower-triangular factor by recursive doubling:
   // inv([[P, 0], [Q, R]]) = [[iP, 0], [-iR Q iP, iR]]
-  X[r][cc] = (r == cc) ? float(1) / A[r][r] : float(0);
+  X[r][cc] = (r == cc) ? 1.f / A[r][r] : 0.f;
   __syncthreads();
   for (int b = 1; b < 32; b <<= 1) {
     // pairs of b x b diagonal blocks at s and s + b, s = multiple of 2b
     const int s = (r / (2 * b)) * (2 * b);
     const bool lower = (r >= s + b) && (cc >= s) && (cc < s + b);   // block (R-row, P-col)
-    float v = float(0);
+    float v = 0.f;
     if (lower) {   // Y = Q iP  (Q = A[s+b.., s..s+b), iP = X[s.., s..])
       for (int k = cc; k < s + b; ++k) v += A[r][k] * X[k][cc];
     }
     Y[r][cc] = v;
     __syncthreads();
     if (lower) {   // X_lower = -iR Y
-      float w = float(0);
+      float w = 0.f;
       for (int k = s + b; k <= r; ++k) w += X[r][k] * Y[k][cc];
       X[r][cc] = -w;
     }
@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(1024) k_chol_diag(const BandLayout *lay, int n
   }
 }
 
-// L(J+d, J) = A(J+d, J) inv(L_JJ)^float for d = 1..w (blockIdx.y = d - 1).
+// L(J+d, J) = A(J+d, J) inv(L_JJ)^T for d = 1..w (blockIdx.y = d - 1).
 __global__ void __launch_bounds__(256) k_chol_trsm(const BandLayout *lay, int nsys, int J,
                                                    float *poolL, float *poolU) {
   int j = blockIdx.x, d = blockIdx.y + 1;
@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(256) k_chol_trsm(const BandLayout *lay, int ns
   float *tu = tile_ptr(poolU, L, J, d);
   for (int e = threadIdx.x; e < 1024; e += 256) {
     int r = e & 31, c = e >> 5;
-    float s = float(0);
+    float s = 0.f;
     for (int k = 0; k <= c; ++k) s += Aa[r][k] * D[c][k];
     ta[e] = s;                 // (r, c) column-major
     tu[r * 32 + c] = s;        // transposed: U(J, d)(c, r) = L(J+d, J)(r, c)
@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(256) k_chol_update(const BandLayout *lay, int 
   float *tc = tile_ptr(poolL, L, J + d1, d1 - d2);
   for (int e = threadIdx.x; e < 1024; e += 256) {
     int r = e & 31, c = e >> 5;
-    float s = float(0);
+    float s = 0.f;
 #pragma unroll 8
     for (int k = 0; k < 32; ++k) s += Aa[r][k] * Bb[c][k];
     tc[e] -= s;

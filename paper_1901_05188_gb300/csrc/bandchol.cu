@@ -491,7 +491,7 @@ __global__ void __launch_bounds__(256)
 // buffer (integers: the result depends on the cluster only through the bits
 // dropped when sums of different scales are aligned, below 2^-57 of the
 // largest), and one cluster barrier ends the row.
-// Bound: the larger of the chain (six barriers and two products, about 3 us a
+// Bound: the larger of the chain (four barriers and two products, about 3 us a
 // row) and a CTA's share of the tiles, where issuing the copies counts for as
 // much as the matrix instructions.  Per launch of half the subdomains (forward
 // or backward, eight right-hand sides): 36 of 14,500
@@ -954,6 +954,12 @@ int launch_band_cholesky64(const BandLayout *d_lay, int nsys, int nt_max, int w_
   GENEO_CUDA_TRY(cudaGetLastError());
   return GENEO_OK;
 }
+
+// Widest half-bandwidth the set-up takes, in tiles: a vector's window of FP64 tile
+// rows filled shared memory there.  This kernel fits up to 1,650.
+constexpr int kSwMaxBand = 872;
+static_assert(sweep_smem(kSwMaxBand, 1) <= 227 * 1024, "every accepted band has a launch");
+bool band_solve_fits(int w_max) { return w_max <= kSwMaxBand; }
 
 size_t band_solve_scratch(int nsys, int w_max, int ncols) {
   return (size_t)nsys * ((ncols + 7) / 8) * (w_max + 2) * kSwY * 4;

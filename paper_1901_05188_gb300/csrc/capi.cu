@@ -948,7 +948,7 @@ static int setup_coarse_zem(geneo_ctx *c, SetupPlan &P, cudaStream_t s) {
   launch_pou_neumann(pc.d_subs, nsub, P.max_nodes_neu, pc.d_cand, pc.cand_off, c->mask, nnx, nny,
                      c->nz + 1, pc.part.px, pc.part.py, pc.pou, pc.Xneu, s);
   launch_rigid_modes(pc.d_subs, nsub, npad, c->X, c->Y, c->Z, pc.P, mcap, sP, s);
-  launch_tsdots(pc.d_subs, nsub, npad, pc.P, mcap, sP, mcap, pc.P, mcap, sP, mcap, pc.Hpart,
+  launch_tsdots(pc.d_subs, nsub, pc.P, mcap, sP, mcap, pc.P, mcap, sP, mcap, pc.Hpart,
                 kDotChunks, pc.G, (long long)mcap * mcap, s);
   launch_normalize_cols(pc.d_subs, nsub, npad, pc.P, mcap, sP, mcap, pc.G, s);
   GENEO_CUDA_TRY(cudaGetLastError());
@@ -1015,7 +1015,7 @@ static int setup_coarse(geneo_ctx *c, SetupPlan &P, cudaStream_t s) {
   launch_random_block(pc.d_subs, nsub, npad, pc.W, p, sW, p, 0x5eed1234ull, s);
   double *const Rinv = pc.Racc + (long long)nsub * p * p;   // second half of Racc's buffer
   for (int pass = 0; pass < 2; ++pass) {
-    launch_tsdots(pc.d_subs, nsub, npad, pc.W, p, sW, p, pc.W, p, sW, p, pc.Hpart, kDotChunks,
+    launch_tsdots(pc.d_subs, nsub, pc.W, p, sW, p, pc.W, p, sW, p, pc.Hpart, kDotChunks,
                   pc.G, (long long)p * p, s);
     launch_cholqr(pc.d_subs, nsub, npad, pc.G, pc.W, p, pc.Racc, Rinv, pass == 0, 0.0, s);
   }
@@ -1076,18 +1076,18 @@ static int setup_coarse(geneo_ctx *c, SetupPlan &P, cudaStream_t s) {
     for (int pass = 0; pass < 2; ++pass) {
       const int *gt = pass == 0 ? nullptr : gate;
       if (pass == 1) {
-        launch_tsdots(subs, n, npad, W, p, sW, p, W, p, sW, p, Hpart, kDotChunks, G,
+        launch_tsdots(subs, n, W, p, sW, p, W, p, sW, p, Hpart, kDotChunks, G,
                       (long long)p * p, gs);
         launch_reorth_gate(n, G, p, Hs, na, (long long)na * p, gate, gs);
       }
-      launch_tsdots(subs, n, npad, V, ldv, sV, na, W, p, sW, p, Hpart, kDotChunks, Hs,
+      launch_tsdots(subs, n, V, ldv, sV, na, W, p, sW, p, Hpart, kDotChunks, Hs,
                     (long long)na * p, gs, gt);
       launch_hm_accum(n, Hm, kdim, Hs, na, k, p, gs);
       launch_tsgemm(subs, n, npad, V, ldv, sV, na, Hs, p, (long long)na * p, W, p, sW, p, -1.0,
                     1.0, gs, gt);
     }
     for (int pass = 0; pass < 2; ++pass) {
-      launch_tsdots(subs, n, npad, W, p, sW, p, W, p, sW, p, Hpart, kDotChunks, G,
+      launch_tsdots(subs, n, W, p, sW, p, W, p, sW, p, Hpart, kDotChunks, G,
                     (long long)p * p, gs);
       launch_cholqr(subs, n, npad, G, W, p, Racc, Ri, pass == 0, abs_tiny, gs);
     }
@@ -1170,7 +1170,7 @@ static int setup_coarse(geneo_ctx *c, SetupPlan &P, cudaStream_t s) {
   if ((st = launch_band_solve64(pc.d_lay_neu, nsub, pc.w_neu_max, pc.dig_neu, pc.solve_scr, pc.P, sP,
                                 mcap, pc.P, sP, mcap, mcap, 2, s)))
     return st;
-  launch_tsdots(pc.d_subs, nsub, npad, pc.P, mcap, sP, mcap, pc.P, mcap, sP, mcap, pc.Hpart,
+  launch_tsdots(pc.d_subs, nsub, pc.P, mcap, sP, mcap, pc.P, mcap, sP, mcap, pc.Hpart,
                 kDotChunks, pc.G, (long long)mcap * mcap, s);
   launch_normalize_cols(pc.d_subs, nsub, npad, pc.P, mcap, sP, mcap, pc.G, s);
   GENEO_CUDA_TRY(cudaGetLastError());

@@ -62,12 +62,7 @@ constexpr long long kDigBias = (1LL << 8) | (1LL << 17) | (1LL << 26) | (1LL << 
 __device__ __forceinline__ uint32_t digit_bits(long long xb, int s) {
   return s == 0 ? (uint32_t)((int)(xb >> 54) + 256) : (uint32_t)(xb >> (9 * (6 - s))) & 511u;
 }
-// 0x6400 | f is the half 1024 + f, exact for f < 1024.
-__device__ __forceinline__ uint32_t digit_pair(long long xb0, long long xb1, int s) {
-  const uint32_t h = 0x64006400u | digit_bits(xb0, s) | (digit_bits(xb1, s) << 16);
-  const __half2 r = __hsub2(*reinterpret_cast<const __half2 *>(&h), __half2half2(__ushort_as_half(0x6500)));
-  return *reinterpret_cast<const uint32_t *>(&r);   // 0x6500 = 1280
-}
+// 0x6400 | f is the half 1024 + f, exact for f < 1024; 0x6500 = 1280.
 __device__ __forceinline__ __half digit_half(long long xb, int s) {
   return __hsub(__ushort_as_half((unsigned short)(0x6400u | digit_bits(xb, s))), __ushort_as_half(0x6500));
 }

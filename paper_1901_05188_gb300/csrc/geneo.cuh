@@ -43,9 +43,9 @@ void launch_random_block(const SubDesc *d_subs, int nsub, int npad, double *V, i
 // pass, H the removed coefficients, na x p per system with stride hs).
 void launch_reorth_gate(int nsub, const double *G, int p, const double *H, int na, long long hs,
                         int *gate, cudaStream_t s);
-void launch_tsdots(const SubDesc *d_subs, int nsub, int npad, const double *A, int lda,
-                   long long sa, int na, const double *B, int ldb, long long sb, int nb,
-                   double *Hpart, int chunks, double *H, long long hs, cudaStream_t s,
+void launch_tsdots(const SubDesc *d_subs, int nsub, const double *A, int lda, long long sa,
+                   int na, const double *B, int ldb, long long sb, int nb, double *Hpart,
+                   int chunks, double *H, long long hs, cudaStream_t s,
                    const int *gate = nullptr);
 
 // C_j = beta C_j + alpha A_j H_j (rows < n_neu).

@@ -541,7 +541,7 @@ static unsigned row_grid(int n, int most) { return std::max(1, std::min(most, (n
 // At most eight warps of rows per SM: latency, not the loads in flight, decides
 // (nine blocks together against one: 6,591 rows 9.5 and 15.5 us, 36,501 rows 9.7
 // and 16.3 us; above, 64 warps per SM of the other form keep more in flight).
-static bool few_rows(int n) { return n <= 152 * 8 * 32; }
+static bool few_rows(int n) { return n <= kRedBlocks / 2 * 8 * 32; }   // kRedBlocks: two per SM
 
 void launch_spmv(const BSR &A, const double *x, double *y, cudaStream_t s) {
   const int n = A.nc * A.nnode;

@@ -1596,8 +1596,6 @@ int launch_schwarz_solve(const SubDesc *d_subs, const BandLayout *d_lay, int nsu
   }
 }
 
-bool band_solve_fits(int w_max) { return smem_bytes_ring<double>(w_max) <= kSmemMax; }
-
 // ---- batch launchers -----------------------------------------------------------
 constexpr long long kBatchSmemMax = kSmemMax - 16;   // beside the item index, in static memory
 

@@ -6,8 +6,12 @@
 // a clock and SM.  Cutting an entry into digits costs about sixty integer
 // instructions once and serves all its products, so the digits are made on the
 // way, from the FP64 arrays, and nothing else changes hands.  Integer sums are
-// exact; a product is rounded once per chunk of rows (k_tsdots) or entry
-// (k_tsgemm), so the results are closer than FP64 sums.
+// exact.  Lost are what the entries have below 2^-60 of the largest of their
+// column (k_tsdots) or row of A and column of H (k_tsgemm), the levels left out,
+// as much again, and one FP64 rounding per entry, chunk of rows, 256 tiles and
+// growth of a column's scale: over n terms 3 n 2^-60 of the product of the largest
+// entries.  An FP64 sum errs by up to n 2^-53 of the sum of |v w|, which is less only
+// where that sum is below 3/128 of the product of the largest.
 //
 // Half of 108 subdomains of 16,000 unknowns: V^T W of 64 columns 0.54 ms, W^T W
 // 0.08 ms, V H of 64 columns 0.45 ms, on the FP64 pipe 0.76 ms (all sizes of V
@@ -23,7 +27,6 @@ namespace geneo {
 namespace {
 
 constexpr int kTsThreads = 256, kTsRows = 32;
-constexpr int kTsCols = 128;                // most columns of V
 constexpr int kTsFlush = 256;               // tiles summed in 32 bits: 256 * 7 * 2^20 < 2^31
 
 // Digits of one entry, at element (r, c) of 32 x 32 tile `dst`.
@@ -46,6 +49,7 @@ __device__ __forceinline__ void ts_b(uint32_t (&b)[4], uint32_t tile, int n0, in
 // too large; only when a column outgrows its scale are the sums so far turned
 // into FP64.  A warp owns one of the 16 x 8 blocks of H and half of the 32
 // rows, as 32-bit level sums.
+// NCG: 32-column groups of V, four at most (kMaxKdim).
 template <int NCG>
 __host__ __device__ constexpr int tsdots_smem() {
   return (NCG + 1) * (int)kDigBytes + 2 * 1024 * 8 + 2 * (32 * NCG + 32) * 4;
@@ -409,11 +413,10 @@ __global__ void __launch_bounds__(kTsThreads, 2)
 
 }  // namespace
 
-void launch_tsdots(const SubDesc *d_subs, int nsub, int npad, const double *A, int lda,
-                   long long sa, int na, const double *B, int ldb, long long sb, int nb,
-                   double *Hpart, int chunks, double *H, long long hs, cudaStream_t s,
+void launch_tsdots(const SubDesc *d_subs, int nsub, const double *A, int lda, long long sa,
+                   int na, const double *B, int ldb, long long sb, int nb, double *Hpart,
+                   int chunks, double *H, long long hs, cudaStream_t s,
                    const int *gate) {
-  (void)npad;
   // One warp for each half of a 16 x 8 block of H, sixteen at most: all 32
   // columns a CTA can stage for up to 32 of A, 16 for up to 64, else eight.
   const int width = na <= 32 ? 32 : na <= 64 ? 16 : 8, groups = (nb + width - 1) / width;
